@@ -63,6 +63,12 @@ def load_library(path: Optional[str] = None):
     lib.osdn_residual_ratio.argtypes = [pp] + [vp] * 7 + [vp]
     lib.osdn_decode_step.restype = ci
     lib.osdn_decode_step.argtypes = [pp] + [vp] * 9 + [vp]
+    lib.osdn_kda_workspace_bytes.restype = sz
+    lib.osdn_kda_workspace_bytes.argtypes = [pp, ci]
+    lib.osdn_kda_fwd.restype = ci
+    lib.osdn_kda_fwd.argtypes = [pp] + [vp] * 11 + [vp, sz, vp]
+    lib.osdn_kda_bwd.restype = ci
+    lib.osdn_kda_bwd.argtypes = [pp] + [vp] * 19 + [vp, sz, vp]
     lib.osdn_step_host.restype = ci
     lib.osdn_step_host.argtypes = [pp] + [vp] * 12 + [vp, sz, vp]
     lib.osdn_read_device_status.restype = ci
@@ -86,6 +92,24 @@ def load_library(path: Optional[str] = None):
     return lib
 
 
+# The hot calls go through the extension module _osdn_call (csrc/call.cpp), which turns tensors into pointers
+# natively; the numbers are its table of calls.
+_FWD, _BWD, _KDA_FWD, _KDA_BWD, _PRECOND, _RATIO, _DECODE, _FWD_STATIC = range(8)
+
+
+def _call(*args) -> int:
+    """Loads the extension on the first call and takes its entry point's place."""
+    global _call
+    load_library()
+    try:
+        from ._osdn_call import call
+    except ImportError as e:
+        raise RuntimeError("the extension module _osdn_call is missing or does not load: build it first "
+                           "(python paper_2605_13473_b200/build.py); there is no fallback path") from e
+    _call = call
+    return call(*args)
+
+
 def status_string(code: int) -> str:
     return load_library().osdn_status_string(code).decode()
 
@@ -100,11 +124,12 @@ def _ptr(t: Optional[torch.Tensor]):
         return None
     if not t.is_contiguous():
         raise ValueError("tensors passed to the OSDN library must be contiguous")
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def _stream_ptr():
-    return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    # the handle itself: building a torch.cuda.Stream object costs more than the rest of a small call
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def make_params(*, B: int, T: int, H: int, K: int, V: int, io_dtype: str, hyper=None,
@@ -178,40 +203,28 @@ def osdn_read_device_status(workspace: torch.Tensor) -> int:
 
 def osdn_fwd(p: OsdnParams, q, k, v, beta, gate, apf_log_ret, init_state, precond_in, out, final_state,
              precond_out, workspace: torch.Tensor):
-    lib = load_library()
-    rc = lib.osdn_fwd(ctypes.byref(p), _ptr(q), _ptr(k), _ptr(v), _ptr(beta), _ptr(gate), _ptr(apf_log_ret),
-                      _ptr(init_state), _ptr(precond_in), _ptr(out), _ptr(final_state), _ptr(precond_out),
-                      _ptr(workspace), ctypes.c_size_t(workspace.numel() * workspace.element_size()),
-                      _stream_ptr())
+    rc = _call(_FWD, p, q, k, v, beta, gate, apf_log_ret, init_state, precond_in, out, final_state, precond_out,
+               workspace)
     _check(rc, "osdn_fwd")
 
 
 def osdn_kda_workspace_bytes(p: OsdnParams, need_bwd: bool) -> int:
-    lib = load_library()
-    lib.osdn_kda_workspace_bytes.restype = ctypes.c_size_t
-    return int(lib.osdn_kda_workspace_bytes(ctypes.byref(p), ctypes.c_int(1 if need_bwd else 0)))
+    return int(load_library().osdn_kda_workspace_bytes(ctypes.byref(p), int(need_bwd)))
 
 
 def osdn_kda_fwd(p: OsdnParams, q, k, v, beta, gate_k, apf_log_ret, init_state, precond_in, out, final_state,
                  precond_out, workspace: torch.Tensor):
     """Channel-gate variant (OSKDA extension): ``gate_k`` is [T,H,K] fp32; the rest as for ``osdn_fwd``."""
-    lib = load_library()
-    rc = lib.osdn_kda_fwd(ctypes.byref(p), _ptr(q), _ptr(k), _ptr(v), _ptr(beta), _ptr(gate_k), _ptr(apf_log_ret),
-                          _ptr(init_state), _ptr(precond_in), _ptr(out), _ptr(final_state), _ptr(precond_out),
-                          _ptr(workspace), ctypes.c_size_t(workspace.numel() * workspace.element_size()),
-                          _stream_ptr())
+    rc = _call(_KDA_FWD, p, q, k, v, beta, gate_k, apf_log_ret, init_state, precond_in, out, final_state, precond_out,
+               workspace)
     _check(rc, "osdn_kda_fwd")
 
 
 def osdn_kda_bwd(p: OsdnParams, q, k, v, beta, gate_k, apf_log_ret, init_state, precond_in, dout, dfinal_state,
                  dprecond_out, dq, dk, dv, dbeta, dgate_k, dapf_log_ret, dinit_state, dprecond_in,
                  workspace: torch.Tensor):
-    lib = load_library()
-    rc = lib.osdn_kda_bwd(ctypes.byref(p), _ptr(q), _ptr(k), _ptr(v), _ptr(beta), _ptr(gate_k), _ptr(apf_log_ret),
-                          _ptr(init_state), _ptr(precond_in), _ptr(dout), _ptr(dfinal_state), _ptr(dprecond_out),
-                          _ptr(dq), _ptr(dk), _ptr(dv), _ptr(dbeta), _ptr(dgate_k), _ptr(dapf_log_ret),
-                          _ptr(dinit_state), _ptr(dprecond_in), _ptr(workspace),
-                          ctypes.c_size_t(workspace.numel() * workspace.element_size()), _stream_ptr())
+    rc = _call(_KDA_BWD, p, q, k, v, beta, gate_k, apf_log_ret, init_state, precond_in, dout, dfinal_state,
+               dprecond_out, dq, dk, dv, dbeta, dgate_k, dapf_log_ret, dinit_state, dprecond_in, workspace)
     _check(rc, "osdn_kda_bwd")
 
 
@@ -223,10 +236,8 @@ def osdn_fwd_static(p: OsdnParams, q, k, v, beta, gate, apf_log_ret, init_state,
     """Forward pass on the library's built-in scratch array: for callers that cannot allocate a
     workspace.  Returns the status code (0 = ok, -6 = the problem does not fit the built-in scratch)
     instead of raising, so that a caller can fall back to ``osdn_fwd`` with its own workspace."""
-    lib = load_library()
-    return int(lib.osdn_fwd_static(ctypes.byref(p), _ptr(q), _ptr(k), _ptr(v), _ptr(beta), _ptr(gate),
-                                   _ptr(apf_log_ret), _ptr(init_state), _ptr(precond_in), _ptr(out),
-                                   _ptr(final_state), _ptr(precond_out), _stream_ptr()))
+    rc = _call(_FWD_STATIC, p, q, k, v, beta, gate, apf_log_ret, init_state, precond_in, out, final_state, precond_out)
+    return rc
 
 
 def osdn_read_static_status() -> int:
@@ -248,34 +259,24 @@ def osdn_selftest_wait_timeout(workspace: torch.Tensor, limit_us: int) -> None:
 def osdn_bwd(p: OsdnParams, q, k, v, beta, gate, apf_log_ret, init_state, precond_in, dout, dfinal_state,
              dprecond_out, dq, dk, dv, dbeta, dgate, dapf_log_ret, dinit_state, dprecond_in,
              workspace: torch.Tensor):
-    lib = load_library()
-    rc = lib.osdn_bwd(ctypes.byref(p), _ptr(q), _ptr(k), _ptr(v), _ptr(beta), _ptr(gate), _ptr(apf_log_ret),
-                      _ptr(init_state), _ptr(precond_in), _ptr(dout), _ptr(dfinal_state), _ptr(dprecond_out),
-                      _ptr(dq), _ptr(dk), _ptr(dv), _ptr(dbeta), _ptr(dgate), _ptr(dapf_log_ret),
-                      _ptr(dinit_state), _ptr(dprecond_in), _ptr(workspace),
-                      ctypes.c_size_t(workspace.numel() * workspace.element_size()), _stream_ptr())
+    rc = _call(_BWD, p, q, k, v, beta, gate, apf_log_ret, init_state, precond_in, dout, dfinal_state, dprecond_out, dq,
+               dk, dv, dbeta, dgate, dapf_log_ret, dinit_state, dprecond_in, workspace)
     _check(rc, "osdn_bwd")
 
 
 def osdn_precond_update(p: OsdnParams, k, beta, gate_or_log_ret, precond_in, k_tilde_out, precond_out):
-    lib = load_library()
-    rc = lib.osdn_precond_update(ctypes.byref(p), _ptr(k), _ptr(beta), _ptr(gate_or_log_ret), _ptr(precond_in),
-                                 _ptr(k_tilde_out), _ptr(precond_out), _stream_ptr())
+    rc = _call(_PRECOND, p, k, beta, gate_or_log_ret, precond_in, k_tilde_out, precond_out)
     _check(rc, "osdn_precond_update")
 
 
 def osdn_residual_ratio(p: OsdnParams, k, beta, gate_or_log_ret, precond_in, ratio_out, log_ratio_sum, precond_out=None):
-    lib = load_library()
-    rc = lib.osdn_residual_ratio(ctypes.byref(p), _ptr(k), _ptr(beta), _ptr(gate_or_log_ret), _ptr(precond_in),
-                                 _ptr(ratio_out), _ptr(log_ratio_sum), _ptr(precond_out), _stream_ptr())
+    rc = _call(_RATIO, p, k, beta, gate_or_log_ret, precond_in, ratio_out, log_ratio_sum, precond_out)
     _check(rc, "osdn_residual_ratio")
 
 
 def osdn_decode_step(p: OsdnParams, q, k, v, beta, gate, apf_log_ret, state, precond, out):
     """``state`` [B,H,V,K] and ``precond`` [B,H,K] (fp32, device) are updated in place."""
-    lib = load_library()
-    rc = lib.osdn_decode_step(ctypes.byref(p), _ptr(q), _ptr(k), _ptr(v), _ptr(beta), _ptr(gate), _ptr(apf_log_ret),
-                              _ptr(state), _ptr(precond), _ptr(out), _stream_ptr())
+    rc = _call(_DECODE, p, q, k, v, beta, gate, apf_log_ret, state, precond, out)
     _check(rc, "osdn_decode_step")
 
 
@@ -285,7 +286,7 @@ def osdn_step_host(p: OsdnParams, q, k, v, beta, gate, dout, out, dq, dk, dv, db
     lib = load_library()
     rc = lib.osdn_step_host(ctypes.byref(p), _ptr(q), _ptr(k), _ptr(v), _ptr(beta), _ptr(gate), _ptr(dout),
                             _ptr(out), _ptr(dq), _ptr(dk), _ptr(dv), _ptr(dbeta), _ptr(dgate), _ptr(staging),
-                            ctypes.c_size_t(staging.numel() * staging.element_size()), _stream_ptr())
+                            staging.nbytes, _stream_ptr())
     _check(rc, "osdn_step_host")
 
 

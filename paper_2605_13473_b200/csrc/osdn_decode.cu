@@ -77,7 +77,7 @@ template <int R> __device__ __forceinline__ void dec_store(float* p, int lane, c
 
 // VEC: vector retention (one log-retention per coordinate, log_ret [B,T,H,K]).
 template <typename T, int K, int V, bool VEC>
-__global__ void __launch_bounds__(DEC_WARPS * 32) decode_kernel(DecArgs a)
+__global__ void __cluster_dims__(V / DEC_VB, 1, 1) __launch_bounds__(DEC_WARPS * 32) decode_kernel(DecArgs a)
 {
     constexpr int R = K / 32;
     constexpr int SLICES = V / DEC_VB;
@@ -196,22 +196,12 @@ __global__ void __launch_bounds__(DEC_WARPS * 32) decode_kernel(DecArgs a)
     if (slice == 0 && warp == 0) dec_store<R>(a.precond + (size_t)chain * K, lane, d);
 }
 
-// One cluster per chain: its V / 16 slices (8 or 4 CTAs, within the portable cluster size).
+// One cluster per chain: its V / 16 slices (8 or 4 CTAs, within the portable cluster size; the size is part of
+// the kernel, so the launch is a plain one).
 template <typename T, int K, int V, bool VEC> bool launch_one(unsigned chains, const DecArgs& a, cudaStream_t st)
 {
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(chains * (unsigned)(V / DEC_VB));
-    cfg.blockDim = dim3(DEC_WARPS * 32);
-    cfg.dynamicSmemBytes = 0;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = V / DEC_VB;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, decode_kernel<T, K, V, VEC>, a) == cudaSuccess;
+    decode_kernel<T, K, V, VEC><<<chains * (unsigned)(V / DEC_VB), DEC_WARPS * 32, 0, st>>>(a);
+    return cudaGetLastError() == cudaSuccess;
 }
 
 template <typename T> int launch_typed(const osdn_params& p, const DecArgs& a, cudaStream_t st)
@@ -229,7 +219,7 @@ template <typename T> int launch_typed(const osdn_params& p, const DecArgs& a, c
         else if (p.K == 64 && p.V == 128) ok = launch_one<T, 64, 128, false>(chains, a, st);
         else ok = launch_one<T, 64, 64, false>(chains, a, st);
     }
-    return ok && cudaGetLastError() == cudaSuccess ? 1 : -1;
+    return ok ? 1 : -1;
 }
 
 }  // namespace
