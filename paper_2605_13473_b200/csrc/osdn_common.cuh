@@ -73,12 +73,12 @@ struct WsLayout {
     size_t U;           // [NT,H,64,V]    f32
     size_t dU;          // [NT,H,64,V]    f32   chunk update (new values)
     size_t Sn;          // [NT,H,V,K]     f32   state at chunk start
+    size_t gvec;        // [NT,H,2,64]    f32   in-chunk gate factors rho, gamma (CUDA-core family)
     // backward only
     size_t ddU;         // [NT,H,64,V]    f32
     size_t dSn;         // [NT,H,V,K]     f32   state cotangent at chunk end
     size_t dktil;       // [T,H,K]        f32
     size_t dkread;      // [T,H,K]        f32
-    size_t scr;         // [NT,H,5,64,max(K,V)] f32 scratch of the chunk-local backward
     size_t out_scratch; // [T,H,V]        f32   forward output when the backward recomputes the forward
     size_t total;
     int S, NTmax;
@@ -97,7 +97,6 @@ inline WsLayout make_layout(const osdn_params& p, bool need_bwd)
     L.NTmax = NTmax;
     L.dense_T = p.nseq > 0 ? 0 : p.T;
     const size_t H = p.H, K = p.K, V = p.V, NT = NTmax;
-    const size_t D = K > V ? K : V;
     size_t off = 0;
     auto take = [&](size_t bytes) { size_t o = off; off = align_up(off + bytes, 256); return o; };
     L.status = take(256);
@@ -118,12 +117,12 @@ inline WsLayout make_layout(const osdn_params& p, bool need_bwd)
     L.U = take(4 * NT * H * CH * V);
     L.dU = take(4 * NT * H * CH * V);
     L.Sn = take(4 * NT * H * V * K);
+    L.gvec = take(4 * NT * H * 2 * CH);
     if (need_bwd) {
         L.ddU = take(4 * NT * H * CH * V);
         L.dSn = take(4 * NT * H * V * K);
         L.dktil = take(4 * Ttot * H * K);
         L.dkread = take(4 * Ttot * H * K);
-        L.scr = take(4 * NT * H * 5 * CH * D);
         L.out_scratch = take(4 * Ttot * H * V);
     }
     L.total = off;
