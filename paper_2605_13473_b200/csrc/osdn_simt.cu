@@ -310,6 +310,7 @@ __device__ __forceinline__ void load_tile(float* dst, int ld, const T* __restric
                                           int H, int h)
 {
     const Rows<T, D> r = rows_of<T, D>(src, tok0, len, H, h);
+#pragma unroll 4
     for (int e = threadIdx.x; e < CH * D / 4; e += NT) {
         const int i = e / (D / 4), c = e % (D / 4) * 4;
         st4(dst + i * ld + c, r(i, c));
@@ -495,7 +496,11 @@ __global__ void __launch_bounds__(CL_NT, K + V == 128 ? 2 : 1) chunk_local_fwd_k
 template <typename T, int K, int V>
 __global__ void __launch_bounds__(256) output_kernel(ChunkArgs a)
 {
-    constexpr int TV = V / 16;
+    extern __shared__ __align__(16) float sm[];
+    constexpr int TV = V / 16, LD = K + 4, NT = 256;
+    float* sQ = sm;                  // [64][LD]
+    float* sS = sQ + CH * LD;        // [V][LD], S_n; then dU [64][V]
+    float* sP = sS + V * LD;         // [64][LC]
     const int c = blockIdx.x, h = blockIdx.y, H = a.H;
     const int len = a.tab.chunk_len(c);
     if (len == 0) return;
@@ -505,28 +510,41 @@ __global__ void __launch_bounds__(256) output_kernel(ChunkArgs a)
     const float* S = a.Sn + tile * V * K;
     const float* P = a.P + tile * CH * CH;
     const float* dU = a.dU + tile * CH * V;
-    const Rows<T, K> q = rows_of<T, K>(a.q, tok0, len, H, h);
+    load_tile<T, K, NT>(sQ, LD, static_cast<const T*>(a.q), tok0, len, H, h);
+#pragma unroll 8
+    for (int e = threadIdx.x; e < V * K / 4; e += NT) st4(sS + e / (K / 4) * LD + e % (K / 4) * 4, ld4(S + e * 4));
+#pragma unroll 4
+    for (int e = threadIdx.x; e < CH * CH / 4; e += NT) st4(sP + e / 16 * LC + e % 16 * 4, ld4(P + e * 4));
+    float4 u[CH * V / 4 / NT];
+#pragma unroll
+    for (int x = 0; x < CH * V / 4 / NT; ++x) u[x] = ld4(dU + (threadIdx.x + x * NT) * 4);
+    __syncthreads();
     float acc[4][TV];
     zero(acc);
-    tile_mm<false, true, TV>(acc, 0, K, l, [&](int m, int k) { return q(m, k); }, [&](int n, int k) { return ld4(S + n * K + k); });
+    tile_mm<false, true, TV>(acc, 0, K, l, [&](int m, int k) { return ld4(sQ + m * LD + k); }, [&](int n, int k) { return ld4(sS + n * LD + k); });
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
         const float g = a.gvec[tile * 2 * CH + CH + row_of(l, i)];
 #pragma unroll
         for (int j = 0; j < TV; ++j) acc[i][j] *= g;
     }
+    __syncthreads();
+    float* sU = sS;
+#pragma unroll
+    for (int x = 0; x < CH * V / 4 / NT; ++x) st4(sU + (threadIdx.x + x * NT) * 4, u[x]);
+    __syncthreads();
     const int jend = (l.tm & ~1) * 4 + 8;
     for (int j4 = 0; j4 < jend; j4 += 4) {   // columns tn + 16 n as above: scalar reads of dU
         float4 pv[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) pv[i] = ld4(P + row_of(l, i) * CH + j4);
+        for (int i = 0; i < 4; ++i) pv[i] = ld4(sP + row_of(l, i) * LC + j4);
 #pragma unroll
         for (int jj = 0; jj < 4; ++jj)
 #pragma unroll
             for (int n = 0; n < TV; ++n) {
-                const float u = dU[(j4 + jj) * V + l.tn + 16 * n];
+                const float x = sU[(j4 + jj) * V + l.tn + 16 * n];
 #pragma unroll
-                for (int i = 0; i < 4; ++i) acc[i][n] = fmaf(comp(pv[i], jj), u, acc[i][n]);
+                for (int i = 0; i < 4; ++i) acc[i][n] = fmaf(comp(pv[i], jj), x, acc[i][n]);
             }
     }
     T* o = static_cast<T*>(a.out);
@@ -842,13 +860,18 @@ __global__ void __launch_bounds__(256) ddu0_kernel(ChunkArgs a)
     const int tok0 = a.tab.chunk_tok0(c);
     const size_t tile = (size_t)c * H + h;
     const Lane l{(int)threadIdx.x >> 4, (int)threadIdx.x & 15};
+    __shared__ __align__(16) float sP[CH * CH];
+    extern __shared__ __align__(16) float sO[];   // [64][V]
     const float* P = a.P + tile * CH * CH;
-    const Rows<T, V> dout = rows_of<T, V>(a.dout, tok0, len, H, h);
+#pragma unroll
+    for (int e = threadIdx.x; e < CH * CH / 4; e += 256) st4(sP + e * 4, ld4(P + e * 4));
+    load_tile<T, V, 256>(sO, V, static_cast<const T*>(a.dout), tok0, len, H, h);
+    __syncthreads();
     float acc[4][TV];
     zero(acc);
     // P is lower triangular: row i of P^T starts at column i
-    tile_mm<true, false, TV>(acc, (l.tm & ~1) * 4, CH, l, [&](int j, int m) { return ld4(P + j * CH + m); },
-                             [&](int j, int n) { return dout(j, n); });
+    tile_mm<true, false, TV>(acc, (l.tm & ~1) * 4, CH, l, [&](int j, int m) { return ld4(sP + j * CH + m); },
+                             [&](int j, int n) { return ld4(sO + j * V + n); });
     float* o = a.ddU + tile * CH * V;
     const float s = a.hy.scale;
 #pragma unroll
@@ -905,6 +928,12 @@ __global__ void __launch_bounds__(CL_NT) chunk_local_bwd_kernel(ChunkArgs a)
     load_tile<float, K, CL_NT>(sKt, LD, a.ktil, tok0, len, H, h);
     load_tile<T, K, CL_NT>(sQ, LD, static_cast<const T*>(a.q), tok0, len, H, h);
     for (int e = threadIdx.x; e < CH * CH / 4; e += CL_NT) st4(sT + (e / 16) * LC + (e % 16) * 4, ld4(a.Tm + tile * CH * CH + e * 4));
+    // dU, then v, are read by rows that differ between lanes: staged in the place of X and Y until those are written
+    constexpr int LU = V + 4;
+    float* sU = sX;
+#pragma unroll 4
+    for (int e = threadIdx.x; e < CH * V / 4; e += CL_NT) st4(sU + e / (V / 4) * LU + e % (V / 4) * 4, ld4(dUg + e * 4));
+    if (V == 64) load_tile<T, V, CL_NT>(sY, LU, static_cast<const T*>(a.v), tok0, len, H, h);
     load_gates(gv, a.gate, a.beta, tok0, len, H, h);
     {   // <dS, S>_F (for the gradient of the chunk-level decay gamma_C)
         float part = 0.f;
@@ -921,7 +950,7 @@ __global__ void __launch_bounds__(CL_NT) chunk_local_bwd_kernel(ChunkArgs a)
     if (grp == 0) {
         float acc[4][4];
         zero(acc);
-        tile_mm<false, true, 4>(acc, 0, V, l, [&](int m, int k) { return dor(m, k); }, [&](int n, int k) { return ld4(dUg + n * V + k); });
+        tile_mm<false, true, 4>(acc, 0, V, l, [&](int m, int k) { return dor(m, k); }, [&](int n, int k) { return ld4(sU + n * LU + k); });
 #pragma unroll
         for (int i = 0; i < 4; ++i)
 #pragma unroll
@@ -980,6 +1009,13 @@ __global__ void __launch_bounds__(CL_NT) chunk_local_bwd_kernel(ChunkArgs a)
         store_rows(acc, static_cast<T*>(a.dq), K);
         row_dots(acc, [&](int m, int n) { return ld4(sQ + m * LD + n); }, sE[0]);
     } else {
+        const float* sV = V == 64 ? sY : sX;
+        if constexpr (V == 128) {   // no room for both before: v takes the place of dU now (this group alone)
+            const int t = threadIdx.x & 255;
+#pragma unroll 4
+            for (int e = t; e < CH * V / 4; e += 256) st4(sX + e / (V / 4) * LU + e % (V / 4) * 4, vr(e / (V / 4), e % (V / 4) * 4));
+            asm volatile("bar.sync 1, 256;" ::: "memory");
+        }
         float acc[4][4];
         zero(acc);
         tile_mm<false, true, 4>(acc, 0, K, l, [&](int m, int k) { return ld4(sW + m * LD + k); }, [&](int n, int k) { return ld4(sK + n * LD + k); });
@@ -987,7 +1023,8 @@ __global__ void __launch_bounds__(CL_NT) chunk_local_bwd_kernel(ChunkArgs a)
         for (int j = 0; j < 4; ++j)
 #pragma unroll
             for (int i = 0; i < 4; ++i) acc[i][j] *= gv.gam[col_of<true>(l, j)];
-        tile_mm<false, true, 4>(acc, 0, V, l, [&](int m, int k) { return ld4(ddUg + m * V + k); }, [&](int n, int k) { return vr(n, k); });
+        tile_mm<false, true, 4>(acc, 0, V, l, [&](int m, int k) { return ld4(ddUg + m * V + k); }, [&](int n, int k) { return ld4(sV + n * LU + k); });
+        if constexpr (V == 128) asm volatile("bar.sync 1, 256;" ::: "memory");   // v has been read
 #pragma unroll
         for (int i = 0; i < 4; ++i)
 #pragma unroll
@@ -1143,8 +1180,10 @@ int fwd_impl(const osdn_params& p, const Hyper& hy, const WsLayout& L, void* ws,
         chain_fwd_kernel<K, V><<<dim3(S * H, V / VS), CNT, smem, st>>>(ch);
         ++launches;
     }
+    const size_t smem_out = sizeof(float) * ((CH + V) * (K + 4) + CH * LC);
+    if (!set_smem(output_kernel<T, K, V>, smem_out)) return -1;
     stage_mark(st, "simt_output");
-    output_kernel<T, K, V><<<dim3(L.NTmax, H), 256, 0, st>>>(ca);
+    output_kernel<T, K, V><<<dim3(L.NTmax, H), 256, smem_out, st>>>(ca);
     ++launches;
     stage_end(st);
     return cudaGetLastError() == cudaSuccess ? launches : -1;
@@ -1166,7 +1205,7 @@ int bwd_impl(const osdn_params& p, const Hyper& hy, const WsLayout& L, void* ws,
     ca.dktil = F(L.dktil); ca.dkread = F(L.dkread);
     ca.dq = a.dq; ca.dv = a.dv; ca.dbeta = a.dbeta; ca.dgate = a.dgate; ca.hy = hy;
     stage_mark(st, "simt_ddu0");
-    ddu0_kernel<T, V><<<dim3(L.NTmax, H), 256, 0, st>>>(ca);
+    ddu0_kernel<T, V><<<dim3(L.NTmax, H), 256, CH * V * sizeof(float), st>>>(ca);
     ++launches;
     {
         ChainArgs ch{};
