@@ -73,7 +73,11 @@ struct WsLayout {
     size_t U;           // [NT,H,64,V]    f32
     size_t dU;          // [NT,H,64,V]    f32   chunk update (new values)
     size_t Sn;          // [NT,H,V,K]     f32   state at chunk start
-    size_t gvec;        // [NT,H,2,64]    f32   in-chunk gate factors rho, gamma (CUDA-core family)
+    // CUDA-core family only
+    size_t R;           // [NT,H,64,64]   f32   masked, decayed k.ktil scores (A without beta)
+    size_t Ktr;         // [NT,H,64,K]    f32   write keys decayed to the chunk's end
+    size_t Qg;          // [NT,H,64,K]    f32   queries decayed from the chunk's start
+    size_t gC;          // [NT,H,K]       f32   decay of the whole chunk
     // backward only
     size_t ddU;         // [NT,H,64,V]    f32
     size_t dSn;         // [NT,H,V,K]     f32   state cotangent at chunk end
@@ -117,7 +121,10 @@ inline WsLayout make_layout(const osdn_params& p, bool need_bwd)
     L.U = take(4 * NT * H * CH * V);
     L.dU = take(4 * NT * H * CH * V);
     L.Sn = take(4 * NT * H * V * K);
-    L.gvec = take(4 * NT * H * 2 * CH);
+    L.R = take(4 * NT * H * CH * CH);
+    L.Ktr = take(4 * NT * H * CH * K);
+    L.Qg = take(4 * NT * H * CH * K);
+    L.gC = take(4 * NT * H * K);
     if (need_bwd) {
         L.ddU = take(4 * NT * H * CH * V);
         L.dSn = take(4 * NT * H * V * K);
