@@ -58,7 +58,8 @@ struct WsLayout {
     size_t status;      // int32 device status word (+ padding)
     size_t table;       // ints, see carve_table
     // phase 1 (shared by both kernel families)
-    size_t p1n;         // [T,H]          f32   1 / max(|k|^2, eps), negated where the floor is active
+    size_t p1sumk;      // [T,H]          f32   |k|^2
+    size_t p1kmax;      // [T,H]          f32   largest k_r^2
     size_t p1rho;       // [T,H]          f32   retention of the preconditioner
     size_t p1al;        // [T,H]          f32   <d_t, k_t^2> of processed tokens                (save only)
     size_t p1flags;     // [NT,H,2]       u32   per token: the step maps d_min*1 to d_min*1, mask all zero
@@ -105,7 +106,8 @@ inline WsLayout make_layout(const osdn_params& p, bool need_bwd)
     auto take = [&](size_t bytes) { size_t o = off; off = align_up(off + bytes, 256); return o; };
     L.status = take(256);
     L.table = take(sizeof(int) * (4 * (size_t)S + 1 + 6 * NT + 4));
-    L.p1n = take(4 * Ttot * H);
+    L.p1sumk = take(4 * Ttot * H);
+    L.p1kmax = take(4 * Ttot * H);
     L.p1rho = take(4 * Ttot * H);
     L.p1flags = take(4 * NT * H * 2);
     if (need_bwd) {
@@ -155,7 +157,7 @@ inline Table carve_table(void* ws, const WsLayout& L)
 }
 
 struct P1Regions {
-    float *n, *rho, *dtraj, *al;
+    float *sumk, *kmax, *rho, *dtraj, *al;
     unsigned *flags, *skipw, *pmask;
 };
 
@@ -163,7 +165,8 @@ inline P1Regions carve_p1(void* ws, const WsLayout& L)
 {
     char* w = static_cast<char*>(ws);
     P1Regions r;
-    r.n = reinterpret_cast<float*>(w + L.p1n);
+    r.sumk = reinterpret_cast<float*>(w + L.p1sumk);
+    r.kmax = reinterpret_cast<float*>(w + L.p1kmax);
     r.rho = reinterpret_cast<float*>(w + L.p1rho);
     r.al = reinterpret_cast<float*>(w + L.p1al);
     r.flags = reinterpret_cast<unsigned*>(w + L.p1flags);

@@ -16,14 +16,11 @@
 //    the gate this removes almost every token from the chain; on inputs where d really moves it
 //    degenerates to the plain sequential scan.
 //
-// The sequential kernels run one warp per chain, so only the warp's own look-ahead hides memory
-// latency: rows are fetched a few tokens ahead into a shared-memory ring with cp.async, whose
-// completion is counted per committed group, first in first out (rows prefetched into registers
-// are held back by the few counters a warp has for outstanding loads).
-//
 // For the backward pass the forward records, per processed token, d_t and the projection mask,
 // and per chunk which tokens were skipped.  A skipped token has an all-zero mask, so the reverse
 // recurrence restarts there: lambda_t = k_t (.) dL/dktil_t, dk_t = dk_read_t + d_min dL/dktil_t.
+#include <type_traits>
+
 #include "osdn_common.cuh"
 
 namespace osdn {
@@ -35,41 +32,6 @@ __device__ __forceinline__ float warp_sum(float x)
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
     return x;
-}
-
-// One step of the recurrence on the warp-distributed vector d (lane l owns coordinates R l + r).
-//   c = eta b (1 - b <d, kap>) / n ;  x = rho d + c kap ;  d <- clip(x)
-// rho is given per owned coordinate (all equal unless the retention is a vector).
-// n_signed: max(sum kap, eps), negated when the floor eps is active.  pass[r]: ballot of the
-// coordinates whose projection passes gradient; all_low: every x strictly below d_min.
-template <int R>
-__device__ __forceinline__ void p1_step(float (&d)[R], const float (&kap)[R], float n, float b,
-                                        const float (&rho)[R], const Hyper& hy, unsigned (&pass)[R], bool& all_low, float& c_out,
-                                        float& al_out)
-{
-    float al = 0.f;
-#pragma unroll
-    for (int r = 0; r < R; ++r) al = fmaf(d[r], kap[r], al);
-    al = warp_sum(al);
-    const float c = hy.eta * b * (1.0f - b * al) / n;
-    bool low = true;
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-        float x = fmaf(c, kap[r], rho[r] * d[r]);
-        bool p = true;
-        if (hy.clamp) {
-            p = (x >= hy.d_min) && (x <= hy.d_max);
-            low = low && (x < hy.d_min);
-            x = fminf(fmaxf(x, hy.d_min), hy.d_max);
-        } else {
-            low = false;
-        }
-        pass[r] = __ballot_sync(0xffffffffu, p);
-        d[r] = x;
-    }
-    all_low = __all_sync(0xffffffffu, low);
-    c_out = c;
-    al_out = al;
 }
 
 // Lane l of the warp owns the R = K / 32 consecutive coordinates R l .. R l + R - 1, so that a
@@ -116,65 +78,17 @@ template <int R> __device__ __forceinline__ void store_row(__nv_bfloat16* p, int
     }
 }
 
-// A row as it sits in memory: loading it does not wait for the data (a conversion right after the
-// load would stall the warp until the load returns, which defeats fetching rows ahead of their use).
-template <typename T, int R> struct RawRow;
-template <> struct RawRow<float, 4> { float4 v; };
-template <> struct RawRow<float, 2> { float2 v; };
-template <> struct RawRow<__nv_bfloat16, 4> { uint2 v; };
-template <> struct RawRow<__nv_bfloat16, 2> { uint32_t v; };
-template <int R> __device__ __forceinline__ void load_raw(const float* p, int lane, RawRow<float, R>& x)
+// Asynchronous copies into shared memory; their completion is counted per committed group, first in first out.
+__device__ __forceinline__ void cp_async4(void* smem, const void* gmem)
 {
-    if constexpr (R == 4) x.v = *reinterpret_cast<const float4*>(p + 4 * lane);
-    else x.v = *reinterpret_cast<const float2*>(p + 2 * lane);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(smem)), "l"(gmem) : "memory");
 }
-template <int R> __device__ __forceinline__ void load_raw(const __nv_bfloat16* p, int lane, RawRow<__nv_bfloat16, R>& x)
+__device__ __forceinline__ void cp_async16_zfill(void* smem, const void* gmem, bool in)   // zeros where !in
 {
-    if constexpr (R == 4) x.v = *reinterpret_cast<const uint2*>(p + 4 * lane);
-    else x.v = *reinterpret_cast<const uint32_t*>(p + 2 * lane);
-}
-template <int R> __device__ __forceinline__ void unpack(const RawRow<float, R>& x, float (&y)[R])
-{
-    if constexpr (R == 4) { y[0] = x.v.x; y[1] = x.v.y; y[2] = x.v.z; y[3] = x.v.w; }
-    else { y[0] = x.v.x; y[1] = x.v.y; }
-}
-template <int R> __device__ __forceinline__ void unpack(const RawRow<__nv_bfloat16, R>& x, float (&y)[R])
-{
-    if constexpr (R == 4) {
-        const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&x.v.x));
-        const float2 b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&x.v.y));
-        y[0] = a.x; y[1] = a.y; y[2] = b.x; y[3] = b.y;
-    } else {
-        const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&x.v));
-        y[0] = a.x; y[1] = a.y;
-    }
-}
-
-// Asynchronous copies into a shared-memory ring: completion is counted per committed group (first in,
-// first out), so a row fetched PF tokens ahead can be waited for without waiting for the more recent
-// ones.  Rows fetched into registers cannot do that: the hardware tracks outstanding loads with a
-// handful of counters per warp, and a counter shared with a load issued one token ago holds back the
-// use of a row issued eight tokens ago (measured: about 300 cycles per token).
-template <int BYTES> __device__ __forceinline__ void cp_async(void* smem, const void* gmem)
-{
-    static_assert(BYTES == 4 || BYTES == 8 || BYTES == 16, "cp.async copies 4, 8 or 16 bytes");
-    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"((uint32_t)__cvta_generic_to_shared(smem)), "l"(gmem),
-                 "n"(BYTES)
-                 : "memory");
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(smem)), "l"(gmem), "r"(in ? 16 : 0) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
-
-template <int R> __device__ __forceinline__ float square_sum(const float (&kk)[R], float (&kap)[R])
-{
-    float sumk = 0.f;
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-        kap[r] = kk[r] * kk[r];
-        sumk += kap[r];
-    }
-    return warp_sum(sumk);
-}
 
 // ---------------------------------------------------------------------------------------------
 // plain streaming sweep (the stand-alone preconditioner update; no workspace)
@@ -310,7 +224,8 @@ __global__ void __launch_bounds__(128) phase1_spec_kernel(P1Fwd a)
             }
         }
         if (in && l8 == 0) {
-            a.r.n[th] = sumk > hy.eps ? 1.0f / n : -1.0f / n;   // reciprocal of the normaliser, signed
+            a.r.sumk[th] = sumk;
+            a.r.kmax[th] = kmax;
             a.r.rho[th] = rho;
         }
         if (low) {   // the write key of a token entered on the face: d_min k
@@ -324,43 +239,57 @@ __global__ void __launch_bounds__(128) phase1_spec_kernel(P1Fwd a)
         const unsigned bal = __ballot_sync(0xffffffffu, low);
         word |= ((bal & 1u) | ((bal >> 7) & 2u) | ((bal >> 14) & 4u) | ((bal >> 21) & 8u)) << (it * 4);
     }
-    if (lane == 0) a.r.flags[tile * 2 + half] = word;
+    if (lane == 0) {
+        a.r.flags[tile * 2 + half] = word;
+        if (a.save) a.r.skipw[tile * 2 + half] = word;   // what the sequential pass skips, if it does not say otherwise
+    }
 }
 
 __device__ __forceinline__ void prefetch_l2(const void* p)
 {
     asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
 }
-// Warms L2 (and the address translation) for a row of `bytes` bytes that starts on a 128-byte line.
-__device__ __forceinline__ void prefetch_row(const void* p, int bytes)
-{
-    for (int o = 0; o < bytes; o += 128) prefetch_l2(static_cast<const char*>(p) + o);
-}
-
-template <int R> __device__ __forceinline__ bool on_lower_face(const float (&d)[R], const Hyper& hy)
-{
-    bool f = hy.clamp != 0;
-#pragma unroll
-    for (int r = 0; r < R; ++r) f = f && (d[r] == hy.d_min);
-    return __all_sync(0xffffffffu, f);
-}
-
 // ---------------------------------------------------------------------------------------------
-// Pipelined stretches of the sequential pass.  Where nearly every token is processed (a preconditioner
-// that really moves), the walk of a chain is bound by the instructions one warp issues per token, most
-// of which do not depend on d: fetching and squaring the key, the step's scalars, forming and storing
-// the write key, the records for the backward.  For such a stretch three warps share the chain:
-//   pre   fetches a block of PB tokens and leaves k, k^2 and the scalars (e, a2, rho) in shared memory;
-//   core  carries d through the block: <d, k^2>, the step, the projection; leaves d_t and the mask;
-//   post  forms ktil_t = d_t (.) k_t and writes ktil, d_t and the mask words to global memory.
-// Blocks go round a ring of PN buffers; the roles meet at mbarriers (full: pre -> core and post,
-// done: core -> post, free: post -> pre).  Every token of a stretch is processed (none is skipped: for a
-// flagged token entered on the face the step returns to the face by construction, so the values are
-// the ones the skipping walk leaves), which keeps the core free of any bookkeeping.
+// The sequential pass, forward.  What it processes are lists of tokens of one chain: a dense run where d is off the
+// lower face, otherwise the unflagged tokens with a few tokens behind each (what lies between is skipped, provided that
+// d is back on the face there).  Walking such a list token by token is bound by the latency of the warp-wide sum
+// <d_t, k_t^2> in the middle of every step (five shuffle rounds of 30 cycles each, or an integer reduction of 75 with its
+// conversions; a multiply-add takes 5).  So the step scalars c_t of a block of PB tokens are solved for together:
+//
+//   guess c for the block; run d through the block with these c (one multiply-add per token and coordinate on the
+//   dependent path); form all PB sums at once; c_t = e_t - a2_t <d_t, k_t^2>; repeat until c does not change.
+//
+// c_t depends on d_t, hence on the c of earlier tokens only: after m rounds the first m tokens are exact whatever the
+// input, so it ends; and the dependence is weak (a change of c_s moves c_t by eta beta^2 <k_s^2, k_t^2>, and
+// <k_s^2, k_t^2> is about 1/128 for unit keys): measured 1.2 rounds at a step size of 0.003, 3.4 at 0.3.
+// A round's c is taken when the d it leads to are unchanged: |change of c_t| max k_t^2 at most 2^-26 of the smallest d
+// the box allows (a quarter of its rounding unit), or a unit in the last place of c_t.
+// In isolation a block of 32 tokens takes 630 + 660 cycles a round with a coordinate per lane (K / 32 warps), against
+// 109 cycles a token for one warp with one integer reduction per token.
+//
+// Warps of a chain's CTA: K / 32 core warps, two that fetch keys and scalars (blocks in turn), four that finish (they
+// repeat a block's steps from its c, the same operations in the same order, and write ktil_t = d_t (.) k_t, d_t and the
+// mask words).  Blocks go round a ring of buffers; the roles meet at mbarriers (full: fetch -> core and finish, done:
+// core -> finish, free: finish -> fetch).  Warp 0 decides between two lists and walks short ones alone.
 // ---------------------------------------------------------------------------------------------
-constexpr int PB = 16, PN = 3;
+constexpr int PB = 32;
 constexpr int P1_ERR_PIPE = 131;
 constexpr long long P1_WAIT_LIMIT = 4000000000ll;   // about two seconds
+constexpr int LIST_MAX = 256;                       // entries of a sparse list
+constexpr int WALK = 16;                            // tokens of a first dense run
+constexpr int SCAN_CHUNKS = 128;                    // chunks whose words warp 0 reads at a time
+
+// A block's way round the ring (fetch, core, finish) takes about six times what the core needs for it, hence that many
+// helpers and a deep ring: with four buffers and two finishing warps the core waited for half of the time.
+template <int K> struct Pipe {
+    static constexpr int CORE = K / 32, FETCH0 = CORE, FETCH = 2, FINISH0 = CORE + FETCH, FINISH = 4, WARPS = FINISH0 + FINISH, THREADS = WARPS * 32;
+};
+constexpr int RING_MAX = 8;
+static_assert(RING_MAX / 2 % Pipe<128>::FETCH == 0 && RING_MAX / 2 % Pipe<128>::FINISH == 0, "a buffer belongs to one fetching and one finishing warp");
+// Buffers of the given size that fit the CTA's shared memory beside the rest: RING_MAX or half of it.  Both are multiples
+// of the numbers of fetching and of finishing warps, so that all uses of a buffer are the same warps' and follow one
+// another in order (a wait tells a barrier's phases apart by their parity only).
+constexpr int ring_depth(size_t bytes) { return bytes * RING_MAX <= 216 * 1024 ? RING_MAX : RING_MAX / 2; }
 
 __device__ __forceinline__ void p1_mbar_init(uint64_t* b, int count)
 {
@@ -370,618 +299,836 @@ __device__ __forceinline__ void p1_mbar_arrive(uint64_t* b)
 {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"((uint32_t)__cvta_generic_to_shared(b)) : "memory");
 }
-// Bounded: gives up after P1_WAIT_LIMIT cycles, records the error and returns false.
+// Bounded: gives up after P1_WAIT_LIMIT cycles, records the error and returns false.  The whole warp calls; the vote at
+// the end brings its lanes together again (lanes that leave the loop in different turns would otherwise run what
+// follows one after the other).
 __device__ __forceinline__ bool p1_mbar_wait(uint64_t* b, uint32_t parity, int* status)
 {
     const uint32_t addr = (uint32_t)__cvta_generic_to_shared(b);
+    uint32_t ok = 0;
     const long long t0 = clock64();
-    while (true) {
-        uint32_t ok;
+    while (!ok) {
         asm volatile("{ .reg .pred p; mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
                      : "=r"(ok)
                      : "r"(addr), "r"(parity)
                      : "memory");
-        if (ok) return true;
-        if (clock64() - t0 > P1_WAIT_LIMIT) {
-            if (status) atomicCAS(status, 0, P1_ERR_PIPE);
-            return false;
-        }
+        if (!ok && clock64() - t0 > P1_WAIT_LIMIT) break;
+    }
+    if (!ok && status) atomicCAS(status, 0, P1_ERR_PIPE);
+    return __all_sync(0xffffffffu, ok != 0);
+}
+template <int NT> __device__ __forceinline__ void bar_sync(int id) { asm volatile("bar.sync %0, %1;" ::"r"(id), "n"(NT) : "memory"); }
+// The barrier with a vote: whether `pred` held everywhere, so that the warps go on, or give up, together.
+template <int NT> __device__ __forceinline__ bool bar_sync_and(int id, bool pred)
+{
+    uint32_t r;
+    asm volatile("{ .reg .pred p, q; setp.ne.u32 p, %1, 0; barrier.cta.red.and.pred q, %2, %3, p; selp.u32 %0, 1, 0, q; }"
+                 : "=r"(r) : "r"((uint32_t)pred), "r"(id), "n"(NT) : "memory");
+    return r != 0;
+}
+__device__ __forceinline__ bool bit_of(unsigned m, int j) { return (m >> j) & 1u; }
+
+struct PipeBars {
+    uint64_t full[RING_MAX], done[RING_MAX], free_[RING_MAX];
+};
+__device__ __forceinline__ void init_bars(PipeBars& bars, int n, int core_warps)
+{
+    for (int i = 0; i < n; ++i) {
+        p1_mbar_init(&bars.full[i], 1);
+        p1_mbar_init(&bars.done[i], core_warps);
+        p1_mbar_init(&bars.free_[i], 1);
     }
 }
 
 template <typename TI, int K, bool VEC> struct PipeBuf {
-    static constexpr int R = K / 32;
-    float kap[PB][K];                       // k^2
-    RawRow<TI, R> kraw[PB][32];             // k as it sits in memory
-    float x[PB][K];                         // the step's value before the projection (d_{t+1} = clip(x_t)), by the core
-    float d0[K];                            // d on entry to the block, by the core
-    float rhov[VEC ? PB : 1][VEC ? K : 1];  // vector retention: exp(l_t) per coordinate
-    float4 scal[PB];                        // e = eta b / n, a2 = e b, rho, fixed-point scale -> <d_t, k^2>
+    TI k[PB][K];                            // as it sits in memory; rows beyond the list are zero
+    float y0[K];                            // core: y on entry to the block
+    float raw[4][PB];                       // sum k^2, max k^2, retention, beta as they sit in memory
+    float rho[PB], off[PB];                 // retention (0 behind a jump: y is 0 there), (retention - 1) d_min / w
+    float4 scal[PB];                        // e', a2, max k^2, sum k^2
+    float2 res[PB];                         // core: c', <y, k^2>
+    unsigned jump;                          // bit j: the token before this one was skipped, d enters on the face
+    int n;                                  // core: tokens of the block that stand
+    alignas(16) float rv[VEC ? PB : 1][VEC ? K : 1];   // vector retention: l_t, then (core) exp(l_t)
+};
+template <typename TI, int K, bool VEC> struct PipeShared {
+    static constexpr int CW = K / 32, PN = ring_depth(sizeof(PipeBuf<TI, K, VEC>));
+    PipeBuf<TI, K, VEC> buf[PN];
+    float y[K];                             // between two lists
+    float c[CW][PB];                        // a core warp's c' of the round
+    float part[2][CW][PB];                  // the core warps' shares of the sums, by round parity
+    unsigned bad[CW];                       // jumps that d enters off the face
+    unsigned long long words[SCAN_CHUNKS];
+    uint16_t list[LIST_MAX];
+    int cmd_tok, cmd_n, cmd_dense;          // first token (a list's offsets count from it), entries; none: finished
+    int stop;                               // entries that stand
+    PipeBars bars;
 };
 
-// What the post role derives from the core's x: d_t of every token (the clipped x of the token before it,
-// the block's entry value for the first) and the projection's pass bits.  The core then carries nothing
-// but the recurrence itself.
-template <int R> __device__ __forceinline__ void clip_row(const float (&x)[R], const Hyper& hy, float (&d)[R], unsigned& bits)
+// The coordinate the recurrence runs in.  With the projection on, y = (d - d_min) / w, w = d_max - d_min: with
+// c' = c / w a step is one saturating multiply-add, y' = sat(rho y + (c' k^2 + (rho - 1) d_min / w)), and
+// c' = e' - a2 <y, k^2>, e' = (e - a2 d_min sum k^2) / w.  With it off, or for a box without width, y = d (w = 1, d_min
+// taken as 0).  Core, finishing warps and the walk use the same functions, hence the same values.
+enum P1Mode { P1_SAT, P1_FREE, P1_CLIP };
+struct P1Coord {
+    float lo, w, iw, k0;   // d = lo + w y; k0 = lo / w
+};
+__device__ __forceinline__ P1Mode p1_mode(const Hyper& hy) { return !hy.clamp ? P1_FREE : hy.d_max > hy.d_min ? P1_SAT : P1_CLIP; }
+__device__ __forceinline__ P1Coord p1_coord(const Hyper& hy)
 {
-    bits = 0;
+    if (p1_mode(hy) != P1_SAT) return {0.f, 1.f, 1.f, 0.f};
+    const float w = hy.d_max - hy.d_min, iw = 1.0f / w;
+    return {hy.d_min, w, iw, hy.d_min * iw};
+}
+__device__ __forceinline__ float p1_y(float d, const P1Coord& q) { return __fmul_rn(d - q.lo, q.iw); }
+__device__ __forceinline__ float p1_d(float y, const P1Coord& q) { return fmaf(q.w, y, q.lo); }
+__device__ __forceinline__ float p1_off(float rho, const P1Coord& q) { return fmaf(rho, q.k0, -q.k0); }
+__device__ __forceinline__ float p1_raw(float y, float kap, float c, float rho, float off) { return fmaf(rho, y, fmaf(c, kap, off)); }
+template <P1Mode M> __device__ __forceinline__ float p1_project(float x, const Hyper& hy)
+{
+    return M == P1_SAT ? __saturatef(x) : M == P1_CLIP ? fminf(fmaxf(x, hy.d_min), hy.d_max) : x;
+}
+__device__ __forceinline__ float p1_project(float x, P1Mode m, const Hyper& hy)
+{
+    return m == P1_SAT ? p1_project<P1_SAT>(x, hy) : m == P1_CLIP ? p1_project<P1_CLIP>(x, hy) : x;
+}
+// e', a2, max k^2, sum k^2 of a token
+__device__ __forceinline__ float4 p1_scalars(float sumk, float kmax, float beta, const Hyper& hy, const P1Coord& q)
+{
+    const float b = hy.beta_aware ? beta : 1.0f;
+    const float e = hy.eta * b / fmaxf(sumk, hy.eps), a2 = e * b;
+    return make_float4(fmaf(-a2 * q.lo, sumk, e) * q.iw, a2, kmax, sumk);
+}
+
+// Lane l gets the warp's sum of x[l % N]: the N sums share their shuffles.
+template <int N> __device__ __forceinline__ float transpose_sum(float (&x)[N], int lane)
+{
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
-        // inside the box (faces included) exactly when clamping leaves the value alone
-        d[r] = hy.clamp ? fminf(fmaxf(x[r], hy.d_min), hy.d_max) : x[r];
-        bits |= d[r] == x[r] ? (1u << r) : 0u;
+    for (int s = N / 2; s > 0; s >>= 1) {
+        const bool up = (lane & s) != 0;
+#pragma unroll
+        for (int i = 0; i < s; ++i) {
+            const float send = up ? x[i] : x[i + s], keep = up ? x[i + s] : x[i];
+            x[i] = keep + __shfl_xor_sync(0xffffffffu, send, s);
+        }
+    }
+    float v = x[0];
+#pragma unroll
+    for (int s = N; s < 32; s <<= 1) v += __shfl_xor_sync(0xffffffffu, v, s);
+    return v;
+}
+
+// One block by the core warps: y of this lane's coordinate goes through it (slots beyond its n tokens leave y alone).
+// r: <y, k^2> / sum k^2 of the latest token, the start of the next guess; rounds: all rounds so far.  Returns the tokens
+// that stand: n, or those before the first jump that d enters off the face (y is then its value there).
+template <typename TI, int K, bool VEC, P1Mode M>
+__device__ __forceinline__ int core_block(PipeShared<TI, K, VEC>& sh, PipeBuf<TI, K, VEC>& B, int n, float& y, float& r, uint32_t& rounds,
+                                          const Hyper& hy, const P1Coord& q, int warp, int lane)
+{
+    constexpr int CW = Pipe<K>::CORE;
+    const int i = warp * 32 + lane;
+    float kap[PB];
+#pragma unroll
+    for (int j = 0; j < PB; ++j) {
+        const float k = ldf(&B.k[j][i]);
+        kap[j] = __fmul_rn(k, k);
+    }
+    if constexpr (VEC) {
+#pragma unroll 4
+        for (int j = 0; j < PB; ++j) {
+            float& v = B.rv[VEC ? j : 0][VEC ? i : 0];
+            v = j < n ? expf(v) : 1.0f;
+        }
+    }
+    B.y0[i] = y;
+    const unsigned jump = B.jump;
+    const float4 sc = B.scal[lane];   // lane j: token j
+    const bool jumped = bit_of(jump, lane);
+    const float tol = M == P1_FREE ? 0.f : 1.4901161e-8f * fmaxf(hy.d_min, 0.f) * q.iw;
+    float c = jumped ? sc.x : fmaf(-sc.y, sc.w * r, sc.x), sum = 0.f, z = y;
+    for (int round = 0; round <= PB; ++round) {   // (round PB + 1 could change nothing)
+        const uint32_t par = rounds++ & 1;
+        sh.c[warp][lane] = c;
+        __syncwarp();
+        float p[PB];
+        z = y;
+#pragma unroll
+        for (int j = 0; j < PB; j += 4) {
+            const float4 c4 = *reinterpret_cast<const float4*>(&sh.c[warp][j]), r4 = *reinterpret_cast<const float4*>(B.rho + j);
+            const float4 o4 = *reinterpret_cast<const float4*>(B.off + j);
+            const float cv[4] = {c4.x, c4.y, c4.z, c4.w}, rv[4] = {r4.x, r4.y, r4.z, r4.w}, ov[4] = {o4.x, o4.y, o4.z, o4.w};
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                float rho = rv[u], off = ov[u];
+                if constexpr (VEC) {   // (rv[u]: 0 behind a jump, else 1)
+                    rho = B.rv[VEC ? j + u : 0][VEC ? i : 0];
+                    off = p1_off(rho, q);
+                    rho *= rv[u];
+                }
+                p[j + u] = z * kap[j + u];
+                z = p1_project<M>(p1_raw(z, kap[j + u], cv[u], rho, off), hy);
+            }
+        }
+        const float mine = transpose_sum(p, lane);
+        float(*part)[PB] = sh.part[par];
+        part[warp][lane] = mine;
+        bar_sync<CW * 32>(3);
+        sum = part[0][lane];
+#pragma unroll
+        for (int x = 1; x < CW; ++x) sum += part[x][lane];
+        if (jumped) sum = 0.f;
+        const float cn = fmaf(-sc.y, sum, sc.x);
+        const float dc = fabsf(cn - c);
+        // the same values in every core warp, so they all leave in the same round
+        if (__all_sync(0xffffffffu, dc * sc.z <= tol || dc <= 1.1920929e-7f * fabsf(cn) || lane >= n)) break;
+        c = cn;
+    }
+    int stand = n;
+    if (jump) {   // was d on the face at the jumps?
+        auto to = [&](int end, unsigned& off_face) {
+            float v = y;
+#pragma unroll 4
+            for (int j = 0; j < end; ++j) {
+                if (bit_of(jump, j) && v != 0.f) off_face |= 1u << j;
+                float rho = B.rho[j], off = B.off[j];
+                if constexpr (VEC) {
+                    const float x = B.rv[VEC ? j : 0][VEC ? i : 0];
+                    off = p1_off(x, q);
+                    rho *= x;
+                }
+                const float k = ldf(&B.k[j][i]);
+                v = p1_project<M>(p1_raw(v, __fmul_rn(k, k), sh.c[warp][j], rho, off), hy);
+            }
+            return v;
+        };
+        unsigned bad = 0;
+        to(n, bad);
+        bad = __reduce_or_sync(0xffffffffu, bad);
+        if (lane == 0) sh.bad[warp] = bad;
+        bar_sync<CW * 32>(3);
+#pragma unroll
+        for (int x = 0; x < CW; ++x) bad |= sh.bad[x];
+        if (bad) {
+            stand = __ffs((int)bad) - 1;
+            unsigned none = 0;
+            z = to(stand, none);
+        }
+    }
+    y = z;
+    if (warp == 0) {
+        B.res[lane] = make_float2(c, sum);
+        if (lane == 0) B.n = stand;
+    }
+    r = __shfl_sync(0xffffffffu, sum / fmaxf(sc.w, 1e-30f), n - 1);
+    return stand;
+}
+template <typename TI, int K, bool VEC>
+__device__ __forceinline__ int core_block(PipeShared<TI, K, VEC>& sh, PipeBuf<TI, K, VEC>& B, int n, float& y, float& r, uint32_t& rounds,
+                                          const Hyper& hy, const P1Coord& q, int warp, int lane)
+{
+    const P1Mode mode = p1_mode(hy);
+    if (mode == P1_SAT) return core_block<TI, K, VEC, P1_SAT>(sh, B, n, y, r, rounds, hy, q, warp, lane);
+    if (mode == P1_FREE) return core_block<TI, K, VEC, P1_FREE>(sh, B, n, y, r, rounds, hy, q, warp, lane);
+    return core_block<TI, K, VEC, P1_CLIP>(sh, B, n, y, r, rounds, hy, q, warp, lane);
+}
+
+// Rows of D elements on their way into a buffer; lane j of the warp holds the number of row j in the source (NO_ROW: the
+// row is filled with zeros).
+constexpr uint32_t NO_ROW = ~0u;
+template <typename T, int D> __device__ __forceinline__ void fetch_rows(T* dst, const T* src, uint32_t mine, int rows, int lane)
+{
+    constexpr int PIECES = D * (int)sizeof(T) / 16, EL = 16 / (int)sizeof(T), STEP = 32 / PIECES;
+    static_assert(PIECES <= 32, "a row is one or a part of a warp-wide copy");
+    const int c = lane % PIECES * EL;
+#pragma unroll 8
+    for (int j = lane / PIECES; j < (rows + STEP - 1) / STEP * STEP; j += STEP) {
+        const uint32_t row = __shfl_sync(0xffffffffu, mine, j);
+        cp_async16_zfill(dst + j * D + c, src + (row == NO_ROW ? 0 : (size_t)row * D) + c, row != NO_ROW);
     }
 }
-constexpr int RING_MAX = 6;   // the deeper of the two rings
-struct PipeBars {
-    uint64_t full[RING_MAX], done[RING_MAX], free_[RING_MAX];
-};
 
-// The core's work on one block: carries d through n tokens; reads kap, the scalars (and the retention
-// vector), leaves d_t, the mask bits and <d_t, k^2> (in scal.w).
-template <typename TI, int K, bool VEC>
-__device__ __forceinline__ void pipe_core_block(PipeBuf<TI, K, VEC>& B, int n, float (&d)[K / 32], const Hyper& hy, int lane)
+// A finishing warp's work on a block: out(j, d_t, k_t, bits) for its n tokens; bit r of `bits`: the projection passed
+// gradient for coordinate R lane + r (inside the box, faces included).
+template <typename TI, int K, bool VEC, P1Mode M, typename OUT>
+__device__ __forceinline__ void finish_block(const PipeBuf<TI, K, VEC>& B, int n, const Hyper& hy, const P1Coord& q, int lane, OUT out)
 {
     constexpr int R = K / 32;
-    store_row<R>(B.d0, lane, d);
-    auto token = [&](int j) {
-        const float4 sc = B.scal[j];
-        float kap[R], rho[R];
-        load_row<R>(B.kap[j], lane, kap);
-        if constexpr (VEC) load_row<R>(B.rhov[VEC ? j : 0], lane, rho);
-        else {
-#pragma unroll
-            for (int r = 0; r < R; ++r) rho[r] = sc.z;
-        }
-        float al0 = d[0] * kap[0], al1 = d[1] * kap[1];   // two short chains instead of one long one
-#pragma unroll
-        for (int r = 2; r < R; r += 2) {
-            al0 = fmaf(d[r], kap[r], al0);
-            al1 = fmaf(d[r + 1], kap[r + 1], al1);
-        }
-        float al;
-        if (hy.clamp) {
-            // With the projection on, 0 <= <d, k^2> <= d_max sum k^2: the lanes' partial sums are added as
-            // fixed-point integers with one warp-wide instruction instead of five shuffle-add rounds.
-            // sc.w = 2^26 / (d_max sum k^2) (from the pre role): the total stays below 2^27, a lane's
-            // rounding is 2^-27 of the bound, 32 of them 2^-22 of it.
-            const unsigned q = __float2uint_rn((al0 + al1) * sc.w);
-            al = __uint2float_rn(__reduce_add_sync(0xffffffffu, q)) * __frcp_rn(sc.w);
-        } else {
-            al = warp_sum(al0 + al1);
-        }
-        const float cc = fmaf(-sc.y, al, sc.x);
-        float x[R];
-#pragma unroll
-        for (int r = 0; r < R; ++r) x[r] = fmaf(cc, kap[r], rho[r] * d[r]);
-        store_row<R>(B.x[j], lane, x);
-#pragma unroll
-        for (int r = 0; r < R; ++r) d[r] = hy.clamp ? fminf(fmaxf(x[r], hy.d_min), hy.d_max) : x[r];
-        if (lane == 0) B.scal[j].w = al;
-    };
-    if (n == PB) {   // partly unrolled: the shared-memory reads of later tokens are issued under the shuffles of earlier ones
+    const unsigned jump = B.jump;
+    float y[R];
+    load_row<R>(B.y0, lane, y);
 #pragma unroll 4
-        for (int j = 0; j < PB; ++j) token(j);
-    } else {
-        for (int j = 0; j < n; ++j) token(j);
+    for (int j = 0; j < n; ++j) {
+        float kk[R], d[R], rho[R], off[R];
+        load_row<R>(B.k[j], lane, kk);
+        const float c = B.res[j].x;
+        if constexpr (VEC) {
+            load_row<R>(B.rv[VEC ? j : 0], lane, rho);
+#pragma unroll
+            for (int r = 0; r < R; ++r) off[r] = p1_off(rho[r], q);
+        } else {
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                rho[r] = B.rho[j];
+                off[r] = B.off[j];
+            }
+        }
+        const float keep = bit_of(jump, j) ? 0.f : 1.f;
+        unsigned bits = 0;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const float v = y[r] * keep;
+            d[r] = p1_d(v, q);
+            const float x = p1_raw(v, __fmul_rn(kk[r], kk[r]), c, rho[r], off[r]);
+            y[r] = p1_project<M>(x, hy);
+            bits |= y[r] == x ? (1u << r) : 0u;
+        }
+        out(j, d, kk, bits);
     }
 }
+template <typename TI, int K, bool VEC, typename OUT>
+__device__ __forceinline__ void finish_block(const PipeBuf<TI, K, VEC>& B, int n, const Hyper& hy, const P1Coord& q, int lane, OUT out)
+{
+    const P1Mode mode = p1_mode(hy);
+    if (mode == P1_SAT) finish_block<TI, K, VEC, P1_SAT>(B, n, hy, q, lane, out);
+    else if (mode == P1_FREE) finish_block<TI, K, VEC, P1_FREE>(B, n, hy, q, lane, out);
+    else finish_block<TI, K, VEC, P1_CLIP>(B, n, hy, q, lane, out);
+}
 
-// tokens [t_a, t_b) of the chain (packed token indices), all three roles; d: the core's registers
+// The list in sh through the ring, all roles.  y travels through sh.y; guess and rounds belong to the core warps.
 template <typename TI, typename TO, int K, bool VEC>
-__device__ __forceinline__ bool pipe_stretch(const P1Fwd& a, int h, int t_a, int t_b, float (&d)[K / 32],
-                                             PipeBuf<TI, K, VEC>* buf, PipeBars& bars, uint32_t& round0, int role, int lane)
+__device__ __forceinline__ bool run_list(const P1Fwd& a, int h, PipeShared<TI, K, VEC>& sh, float& guess, uint32_t& rounds, uint32_t& uses,
+                                         int warp, int lane)
+{
+    constexpr int R = K / 32;
+    using P = Pipe<K>;
+    constexpr int PN = PipeShared<TI, K, VEC>::PN;
+    const int H = a.H;
+    const Hyper hy = a.hy;
+    const P1Coord q = p1_coord(hy);
+    const int tok0 = sh.cmd_tok, total = sh.cmd_n;
+    const bool dense = sh.cmd_dense != 0;
+    const int nblk = (total + PB - 1) / PB;
+    bool ok = true;
+    // block b uses buffer (base + b) % PN; its barriers complete once per use: parity of the use count
+    const uint32_t base = uses;
+    auto tok_of = [&](int idx) { return tok0 + (dense ? idx : (int)sh.list[idx] & 0x7fff); };
+    auto len_of = [&](int b) { return min(PB, total - b * PB); };
+    auto th_of = [&](int b) { return lane < len_of(b) ? (uint32_t)(tok_of(b * PB + lane) * H + h) : NO_ROW; };   // lane j: token j
+    if (warp < P::CORE) {
+        float y = sh.y[warp * 32 + lane];
+        int stop = total;
+        bool dead = false;   // d left the list: what follows in it is dropped
+        for (int b = 0; b < nblk; ++b) {
+            const int bi = (base + b) % PN;
+            ok = bar_sync_and<P::CORE * 32>(3, p1_mbar_wait(&sh.bars.full[bi], ((base + b) / PN) & 1, a.status));
+            if (!ok) break;
+            PipeBuf<TI, K, VEC>& B = sh.buf[bi];
+            if (!dead) {
+                const int n = len_of(b), stand = core_block<TI, K, VEC>(sh, B, n, y, guess, rounds, hy, q, warp, lane);
+                if (stand < n) {
+                    dead = true;
+                    stop = b * PB + stand;
+                }
+            } else if (warp == 0 && lane == 0) {
+                B.n = 0;
+            }
+            __syncwarp();
+            if (lane == 0) p1_mbar_arrive(&sh.bars.done[bi]);
+        }
+        sh.y[warp * 32 + lane] = y;
+        if (warp == 0 && lane == 0) sh.stop = ok ? stop : 0;
+    } else if (warp < P::FINISH0) {
+        // the warps take the blocks in turn
+        auto start = [&](int b) {
+            const uint32_t use = base + b;
+            const int bi = use % PN;
+            if (use >= PN) ok = p1_mbar_wait(&sh.bars.free_[bi], ((use / PN) - 1) & 1, a.status);
+            if (!ok) return;
+            PipeBuf<TI, K, VEC>& B = sh.buf[bi];
+            const uint32_t th = th_of(b);
+            fetch_rows<TI, K>(&B.k[0][0], static_cast<const TI*>(a.k), th, PB, lane);
+            if constexpr (VEC) fetch_rows<float, K>(&B.rv[0][0], a.retsrc, th, PB, lane);
+            if (th != NO_ROW) {
+                cp_async4(&B.raw[0][lane], a.r.sumk + th);
+                cp_async4(&B.raw[1][lane], a.r.kmax + th);
+                cp_async4(&B.raw[2][lane], a.r.rho + th);
+                cp_async4(&B.raw[3][lane], a.beta + th);
+            }
+            cp_async_commit();
+        };
+        auto complete = [&](int b) {   // the step's scalars from the raw ones
+            const int bi = (base + b) % PN;
+            PipeBuf<TI, K, VEC>& B = sh.buf[bi];
+            const int n = len_of(b), idx = b * PB + lane;
+            float4 sc = make_float4(0.f, 0.f, 0.f, 0.f);   // an empty slot: c' = 0, k^2 = 0, rho = 1
+            float rho = 1.f;
+            bool jump = false;
+            if (lane < n) {
+                sc = p1_scalars(B.raw[0][lane], B.raw[1][lane], B.raw[3][lane], hy, q);
+                rho = B.raw[2][lane];
+                jump = !dense && idx > 0 && tok_of(idx) != tok_of(idx - 1) + 1;
+            }
+            const unsigned jumps = __ballot_sync(0xffffffffu, jump);
+            B.scal[lane] = sc;
+            B.off[lane] = p1_off(rho, q);
+            B.rho[lane] = jump ? 0.f : VEC ? 1.f : rho;
+            if (lane == 0) B.jump = jumps;
+            __syncwarp();
+            if (lane == 0) p1_mbar_arrive(&sh.bars.full[bi]);
+        };
+        int b = (int)((warp - P::FETCH0 + base) & 1);
+        if (b < nblk) start(b);
+        for (; b < nblk && ok; b += 2) {
+            cp_async_wait<0>();
+            __syncwarp();
+            complete(b);
+            if (b + 2 < nblk) start(b + 2);
+        }
+        cp_async_wait<0>();
+    } else {
+        TO* kt = static_cast<TO*>(a.ktil);
+        for (int b = (int)((warp - P::FINISH0 - base) & (P::FINISH - 1)); b < nblk; b += P::FINISH) {
+            const int bi = (base + b) % PN;
+            ok = p1_mbar_wait(&sh.bars.done[bi], ((base + b) / PN) & 1, a.status);
+            if (!ok) break;
+            const PipeBuf<TI, K, VEC>& B = sh.buf[bi];
+            const int n = B.n;
+            const uint32_t mine = th_of(b);
+            finish_block<TI, K, VEC>(B, n, hy, q, lane, [&](int j, const float (&d)[R], const float (&kk)[R], unsigned bits) {
+                const size_t th = __shfl_sync(0xffffffffu, mine, j);
+                float wk[R];
+#pragma unroll
+                for (int r = 0; r < R; ++r) wk[r] = d[r] * kk[r];
+                store_row<R>(kt + th * K, lane, wk);
+                if (a.save) {
+                    store_row<R>(a.r.dtraj + th * K, lane, d);
+                    a.r.pmask[th * 32 + lane] = bits;
+                }
+            });
+            if (a.save && lane < n) a.r.al[mine] = fmaf(q.w, B.res[lane].y, q.lo * B.scal[lane].w);
+            __syncwarp();
+            if (lane == 0) p1_mbar_arrive(&sh.bars.free_[bi]);
+        }
+    }
+    uses = base + nblk;
+    return ok;
+}
+
+// A list of at most PB entries by warp 0 alone, token by token (a few tokens are done before a ring would be full, and
+// the code is short).  An entry marked with bit 15 is skipped when d enters it on the face.  Returns the entries
+// that stand (fewer than n where d is off the face at a jump); sets the bits of the processed tokens in `proc`.
+template <typename TI, typename TO, int K, bool VEC>
+__device__ __forceinline__ int walk_list(const P1Fwd& a, int h, PipeShared<TI, K, VEC>& sh, int tok0, int n, bool& face, unsigned long long& proc, int lane)
 {
     constexpr int R = K / 32;
     const int H = a.H;
     const Hyper hy = a.hy;
-    const int nblk = (t_b - t_a + PB - 1) / PB;
-    const TI* kp = static_cast<const TI*>(a.k);
-    bool ok = true;
-    // block b uses buffer b % PN; its barriers complete once per use: parity of the use count
-    const uint32_t base = round0;   // uses of the ring before this stretch (a multiple of PN blocks is not required)
-    if (role == 1) {
-        // ------------------------------------------------------------------ pre
-        for (int b = 0; b < nblk && ok; ++b) {
-            const uint32_t use = base + b;
-            const int bi = use % PN;
-            if (use >= PN) ok = p1_mbar_wait(&bars.free_[bi], ((use / PN) - 1) & 1, a.status);
-            if (!ok) break;
-            PipeBuf<TI, K, VEC>& B = buf[bi];
-            const int t0 = t_a + b * PB, n = min(PB, t_b - t0);
-            RawRow<TI, R> raw[PB];
-#pragma unroll
-            for (int j = 0; j < PB; ++j) {
-                const size_t th = (size_t)(t0 + min(j, n - 1)) * H + h;
-                load_raw<R>(kp + th * K, lane, raw[j]);
-            }
-            if (lane < n) {
-                const size_t th = (size_t)(t0 + lane) * H + h;
-                const float rn = fabsf(a.r.n[th]), bb = hy.beta_aware ? a.beta[th] : 1.0f;
-                const float e = hy.eta * bb * rn;
-                // .w: the fixed-point scale of the core's sum, 2^26 / (d_max max(sum k^2, eps)); the core
-                // replaces it by <d_t, k^2>
-                B.scal[lane] = make_float4(e, e * bb, a.r.rho[th], 67108864.0f * rn / hy.d_max);
-            }
-#pragma unroll
-            for (int j = 0; j < PB; ++j) {
-                float kk[R], kap[R];
-                unpack<R>(raw[j], kk);
-#pragma unroll
-                for (int r = 0; r < R; ++r) kap[r] = kk[r] * kk[r];
-                store_row<R>(B.kap[j], lane, kap);
-                B.kraw[j][lane] = raw[j];
-            }
-            if constexpr (VEC) {
-                for (int j = 0; j < n; ++j) {
-                    const size_t th = (size_t)(t0 + j) * H + h;
-                    float lr[R];
-                    load_row<R>(a.retsrc + th * K, lane, lr);
-#pragma unroll
-                    for (int r = 0; r < R; ++r) lr[r] = expf(lr[r]);
-                    store_row<R>(B.rhov[VEC ? j : 0], lane, lr);
-                }
-            }
-            __syncwarp();
-            if (lane == 0) p1_mbar_arrive(&bars.full[bi]);
-        }
-    } else if (role == 0) {
-        // ------------------------------------------------------------------ core
-        for (int b = 0; b < nblk && ok; ++b) {
-            const uint32_t use = base + b;
-            const int bi = use % PN;
-            ok = p1_mbar_wait(&bars.full[bi], (use / PN) & 1, a.status);
-            if (!ok) break;
-            const int n = min(PB, t_b - (t_a + b * PB));
-            pipe_core_block<TI, K, VEC>(buf[bi], n, d, hy, lane);
-            __syncwarp();
-            if (lane == 0) p1_mbar_arrive(&bars.done[bi]);
-        }
-    } else {
-        // ------------------------------------------------------------------ post
-        TO* kt = static_cast<TO*>(a.ktil);
-        for (int b = 0; b < nblk && ok; ++b) {
-            const uint32_t use = base + b;
-            const int bi = use % PN;
-            ok = p1_mbar_wait(&bars.done[bi], (use / PN) & 1, a.status);
-            if (!ok) break;
-            const PipeBuf<TI, K, VEC>& B = buf[bi];
-            const int t0 = t_a + b * PB, n = min(PB, t_b - t0);
-            float dd[R];   // d_t of the token in hand
-            load_row<R>(B.d0, lane, dd);
-            auto token = [&](int j) {
-                const size_t th = (size_t)(t0 + j) * H + h;
-                float kk[R], wk[R], xx[R];
-                unpack<R>(B.kraw[j][lane], kk);
-#pragma unroll
-                for (int r = 0; r < R; ++r) wk[r] = dd[r] * kk[r];
-                store_row<R>(kt + th * K, lane, wk);
-                if (a.save) store_row<R>(a.r.dtraj + th * K, lane, dd);
-                load_row<R>(B.x[j], lane, xx);
-                unsigned bits;
-                clip_row<R>(xx, hy, dd, bits);   // the next token's d, this token's pass bits
-                if (a.save) a.r.pmask[th * 32 + lane] = bits;
-            };
-            if (a.save && lane < n) a.r.al[(size_t)(t0 + lane) * H + h] = B.scal[lane].w;   // lane j: token j
-            if (n == PB) {
-#pragma unroll 4
-                for (int j = 0; j < PB; ++j) token(j);
-            } else {
-                for (int j = 0; j < n; ++j) token(j);
-            }
-            __syncwarp();
-            if (lane == 0) p1_mbar_arrive(&bars.free_[bi]);
-        }
+    const P1Coord q = p1_coord(hy);
+    const P1Mode mode = p1_mode(hy);
+    PipeBuf<TI, K, VEC>& B = sh.buf[0];
+    const uint32_t mine = lane < n ? (uint32_t)((tok0 + ((int)sh.list[lane] & 0x7fff)) * H + h) : NO_ROW;
+    fetch_rows<TI, K>(&B.k[0][0], static_cast<const TI*>(a.k), mine, n, lane);
+    if constexpr (VEC) fetch_rows<float, K>(&B.rv[0][0], a.retsrc, mine, n, lane);
+    cp_async_commit();
+    if (lane < n) {
+        const float rho = a.r.rho[mine];
+        B.scal[lane] = p1_scalars(a.r.sumk[mine], a.r.kmax[mine], a.beta[mine], hy, q);
+        B.rho[lane] = rho;
+        B.off[lane] = p1_off(rho, q);
     }
-    round0 = base + nblk;
-    return ok;
+    float y[R];
+    load_row<R>(sh.y, lane, y);
+    cp_async_wait<0>();
+    __syncwarp();
+    int prev = -1, j = 0;
+#pragma unroll 1
+    for (; j < n; ++j) {
+        const int e = sh.list[j], at = e & 0x7fff;
+        if (face && (e & 0x8000)) continue;
+        if (!face && prev >= 0 && at != prev + 1) break;
+        prev = at;
+        const size_t th = (size_t)(tok0 + at) * H + h;
+        const float4 sc = B.scal[j];
+        float kk[R], rho[R], off[R], d[R], wk[R], s = 0.f;
+        load_row<R>(B.k[j], lane, kk);
+        if constexpr (VEC) {
+            load_row<R>(B.rv[VEC ? j : 0], lane, rho);
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                rho[r] = expf(rho[r]);
+                off[r] = p1_off(rho[r], q);
+            }
+        } else {
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                rho[r] = B.rho[j];
+                off[r] = B.off[j];
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < R; ++r) s = fmaf(y[r], __fmul_rn(kk[r], kk[r]), s);
+        s = warp_sum(s);
+        const float c = fmaf(-sc.y, s, sc.x);
+        unsigned bits = 0;
+        bool on = mode == P1_SAT;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            d[r] = p1_d(y[r], q);
+            wk[r] = d[r] * kk[r];
+            const float x = p1_raw(y[r], __fmul_rn(kk[r], kk[r]), c, rho[r], off[r]);
+            y[r] = p1_project(x, mode, hy);
+            bits |= y[r] == x ? (1u << r) : 0u;
+            on = on && y[r] == 0.f;
+        }
+        store_row<R>(static_cast<TO*>(a.ktil) + th * K, lane, wk);
+        if (a.save) {
+            store_row<R>(a.r.dtraj + th * K, lane, d);
+            a.r.pmask[th * 32 + lane] = bits;
+            if (lane == 0) a.r.al[th] = fmaf(q.w, s, q.lo * sc.w);
+        }
+        if (lane == at >> 6) proc |= 1ull << (at & 63);
+        face = __all_sync(0xffffffffu, on);
+    }
+    store_row<R>(sh.y, lane, y);
+    __syncwarp();
+    return j;
 }
 
-// The stand-alone sweep processes every token: the whole sequence is one pipelined stretch (see the
-// forward's stretches below the parallel pass).  pre also forms the normaliser here (there is no parallel
-// pass before this kernel); post forms the write keys and the residual ratios.
+// The tokens of 32 chunks from bit `pos` on, for the lane that holds chunk `lane`.
+__device__ __forceinline__ unsigned long long from_bit(int pos, int lane)
+{
+    const int rel = pos - 64 * lane;
+    return rel <= 0 ? ~0ull : rel >= 64 ? 0ull : ~0ull << rel;
+}
+__device__ __forceinline__ unsigned long long valid_bits(int len) { return len >= 64 ? ~0ull : len <= 0 ? 0ull : (1ull << len) - 1ull; }
+
+// Set bits of the lanes' words, in order, into a list of at most `most` offsets (those that are set in `mark` too with
+// bit 15); returns how many there were.
+__device__ __forceinline__ int write_list(uint16_t* list, unsigned long long w, unsigned long long mark, int most, int lane)
+{
+    const int mine = __popcll(w);
+    int end = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int u = __shfl_up_sync(0xffffffffu, end, o);
+        if (lane >= o) end += u;
+    }
+    for (int at = end - mine; w && at < most; ++at) {
+        const int t = __ffsll((long long)w) - 1;
+        w &= w - 1;
+        list[at] = (uint16_t)((64 * lane + t) | (int)((mark >> t) & 1ull) << 15);
+    }
+    __syncwarp();
+    return __shfl_sync(0xffffffffu, end, 31);
+}
+
+// The words of SCAN_CHUNKS chunks from c on, complemented (set: unflagged, or processed) and cut to the sequence, into
+// shared memory, four loads in flight per lane (one group of 32 at a time made a long sequence wait for memory once per 2048
+// tokens).  Chunks [c0, c1); word of chunk c + x at words[x].
+__device__ __forceinline__ void scan_words(unsigned long long* words, const unsigned* src, int c, int c0, int c1, int seq_len, int H, int h, int lane)
+{
+    uint2 w[SCAN_CHUNKS / 32];
+#pragma unroll
+    for (int g = 0; g < SCAN_CHUNKS / 32; ++g) {
+        const int x = c + g * 32 + lane;
+        w[g] = x < c1 ? *reinterpret_cast<const uint2*>(src + ((size_t)x * H + h) * 2) : make_uint2(~0u, ~0u);
+    }
+#pragma unroll
+    for (int g = 0; g < SCAN_CHUNKS / 32; ++g)
+        words[g * 32 + lane] = ~((unsigned long long)w[g].x | (unsigned long long)w[g].y << 32) & valid_bits(seq_len - (c + g * 32 + lane - c0) * CH);
+    __syncwarp();
+}
+
+// Which tokens are processed, decided by warp 0.
+//   on the face   the next unflagged tokens with `follow` tokens behind each, at most LIST_MAX; d is expected back on
+//                 the face where the list jumps (where it is not, the list ends there, and the chain's later lists
+//                 take more tokens behind each)
+//   off the face  every token, WALK at first, then 128 and twice as many each time d is still off at the end
+// What is not listed is skipped: its write key d_min k is there already and its projection mask is all zero.
+// Lists of up to PB entries are walked, unless they are dense and mostly unflagged (d will not be back soon).
+template <typename TI, typename TO, int K, bool VEC> struct ListPlan {
+    const P1Fwd& a;
+    PipeShared<TI, K, VEC>& sh;
+    const int h, lane, c0, c1, seq_t0, seq_len;
+    const bool sat;
+    // the group of 32 chunks in hand: unflagged and processed tokens (a chunk per lane), tokens, first token, next one
+    int cbase, base = 0, glen = 0, pos = 0;
+    unsigned long long unf = 0ull, proc = 0ull, cand = 0ull;
+    int follow = 3, run = WALK;
+    bool face, listed = false, touched = false;
+
+    __device__ __forceinline__ ListPlan(const P1Fwd& a_, PipeShared<TI, K, VEC>& sh_, int s, int h_, int lane_)
+        : a(a_), sh(sh_), h(h_), lane(lane_), c0(a_.tab.seq_chunk0(s)), c1(a_.tab.seq_chunk0(s + 1)), seq_t0(a_.tab.seq_tok0(s)),
+          seq_len(a_.tab.seq_len(s)), sat(p1_mode(a_.hy) == P1_SAT), cbase(c0 - 32)
+    {
+        face = on_face();
+    }
+    __device__ __forceinline__ bool on_face() const
+    {
+        constexpr int R = K / 32;
+        float y[R];
+        load_row<R>(sh.y, lane, y);
+        bool on = sat;
+#pragma unroll
+        for (int r = 0; r < R; ++r) on = on && y[r] == 0.f;
+        return __all_sync(0xffffffffu, on) != 0;
+    }
+    __device__ __forceinline__ bool next_group()
+    {
+        if (cbase >= c0 && a.save && cbase + lane < c1 && (unf ^ proc) != 0ull) {   // (the parallel pass left the flags there)
+            const unsigned long long skipped = valid_bits(glen - 64 * lane) & ~proc;
+            *reinterpret_cast<uint2*>(a.r.skipw + ((size_t)(cbase + lane) * a.H + h) * 2) =
+                make_uint2((unsigned)(skipped & 0xffffffffull), (unsigned)(skipped >> 32));
+        }
+        cbase += 32;
+        if (cbase >= c1) return false;
+        const int at = (cbase - c0) % SCAN_CHUNKS;
+        if (at == 0) scan_words(sh.words, a.r.flags, cbase, c0, c1, seq_len, a.H, h, lane);
+        base = (cbase - c0) * CH;
+        glen = min(32 * CH, seq_len - base);
+        unf = sh.words[at + lane];
+        proc = 0ull;
+        pos = 0;
+        return true;
+    }
+    // Leaves the next list for run_list in sh; cmd_n 0: the chain is finished (cmd_dense: anything was processed).
+    __device__ __forceinline__ void next()
+    {
+        if (sh.cmd_n != 0) {   // the list before has been worked off
+            const int stop = sh.stop, n = sh.cmd_n;
+            face = on_face();
+            if (listed) {
+                if (stop) pos = ((int)sh.list[stop - 1] & 0x7fff) + 1;
+                proc |= cand & ~from_bit(pos, lane);
+                if (stop < n) follow = min(2 * follow + 1, 15);
+                run = WALK;
+            } else {
+                pos += stop;
+                proc |= cand;
+                run = face ? WALK : min(max(2 * run, 4 * PB), 32 * CH);
+            }
+            if (stop == 0) {   // a wait ran out
+                pos = glen;
+                cbase = c1;
+            }
+        }
+        while (true) {
+            if (pos >= glen) {
+                if (next_group()) continue;
+                __syncwarp();
+                if (lane == 0) {
+                    sh.cmd_n = 0;
+                    sh.cmd_dense = touched;
+                }
+                return;
+            }
+            const unsigned long long valid = valid_bits(glen - 64 * lane);
+            int n;
+            bool walk;
+            listed = face;
+            if (face) {
+                const unsigned long long my = unf & from_bit(pos, lane);
+                if (!__any_sync(0xffffffffu, my != 0ull)) {   // the rest of the group is skipped
+                    pos = glen;
+                    continue;
+                }
+                cand = my;
+                for (int f = 0; f < follow; ++f) {
+                    unsigned long long up = __shfl_up_sync(0xffffffffu, cand, 1) >> 63;
+                    if (lane == 0) up = 0ull;
+                    cand = my | (cand << 1) | up;
+                }
+                cand &= valid;
+                n = write_list(sh.list, cand, ~unf, LIST_MAX, lane);
+                walk = n <= PB;
+                n = min(n, LIST_MAX);
+            } else {
+                n = min(glen - pos, run);
+                cand = from_bit(pos, lane) & ~from_bit(pos + n, lane) & valid;
+                walk = run == WALK && __reduce_add_sync(0xffffffffu, __popcll(unf & cand)) * 2 < n;
+                if (walk) write_list(sh.list, cand, ~unf, LIST_MAX, lane);
+            }
+            touched = true;
+            if (walk) {
+                const int stop = walk_list<TI, TO, K, VEC>(a, h, sh, seq_t0 + base, n, face, proc, lane);
+                pos = ((int)sh.list[stop - 1] & 0x7fff) + 1;
+                run = face || listed ? WALK : 4 * PB;
+                continue;
+            }
+            __syncwarp();
+            if (lane == 0) {
+                sh.cmd_tok = seq_t0 + base + (listed ? 0 : pos);
+                sh.cmd_n = n;
+                sh.cmd_dense = !listed;
+            }
+            return;
+        }
+    }
+};
+
+// One chain per CTA.
 template <typename TI, typename TO, int K, bool VEC>
-__global__ void __launch_bounds__(96) phase1_stream_kernel(P1Args a)
+__global__ void __launch_bounds__(Pipe<K>::THREADS, 1) phase1_seq_kernel(P1Fwd a)
+{
+    using P = Pipe<K>;
+    extern __shared__ __align__(16) uint8_t p1_dyn[];
+    PipeShared<TI, K, VEC>& sh = *reinterpret_cast<PipeShared<TI, K, VEC>*>(p1_dyn);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int chain = blockIdx.x;
+    const int s = chain / a.H, h = chain % a.H, H = a.H;
+    const P1Coord q = p1_coord(a.hy);
+    const int coord = warp * 32 + lane;   // core warps
+    if (threadIdx.x == 0) {
+        init_bars(sh.bars, PipeShared<TI, K, VEC>::PN, P::CORE);
+        sh.cmd_n = 0;
+    }
+    float d_in = 1.0f, guess = 0.f;
+    if (warp < P::CORE) {
+        if (a.d0) d_in = a.d0[((size_t)s * H + h) * K + coord];
+        sh.y[coord] = p1_y(d_in, q);
+    }
+    uint32_t rounds = 0, uses = 0;
+    __syncthreads();
+    ListPlan<TI, TO, K, VEC> plan(a, sh, s, h, lane);
+    while (true) {   // warp 0 announces a list, all work it off (one call site: the warps share the code)
+        if (warp == 0) plan.next();
+        bar_sync<P::THREADS>(1);
+        if (sh.cmd_n == 0) break;
+        run_list<TI, TO, K, VEC>(a, h, sh, guess, rounds, uses, warp, lane);
+        bar_sync<P::THREADS>(2);
+    }
+    if (a.d_final && warp < P::CORE) a.d_final[((size_t)s * H + h) * K + coord] = sh.cmd_dense ? p1_d(sh.y[coord], q) : d_in;
+}
+
+// The stand-alone sweep processes every token: the whole sequence is one list (see above).  The fetching warps also
+// form the normalisers here (there is no parallel pass before this kernel; max k^2, which only the rounds' tolerance
+// needs, is taken as sum k^2); the finishing ones form the write keys and the residual ratios.
+template <typename TI, typename TO, int K, bool VEC>
+__global__ void __launch_bounds__(Pipe<K>::THREADS, 1) phase1_stream_kernel(P1Args a)
 {
     constexpr int R = K / 32;
-    extern __shared__ __align__(16) uint8_t p1_dyn[];   // PipeBuf[PN], then the write strengths beta[PN][PB]
-    PipeBuf<TI, K, VEC>* buf = reinterpret_cast<PipeBuf<TI, K, VEC>*>(p1_dyn);
-    float(*sbeta)[PB] = reinterpret_cast<float(*)[PB]>(p1_dyn + PN * sizeof(PipeBuf<TI, K, VEC>));
-    __shared__ PipeBars bars;
-    const int lane = threadIdx.x & 31, role = threadIdx.x >> 5;   // 0 core, 1 pre, 2 post
+    using P = Pipe<K>;
+    constexpr int PN = PipeShared<TI, K, VEC>::PN;
+    extern __shared__ __align__(16) uint8_t p1_dyn[];
+    PipeShared<TI, K, VEC>& sh = *reinterpret_cast<PipeShared<TI, K, VEC>*>(p1_dyn);
+    __shared__ float log_part[P::FINISH];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int chain = blockIdx.x;
     const int s = chain / a.H, h = chain % a.H, H = a.H;
     // packed batch: T_dense is the packed token count; a malformed offset pair is clamped into it
     const int t0 = a.cu ? min(max(a.cu[s], 0), a.T_dense) : s * a.T_dense;
     const int len = a.cu ? min(max(a.cu[s + 1], t0), a.T_dense) - t0 : a.T_dense;
-    const TI* kp = static_cast<const TI*>(a.k);
     const Hyper hy = a.hy;
-    if (threadIdx.x == 0) {
-        for (int i = 0; i < PN; ++i) {
-            p1_mbar_init(&bars.full[i], 1);
-            p1_mbar_init(&bars.done[i], 1);
-            p1_mbar_init(&bars.free_[i], 1);
-        }
-    }
+    const P1Coord q = p1_coord(hy);
+    if (threadIdx.x == 0) init_bars(sh.bars, PN, P::CORE);
     __syncthreads();
     const int nblk = (len + PB - 1) / PB;
     const bool scalar_ret = !VEC && hy.apf_mode != 0;
     bool ok = true;
-    if (role == 1) {
-        for (int b = 0; b < nblk && ok; ++b) {
-            const int bi = b % PN;
-            if (b >= PN) ok = p1_mbar_wait(&bars.free_[bi], ((b / PN) - 1) & 1, nullptr);
+    float lsum = 0.f;
+    auto len_of = [&](int b) { return min(PB, len - b * PB); };
+    auto th_of = [&](int b) { return lane < len_of(b) ? (uint32_t)((t0 + b * PB + lane) * H + h) : NO_ROW; };   // lane j: token j
+    if (warp < P::CORE) {
+        const size_t at = ((size_t)s * H + h) * K + warp * 32 + lane;
+        const float d0 = a.d0 ? a.d0[at] : 1.0f;
+        float y = p1_y(d0, q), guess = 0.f;
+        uint32_t rounds = 0;
+        for (int b = 0; b < nblk; ++b) {
+            ok = bar_sync_and<P::CORE * 32>(3, p1_mbar_wait(&sh.bars.full[b % PN], (b / PN) & 1, nullptr));
             if (!ok) break;
-            PipeBuf<TI, K, VEC>& B = buf[bi];
-            const int tb0 = t0 + b * PB, n = min(PB, len - b * PB);
-            RawRow<TI, R> raw[PB];
-#pragma unroll
-            for (int j = 0; j < PB; ++j) load_raw<R>(kp + ((size_t)(tb0 + min(j, n - 1)) * H + h) * K, lane, raw[j]);
-            float beta = 0.f, ret = 0.f;
-            if (lane < n) {
-                const size_t th = (size_t)(tb0 + lane) * H + h;
-                beta = a.beta[th];
-                if (scalar_ret) ret = a.retsrc[th];
+            core_block<TI, K, VEC>(sh, sh.buf[b % PN], len_of(b), y, guess, rounds, hy, q, warp, lane);
+            __syncwarp();
+            if (lane == 0) p1_mbar_arrive(&sh.bars.done[b % PN]);
+        }
+        if (a.d_final && ok) a.d_final[at] = nblk > 0 ? p1_d(y, q) : d0;
+    } else if (warp < P::FINISH0) {
+        auto start = [&](int b) {
+            if (b >= PN) ok = p1_mbar_wait(&sh.bars.free_[b % PN], ((b / PN) - 1) & 1, nullptr);
+            if (!ok) return;
+            PipeBuf<TI, K, VEC>& B = sh.buf[b % PN];
+            const uint32_t th = th_of(b);
+            fetch_rows<TI, K>(&B.k[0][0], static_cast<const TI*>(a.k), th, PB, lane);
+            if constexpr (VEC) fetch_rows<float, K>(&B.rv[0][0], a.retsrc, th, PB, lane);
+            if (th != NO_ROW) {
+                cp_async4(&B.raw[3][lane], a.beta + th);
+                if (scalar_ret) cp_async4(&B.raw[2][lane], a.retsrc + th);
             }
-            float sums[PB];
+            cp_async_commit();
+        };
+        int b = warp - P::FETCH0;
+        if (b < nblk) start(b);
+        for (; b < nblk && ok; b += 2) {
+            cp_async_wait<0>();
+            __syncwarp();
+            PipeBuf<TI, K, VEC>& B = sh.buf[b % PN];
+            float x[PB];
 #pragma unroll
             for (int j = 0; j < PB; ++j) {
-                float kk[R], kap[R];
-                unpack<R>(raw[j], kk);
-                sums[j] = 0.f;
+                float kk[R];
+                load_row<R>(B.k[j], lane, kk);
+                x[j] = 0.f;
 #pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    kap[r] = kk[r] * kk[r];
-                    sums[j] += kap[r];
-                }
-                store_row<R>(B.kap[j], lane, kap);
-                B.kraw[j][lane] = raw[j];
+                for (int r = 0; r < R; ++r) x[j] = fmaf(kk[r], kk[r], x[j]);
             }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1)   // the sixteen sums together: their shuffle rounds overlap
-#pragma unroll
-                for (int j = 0; j < PB; ++j) sums[j] += __shfl_xor_sync(0xffffffffu, sums[j], o);
-            float mine = 0.f;
-#pragma unroll
-            for (int j = 0; j < PB; ++j) mine = lane == j ? sums[j] : mine;
-            if (lane < n) {
-                const float nn = fmaxf(mine, hy.eps), bb = hy.beta_aware ? beta : 1.0f;
-                const float e = hy.eta * bb / nn;
-                B.scal[lane] = make_float4(e, e * bb, scalar_ret ? expf(ret) : 1.0f, 67108864.0f / (nn * hy.d_max));
-                sbeta[bi][lane] = beta;
+            const float sumk = transpose_sum(x, lane);
+            float4 sc = make_float4(0.f, 0.f, 0.f, 0.f);
+            float rho = 1.f;
+            if (lane < len_of(b)) {
+                sc = p1_scalars(sumk, sumk, B.raw[3][lane], hy, q);
+                if (scalar_ret) rho = expf(B.raw[2][lane]);
             }
-            if constexpr (VEC) {
-                for (int j = 0; j < n; ++j) {
-                    float lr[R];
-                    load_row<R>(a.retsrc + ((size_t)(tb0 + j) * H + h) * K, lane, lr);
-#pragma unroll
-                    for (int r = 0; r < R; ++r) lr[r] = expf(lr[r]);
-                    store_row<R>(B.rhov[VEC ? j : 0], lane, lr);
-                }
-            }
+            B.scal[lane] = sc;
+            B.rho[lane] = rho;
+            B.off[lane] = p1_off(rho, q);
+            if (lane == 0) B.jump = 0u;
             __syncwarp();
-            if (lane == 0) p1_mbar_arrive(&bars.full[bi]);
+            if (lane == 0) p1_mbar_arrive(&sh.bars.full[b % PN]);
+            if (b + 2 < nblk) start(b + 2);
         }
-    } else if (role == 0) {
-        float d[R];
-        if (a.d0) load_row<R>(a.d0 + ((size_t)s * H + h) * K, lane, d);
-        else {
-#pragma unroll
-            for (int r = 0; r < R; ++r) d[r] = 1.0f;
-        }
-        for (int b = 0; b < nblk && ok; ++b) {
-            const int bi = b % PN;
-            ok = p1_mbar_wait(&bars.full[bi], (b / PN) & 1, nullptr);
-            if (!ok) break;
-            pipe_core_block<TI, K, VEC>(buf[bi], min(PB, len - b * PB), d, hy, lane);
-            __syncwarp();
-            if (lane == 0) p1_mbar_arrive(&bars.done[bi]);
-        }
-        if (a.d_final && ok) store_row<R>(a.d_final + ((size_t)s * H + h) * K, lane, d);
+        cp_async_wait<0>();
     } else {
         TO* kt = static_cast<TO*>(a.ktil);
-        float lsum = 0.f;
-        for (int b = 0; b < nblk && ok; ++b) {
-            const int bi = b % PN;
-            ok = p1_mbar_wait(&bars.done[bi], (b / PN) & 1, nullptr);
+        for (int b = warp - P::FINISH0; b < nblk; b += P::FINISH) {
+            ok = p1_mbar_wait(&sh.bars.done[b % PN], (b / PN) & 1, nullptr);
             if (!ok) break;
-            const PipeBuf<TI, K, VEC>& B = buf[bi];
-            const int tb0 = t0 + b * PB, n = min(PB, len - b * PB);
-            if (kt) {
-                float dd[R];
-                load_row<R>(B.d0, lane, dd);
-                for (int j = 0; j < n; ++j) {
-                    float kk[R], wk[R], xx[R];
-                    unpack<R>(B.kraw[j][lane], kk);
+            const PipeBuf<TI, K, VEC>& B = sh.buf[b % PN];
+            const int n = len_of(b);
+            const uint32_t mine = th_of(b);
+            if (kt)
+                finish_block<TI, K, VEC>(B, n, hy, q, lane, [&](int j, const float (&d)[R], const float (&kk)[R], unsigned) {
+                    const size_t th = __shfl_sync(0xffffffffu, mine, j);
+                    float wk[R];
 #pragma unroll
-                    for (int r = 0; r < R; ++r) wk[r] = dd[r] * kk[r];
-                    store_row<R>(kt + ((size_t)(tb0 + j) * H + h) * K, lane, wk);
-                    load_row<R>(B.x[j], lane, xx);
-                    unsigned bits;
-                    clip_row<R>(xx, hy, dd, bits);
-                }
-            }
+                    for (int r = 0; r < R; ++r) wk[r] = d[r] * kk[r];
+                    store_row<R>(kt + th * K, lane, wk);
+                });
             if (a.ratio || a.log_sum) {
                 // residual ratio of the write of a token (token-local theorem): the loss |S k - v|^2 after the
                 // write over the loss before it is (1 - beta <d_t, k^2>)^2, with the write strength beta itself
                 // (whether or not the step of d is beta-aware) and the d the write key was formed with
                 float lq = 0.f;
                 if (lane < n) {
-                    const float fac = 1.0f - sbeta[bi][lane] * B.scal[lane].w;
+                    const float fac = 1.0f - B.raw[3][lane] * fmaf(q.w, B.res[lane].y, q.lo * B.scal[lane].w);
                     const float qt = fac * fac;
-                    if (a.ratio) a.ratio[(size_t)(tb0 + lane) * H + h] = qt;
+                    if (a.ratio) a.ratio[mine] = qt;
                     lq = logf(fmaxf(qt, 1.17549435e-38f));
                 }
                 lsum += warp_sum(lq);
             }
             __syncwarp();
-            if (lane == 0) p1_mbar_arrive(&bars.free_[bi]);
-        }
-        if (a.log_sum && lane == 0) a.log_sum[(size_t)s * H + h] = lsum;
-    }
-}
-
-// one warp per chain.  Flag words are fetched for 32 chunks at a time (one chunk per lane); the
-// rows of the tokens that are really processed are prefetched a few tokens ahead.
-// A chunk of which at least PIPE_TRIGGER tokens had to be processed starts a pipelined stretch of up to
-// PIPE_CHUNKS chunks; stretches follow one another while d stays off the lower face.
-constexpr int PIPE_TRIGGER = 32, PIPE_CHUNKS = 8;
-
-template <typename TI, typename TO, int K, bool VEC>
-__global__ void __launch_bounds__(96) phase1_seq_kernel(P1Fwd a)
-{
-    constexpr int R = K / 32;
-    // prefetch distance in tokens: short, because the long runs go through the pipelined stretches and a
-    // run's start waits for whatever the run before it still had in flight (8 -> 4: osdn_1p3b 452 -> 401 us)
-    constexpr int PF = 4;
-    struct RingSlot {
-        RawRow<TI, R> k[32];
-        RawRow<float, R> lr[VEC ? 32 : 1];
-        float n[32], rho[32], beta[32];
-    };
-    extern __shared__ __align__(16) uint8_t p1_dyn[];   // PipeBuf[PN]
-    PipeBuf<TI, K, VEC>* pbuf = reinterpret_cast<PipeBuf<TI, K, VEC>*>(p1_dyn);
-    __shared__ __align__(16) RingSlot ring[PF];
-    __shared__ PipeBars bars;
-    __shared__ int cmd[2];   // token range of the next pipelined stretch; empty: the chain is finished
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int chain = blockIdx.x;
-    const int s = chain / a.H, h = chain % a.H, H = a.H;
-    if (threadIdx.x == 0) {
-        for (int i = 0; i < PN; ++i) {
-            p1_mbar_init(&bars.full[i], 1);
-            p1_mbar_init(&bars.done[i], 1);
-            p1_mbar_init(&bars.free_[i], 1);
+            if (lane == 0) p1_mbar_arrive(&sh.bars.free_[b % PN]);
         }
     }
-    __syncthreads();
-    uint32_t pipe_uses = 0;   // blocks that have gone through the ring so far (the same in all three warps)
-    if (warp != 0) {
-        // helper warps (1: pre, 2: post) serve the stretches warp 0 announces
-        float none[R];
-        while (true) {
-            asm volatile("bar.sync 1, 96;" ::: "memory");
-            const int t_a = cmd[0], t_b = cmd[1];
-            if (t_b <= t_a) break;
-            pipe_stretch<TI, TO, K, VEC>(a, h, t_a, t_b, none, pbuf, bars, pipe_uses, warp, lane);
-            asm volatile("bar.sync 2, 96;" ::: "memory");
-        }
-        return;
-    }
-    bool pipe_next = false;
-    const TI* kp = static_cast<const TI*>(a.k);
-    TO* kt = static_cast<TO*>(a.ktil);
-    const Hyper hy = a.hy;
-    float d[R];
-    if (a.d0) load_row<R>(a.d0 + ((size_t)s * H + h) * K, lane, d);
-    else {
+    if (a.log_sum) {   // the finishing warps' shares, always in the same order
+        if (warp >= P::FINISH0 && lane == 0) log_part[warp - P::FINISH0] = lsum;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            float sum = log_part[0];
 #pragma unroll
-        for (int r = 0; r < R; ++r) d[r] = 1.0f;
-    }
-    bool face = on_lower_face<R>(d, hy);
-    const int c0 = a.tab.seq_chunk0(s), c1 = a.tab.seq_chunk0(s + 1);
-    const int seq_t0 = a.tab.seq_tok0(s), seq_len = a.tab.seq_len(s);
-    for (int cbase = c0; cbase < c1; cbase += 32) {
-        unsigned w0 = 0, w1 = 0;
-        if (cbase + lane < c1) {
-            const size_t tl = (size_t)(cbase + lane) * H + h;
-            w0 = a.r.flags[tl * 2];
-            w1 = a.r.flags[tl * 2 + 1];
-            // Sparse work: unflagged tokens are processed for certain; warm L2 with their rows now.
-            const int cl = cbase + lane;
-            const int lenl = min(CH, seq_len - (cl - c0) * CH);
-            unsigned long long m = ~((unsigned long long)w0 | ((unsigned long long)w1 << 32)) &
-                                   (lenl >= 64 ? ~0ull : ((1ull << lenl) - 1ull));
-            if (__popcll(m) <= 16) {
-                while (m) {
-                    const int t = __ffsll((long long)m) - 1;
-                    m &= m - 1;
-                    const size_t th = (size_t)(seq_t0 + (cl - c0) * CH + t) * H + h;
-                    prefetch_row(kp + th * K, K * (int)sizeof(TI));
-                    if constexpr (VEC) prefetch_row(a.retsrc + th * K, K * 4);
-                    prefetch_l2(a.r.n + th);
-                    prefetch_l2(a.r.rho + th);
-                    prefetch_l2(a.beta + th);
-                }
-            }
-        }
-        const int cend = min(cbase + 32, c1);
-        // chunks of this group whose every token is flagged (lane = chunk)
-        unsigned allflag;
-        {
-            const int cl = cbase + lane;
-            const int lenl = cl < c1 ? min(CH, seq_len - (cl - c0) * CH) : 0;
-            const unsigned long long bl = (unsigned long long)w0 | ((unsigned long long)w1 << 32);
-            const unsigned long long vl = lenl >= 64 ? ~0ull : ((1ull << lenl) - 1ull);
-            allflag = __ballot_sync(0xffffffffu, cl < c1 && (bl & vl) == vl);
-            // The first chunk of a sequence that enters off the face with at least PIPE_TRIGGER tokens that
-            // are processed for certain (unflagged) starts pipelined right away.
-            if (cbase == c0 && !face) {
-                const int sure = __shfl_sync(0xffffffffu, __popcll(~bl & vl), 0);
-                pipe_next = sure >= PIPE_TRIGGER;
-            }
-        }
-        for (int c = cbase; c < cend; ++c) {
-            if (pipe_next) {
-                // a pipelined stretch: every token of the next chunks (of this group) is processed
-                const int np = min(PIPE_CHUNKS, cend - c);
-                const int nrel = c - c0;
-                const int t_a = seq_t0 + nrel * CH, t_b = seq_t0 + min(seq_len, (nrel + np) * CH);
-                if (lane == 0) {
-                    cmd[0] = t_a;
-                    cmd[1] = t_b;
-                }
-                cp_async_wait<0>();   // nothing of the token-by-token walk is still on its way
-                asm volatile("bar.sync 1, 96;" ::: "memory");
-                const bool okp = pipe_stretch<TI, TO, K, VEC>(a, h, t_a, t_b, d, pbuf, bars, pipe_uses, 0, lane);
-                asm volatile("bar.sync 2, 96;" ::: "memory");
-                if (a.save && lane < np) {
-                    const size_t tl = (size_t)(c + lane) * H + h;
-                    a.r.skipw[tl * 2] = 0u;
-                    a.r.skipw[tl * 2 + 1] = 0u;
-                }
-                face = on_lower_face<R>(d, hy);
-                pipe_next = okp && !face;
-                c += np - 1;
-                continue;
-            }
-            if (face) {
-                // a run of fully flagged chunks entered on the face is skipped in one go
-                const unsigned rest = ~allflag >> (c - cbase);
-                const int run = min(rest ? __ffs((int)rest) - 1 : 32, cend - c);
-                if (run > 0) {
-                    if (a.save && lane < run) {
-                        const int cl = c + lane;
-                        const int lenl = min(CH, seq_len - (cl - c0) * CH);
-                        const unsigned long long vl = lenl >= 64 ? ~0ull : ((1ull << lenl) - 1ull);
-                        const size_t tl = (size_t)cl * H + h;
-                        a.r.skipw[tl * 2] = (unsigned)(vl & 0xffffffffull);
-                        a.r.skipw[tl * 2 + 1] = (unsigned)(vl >> 32);
-                    }
-                    c += run - 1;
-                    continue;
-                }
-            }
-            const int nrel = c - c0;
-            const int tok0 = seq_t0 + nrel * CH, len = min(CH, seq_len - nrel * CH);
-            const size_t tile = (size_t)c * H + h;
-            const unsigned long long bits = (unsigned long long)__shfl_sync(0xffffffffu, w0, c - cbase) |
-                                            ((unsigned long long)__shfl_sync(0xffffffffu, w1, c - cbase) << 32);
-            const unsigned long long valid = len >= 64 ? ~0ull : ((1ull << len) - 1ull);
-            unsigned long long skipped = 0ull;
-            int processed = 0;
-            if (face && (bits & valid) == valid) {
-                skipped = valid;
-            } else {
-                // ring of prefetched rows and scalars in shared memory (every lane copies and later reads
-                // its own bytes, the three scalars included, so no lane waits for another)
-                auto fetch = [&](int i, int slot) {
-                    const int ii = min(i, len - 1);
-                    const size_t th = (size_t)(tok0 + ii) * H + h;
-                    RingSlot& rs = ring[slot];
-                    cp_async<R * (int)sizeof(TI)>(&rs.k[lane], kp + th * K + R * lane);
-                    if constexpr (VEC) cp_async<R * 4>(&rs.lr[VEC ? lane : 0], a.retsrc + th * K + R * lane);
-                    cp_async<4>(&rs.n[lane], a.r.n + th);
-                    cp_async<4>(&rs.rho[lane], a.r.rho + th);
-                    cp_async<4>(&rs.beta[lane], a.beta + th);
-                    cp_async_commit();
-                };
-                int i = 0;
-                while (i < len) {
-                    if (face) {
-                        // jump over the flagged tokens that follow while d stays on the face
-                        const unsigned long long rest = (~bits & valid) >> i;
-                        const int run = rest ? __ffsll((long long)rest) - 1 : len - i;
-                        if (run > 0) {
-                            skipped |= (run >= 64 ? ~0ull : ((1ull << run) - 1ull)) << i;
-                            i += run;
-                            continue;
-                        }
-                    }
-                    // process tokens i, i+1, ... until d is back on the face (or the chunk ends)
-                    cp_async_wait<0>();   // nothing of an earlier run is still on its way into the ring
-#pragma unroll
-                    for (int u = 0; u < PF; ++u) fetch(i + u, u);
-                    bool stop = false;
-                    while (i < len && !stop) {
-#pragma unroll
-                        for (int u = 0; u < PF; ++u) {
-                            if (i < len && !stop) {
-                                cp_async_wait<PF - 1>();   // the oldest group, this token's, has landed
-                                const RingSlot& rs = ring[u];
-                                float kk[R];
-                                unpack<R>(rs.k[lane], kk);
-                                const float rn = fabsf(rs.n[lane]), b = hy.beta_aware ? rs.beta[lane] : 1.0f;
-                                // c = e - a2 <d, k^2>: e and a2 do not depend on d (1 / n comes from the
-                                // parallel pass), so nothing but one multiply-add follows the warp sum
-                                const float e = hy.eta * b * rn, a2 = e * b;
-                                float rho[R];
-                                if constexpr (VEC) {
-                                    float lr[R];
-                                    unpack<R>(rs.lr[VEC ? lane : 0], lr);
-#pragma unroll
-                                    for (int r = 0; r < R; ++r) rho[r] = expf(lr[r]);
-                                } else {
-                                    const float r1 = rs.rho[lane];
-#pragma unroll
-                                    for (int r = 0; r < R; ++r) rho[r] = r1;
-                                }
-                                fetch(i + PF, u);
-                                const size_t th = (size_t)(tok0 + i) * H + h;
-                                float kap[R], wk[R], rd[R], al = 0.f;
-#pragma unroll
-                                for (int r = 0; r < R; ++r) {
-                                    kap[r] = kk[r] * kk[r];
-                                    wk[r] = d[r] * kk[r];
-                                    rd[r] = rho[r] * d[r];
-                                    al = fmaf(d[r], kap[r], al);
-                                }
-                                al = warp_sum(al);
-                                store_row<R>(kt + th * K, lane, wk);
-                                if (a.save) store_row<R>(a.r.dtraj + th * K, lane, d);
-                                const float cc = fmaf(-a2, al, e);
-                                unsigned mybits = 0;         // bit r: the projection passes gradient for coordinate R lane + r
-                                bool at_min = hy.clamp != 0;
-#pragma unroll
-                                for (int r = 0; r < R; ++r) {
-                                    float x = fmaf(cc, kap[r], rd[r]);
-                                    bool pz = true;
-                                    if (hy.clamp) {
-                                        pz = (x >= hy.d_min) && (x <= hy.d_max);
-                                        x = fminf(fmaxf(x, hy.d_min), hy.d_max);
-                                    }
-                                    mybits |= pz ? (1u << r) : 0u;
-                                    at_min = at_min && (x == hy.d_min);
-                                    d[r] = x;
-                                }
-                                if (a.save) {
-                                    a.r.pmask[th * 32 + lane] = mybits;
-                                    if (lane == 0) a.r.al[th] = al;
-                                }
-                                face = __all_sync(0xffffffffu, at_min);
-                                ++i;
-                                ++processed;
-                                // back on the face with a flagged token next: leave the run
-                                stop = face && i < len && ((bits >> i) & 1ull);
-                            }
-                        }
-                    }
-                }
-            }
-            if (a.save && lane == 0) {
-                a.r.skipw[tile * 2] = (unsigned)(skipped & 0xffffffffull);
-                a.r.skipw[tile * 2 + 1] = (unsigned)(skipped >> 32);
-            }
-            pipe_next = processed >= PIPE_TRIGGER && !face;
+            for (int x = 1; x < P::FINISH; ++x) sum += log_part[x];
+            a.log_sum[(size_t)s * H + h] = sum;
         }
     }
-    if (a.d_final) store_row<R>(a.d_final + ((size_t)s * H + h) * K, lane, d);
-    cp_async_wait<0>();   // rows fetched past the last processed token are not used, but must have landed
-    if (lane == 0) {      // release the helper warps
-        cmd[0] = 0;
-        cmd[1] = 0;
-    }
-    asm volatile("bar.sync 1, 96;" ::: "memory");
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1029,546 +1176,457 @@ __global__ void __launch_bounds__(128) phase1_bwd_bulk_kernel(P1Bwd a)
 }
 
 // ---------------------------------------------------------------------------------------------
-// Pipelined stretches of the reverse pass, the mirror image of the forward ones: over chunks in which
-// every token was processed, lambda = dL/dd flows without a restart, and of a token's work only
-//     lambda <- mask (.) lambda ;  dc = <lambda, k^2> ;  lambda <- rho lambda - a2 dc k^2 + k (.) dL/dktil
-// depends on lambda.  Three warps share the chain:
-//   pre   fetches a block of QB tokens (k, d_t, dL/dktil, dk_read, mask, scalars) and recomputes the
-//         step's own scalars (<d_t, k^2>, c, the factors of the beta and normaliser gradients);
-//   core  carries lambda through the block (top token first) and leaves the masked lambda and dc;
-//   post  forms dk, the retention and beta gradients from those and writes them out.
+// The reverse pass over the processed tokens of a chain, last one first:
+//   lambda <- mask (.) lambda ;  u = <lambda, k^2> ;  lambda <- rho lambda - a2 u k^2 + k (.) dL/dktil
+// (lambda = dL/dd behind the token).  It is the forward pass's problem once more (u_t depends on lambda_t, hence on the u
+// of the tokens behind it, by the same weak coupling), linear this time, and is solved the same way: the u of a block of
+// PB tokens together, in rounds.  A round's u is taken when lambda is unchanged to its precision: a2 |change of u| max k^2
+// at most 2^-24 of the block's largest |u| / n (a weighted mean of |lambda|), or a unit in the last place of u.
+// A skipped token's mask is all zero, so lambda restarts there from k (.) dL/dktil: where a processed token's upper
+// neighbour was skipped, that neighbour goes into the list as well, with its mask and its step taken as zero, and
+// nothing is written for it.  Warps and ring as in the forward pass (the finishing warps form dk and the retention and
+// beta gradients and read d_t and dk_read, which the core does not need, from global memory, four tokens ahead).
+// In isolation a block of 32 takes 2200 cycles at a step size of 0.003 (two rounds), 3700 at 0.3 (four).
 // ---------------------------------------------------------------------------------------------
-// Five buffers: the pre role holds two (one landing, one being finished), core and post one each, one spare.
-constexpr int QB = 8, QN = 5;
-static_assert(QN <= RING_MAX && PN <= RING_MAX, "barrier arrays");
-
 template <typename T, int K, bool VEC> struct RevBuf {
-    static constexpr int R = K / 32;
-    RawRow<T, R> kraw[QB][32];
-    float dt[QB][K], dkt[QB][K], dkr[QB][K];
-    float lam[QB][K];                       // lambda on entry to the token (before the mask), written by the core
-    // what the core reads, prepared by the pre role so that nothing but the recurrence is left to the core:
-    float kap[QB][K], mkap[QB][K];          // k^2, and k^2 where the projection passed (else 0)
-    float rm[QB][K];                        // retention where the projection passed (else 0)
-    float w[QB][K];                         // k (.) dL/dktil
-    float rv[VEC ? QB : 1][VEC ? K : 1];    // vector retention: exp(l_t)
-    unsigned mask[QB][32];
-    float4 sc0[QB];                         // a2, rho, cc, g1
-    float4 sc1[QB];                         // g2, dc (written by the core), -, -
-    float raw[4][QB];                       // n (signed), rho, beta, <d_t, k^2> as they sit in memory
+    T k[PB][K];
+    float dkt[PB][K];
+    unsigned mask[PB][32];
+    float lam0[K];                          // core: lambda on entry to the block
+    float raw[5][PB];                       // sum k^2, max k^2, retention, beta, <d_t, k^2> as they sit in memory
+    float4 scal[PB];                        // a2, rho, max k^2, 1 / n
+    float4 grad[PB];                        // c, factor of the beta gradient, of the normaliser's, u (by the core)
+    float rho[PB];
+    unsigned restart;                       // bit j: a skipped token, there to restart lambda
+    alignas(16) float rv[VEC ? PB : 1][VEC ? K : 1];   // vector retention: l_t, then (core) exp(l_t)
+};
+template <typename T, int K, bool VEC> struct RevShared {
+    static constexpr int CW = K / 32, QN = ring_depth(sizeof(RevBuf<T, K, VEC>));
+    RevBuf<T, K, VEC> buf[QN];
+    float lam[K];                           // between two lists
+    float au[CW][PB];                       // a core warp's -a2 u of the round
+    float part[2][CW][PB];
+    unsigned long long words[SCAN_CHUNKS];
+    uint16_t list[32 * CH + 8];             // bit 15: a restart
+    int cmd_tok, cmd_n, live;
+    PipeBars bars;
 };
 
-// tokens [t_lo, t_hi) of the chain in reverse, all three roles; lam: the core's registers
-template <typename T, int K, bool VEC>
-__device__ __forceinline__ bool rev_stretch(const P1Bwd& a, int h, int t_lo, int t_hi, float (&lam)[K / 32],
-                                            RevBuf<T, K, VEC>* buf, PipeBars& bars, uint32_t& round0, int role, int lane)
+// The factors of a processed token: scal and grad (without u).
+__device__ __forceinline__ void rev_scalars(float sumk, float kmax, float rho, float beta, float al, const Hyper& hy, float4& sc, float4& gr)
 {
-    constexpr int R = K / 32;
-    const int H = a.H;
-    const Hyper hy = a.hy;
-    const int nblk = (t_hi - t_lo + QB - 1) / QB;
-    const T* kp = static_cast<const T*>(a.k);
-    bool ok = true;
-    const uint32_t base = round0;
-    // block b: tokens t_hi - 1 - (b QB + j), j = 0 .. n - 1 (slot j of the buffer)
-    if (role == 1) {
-        // Rows go straight into the buffer with cp.async (nothing of them is converted here), one committed
-        // group per block and one block ahead: while block b is on its way, block b - 1 is finished (the
-        // step's own scalars formed from the raw ones, the retention vector exponentiated) and handed over.
-        auto finish = [&](int b) {
-            const uint32_t use = base + b;
-            const int bi = use % QN;
-            RevBuf<T, K, VEC>& B = buf[bi];
-            const int ttop = t_hi - 1 - b * QB, n = min(QB, ttop - t_lo + 1);
-            if (lane < n) {
-                const float ns = B.raw[0][lane], rho = B.raw[1][lane], alv = B.raw[3][lane];
-                const float bb = hy.beta_aware ? B.raw[2][lane] : 1.0f;
-                const float rn = fabsf(ns);
-                const float e = hy.eta * bb * rn, a2 = e * bb;
-                const float cc = fmaf(-a2, alv, e);
-                const float g1 = hy.eta * (1.0f - 2.0f * bb * alv) * rn;
-                const float g2 = ns > 0.f ? -cc * rn : 0.f;
-                B.sc0[lane] = make_float4(a2, rho, cc, g1);
-                B.sc1[lane].x = g2;
-            }
-            if constexpr (VEC) {
-                for (int j = 0; j < n; ++j) {
-                    float lr[R];
-                    load_row<R>(B.rv[VEC ? j : 0], lane, lr);
+    const float b = hy.beta_aware ? beta : 1.0f, rn = 1.0f / fmaxf(sumk, hy.eps);
+    const float e = hy.eta * b * rn, a2 = e * b, cc = fmaf(-a2, al, e);
+    sc = make_float4(a2, rho, kmax, rn);
+    gr = make_float4(cc, hy.eta * (1.0f - 2.0f * b * al) * rn, sumk > hy.eps ? -cc * rn : 0.f, 0.f);
+}
+__device__ __forceinline__ float rev_step(float lm, float kap, float w, float au, float rho) { return fmaf(rho, lm, fmaf(au, kap, w)); }
+
+template <typename T, int K, bool VEC>
+__device__ __forceinline__ void rev_core_block(RevShared<T, K, VEC>& sh, RevBuf<T, K, VEC>& B, int n, float& lam, uint32_t& rounds, int warp, int lane)
+{
+    constexpr int CW = K / 32, R = K / 32;
+    const int i = warp * 32 + lane;
+    float kap[PB], w[PB];
+    unsigned pass = 0;
 #pragma unroll
-                    for (int r = 0; r < R; ++r) lr[r] = expf(lr[r]);
-                    store_row<R>(B.rv[VEC ? j : 0], lane, lr);
-                }
-            }
+    for (int j = 0; j < PB; ++j) {
+        const float k = ldf(&B.k[j][i]);
+        kap[j] = __fmul_rn(k, k);
+        w[j] = __fmul_rn(k, B.dkt[j][i]);
+        pass |= ((B.mask[j][i / R] >> (i % R)) & 1u) << j;
+    }
+    pass &= ~B.restart;
+    if constexpr (VEC) {
 #pragma unroll 4
-            for (int j = 0; j < QB; ++j) {   // (slots beyond n repeat the last token: harmless)
-                float kk[R], dkt[R], kap[R], mkap[R], rm[R], w[R], rv[R];
-                unpack<R>(B.kraw[j][lane], kk);
-                load_row<R>(B.dkt[j], lane, dkt);
-                const unsigned mw = B.mask[j][lane];
-                if constexpr (VEC) load_row<R>(B.rv[VEC ? j : 0], lane, rv);
-                else {
-                    const float rho = B.raw[1][min(j, n - 1)];
-#pragma unroll
-                    for (int r = 0; r < R; ++r) rv[r] = rho;
-                }
-#pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    const bool pass = (mw >> r) & 1u;
-                    kap[r] = kk[r] * kk[r];
-                    mkap[r] = pass ? kap[r] : 0.f;
-                    rm[r] = pass ? rv[r] : 0.f;
-                    w[r] = kk[r] * dkt[r];
-                }
-                store_row<R>(B.kap[j], lane, kap);
-                store_row<R>(B.mkap[j], lane, mkap);
-                store_row<R>(B.rm[j], lane, rm);
-                store_row<R>(B.w[j], lane, w);
-            }
-            __syncwarp();
-            if (lane == 0) p1_mbar_arrive(&bars.full[bi]);
-        };
-        for (int b = 0; b < nblk && ok; ++b) {
-            const uint32_t use = base + b;
-            const int bi = use % QN;
-            if (use >= QN) ok = p1_mbar_wait(&bars.free_[bi], ((use / QN) - 1) & 1, a.status);
-            if (!ok) break;
-            RevBuf<T, K, VEC>& B = buf[bi];
-            const int ttop = t_hi - 1 - b * QB, n = min(QB, ttop - t_lo + 1);
-#pragma unroll
-            for (int j = 0; j < QB; ++j) {
-                const size_t th = (size_t)(ttop - min(j, n - 1)) * H + h;
-                cp_async<R * (int)sizeof(T)>(&B.kraw[j][lane], kp + th * K + R * lane);
-                cp_async<R * 4>(&B.dt[j][R * lane], a.r.dtraj + th * K + R * lane);
-                cp_async<R * 4>(&B.dkt[j][R * lane], a.dktil + th * K + R * lane);
-                cp_async<R * 4>(&B.dkr[j][R * lane], a.dkread + th * K + R * lane);
-                cp_async<4>(&B.mask[j][lane], a.r.pmask + th * 32 + lane);
-                if constexpr (VEC) cp_async<R * 4>(&B.rv[VEC ? j : 0][R * lane], a.log_ret + th * K + R * lane);
-            }
-            if (lane < n) {
-                const size_t th = (size_t)(ttop - lane) * H + h;
-                cp_async<4>(&B.raw[0][lane], a.r.n + th);
-                cp_async<4>(&B.raw[1][lane], a.r.rho + th);
-                cp_async<4>(&B.raw[2][lane], a.beta + th);
-                cp_async<4>(&B.raw[3][lane], a.r.al + th);
-            }
-            cp_async_commit();
-            if (b > 0) {
-                cp_async_wait<1>();   // block b - 1 has landed
-                __syncwarp();
-                finish(b - 1);
-            }
-        }
-        cp_async_wait<0>();
-        __syncwarp();
-        if (ok && nblk > 0) finish(nblk - 1);
-    } else if (role == 0) {
-        for (int b = 0; b < nblk && ok; ++b) {
-            const uint32_t use = base + b;
-            const int bi = use % QN;
-            ok = p1_mbar_wait(&bars.full[bi], (use / QN) & 1, a.status);
-            if (!ok) break;
-            RevBuf<T, K, VEC>& B = buf[bi];
-            const int ttop = t_hi - 1 - b * QB, n = min(QB, ttop - t_lo + 1);
-            auto token = [&](int j) {
-                const float a2 = B.sc0[j].x;
-                float kap[R], mkap[R], rm[R], w[R];
-                load_row<R>(B.mkap[j], lane, mkap);
-                load_row<R>(B.kap[j], lane, kap);
-                load_row<R>(B.rm[j], lane, rm);
-                load_row<R>(B.w[j], lane, w);
-                float dc0 = lam[0] * mkap[0], dc1 = lam[1] * mkap[1];
-#pragma unroll
-                for (int r = 2; r < R; r += 2) {
-                    dc0 = fmaf(lam[r], mkap[r], dc0);
-                    dc1 = fmaf(lam[r + 1], mkap[r + 1], dc1);
-                }
-                store_row<R>(B.lam[j], lane, lam);
-                const float dc = warp_sum(dc0 + dc1);
-                const float da = -a2 * dc;
-#pragma unroll
-                for (int r = 0; r < R; ++r) lam[r] = fmaf(rm[r], lam[r], fmaf(da, kap[r], w[r]));
-                if (lane == 0) B.sc1[j].y = dc;
-            };
-            if (n == QB) {
-#pragma unroll
-                for (int j = 0; j < QB; ++j) token(j);
-            } else {
-                for (int j = 0; j < n; ++j) token(j);
-            }
-            __syncwarp();
-            if (lane == 0) p1_mbar_arrive(&bars.done[bi]);
-        }
-    } else {
-        T* dkp = static_cast<T*>(a.dk);
-        for (int b = 0; b < nblk && ok; ++b) {
-            const uint32_t use = base + b;
-            const int bi = use % QN;
-            ok = p1_mbar_wait(&bars.done[bi], (use / QN) & 1, a.status);
-            if (!ok) break;
-            const RevBuf<T, K, VEC>& B = buf[bi];
-            const int ttop = t_hi - 1 - b * QB, n = min(QB, ttop - t_lo + 1);
-            // <lambda, d_t> of the block's tokens first, all slots at once: the shuffle rounds of the eight
-            // sums overlap instead of following one another
-            float drv[QB];
-#pragma unroll
-            for (int j = 0; j < QB; ++j) {
-                float dt[R], lm[R];
-                load_row<R>(B.dt[j], lane, dt);
-                load_row<R>(B.lam[j], lane, lm);
-                const unsigned mw = B.mask[j][lane];
-                drv[j] = 0.f;
-#pragma unroll
-                for (int r = 0; r < R; ++r) drv[j] = fmaf((mw >> r) & 1u ? lm[r] : 0.f, dt[r], drv[j]);
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-                for (int j = 0; j < QB; ++j) drv[j] += __shfl_xor_sync(0xffffffffu, drv[j], o);
-            // the per-token scalars (beta and retention gradients): lane j takes token j
-            {
-                float mine = 0.f;
-#pragma unroll
-                for (int j = 0; j < QB; ++j) mine = lane == j ? drv[j] : mine;
-                if (lane < n) {
-                    const size_t th = (size_t)(ttop - lane) * H + h;
-                    const float4 s0 = B.sc0[lane];
-                    const float dc = B.sc1[lane].y;
-                    if (hy.beta_aware) atomicAdd(&a.dbeta[th], s0.w * dc);
-                    if (hy.apf_mode == 1) atomicAdd(&a.dgate[th], s0.y * mine);
-                    if (hy.apf_mode == 2 && a.dlog_ret) a.dlog_ret[th] = s0.y * mine;
-                }
-            }
-            auto token = [&](int j) {
-                const size_t th = (size_t)(ttop - j) * H + h;
-                const float4 s0 = B.sc0[j], s1 = B.sc1[j];
-                const float a2 = s0.x, cc = s0.z, g2 = s1.x, dc = s1.y;
-                float kk[R], dt[R], dkt[R], dkr[R], lm[R];
-                unpack<R>(B.kraw[j][lane], kk);
-                load_row<R>(B.dt[j], lane, dt);
-                load_row<R>(B.dkt[j], lane, dkt);
-                load_row<R>(B.dkr[j], lane, dkr);
-                load_row<R>(B.lam[j], lane, lm);
-                {
-                    const unsigned mw = B.mask[j][lane];
-#pragma unroll
-                    for (int r = 0; r < R; ++r) lm[r] = (mw >> r) & 1u ? lm[r] : 0.f;
-                }
-                const float da = -a2 * dc, dn = g2 * dc;
-                if constexpr (VEC) {
-                    if (a.dlog_ret) {
-                        float rv[R], dl[R];
-                        load_row<R>(B.rv[VEC ? j : 0], lane, rv);
-#pragma unroll
-                        for (int r = 0; r < R; ++r) dl[r] = rv[r] * lm[r] * dt[r];
-                        store_row<R>(a.dlog_ret + th * K, lane, dl);
-                    }
-                }
-                float out[R];
-#pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    const float dkap = cc * lm[r] + da * dt[r] + dn;
-                    out[r] = dkr[r] + dt[r] * dkt[r] + 2.0f * kk[r] * dkap;
-                }
-                store_row<R>(dkp + th * K, lane, out);
-            };
-            if (n == QB) {   // unrolled without a branch between the tokens: their reads and products interleave
-#pragma unroll
-                for (int j = 0; j < QB; ++j) token(j);
-            } else {
-                for (int j = 0; j < n; ++j) token(j);
-            }
-            __syncwarp();
-            if (lane == 0) p1_mbar_arrive(&bars.free_[bi]);
+        for (int j = 0; j < PB; ++j) {
+            float& v = B.rv[VEC ? j : 0][VEC ? i : 0];
+            v = j < n ? expf(v) : 1.0f;
         }
     }
-    round0 = base + nblk;
+    B.lam0[i] = lam;
+    const float4 sc = B.scal[lane];   // lane j: token j
+    float u = 0.f, l = lam;
+    for (int round = 0; round <= PB; ++round) {
+        const uint32_t par = rounds++ & 1;
+        sh.au[warp][lane] = -sc.x * u;
+        __syncwarp();
+        float p[PB];
+        l = lam;
+#pragma unroll
+        for (int j = 0; j < PB; j += 4) {
+            const float4 u4 = *reinterpret_cast<const float4*>(&sh.au[warp][j]), r4 = *reinterpret_cast<const float4*>(B.rho + j);
+            const float au[4] = {u4.x, u4.y, u4.z, u4.w}, rs[4] = {r4.x, r4.y, r4.z, r4.w};
+#pragma unroll
+            for (int x = 0; x < 4; ++x) {
+                const float rho = VEC ? B.rv[VEC ? j + x : 0][VEC ? i : 0] : rs[x];
+                const float lm = bit_of(pass, j + x) ? l : 0.f;
+                p[j + x] = lm * kap[j + x];
+                l = rev_step(lm, kap[j + x], w[j + x], au[x], rho);
+            }
+        }
+        const float mine = transpose_sum(p, lane);
+        float(*part)[PB] = sh.part[par];
+        part[warp][lane] = mine;
+        bar_sync<CW * 32>(3);
+        float un = part[0][lane];
+#pragma unroll
+        for (int x = 1; x < CW; ++x) un += part[x][lane];
+        const float du = fabsf(un - u);
+        const float size = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(fabsf(un) * sc.w)));
+        if (__all_sync(0xffffffffu, du * sc.x * sc.z <= 5.9604645e-8f * size || du <= 1.1920929e-7f * fabsf(un) || lane >= n)) break;
+        u = un;
+    }
+    lam = l;
+    if (warp == 0) B.grad[lane].w = u;
+}
+
+// What a processed token leaves: dk and, where one per coordinate is asked for, the retention gradient.
+template <typename T, int K, bool VEC>
+__device__ __forceinline__ void rev_outputs(const P1Bwd& a, size_t th, int lane, const float4& g, float a2, const float (&kk)[K / 32],
+                                            const float (&dt)[K / 32], const float (&dkt)[K / 32], const float (&dkr)[K / 32],
+                                            const float (&lm)[K / 32], const float (&rv)[K / 32])
+{
+    constexpr int R = K / 32;
+    const float da = -a2 * g.w, dn = g.z * g.w;
+    if constexpr (VEC) {   // r_i lambda_i d_i
+        if (a.dlog_ret) {
+            float dl[R];
+#pragma unroll
+            for (int r = 0; r < R; ++r) dl[r] = rv[r] * lm[r] * dt[r];
+            store_row<R>(a.dlog_ret + th * K, lane, dl);
+        }
+    }
+    float out[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const float dkap = g.x * lm[r] + da * dt[r] + dn;
+        out[r] = dkr[r] + dt[r] * dkt[r] + 2.0f * kk[r] * dkap;
+    }
+    store_row<R>(static_cast<T*>(a.dk) + th * K, lane, out);
+}
+// The per-token scalar gradients, added on top of what the chunk-local backward wrote (as reductions without a return
+// value, so that nobody waits for memory); dr = <lambda, d_t>.
+__device__ __forceinline__ void rev_scalar_grads(const P1Bwd& a, size_t th, const float4& g, float rho, float dr)
+{
+    if (a.hy.beta_aware) atomicAdd(&a.dbeta[th], g.y * g.w);
+    if (a.hy.apf_mode == 1) atomicAdd(&a.dgate[th], rho * dr);
+    if (a.hy.apf_mode == 2 && a.dlog_ret) a.dlog_ret[th] = rho * dr;
+}
+
+template <typename T, int K, bool VEC>
+__device__ __forceinline__ bool run_rev_list(const P1Bwd& a, int h, RevShared<T, K, VEC>& sh, uint32_t& rounds, uint32_t& uses, int warp, int lane)
+{
+    constexpr int R = K / 32;
+    using P = Pipe<K>;
+    constexpr int QN = RevShared<T, K, VEC>::QN;
+    const int H = a.H;
+    const int tok0 = sh.cmd_tok, total = sh.cmd_n;
+    const int nblk = (total + PB - 1) / PB;
+    bool ok = true;
+    const uint32_t base = uses;
+    auto entry = [&](int idx) { return (int)sh.list[total - 1 - idx]; };   // from the last token on
+    auto len_of = [&](int b) { return min(PB, total - b * PB); };
+    auto th_of = [&](int b) {   // lane j: token j
+        return lane < len_of(b) ? (uint32_t)((tok0 + (entry(b * PB + lane) & 0x7fff)) * H + h) : NO_ROW;
+    };
+    if (warp < P::CORE) {
+        float lam = sh.lam[warp * 32 + lane];
+        for (int b = 0; b < nblk; ++b) {
+            const int bi = (base + b) % QN;
+            ok = bar_sync_and<P::CORE * 32>(3, p1_mbar_wait(&sh.bars.full[bi], ((base + b) / QN) & 1, a.status));
+            if (!ok) break;
+            rev_core_block<T, K, VEC>(sh, sh.buf[bi], len_of(b), lam, rounds, warp, lane);
+            __syncwarp();
+            if (lane == 0) p1_mbar_arrive(&sh.bars.done[bi]);
+        }
+        sh.lam[warp * 32 + lane] = lam;
+    } else if (warp < P::FINISH0) {
+        auto start = [&](int b) {
+            const uint32_t use = base + b;
+            const int bi = use % QN;
+            if (use >= QN) ok = p1_mbar_wait(&sh.bars.free_[bi], ((use / QN) - 1) & 1, a.status);
+            if (!ok) return;
+            RevBuf<T, K, VEC>& B = sh.buf[bi];
+            const uint32_t th = th_of(b);
+            fetch_rows<T, K>(&B.k[0][0], static_cast<const T*>(a.k), th, PB, lane);
+            fetch_rows<float, K>(&B.dkt[0][0], a.dktil, th, PB, lane);
+            fetch_rows<unsigned, 32>(&B.mask[0][0], a.r.pmask, th, PB, lane);
+            if constexpr (VEC) fetch_rows<float, K>(&B.rv[0][0], a.log_ret, th, PB, lane);
+            if (th != NO_ROW) {
+                cp_async4(&B.raw[0][lane], a.r.sumk + th);
+                cp_async4(&B.raw[1][lane], a.r.kmax + th);
+                cp_async4(&B.raw[2][lane], a.r.rho + th);
+                cp_async4(&B.raw[3][lane], a.beta + th);
+                cp_async4(&B.raw[4][lane], a.r.al + th);
+                for (int o = 0; o < K * 4; o += 128) {   // what the finishing warps will read
+                    prefetch_l2(reinterpret_cast<const char*>(a.r.dtraj + (size_t)th * K) + o);
+                    prefetch_l2(reinterpret_cast<const char*>(a.dkread + (size_t)th * K) + o);
+                }
+            }
+            cp_async_commit();
+        };
+        auto complete = [&](int b) {
+            const int bi = (base + b) % QN;
+            RevBuf<T, K, VEC>& B = sh.buf[bi];
+            const int n = len_of(b);
+            // an empty slot has to leave lambda alone: mask all ones, rho = 1 (k = 0)
+            float4 sc = make_float4(0.f, 1.f, 0.f, 0.f), gr = make_float4(0.f, 0.f, 0.f, 0.f);
+            bool skipped = false;
+            if (lane < n) {
+                skipped = (entry(b * PB + lane) & 0x8000) != 0;
+                if (!skipped) rev_scalars(B.raw[0][lane], B.raw[1][lane], B.raw[2][lane], B.raw[3][lane], B.raw[4][lane], a.hy, sc, gr);
+            }
+            const unsigned restarts = __ballot_sync(0xffffffffu, skipped);
+            B.scal[lane] = sc;
+            B.grad[lane] = gr;
+            B.rho[lane] = sc.y;
+            if (lane == 0) B.restart = restarts;
+            for (int j = n; j < PB; ++j) B.mask[j][lane] = 0xffffffffu;
+            __syncwarp();
+            if (lane == 0) p1_mbar_arrive(&sh.bars.full[bi]);
+        };
+        int b = (int)((warp - P::FETCH0 + base) & 1);
+        if (b < nblk) start(b);
+        for (; b < nblk && ok; b += 2) {
+            cp_async_wait<0>();
+            __syncwarp();
+            complete(b);
+            if (b + 2 < nblk) start(b + 2);
+        }
+        cp_async_wait<0>();
+    } else {
+        for (int b = (int)((warp - P::FINISH0 - base) & (P::FINISH - 1)); b < nblk; b += P::FINISH) {
+            const int bi = (base + b) % QN;
+            const RevBuf<T, K, VEC>& B = sh.buf[bi];
+            const int n = len_of(b);
+            const uint32_t mine = th_of(b);
+            struct Ahead {
+                float dt[4][R], dkr[4][R];
+            } even, odd;
+            auto load = [&](int j0, Ahead& x) {
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const size_t th = __shfl_sync(0xffffffffu, mine, min(j0 + j, n - 1));
+                    load_row<R>(a.r.dtraj + th * K, lane, x.dt[j]);
+                    load_row<R>(a.dkread + th * K, lane, x.dkr[j]);
+                }
+            };
+            load(0, even);
+            ok = p1_mbar_wait(&sh.bars.done[bi], ((base + b) / QN) & 1, a.status);
+            if (!ok) break;
+            const unsigned restart = B.restart;
+            float lam[R];
+            load_row<R>(B.lam0, lane, lam);
+            auto work = [&](int j0, const Ahead& x) {
+                float drv[4];
+#pragma unroll
+                for (int jj = 0; jj < 4; ++jj) {
+                    const int j = j0 + jj;
+                    float kk[R], dkt[R], lm[R], rv[R];
+                    load_row<R>(B.k[j], lane, kk);
+                    load_row<R>(B.dkt[j], lane, dkt);
+                    const unsigned mw = bit_of(restart, j) ? 0u : B.mask[j][lane];
+                    const float4 sc = B.scal[j], g = B.grad[j];
+                    if constexpr (VEC) load_row<R>(B.rv[VEC ? j : 0], lane, rv);
+                    else {
+#pragma unroll
+                        for (int r = 0; r < R; ++r) rv[r] = sc.y;
+                    }
+                    drv[jj] = 0.f;
+                    const float au = -sc.x * g.w;
+#pragma unroll
+                    for (int r = 0; r < R; ++r) {
+                        lm[r] = bit_of(mw, r) ? lam[r] : 0.f;
+                        drv[jj] = fmaf(lm[r], x.dt[jj][r], drv[jj]);
+                        lam[r] = rev_step(lm[r], __fmul_rn(kk[r], kk[r]), __fmul_rn(kk[r], dkt[r]), au, rv[r]);
+                    }
+                    const size_t th = __shfl_sync(0xffffffffu, mine, j);
+                    if (j < n && !bit_of(restart, j)) rev_outputs<T, K, VEC>(a, th, lane, g, sc.x, kk, x.dt[jj], dkt, x.dkr[jj], lm, rv);
+                }
+                const float dr = transpose_sum(drv, lane);   // lane j: token j0 + j
+                const int j = (j0 + lane) & (PB - 1);
+                const size_t th = __shfl_sync(0xffffffffu, mine, j);
+                if (lane < 4 && j < n && !bit_of(restart, j)) rev_scalar_grads(a, th, B.grad[j], B.scal[j].y, dr);
+            };
+#pragma unroll 1
+            for (int j0 = 0; j0 < n; j0 += 8) {
+                load(j0 + 4, odd);
+                work(j0, even);
+                load(j0 + 8, even);
+                if (j0 + 4 < n) work(j0 + 4, odd);
+            }
+            __syncwarp();
+            if (lane == 0) p1_mbar_arrive(&sh.bars.free_[bi]);
+        }
+    }
+    uses = base + nblk;
     return ok;
 }
 
-// processed tokens, in reverse; one chain per CTA: warp 0 walks the chain, warps 1 and 2 serve its
-// pipelined stretches.  Skip words are fetched for 32 chunks at a time.
-
+// A list of at most PB entries by warp 0 alone, token by token.
 template <typename T, int K, bool VEC>
-__global__ void __launch_bounds__(96) phase1_bwd_seq_kernel(P1Bwd a)
+__device__ __forceinline__ void walk_rev_list(const P1Bwd& a, int h, RevShared<T, K, VEC>& sh, int tok0, int n, int lane)
 {
     constexpr int R = K / 32;
-    constexpr int PF = 4;   // prefetch distance in processed tokens
-    // ring of prefetched rows and scalars (cp.async; every lane copies and later reads its own bytes)
-    struct BSlot {
-        RawRow<T, R> k[32], sk_k[32];
-        RawRow<float, R> dt[32], dkt[32], dkr[32], sk_t[32], lr[VEC ? 32 : 1];
-        unsigned m[32];
-        float n[32], rho[32], beta[32], al[32];
-    };
-    extern __shared__ __align__(16) uint8_t p1_dyn[];   // RevBuf[QN]
-    RevBuf<T, K, VEC>* rbuf = reinterpret_cast<RevBuf<T, K, VEC>*>(p1_dyn);
-    __shared__ __align__(16) BSlot ring[PF];
-    __shared__ PipeBars bars;
-    __shared__ int cmd[2];
+    const int H = a.H;
+    RevBuf<T, K, VEC>& B = sh.buf[0];
+    const uint32_t mine = lane < n ? (uint32_t)((tok0 + ((int)sh.list[n - 1 - lane] & 0x7fff)) * H + h) : NO_ROW;
+    fetch_rows<T, K>(&B.k[0][0], static_cast<const T*>(a.k), mine, n, lane);
+    fetch_rows<float, K>(&B.dkt[0][0], a.dktil, mine, n, lane);
+    fetch_rows<unsigned, 32>(&B.mask[0][0], a.r.pmask, mine, n, lane);
+    fetch_rows<float, K>(&sh.buf[1].dkt[0][0], a.r.dtraj, mine, n, lane);
+    fetch_rows<float, K>(&sh.buf[2].dkt[0][0], a.dkread, mine, n, lane);
+    if constexpr (VEC) fetch_rows<float, K>(&B.rv[0][0], a.log_ret, mine, n, lane);
+    cp_async_commit();
+    if (lane < n) {
+        float4 sc, gr;
+        rev_scalars(a.r.sumk[mine], a.r.kmax[mine], a.r.rho[mine], a.beta[mine], a.r.al[mine], a.hy, sc, gr);
+        B.scal[lane] = sc;
+        B.grad[lane] = gr;
+    }
+    float lam[R];
+    load_row<R>(sh.lam, lane, lam);
+    cp_async_wait<0>();
+    __syncwarp();
+#pragma unroll 1
+    for (int j = 0; j < n; ++j) {
+        const float4 sc = B.scal[j];
+        float4 g = B.grad[j];
+        float kk[R], dkt[R], dt[R], dkr[R], lm[R], rv[R], u = 0.f, dr = 0.f;
+        load_row<R>(B.k[j], lane, kk);
+        load_row<R>(B.dkt[j], lane, dkt);
+        if (sh.list[n - 1 - j] & 0x8000) {   // a restart
+#pragma unroll
+            for (int r = 0; r < R; ++r) lam[r] = kk[r] * dkt[r];
+            continue;
+        }
+        load_row<R>(sh.buf[1].dkt[j], lane, dt);
+        load_row<R>(sh.buf[2].dkt[j], lane, dkr);
+        if constexpr (VEC) {
+            load_row<R>(B.rv[VEC ? j : 0], lane, rv);
+#pragma unroll
+            for (int r = 0; r < R; ++r) rv[r] = expf(rv[r]);
+        } else {
+#pragma unroll
+            for (int r = 0; r < R; ++r) rv[r] = sc.y;
+        }
+        const unsigned mw = B.mask[j][lane];
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            lm[r] = bit_of(mw, r) ? lam[r] : 0.f;
+            u = fmaf(lm[r], kk[r] * kk[r], u);
+            dr = fmaf(lm[r], dt[r], dr);
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            u += __shfl_xor_sync(0xffffffffu, u, o);
+            dr += __shfl_xor_sync(0xffffffffu, dr, o);
+        }
+        g.w = u;
+        const float au = -sc.x * u;
+#pragma unroll
+        for (int r = 0; r < R; ++r) lam[r] = rev_step(lm[r], kk[r] * kk[r], kk[r] * dkt[r], au, rv[r]);
+        const size_t th = __shfl_sync(0xffffffffu, mine, j);
+        rev_outputs<T, K, VEC>(a, th, lane, g, sc.x, kk, dt, dkt, dkr, lm, rv);
+        if (lane == 0) rev_scalar_grads(a, th, g, sc.y, dr);
+    }
+    store_row<R>(sh.lam, lane, lam);
+    __syncwarp();
+}
+
+// Skip words are taken 32 chunks at a time, the last ones first, and their processed tokens (with the restarts
+// between them) are one list.  Warp 0 walks short lists itself.
+template <typename T, int K, bool VEC> struct RevPlan {
+    const P1Bwd& a;
+    RevShared<T, K, VEC>& sh;
+    const int h, lane, c0, c1, seq_t0, seq_len;
+    int g, scanned = -1;
+    bool live = true;   // the token above the group was processed (at the end: the sequence's first one): lambda holds
+
+    __device__ __forceinline__ RevPlan(const P1Bwd& a_, RevShared<T, K, VEC>& sh_, int s, int h_, int lane_)
+        : a(a_), sh(sh_), h(h_), lane(lane_), c0(a_.tab.seq_chunk0(s)), c1(a_.tab.seq_chunk0(s + 1)), seq_t0(a_.tab.seq_tok0(s)),
+          seq_len(a_.tab.seq_len(s)), g(c1 > c0 ? (c1 - c0 - 1) >> 5 : -1)
+    {
+    }
+    __device__ __forceinline__ void next()
+    {
+        for (; g >= 0; --g) {
+            const int top = g * 32 / SCAN_CHUNKS;
+            if (top != scanned) scan_words(sh.words, a.r.skipw, c0 + top * SCAN_CHUNKS, c0, c1, seq_len, a.H, h, lane);
+            scanned = top;
+            const int base = g * 32 * CH, glen = min(32 * CH, seq_len - base);
+            const unsigned long long valid = valid_bits(glen - 64 * lane), proc = sh.words[g * 32 % SCAN_CHUNKS + lane];
+            unsigned long long up = __shfl_up_sync(0xffffffffu, proc, 1) >> 63;
+            if (lane == 0) up = 0ull;
+            const unsigned long long restart = ((proc << 1) | up) & ~proc & valid;
+            const bool above = live;
+            const unsigned long long last = __shfl_sync(0xffffffffu, proc, (glen - 1) / CH);
+            live = (__shfl_sync(0xffffffffu, proc, 0) & 1ull) != 0ull;
+            if (!__any_sync(0xffffffffu, proc != 0ull)) continue;
+            int n = write_list(sh.list, proc | restart, restart, 32 * CH, lane);
+            if (((last >> ((glen - 1) % CH)) & 1ull) && !above) {   // (the sequence goes on above: `above` starts out true)
+                if (lane == 0) sh.list[n] = (uint16_t)(glen | 0x8000);
+                __syncwarp();
+                ++n;
+            }
+            if (n <= PB) {
+                walk_rev_list<T, K, VEC>(a, h, sh, seq_t0 + base, n, lane);
+                continue;
+            }
+            if (lane == 0) {
+                sh.cmd_tok = seq_t0 + base;
+                sh.cmd_n = n;
+            }
+            --g;
+            return;
+        }
+        if (lane == 0) {
+            sh.cmd_n = 0;
+            sh.live = live;
+        }
+    }
+};
+
+// One chain per CTA.
+template <typename T, int K, bool VEC>
+__global__ void __launch_bounds__(Pipe<K>::THREADS, 1) phase1_bwd_seq_kernel(P1Bwd a)
+{
+    using P = Pipe<K>;
+    extern __shared__ __align__(16) uint8_t p1_dyn[];
+    RevShared<T, K, VEC>& sh = *reinterpret_cast<RevShared<T, K, VEC>*>(p1_dyn);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int chain = blockIdx.x;
     const int s = chain / a.H, h = chain % a.H, H = a.H;
-    const Hyper hy = a.hy;
-    const T* kp = static_cast<const T*>(a.k);
-    T* dkp = static_cast<T*>(a.dk);
-    if (threadIdx.x == 0) {
-        for (int i = 0; i < QN; ++i) {
-            p1_mbar_init(&bars.full[i], 1);
-            p1_mbar_init(&bars.done[i], 1);
-            p1_mbar_init(&bars.free_[i], 1);
-        }
-    }
+    const int coord = warp * 32 + lane;   // core warps
+    const size_t mine = ((size_t)s * H + h) * K + coord;
+    if (threadIdx.x == 0) init_bars(sh.bars, RevShared<T, K, VEC>::QN, P::CORE);
+    if (warp < P::CORE) sh.lam[coord] = a.dprecond_out ? a.dprecond_out[mine] : 0.f;
+    uint32_t rounds = 0, uses = 0;
     __syncthreads();
-    uint32_t pipe_uses = 0;
-    if (warp != 0) {
-        float none[R];
-        while (true) {
-            asm volatile("bar.sync 1, 96;" ::: "memory");
-            const int t_lo = cmd[0], t_hi = cmd[1];
-            if (t_hi <= t_lo) break;
-            rev_stretch<T, K, VEC>(a, h, t_lo, t_hi, none, rbuf, bars, pipe_uses, warp, lane);
-            asm volatile("bar.sync 2, 96;" ::: "memory");
+    RevPlan<T, K, VEC> plan(a, sh, s, h, lane);
+    while (true) {
+        if (warp == 0) plan.next();
+        bar_sync<P::THREADS>(1);
+        if (sh.cmd_n == 0) break;
+        if (!run_rev_list<T, K, VEC>(a, h, sh, rounds, uses, warp, lane)) plan.g = -1;
+        bar_sync<P::THREADS>(2);
+    }
+    if (a.dprecond_in && warp < P::CORE) {
+        float lam = sh.lam[coord];
+        if (!sh.live) {   // the first token was skipped: lambda restarts there
+            const size_t th = (size_t)a.tab.seq_tok0(s) * H + h;
+            lam = ldf(static_cast<const T*>(a.k) + th * K + coord) * a.dktil[th * K + coord];
         }
-        return;
+        a.dprecond_in[mine] = lam;
     }
-    float lam[R];
-    if (a.dprecond_out) load_row<R>(a.dprecond_out + ((size_t)s * H + h) * K, lane, lam);
-    else {
-#pragma unroll
-        for (int r = 0; r < R; ++r) lam[r] = 0.f;
-    }
-    bool lam_valid = true;     // lam holds dL/dd_{t+1} for the token about to be processed
-    long src = -1;             // otherwise it is k (.) dktil of this (skipped) token
-    auto restart = [&](long tsrc) {
-        const size_t ts = (size_t)tsrc * H + h;
-        float kk[R], dk[R];
-        load_row<R>(kp + ts * K, lane, kk);
-        load_row<R>(a.dktil + ts * K, lane, dk);
-#pragma unroll
-        for (int r = 0; r < R; ++r) lam[r] = kk[r] * dk[r];
-    };
-    const int c0 = a.tab.seq_chunk0(s), c1 = a.tab.seq_chunk0(s + 1);
-    const int seq_t0 = a.tab.seq_tok0(s), seq_len = a.tab.seq_len(s);
-    for (int ctop = c1; ctop > c0; ctop -= 32) {
-        // lane j holds the words of chunk ctop - 1 - j
-        unsigned w0 = 0, w1 = 0;
-        if (ctop - 1 - lane >= c0) {
-            const size_t tl = (size_t)(ctop - 1 - lane) * H + h;
-            w0 = a.r.skipw[tl * 2];
-            w1 = a.r.skipw[tl * 2 + 1];
-            // Sparse work (a few processed tokens per chunk): each lane warms L2 with the rows its
-            // chunk's tokens will need, long before the sequential walk gets there.  These rows sit in
-            // large arrays that were last touched several kernels ago; a cold access costs microseconds.
-            const int cl = ctop - 1 - lane;
-            const int lenl = min(CH, seq_len - (cl - c0) * CH);
-            unsigned long long m = ~((unsigned long long)w0 | ((unsigned long long)w1 << 32)) &
-                                   (lenl >= 64 ? ~0ull : ((1ull << lenl) - 1ull));
-            if (__popcll(m) <= 16) {
-                while (m) {
-                    const int t = __ffsll((long long)m) - 1;
-                    m &= m - 1;
-                    const size_t th = (size_t)(seq_t0 + (cl - c0) * CH + t) * H + h;
-                    prefetch_row(kp + th * K, K * (int)sizeof(T));
-                    prefetch_row(a.r.dtraj + th * K, K * 4);
-                    prefetch_row(a.dktil + th * K, K * 4);
-                    prefetch_row(a.dkread + th * K, K * 4);
-                    if constexpr (VEC) prefetch_row(a.log_ret + th * K, K * 4);
-                    prefetch_l2(a.r.pmask + th * 32);
-                    prefetch_l2(a.r.n + th);
-                    prefetch_l2(a.r.rho + th);
-                    prefetch_l2(a.beta + th);
-                    if (t + 1 < lenl) {   // rows a restart above this token would read
-                        prefetch_row(kp + (th + H) * K, K * (int)sizeof(T));
-                        prefetch_row(a.dktil + (th + H) * K, K * 4);
-                    }
-                }
-            }
-        }
-        const int cbot = max(ctop - 32, c0);
-        for (int c = ctop - 1; c >= cbot; --c) {
-            const int nrel = c - c0;
-            const int tok0 = seq_t0 + nrel * CH, len = min(CH, seq_len - nrel * CH);
-            const unsigned long long sk = (unsigned long long)__shfl_sync(0xffffffffu, w0, ctop - 1 - c) |
-                                          ((unsigned long long)__shfl_sync(0xffffffffu, w1, ctop - 1 - c) << 32);
-            const unsigned long long valid = len >= 64 ? ~0ull : ((1ull << len) - 1ull);
-            if ((sk & valid) == valid) {
-                lam_valid = false;
-                src = tok0;
-                continue;
-            }
-            if ((sk & valid) == 0ull) {
-                // every token of the chunk was processed: a pipelined stretch over this chunk and the ones
-                // below it of which the same holds (within this group of skip words, at most PIPE_CHUNKS)
-                int np = 1;
-                while (np < PIPE_CHUNKS && c - np >= cbot) {
-                    const int cc2 = c - np;
-                    const unsigned long long s2 = (unsigned long long)__shfl_sync(0xffffffffu, w0, ctop - 1 - cc2) |
-                                                  ((unsigned long long)__shfl_sync(0xffffffffu, w1, ctop - 1 - cc2) << 32);
-                    if (s2 != 0ull) break;   // chunks below the top one of a sequence are full
-                    ++np;
-                }
-                const int t_hi = tok0 + len, t_lo = seq_t0 + (nrel - (np - 1)) * CH;
-                if (!lam_valid) restart(src);
-                if (lane == 0) {
-                    cmd[0] = t_lo;
-                    cmd[1] = t_hi;
-                }
-                cp_async_wait<0>();
-                asm volatile("bar.sync 1, 96;" ::: "memory");
-                rev_stretch<T, K, VEC>(a, h, t_lo, t_hi, lam, rbuf, bars, pipe_uses, 0, lane);
-                asm volatile("bar.sync 2, 96;" ::: "memory");
-                lam_valid = true;
-                c -= np - 1;
-                continue;
-            }
-            // The tokens to process are known up front (the clear bits of the skip word), so the rows of
-            // the next PF of them are always in flight, across runs of skipped tokens.  Where the
-            // recurrence restarts before a token (its upper neighbour was skipped), the two rows the
-            // restart needs travel with that token's rows.
-            const unsigned long long todo = ~sk & valid;
-            const bool valid_in = lam_valid;
-            const long src_in = src;
-            auto pop_top = [](unsigned long long& m) {
-                const int t = 63 - __clzll((long long)m);
-                m &= ~(1ull << t);
-                return t;
-            };
-            // one committed group per ring slot use (an empty one when nothing is left to fetch), so
-            // that "all but the PF - 1 most recent groups" is always the slot about to be read
-            auto fetch = [&](int i, int slot) {
-                const size_t th = (size_t)(tok0 + i) * H + h;
-                BSlot& rs = ring[slot];
-                cp_async<R * (int)sizeof(T)>(&rs.k[lane], kp + th * K + R * lane);
-                cp_async<R * 4>(&rs.dt[lane], a.r.dtraj + th * K + R * lane);
-                cp_async<R * 4>(&rs.dkt[lane], a.dktil + th * K + R * lane);
-                cp_async<R * 4>(&rs.dkr[lane], a.dkread + th * K + R * lane);
-                if constexpr (VEC) cp_async<R * 4>(&rs.lr[VEC ? lane : 0], a.log_ret + th * K + R * lane);
-                cp_async<4>(&rs.m[lane], a.r.pmask + th * 32 + lane);
-                cp_async<4>(&rs.n[lane], a.r.n + th);
-                cp_async<4>(&rs.rho[lane], a.r.rho + th);
-                cp_async<4>(&rs.beta[lane], a.beta + th);
-                cp_async<4>(&rs.al[lane], a.r.al + th);
-                const bool top = i == len - 1;
-                const bool need = top ? !valid_in : (((sk >> (i + 1)) & 1ull) != 0ull);
-                if (need) {   // lambda restarts at the lowest token of the skipped run above
-                    const size_t ts = (size_t)(top ? src_in : (long)(tok0 + i + 1)) * H + h;
-                    cp_async<R * (int)sizeof(T)>(&rs.sk_k[lane], kp + ts * K + R * lane);
-                    cp_async<R * 4>(&rs.sk_t[lane], a.dktil + ts * K + R * lane);
-                }
-                cp_async_commit();
-                return need;
-            };
-            bool needr[PF];
-            unsigned long long pfm = todo, rem = todo;
-            cp_async_wait<0>();
-#pragma unroll
-            for (int u = 0; u < PF; ++u) {
-                needr[u] = false;
-                if (pfm) needr[u] = fetch(pop_top(pfm), u);
-                else cp_async_commit();
-            }
-            while (rem) {
-#pragma unroll
-                for (int u = 0; u < PF; ++u) {
-                    if (rem) {
-                        const int i = pop_top(rem);
-                        cp_async_wait<PF - 1>();
-                        const BSlot& rs = ring[u];
-                        float kk[R], kap[R], dt[R], dkt[R], dkr[R], drho = 0.f, dc = 0.f, al = 0.f;
-                        unpack<R>(rs.k[lane], kk);
-                        unpack<R>(rs.dt[lane], dt);
-                        unpack<R>(rs.dkt[lane], dkt);
-                        unpack<R>(rs.dkr[lane], dkr);
-                        if (needr[u]) {
-                            float rk[R], rt[R];
-                            unpack<R>(rs.sk_k[lane], rk);
-                            unpack<R>(rs.sk_t[lane], rt);
-#pragma unroll
-                            for (int r = 0; r < R; ++r) lam[r] = rk[r] * rt[r];
-                        }
-                        const unsigned mw = rs.m[lane];
-                        const float ns = rs.n[lane], rn = fabsf(ns), rho = rs.rho[lane];
-                        const float b = hy.beta_aware ? rs.beta[lane] : 1.0f;
-                        float rv[R];
-                        if constexpr (VEC) {
-                            float lr[R];
-                            unpack<R>(rs.lr[VEC ? lane : 0], lr);
-#pragma unroll
-                            for (int r = 0; r < R; ++r) rv[r] = expf(lr[r]);
-                        } else {
-#pragma unroll
-                            for (int r = 0; r < R; ++r) rv[r] = rho;
-                        }
-                        if (pfm) needr[u] = fetch(pop_top(pfm), u);
-                        else cp_async_commit();
-                        const size_t th = (size_t)(tok0 + i) * H + h;
-                        // what does not depend on lambda first: the step's own scalars (<d_t, k^2> was
-                        // recorded by the forward pass)
-#pragma unroll
-                        for (int r = 0; r < R; ++r) kap[r] = kk[r] * kk[r];
-                        al = rs.al[lane];
-                        const float e = hy.eta * b * rn, a2 = e * b;
-                        const float cc = fmaf(-a2, al, e);
-                        const float g1 = hy.eta * (1.0f - 2.0f * b * al) * rn;
-                        const float g2 = ns > 0.f ? -cc * rn : 0.f;
-#pragma unroll
-                        for (int r = 0; r < R; ++r) {
-                            if (!((mw >> r) & 1u)) lam[r] = 0.f;
-                            drho = fmaf(lam[r], dt[r], drho);
-                            dc = fmaf(lam[r], kap[r], dc);
-                        }
-                        dc = warp_sum(dc);
-                        drho = warp_sum(drho);
-                        const float da = -a2 * dc, dbt = g1 * dc, dn = g2 * dc;
-                        float out[R];
-                        if constexpr (VEC) {   // one gradient per coordinate: r_i lambda_i d_i
-                            if (a.dlog_ret) {
-                                float dl[R];
-#pragma unroll
-                                for (int r = 0; r < R; ++r) dl[r] = rv[r] * lam[r] * dt[r];
-                                store_row<R>(a.dlog_ret + th * K, lane, dl);
-                            }
-                        }
-#pragma unroll
-                        for (int r = 0; r < R; ++r) {
-                            const float dkap = cc * lam[r] + da * dt[r] + dn;
-                            out[r] = dkr[r] + dt[r] * dkt[r] + 2.0f * kk[r] * dkap;
-                            lam[r] = rv[r] * lam[r] + da * kap[r] + kk[r] * dkt[r];
-                        }
-                        store_row<R>(dkp + th * K, lane, out);
-                        if (lane == 0) {
-                            // added on top of what the chunk-local backward wrote; as reductions
-                            // without a return value, so that the sweep does not wait for memory
-                            if (hy.beta_aware) atomicAdd(&a.dbeta[th], dbt);
-                            if (hy.apf_mode == 1) atomicAdd(&a.dgate[th], rho * drho);
-                            if (hy.apf_mode == 2 && a.dlog_ret) a.dlog_ret[th] = rho * drho;
-                        }
-                    }
-                }
-            }
-            // state handed to the chunk below: lambda is live iff the chunk's first token was processed
-            lam_valid = (todo & 1ull) != 0ull;
-            if (!lam_valid) src = tok0;
-        }
-    }
-    if (a.dprecond_in) {
-        if (!lam_valid) restart(src);
-        store_row<R>(a.dprecond_in + ((size_t)s * H + h) * K, lane, lam);
-    }
-    cp_async_wait<0>();
-    if (lane == 0) {   // release the helper warps
-        cmd[0] = 0;
-        cmd[1] = 0;
-    }
-    asm volatile("bar.sync 1, 96;" ::: "memory");
 }
 
 template <typename TI, typename TO, int K>
 int fwd_launch(const P1Fwd& a, cudaStream_t st)
 {
     const long warps = (long)a.NT * a.H * 2;
-    const unsigned gspec = (unsigned)((warps + 3) / 4), gseq = (unsigned)((a.S * a.H + 3) / 4);
+    const unsigned gspec = (unsigned)((warps + 3) / 4);
     stage_mark(st, "phase1_spec");
     if (a.hy.apf_mode == 3) phase1_spec_kernel<TI, TO, K, true><<<gspec, 128, 0, st>>>(a);
     else phase1_spec_kernel<TI, TO, K, false><<<gspec, 128, 0, st>>>(a);
@@ -1576,11 +1634,11 @@ int fwd_launch(const P1Fwd& a, cudaStream_t st)
     const unsigned chains = (unsigned)(a.S * a.H);
     auto launch_seq = [&](auto kernel, size_t smem) {
         if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return false;
-        kernel<<<chains, 96, smem, st>>>(a);
+        kernel<<<chains, Pipe<K>::THREADS, smem, st>>>(a);
         return true;
     };
-    const bool okl = a.hy.apf_mode == 3 ? launch_seq(phase1_seq_kernel<TI, TO, K, true>, PN * sizeof(PipeBuf<TI, K, true>))
-                                        : launch_seq(phase1_seq_kernel<TI, TO, K, false>, PN * sizeof(PipeBuf<TI, K, false>));
+    const bool okl = a.hy.apf_mode == 3 ? launch_seq(phase1_seq_kernel<TI, TO, K, true>, sizeof(PipeShared<TI, K, true>))
+                                        : launch_seq(phase1_seq_kernel<TI, TO, K, false>, sizeof(PipeShared<TI, K, false>));
     if (!okl) return -1;
     return cudaGetLastError() == cudaSuccess ? 2 : -1;
 }
@@ -1599,11 +1657,11 @@ int bwd_launch(const P1Bwd& a, bool bulk, cudaStream_t st)
     const unsigned chains = (unsigned)(a.S * a.H);
     auto launch_seq = [&](auto kernel, size_t smem) {
         if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return false;
-        kernel<<<chains, 96, smem, st>>>(a);
+        kernel<<<chains, Pipe<K>::THREADS, smem, st>>>(a);
         return true;
     };
-    if (!(a.hy.apf_mode == 3 ? launch_seq(phase1_bwd_seq_kernel<T, K, true>, QN * sizeof(RevBuf<T, K, true>))
-                             : launch_seq(phase1_bwd_seq_kernel<T, K, false>, QN * sizeof(RevBuf<T, K, false>))))
+    if (!(a.hy.apf_mode == 3 ? launch_seq(phase1_bwd_seq_kernel<T, K, true>, sizeof(RevShared<T, K, true>))
+                             : launch_seq(phase1_bwd_seq_kernel<T, K, false>, sizeof(RevShared<T, K, false>))))
         return -1;
     ++n;
     return cudaGetLastError() == cudaSuccess ? n : -1;
@@ -1662,29 +1720,21 @@ int phase1_update(const osdn_params& p, const Hyper& hy, const void* k, const fl
     const unsigned chains = (unsigned)(pa.S * pa.H);
     stage_mark(st, "phase1_stream");
     const bool vec = hy.apf_mode == 3;
-    auto launch = [&](auto kernel, size_t buf_bytes) {
-        const size_t smem = PN * buf_bytes + PN * PB * sizeof(float);
+    auto launch = [&](auto kernel, size_t smem, int threads) {
         if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return false;
-        kernel<<<chains, 96, smem, st>>>(pa);
+        kernel<<<chains, threads, smem, st>>>(pa);
         return true;
     };
-    bool ok;
-    if (p.io_dtype == OSDN_FP32) {
-        if (p.K == 64)
-            ok = vec ? launch(phase1_stream_kernel<float, float, 64, true>, sizeof(PipeBuf<float, 64, true>))
-                     : launch(phase1_stream_kernel<float, float, 64, false>, sizeof(PipeBuf<float, 64, false>));
-        else
-            ok = vec ? launch(phase1_stream_kernel<float, float, 128, true>, sizeof(PipeBuf<float, 128, true>))
-                     : launch(phase1_stream_kernel<float, float, 128, false>, sizeof(PipeBuf<float, 128, false>));
-    } else {
-        using B16 = __nv_bfloat16;
-        if (p.K == 64)
-            ok = vec ? launch(phase1_stream_kernel<B16, B16, 64, true>, sizeof(PipeBuf<B16, 64, true>))
-                     : launch(phase1_stream_kernel<B16, B16, 64, false>, sizeof(PipeBuf<B16, 64, false>));
-        else
-            ok = vec ? launch(phase1_stream_kernel<B16, B16, 128, true>, sizeof(PipeBuf<B16, 128, true>))
-                     : launch(phase1_stream_kernel<B16, B16, 128, false>, sizeof(PipeBuf<B16, 128, false>));
-    }
+    auto typed = [&](auto t, auto kk) {
+        using T = decltype(t);
+        constexpr int K = decltype(kk)::value;
+        return vec ? launch(phase1_stream_kernel<T, T, K, true>, sizeof(PipeShared<T, K, true>), Pipe<K>::THREADS)
+                   : launch(phase1_stream_kernel<T, T, K, false>, sizeof(PipeShared<T, K, false>), Pipe<K>::THREADS);
+    };
+    using K64 = std::integral_constant<int, 64>;
+    using K128 = std::integral_constant<int, 128>;
+    const bool ok = p.io_dtype == OSDN_FP32 ? (p.K == 64 ? typed(float(), K64()) : typed(float(), K128()))
+                                            : (p.K == 64 ? typed(__nv_bfloat16(), K64()) : typed(__nv_bfloat16(), K128()));
     if (!ok) return -1;
     stage_end(st);
     return cudaGetLastError() == cudaSuccess ? 1 : -1;
