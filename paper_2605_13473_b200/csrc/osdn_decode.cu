@@ -11,24 +11,25 @@
 // exactly the recurrence the chunk path evaluates chunk by chunk, so that a prefill with osdn_fwd
 // followed by osdn_decode_step continues the same sequence.
 //
-// The work is bound by reading and writing the state once (V x K fp32 per chain).  Rows of S are
-// independent, so a chain is cut into V / 16 slices of 16 rows, one CTA each (4 warps x 4 rows); every
-// CTA repeats the tiny preconditioner update for its own use and slice 0 stores it.  The slices of a
-// chain form one thread-block cluster: the preconditioner is updated in place, so slice 0 may only
-// store the advanced vector once every slice of the chain has read the old one; a cluster barrier
-// (arrive after the read, wait before the store) gives exactly that order within the one launch,
-// however many waves the grid takes.  Lane l of a warp owns the R = K / 32 consecutive columns
-// R l .. R l + R - 1 of its rows (one vector access per row), the rows stay in registers over all
-// tokens of the call.
+// The work is bound by reading and writing the state once (V x K fp32 per chain).  Rows of S are independent; lane l of a
+// warp owns the R = K / 32 consecutive columns R l .. R l + R - 1 of its rows (one vector access per row), the rows stay
+// in registers over all tokens of the call, and every CTA repeats the preconditioner update for its own use.  Two shapes:
+//   few chains     V / 16 CTAs of 4 warps x 4 rows per chain: a call of a few sequences is bound by latency and is spread
+//                  over the chip.  They form one thread-block cluster: the preconditioner is updated in place, so the
+//                  CTA that stores the advanced vector may do so only once every CTA of the chain has read the old one;
+//                  a cluster barrier (arrive after the read, wait before the store) gives exactly that order.
+//   many chains    one CTA of 8 warps per chain (from one chain per SM on): no cluster to schedule, the preconditioner
+//                  update once per chain instead of eight times, a row's two sums share their shuffles with fifteen
+//                  other rows'.
+// Calls of several tokens stage the tokens' rows through shared memory, eight tokens at a time and one block ahead
+// (fetched one token ahead, a token cost a trip to memory).
 #include "osdn_common.cuh"
 
 namespace osdn {
 
 namespace {
 
-constexpr int DEC_RW = 4;        // rows per warp
-constexpr int DEC_WARPS = 4;     // warps per CTA
-constexpr int DEC_VB = DEC_RW * DEC_WARPS;
+constexpr int DEC_TB = 8;        // tokens of a staged block
 
 struct DecArgs {
     int B, L, H;
@@ -75,67 +76,109 @@ template <int R> __device__ __forceinline__ void dec_store(float* p, int lane, c
     else *reinterpret_cast<float2*>(p + 2 * lane) = make_float2(x[0], x[1]);
 }
 
-// VEC: vector retention (one log-retention per coordinate, log_ret [B,T,H,K]).
-template <typename T, int K, int V, bool VEC>
-__global__ void __cluster_dims__(V / DEC_VB, 1, 1) __launch_bounds__(DEC_WARPS * 32) decode_kernel(DecArgs a)
+// Two floats in one 64-bit register: the packed multiply and multiply-add issue once for both.
+struct F2 {
+    unsigned long long v;
+};
+__device__ __forceinline__ F2 pack2(float x, float y)
 {
-    constexpr int R = K / 32;
-    constexpr int SLICES = V / DEC_VB;
+    F2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(x), "f"(y));
+    return r;
+}
+__device__ __forceinline__ float2 unpack2(F2 a)
+{
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a.v));
+    return r;
+}
+__device__ __forceinline__ F2 mul2(F2 a, F2 b)
+{
+    F2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c)
+{
+    F2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+    return r;
+}
+
+// Lane l gets the warp's sum of x[l % N]: the N sums share their shuffles.
+template <int N> __device__ __forceinline__ float dec_row_sums(float (&x)[N], int lane)
+{
+#pragma unroll
+    for (int s = N / 2; s > 0; s >>= 1) {
+        const bool up = (lane & s) != 0;
+#pragma unroll
+        for (int i = 0; i < s; ++i) {
+            const float send = up ? x[i] : x[i + s], keep = up ? x[i + s] : x[i];
+            x[i] = keep + __shfl_xor_sync(0xffffffffu, send, s);
+        }
+    }
+    float v = x[0];
+#pragma unroll
+    for (int s = N; s < 32; s <<= 1) v += __shfl_xor_sync(0xffffffffu, v, s);
+    return v;
+}
+
+__device__ __forceinline__ void dec_cp16(void* dst, const void* src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void dec_cp4(void* dst, const void* src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+
+template <typename T, int K, int VB, bool VEC> struct alignas(16) DecBlock {
+    T k[DEC_TB][K], q[DEC_TB][K], v[DEC_TB][VB];
+    float beta[DEC_TB], gate[DEC_TB], lr[DEC_TB];
+    alignas(16) float lrv[VEC ? DEC_TB : 1][VEC ? K : 1];
+};
+
+// RW rows per warp, WARPS warps per CTA.  VEC: vector retention (one log-retention per coordinate, log_ret [B,T,H,K]).
+// MULTI: the call has several tokens per sequence.
+template <typename T, int K, int V, bool VEC, int RW, int WARPS, bool MULTI> __device__ __forceinline__ void decode_body(const DecArgs& a)
+{
+    constexpr int R = K / 32, VB = RW * WARPS, SLICES = V / VB, NT = WARPS * 32;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int chain = blockIdx.x / SLICES, slice = blockIdx.x % SLICES;
     const int b = chain / a.H, h = chain % a.H;
-    const int v0 = slice * DEC_VB + warp * DEC_RW;
+    const int vb0 = slice * VB, vw = warp * RW, row = lane % RW;   // the CTA's first row, the warp's first of these, this lane's
     const Hyper hy = a.hy;
     const T* qp = static_cast<const T*>(a.q);
     const T* kp = static_cast<const T*>(a.k);
     const T* vp = static_cast<const T*>(a.v);
     T* op = static_cast<T*>(a.out);
+    auto th_of = [&](int t) { return ((size_t)b * a.L + t) * a.H + h; };
 
-    float S[DEC_RW][R], d[R];
-    float* srow = a.state + ((size_t)chain * V + v0) * K;
+    float d[R];
+    F2 S[RW][R / 2];
+    float* srow = a.state + ((size_t)chain * V + vb0 + vw) * K;
     dec_load<R>(a.precond + (size_t)chain * K, lane, d);
 #pragma unroll
-    for (int r = 0; r < DEC_RW; ++r) dec_load<R>(srow + (size_t)r * K, lane, S[r]);
-    // This slice has read the chain's preconditioner: the arrival takes the loaded values as an operand, so
-    // it cannot issue before they have come back, and a load that has returned cannot see a later store.
-    // (A releasing arrival would also wait for the state rows, which are still in flight here.)
-    {
+    for (int r = 0; r < RW; ++r) {
+        float x[R];
+        dec_load<R>(srow + (size_t)r * K, lane, x);
+#pragma unroll
+        for (int j = 0; j < R / 2; ++j) S[r][j] = pack2(x[2 * j], x[2 * j + 1]);
+    }
+    if constexpr (SLICES > 1) {
+        // This slice has read the chain's preconditioner: the arrival takes the loaded values as an operand, so
+        // it cannot issue before they have come back, and a load that has returned cannot see a later store.
+        // (A releasing arrival would also wait for the state rows, which are still in flight here.)
         float seen = d[0];
 #pragma unroll
         for (int j = 1; j < R; ++j) seen += d[j];
         asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::"f"(seen) : "memory");
     }
 
-    // inputs of a token, fetched one token ahead
-    float kk[R], qq[R], vv[DEC_RW], bt, gt, lr, lrv[VEC ? R : 1];
-    auto fetch = [&](int t) {
-        const size_t th = ((size_t)b * a.L + t) * a.H + h;
-        dec_load<R>(kp + th * K, lane, kk);
-        dec_load<R>(qp + th * K, lane, qq);
-#pragma unroll
-        for (int r = 0; r < DEC_RW; ++r) vv[r] = ldf(vp + th * V + v0 + r);
-        bt = a.beta[th];
-        gt = a.gate[th];
-        lr = hy.apf_mode == 2 ? a.log_ret[th] : 0.f;
-        if constexpr (VEC) dec_load<R>(a.log_ret + th * K, lane, lrv);   // one log-retention per coordinate
-    };
-    fetch(0);
-    for (int t = 0; t < a.L; ++t) {
-        float k1[R], q1[R], v1[DEC_RW];
-#pragma unroll
-        for (int j = 0; j < R; ++j) { k1[j] = kk[j]; q1[j] = qq[j]; }
-#pragma unroll
-        for (int r = 0; r < DEC_RW; ++r) v1[r] = vv[r];
-        const float beta = bt, alpha = expf(gt);
+    // v: of this lane's row; lrv: the log-retention vector (VEC)
+    auto step = [&](int t, const float (&k1)[R], const float (&q1)[R], float v, float beta, float gate, float lr, const float (&lrv)[VEC ? R : 1]) {
+        const float alpha = expf(gate);
         const float rho1 = hy.apf_mode == 0 ? 1.0f : (hy.apf_mode == 1 ? alpha : expf(lr));
-        float rho[R];
-#pragma unroll
-        for (int j = 0; j < R; ++j) {
-            if constexpr (VEC) rho[j] = expf(lrv[j]);
-            else rho[j] = rho1;
-        }
-        if (t + 1 < a.L) fetch(t + 1);
-
         // preconditioner step
         float kap[R], ktil[R], sumk = 0.f, al = 0.f;
 #pragma unroll
@@ -152,55 +195,132 @@ __global__ void __cluster_dims__(V / DEC_VB, 1, 1) __launch_bounds__(DEC_WARPS *
         const float c = hy.eta * bb * (1.0f - bb * al) / n;
 #pragma unroll
         for (int j = 0; j < R; ++j) {
-            float x = fmaf(c, kap[j], rho[j] * d[j]);
+            float rho = rho1;
+            if constexpr (VEC) rho = expf(lrv[j]);
+            float x = fmaf(c, kap[j], rho * d[j]);
             if (hy.clamp) x = fminf(fmaxf(x, hy.d_min), hy.d_max);
             d[j] = x;
         }
-
-        // rank-1 write and read-out, row by row (the four reductions of a step are independent)
-        float dot[DEC_RW], o[DEC_RW];
+        // rank-1 write and read-out
+        F2 k2[R / 2], q2[R / 2], t2[R / 2];
 #pragma unroll
-        for (int r = 0; r < DEC_RW; ++r) {
-            float s = 0.f;
-#pragma unroll
-            for (int j = 0; j < R; ++j) s = fmaf(S[r][j], k1[j], s);
-            dot[r] = s;
+        for (int j = 0; j < R / 2; ++j) {
+            k2[j] = pack2(k1[2 * j], k1[2 * j + 1]);
+            q2[j] = pack2(q1[2 * j], q1[2 * j + 1]);
+            t2[j] = pack2(ktil[2 * j], ktil[2 * j + 1]);
         }
+        auto dots = [&](const F2 (&x)[R / 2]) {   // lane l: row l % RW
+            float p[RW];
 #pragma unroll
-        for (int r = 0; r < DEC_RW; ++r) dot[r] = dec_warp_sum(dot[r]);
+            for (int r = 0; r < RW; ++r) {
+                F2 s = mul2(S[r][0], x[0]);
 #pragma unroll
-        for (int r = 0; r < DEC_RW; ++r) {
-            const float rv = beta * (v1[r] - alpha * dot[r]);
-            float s = 0.f;
-#pragma unroll
-            for (int j = 0; j < R; ++j) {
-                S[r][j] = fmaf(alpha, S[r][j], rv * ktil[j]);
-                s = fmaf(S[r][j], q1[j], s);
+                for (int j = 1; j < R / 2; ++j) s = fma2(S[r][j], x[j], s);
+                const float2 u = unpack2(s);
+                p[r] = u.x + u.y;
             }
-            o[r] = s;
+            return dec_row_sums(p, lane);
+        };
+        const float rv = beta * (v - alpha * dots(k2));
+        const F2 alpha2 = pack2(alpha, alpha);
+#pragma unroll
+        for (int r = 0; r < RW; ++r) {
+            const float x = __shfl_sync(0xffffffffu, rv, r);
+            const F2 x2 = pack2(x, x);
+#pragma unroll
+            for (int j = 0; j < R / 2; ++j) S[r][j] = fma2(alpha2, S[r][j], mul2(x2, t2[j]));
         }
-#pragma unroll
-        for (int r = 0; r < DEC_RW; ++r) o[r] = dec_warp_sum(o[r]);
-        if (lane < DEC_RW) {
-            float mine = o[0];
-#pragma unroll
-            for (int r = 1; r < DEC_RW; ++r) mine = lane == r ? o[r] : mine;
-            const size_t th = ((size_t)b * a.L + t) * a.H + h;
-            stf(op + th * V + v0 + lane, hy.scale * mine);
+        const float o = dots(q2);
+        if (lane < RW) stf(op + th_of(t) * V + vb0 + vw + lane, hy.scale * o);
+    };
+
+    if constexpr (!MULTI) {
+        const size_t th = th_of(0);
+        float k1[R], q1[R], lrv[VEC ? R : 1];
+        dec_load<R>(kp + th * K, lane, k1);
+        dec_load<R>(qp + th * K, lane, q1);
+        if constexpr (VEC) dec_load<R>(a.log_ret + th * K, lane, lrv);
+        step(0, k1, q1, ldf(vp + th * V + vb0 + vw + row), a.beta[th], a.gate[th], hy.apf_mode == 2 ? a.log_ret[th] : 0.f, lrv);
+    } else {
+        __shared__ DecBlock<T, K, VB, VEC> blk[2];
+        auto stage = [&](int t0) {
+            DecBlock<T, K, VB, VEC>& B = blk[(t0 / DEC_TB) & 1];
+            const int n = min(DEC_TB, a.L - t0);
+            constexpr int PK = K * (int)sizeof(T) / 16, PV = VB * (int)sizeof(T) / 16, PL = VEC ? K / 4 : 0, PER = 2 * PK + PV + PL, EL = 16 / (int)sizeof(T);
+            for (int e = threadIdx.x; e < n * PER; e += NT) {
+                const int j = e / PER, p = e % PER;
+                const size_t th = th_of(t0 + j);
+                if (p < PK) dec_cp16(&B.k[j][p * EL], kp + th * K + p * EL);
+                else if (p < 2 * PK) dec_cp16(&B.q[j][(p - PK) * EL], qp + th * K + (p - PK) * EL);
+                else if (p < 2 * PK + PV) dec_cp16(&B.v[j][(p - 2 * PK) * EL], vp + th * V + vb0 + (p - 2 * PK) * EL);
+                else dec_cp16(&B.lrv[VEC ? j : 0][VEC ? (p - 2 * PK - PV) * 4 : 0], a.log_ret + th * K + (p - 2 * PK - PV) * 4);
+            }
+            if ((int)threadIdx.x < n) {
+                const size_t th = th_of(t0 + threadIdx.x);
+                dec_cp4(&B.beta[threadIdx.x], a.beta + th);
+                dec_cp4(&B.gate[threadIdx.x], a.gate + th);
+                if (hy.apf_mode == 2) dec_cp4(&B.lr[threadIdx.x], a.log_ret + th);
+            }
+            asm volatile("cp.async.commit_group;" ::: "memory");
+        };
+        stage(0);
+        for (int t0 = 0; t0 < a.L; t0 += DEC_TB) {
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+            __syncthreads();   // the block is there for everybody, and everybody is done with the one before
+            if (t0 + DEC_TB < a.L) stage(t0 + DEC_TB);
+            const DecBlock<T, K, VB, VEC>& B = blk[(t0 / DEC_TB) & 1];
+            const int n = min(DEC_TB, a.L - t0);
+            for (int j = 0; j < n; ++j) {
+                float k1[R], q1[R], lrv[VEC ? R : 1];
+                dec_load<R>(B.k[j], lane, k1);
+                dec_load<R>(B.q[j], lane, q1);
+                if constexpr (VEC) dec_load<R>(B.lrv[VEC ? j : 0], lane, lrv);
+                step(t0 + j, k1, q1, ldf(&B.v[j][vw + row]), B.beta[j], B.gate[j], hy.apf_mode == 2 ? B.lr[j] : 0.f, lrv);
+            }
         }
     }
 #pragma unroll
-    for (int r = 0; r < DEC_RW; ++r) dec_store<R>(srow + (size_t)r * K, lane, S[r]);
-    // every slice of the chain has read the old preconditioner before slice 0 overwrites it
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    for (int r = 0; r < RW; ++r) {
+        float x[R];
+#pragma unroll
+        for (int j = 0; j < R / 2; ++j) {
+            const float2 u = unpack2(S[r][j]);
+            x[2 * j] = u.x;
+            x[2 * j + 1] = u.y;
+        }
+        dec_store<R>(srow + (size_t)r * K, lane, x);
+    }
+    // every warp (of every slice) of the chain has read the old preconditioner before it is overwritten
+    if constexpr (SLICES > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    else __syncthreads();
     if (slice == 0 && warp == 0) dec_store<R>(a.precond + (size_t)chain * K, lane, d);
 }
 
-// One cluster per chain: its V / 16 slices (8 or 4 CTAs, within the portable cluster size; the size is part of
-// the kernel, so the launch is a plain one).
+constexpr int FEW_RW = 4, FEW_WARPS = 4, MANY_WARPS = 8;
+
+template <typename T, int K, int V, bool VEC, bool MULTI>
+__global__ void __cluster_dims__(V / (FEW_RW * FEW_WARPS), 1, 1) __launch_bounds__(FEW_WARPS * 32) decode_few_kernel(DecArgs a)
+{
+    decode_body<T, K, V, VEC, FEW_RW, FEW_WARPS, MULTI>(a);
+}
+template <typename T, int K, int V, bool VEC, bool MULTI>
+__global__ void __launch_bounds__(MANY_WARPS * 32, 2) decode_many_kernel(DecArgs a)
+{
+    decode_body<T, K, V, VEC, V / MANY_WARPS, MANY_WARPS, MULTI>(a);
+}
+
+// From one chain per SM on, a CTA per chain fills the chip.
+constexpr unsigned MANY_CHAINS = 148;
 template <typename T, int K, int V, bool VEC> bool launch_one(unsigned chains, const DecArgs& a, cudaStream_t st)
 {
-    decode_kernel<T, K, V, VEC><<<chains * (unsigned)(V / DEC_VB), DEC_WARPS * 32, 0, st>>>(a);
+    constexpr unsigned SLICES = V / (FEW_RW * FEW_WARPS);
+    if (chains >= MANY_CHAINS) {
+        if (a.L > 1) decode_many_kernel<T, K, V, VEC, true><<<chains, MANY_WARPS * 32, 0, st>>>(a);
+        else decode_many_kernel<T, K, V, VEC, false><<<chains, MANY_WARPS * 32, 0, st>>>(a);
+    } else {
+        if (a.L > 1) decode_few_kernel<T, K, V, VEC, true><<<chains * SLICES, FEW_WARPS * 32, 0, st>>>(a);
+        else decode_few_kernel<T, K, V, VEC, false><<<chains * SLICES, FEW_WARPS * 32, 0, st>>>(a);
+    }
     return cudaGetLastError() == cudaSuccess;
 }
 
