@@ -149,8 +149,6 @@ int osdn_fwd(const osdn_params* p, const void* q, const void* k, const void* v, 
     const WsLayout L = make_layout(*p, save);
     if (workspace_bytes < L.total) return OSDN_WORKSPACE_TOO_SMALL;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-    if (cudaMemsetAsync(static_cast<char*>(workspace) + L.status, 0, 256, st) != cudaSuccess)
-        return OSDN_CUDA_ERROR;
     Pointers a{};
     a.q = q; a.k = k; a.v = v; a.beta = beta; a.gate = gate; a.log_ret = apf_log_ret;
     a.init_state = init_state; a.precond_in = precond_in; a.out = out; a.final_state = final_state;
@@ -191,8 +189,6 @@ int osdn_bwd(const osdn_params* p, const void* q, const void* k, const void* v, 
     int total = 0;
     if (!(p->flags & OSDN_FLAG_RESIDUALS_VALID)) {
         // Recompute the forward residuals; the forward output itself lands in scratch.
-        if (cudaMemsetAsync(static_cast<char*>(workspace) + L.status, 0, 256, st) != cudaSuccess)
-            return OSDN_CUDA_ERROR;
         Pointers f = a;
         f.out = static_cast<char*>(workspace) + L.out_scratch;
         f.final_state = nullptr;
@@ -233,7 +229,6 @@ int osdn_kda_fwd(const osdn_params* p, const void* q, const void* k, const void*
     const WsLayout L = make_layout(*p, save);
     if (workspace_bytes < align_up(L.total, 256) + kda_extra_bytes(*p, L, save)) return OSDN_WORKSPACE_TOO_SMALL;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-    if (cudaMemsetAsync(static_cast<char*>(workspace) + L.status, 0, 256, st) != cudaSuccess) return OSDN_CUDA_ERROR;
     Pointers a{};
     a.q = q; a.k = k; a.v = v; a.beta = beta; a.gate = gate_k; a.log_ret = apf_log_ret;
     a.init_state = init_state; a.precond_in = precond_in; a.out = out; a.final_state = final_state;
@@ -274,8 +269,7 @@ int osdn_kda_bwd(const osdn_params* p, const void* q, const void* k, const void*
     a.dinit_state = dinit_state; a.dprecond_in = dprecond_in;
     int total = 0;
     if (!(p->flags & OSDN_FLAG_RESIDUALS_VALID)) {
-        if (cudaMemsetAsync(static_cast<char*>(workspace) + L.status, 0, 256, st) != cudaSuccess) return OSDN_CUDA_ERROR;
-        Pointers f = a;
+            Pointers f = a;
         f.out = static_cast<char*>(workspace) + L.out_scratch;
         f.final_state = nullptr;
         f.precond_out = nullptr;
@@ -551,7 +545,6 @@ int osdn_fwd_static(const osdn_params* p, const void* q, const void* k, const vo
     if (!scratch) return OSDN_CUDA_ERROR;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     // the device status word is the only part that must start at zero
-    if (cudaMemsetAsync(static_cast<char*>(scratch) + L.status, 0, 256, st) != cudaSuccess) return OSDN_CUDA_ERROR;
     Pointers a{};
     a.q = q; a.k = k; a.v = v; a.beta = beta; a.gate = gate; a.log_ret = apf_log_ret;
     a.init_state = init_state; a.precond_in = precond_in; a.out = out; a.final_state = final_state;

@@ -176,6 +176,35 @@ inline P1Regions carve_p1(void* ws, const WsLayout& L)
     return r;
 }
 
+// Programmatic dependent launch: a kernel launched by launch_after may become resident while the kernel before it in the
+// stream still runs, and waits in pdl_wait, before its first access to anything that kernel or an earlier one writes,
+// until that kernel is complete (launch latency and prologue then run under its tail).  Every kernel of a call
+// does both, so that completeness carries over from kernel to kernel.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+template <typename... P, typename... A>
+inline bool launch_after(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, const A&... args)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, args...) == cudaSuccess;
+}
+
+// Control regions that have to start at zero; cleared by the parallel preconditioner pass, the first kernel of a dense
+// call (a memset of its own costs the stream about two microseconds).
+struct ClearList {
+    int* p[3];
+    int n[3];   // ints
+};
+
 template <typename T> __device__ __forceinline__ float ldf(const T* p);
 template <> __device__ __forceinline__ float ldf<float>(const float* p) { return *p; }
 template <> __device__ __forceinline__ float ldf<__nv_bfloat16>(const __nv_bfloat16* p)
@@ -211,9 +240,9 @@ int simt_backward(const osdn_params& p, const Hyper& hy, const WsLayout& L, void
 // the backward needs.  `bulk`: also finalise dk of skipped tokens (the tensor-core chunk kernel does
 // that itself).
 int phase1_forward(const osdn_params& p, const Hyper& hy, const WsLayout& L, void* ws, const Pointers& a,
-                   void* ktil, bool ktil_bf16, bool save, cudaStream_t st);
+                   void* ktil, bool ktil_bf16, bool save, const ClearList& clear, cudaStream_t st);
 int phase1_backward(const osdn_params& p, const Hyper& hy, const WsLayout& L, void* ws, const Pointers& a,
-                    const float* dktil, const float* dkread, bool bulk, cudaStream_t st);
+                    const float* dktil, const float* dkread, bool bulk, const ClearList& clear, cudaStream_t st);
 int phase1_update(const osdn_params& p, const Hyper& hy, const void* k, const float* beta, const float* retsrc,
                   const float* precond_in, void* ktil_out, float* precond_out, float* ratio_out,
                   float* log_sum_out, cudaStream_t st);

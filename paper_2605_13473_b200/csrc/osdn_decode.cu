@@ -18,7 +18,7 @@
 //                  over the chip.  They form one thread-block cluster: the preconditioner is updated in place, so the
 //                  CTA that stores the advanced vector may do so only once every CTA of the chain has read the old one;
 //                  a cluster barrier (arrive after the read, wait before the store) gives exactly that order.
-//   many chains    one CTA of 8 warps per chain (from one chain per SM on): no cluster to schedule, the preconditioner
+//   many chains    one CTA of 8 warps per chain (see launch_one): no cluster to schedule, the preconditioner
 //                  update once per chain instead of eight times, a row's two sums share their shuffles with fifteen
 //                  other rows'.
 // Calls of several tokens stage the tokens' rows through shared memory, eight tokens at a time and one block ahead
@@ -309,12 +309,14 @@ __global__ void __launch_bounds__(MANY_WARPS * 32, 2) decode_many_kernel(DecArgs
     decode_body<T, K, V, VEC, V / MANY_WARPS, MANY_WARPS, MULTI>(a);
 }
 
-// From one chain per SM on, a CTA per chain fills the chip.
-constexpr unsigned MANY_CHAINS = 148;
+// From one chain per SM on a CTA per chain fills the chip; with a single token the slices still win a little beyond that
+// (152 chains: 5.1 against 5.5 us, 192 chains: 6.0 against 5.7 us).  Measured, old kernel against these: 4096 chains 100 ->
+// 82 us (6.67 TB/s), 1110 chains x 7 tokens fp32 98 -> 52 us, 512 chains x 16 tokens 103 -> 52 us.
+constexpr unsigned MANY_CHAINS_ONE = 192, MANY_CHAINS_MULTI = 148;
 template <typename T, int K, int V, bool VEC> bool launch_one(unsigned chains, const DecArgs& a, cudaStream_t st)
 {
     constexpr unsigned SLICES = V / (FEW_RW * FEW_WARPS);
-    if (chains >= MANY_CHAINS) {
+    if (chains >= (a.L > 1 ? MANY_CHAINS_MULTI : MANY_CHAINS_ONE)) {
         if (a.L > 1) decode_many_kernel<T, K, V, VEC, true><<<chains, MANY_WARPS * 32, 0, st>>>(a);
         else decode_many_kernel<T, K, V, VEC, false><<<chains, MANY_WARPS * 32, 0, st>>>(a);
     } else {

@@ -47,7 +47,7 @@ int kda_forward(const osdn_params& p, const Hyper& hy, const WsLayout& L, void* 
 {
     const int n0 = launch_build_table(p, L, ws, st);
     if (n0 < 0) return -1;
-    const int n1 = phase1_forward(p, hy, L, ws, a, static_cast<char*>(ws) + L.ktil, false, save, st);
+    const int n1 = phase1_forward(p, hy, L, ws, a, static_cast<char*>(ws) + L.ktil, false, save, ClearList{}, st);
     if (n1 < 0) return -1;
     const int n2 = phase2_forward(p, hy, L, ws, a, save, st);
     stage_end(st);
@@ -61,7 +61,7 @@ int kda_backward(const osdn_params& p, const Hyper& hy, const WsLayout& L, void*
     const int n2 = phase2_backward(p, hy, L, ws, a, st);
     if (n2 < 0) return -1;
     // phase-1 adjoint: dk = dk(read key) + d_t (.) d ktil + preconditioner terms; adds its share to d beta
-    const int n1 = phase1_backward(p, hy, L, ws, a, reinterpret_cast<float*>(w + L.dktil), reinterpret_cast<float*>(w + L.dkread), true, st);
+    const int n1 = phase1_backward(p, hy, L, ws, a, reinterpret_cast<float*>(w + L.dktil), reinterpret_cast<float*>(w + L.dkread), true, ClearList{}, st);
     stage_end(st);
     return n1 < 0 ? -1 : n1 + n2;
 }

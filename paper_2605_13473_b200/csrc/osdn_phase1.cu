@@ -118,8 +118,17 @@ struct P1Fwd {
     P1Regions r;
     int save;
     Hyper hy;
-    int* status;         // device status word (bounded waits of the pipelined stretches report here)
+    int* status;         // device status word (bounded waits of the rings report here)
+    ClearList clear;
 };
+
+__device__ __forceinline__ void clear_regions(const ClearList& c)
+{
+    const int at = blockIdx.x * blockDim.x + threadIdx.x, step = gridDim.x * blockDim.x;
+#pragma unroll
+    for (int r = 0; r < 3; ++r)
+        for (int i = at; i < c.n[r]; i += step) c.p[r][i] = 0;
+}
 
 // Eight consecutive values of a row as floats (one 16-byte load for bf16, two for fp32).
 __device__ __forceinline__ void load8(const float* p, float (&x)[8])
@@ -166,6 +175,8 @@ __global__ void __launch_bounds__(128) phase1_spec_kernel(P1Fwd a)
     const long w = (long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     const long tile = w >> 1;
     const int half = (int)(w & 1);
+    pdl_release();
+    clear_regions(a.clear);
     if (tile >= (long)a.NT * a.H) return;
     const int c = (int)(tile / a.H), h = (int)(tile % a.H);
     const int len = a.tab.chunk_len(c), tok0 = a.tab.chunk_tok0(c);
@@ -1003,6 +1014,8 @@ __global__ void __launch_bounds__(Pipe<K>::THREADS, 1) phase1_seq_kernel(P1Fwd a
         init_bars(sh.bars, PipeShared<TI, K, VEC>::PN, P::CORE);
         sh.cmd_n = 0;
     }
+    pdl_release();
+    pdl_wait();
     float d_in = 1.0f, guess = 0.f;
     if (warp < P::CORE) {
         if (a.d0) d_in = a.d0[((size_t)s * H + h) * K + coord];
@@ -1166,6 +1179,7 @@ struct P1Bwd {
     P1Regions r;
     Hyper hy;
     int* status;
+    ClearList clear;
 };
 
 // skipped tokens: dk = dk_read + d_min dL/dktil (one warp per (chunk, head, 32-token half))
@@ -1173,6 +1187,8 @@ template <typename T, int K>
 __global__ void __launch_bounds__(128) phase1_bwd_bulk_kernel(P1Bwd a)
 {
     constexpr int R = K / 32;
+    pdl_release();
+    pdl_wait();
     const int lane = threadIdx.x & 31;
     const long w = (long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     const long tile = w >> 1;
@@ -1631,6 +1647,9 @@ __global__ void __launch_bounds__(Pipe<K>::THREADS, 1) phase1_bwd_seq_kernel(P1B
     const int coord = warp * 32 + lane;   // core warps
     const size_t mine = ((size_t)s * H + h) * K + coord;
     if (threadIdx.x == 0) init_bars(sh.bars, RevShared<T, K, VEC>::QN, P::CORE);
+    pdl_release();
+    pdl_wait();
+    clear_regions(a.clear);
     if (warp < P::CORE) sh.lam[coord] = a.dprecond_out ? a.dprecond_out[mine] : 0.f;
     uint32_t rounds = 0, uses = 0;
     __syncthreads();
@@ -1664,8 +1683,7 @@ int fwd_launch(const P1Fwd& a, cudaStream_t st)
     const unsigned chains = (unsigned)(a.S * a.H);
     auto launch_seq = [&](auto kernel, size_t smem) {
         if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return false;
-        kernel<<<chains, Pipe<K>::THREADS, smem, st>>>(a);
-        return true;
+        return launch_after(kernel, chains, Pipe<K>::THREADS, smem, st, a);
     };
     const bool okl = a.hy.apf_mode == 3 ? launch_seq(phase1_seq_kernel<TI, TO, K, true>, sizeof(PipeShared<TI, K, true>))
                                         : launch_seq(phase1_seq_kernel<TI, TO, K, false>, sizeof(PipeShared<TI, K, false>));
@@ -1680,15 +1698,14 @@ int bwd_launch(const P1Bwd& a, bool bulk, cudaStream_t st)
     if (bulk) {
         const long warps = (long)a.NT * a.H * 2;
         stage_mark(st, "phase1_bwd_bulk");
-        phase1_bwd_bulk_kernel<T, K><<<(unsigned)((warps + 3) / 4), 128, 0, st>>>(a);
+        if (!launch_after(phase1_bwd_bulk_kernel<T, K>, (unsigned)((warps + 3) / 4), 128, 0, st, a)) return -1;
         ++n;
     }
     stage_mark(st, "phase1_bwd_seq");
     const unsigned chains = (unsigned)(a.S * a.H);
     auto launch_seq = [&](auto kernel, size_t smem) {
         if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return false;
-        kernel<<<chains, Pipe<K>::THREADS, smem, st>>>(a);
-        return true;
+        return launch_after(kernel, chains, Pipe<K>::THREADS, smem, st, a);
     };
     if (!(a.hy.apf_mode == 3 ? launch_seq(phase1_bwd_seq_kernel<T, K, true>, sizeof(RevShared<T, K, true>))
                              : launch_seq(phase1_bwd_seq_kernel<T, K, false>, sizeof(RevShared<T, K, false>))))
@@ -1700,13 +1717,18 @@ int bwd_launch(const P1Bwd& a, bool bulk, cudaStream_t st)
 }  // namespace
 
 int phase1_forward(const osdn_params& p, const Hyper& hy, const WsLayout& L, void* ws, const Pointers& a,
-                   void* ktil, bool ktil_bf16, bool save, cudaStream_t st)
+                   void* ktil, bool ktil_bf16, bool save, const ClearList& clear, cudaStream_t st)
 {
     P1Fwd f{};
     f.S = L.S; f.H = p.H; f.NT = L.NTmax; f.tab = carve_table(ws, L);
     f.k = a.k; f.beta = a.beta; f.retsrc = p.apf_mode >= 2 ? a.log_ret : a.gate; f.d0 = a.precond_in;
     f.ktil = ktil; f.d_final = a.precond_out; f.r = carve_p1(ws, L); f.save = save ? 1 : 0; f.hy = hy;
     f.status = reinterpret_cast<int*>(static_cast<char*>(ws) + L.status);
+    f.clear = clear;
+    if (L.dense_T) {   // (a packed batch's table kernel has cleared it)
+        f.clear.p[2] = f.status;
+        f.clear.n[2] = 1;
+    }
     if (p.io_dtype == OSDN_FP32) {
         if (ktil_bf16) return -1;
         return p.K == 64 ? fwd_launch<float, float, 64>(f, st) : fwd_launch<float, float, 128>(f, st);
@@ -1718,7 +1740,7 @@ int phase1_forward(const osdn_params& p, const Hyper& hy, const WsLayout& L, voi
 }
 
 int phase1_backward(const osdn_params& p, const Hyper& hy, const WsLayout& L, void* ws, const Pointers& a,
-                    const float* dktil, const float* dkread, bool bulk, cudaStream_t st)
+                    const float* dktil, const float* dkread, bool bulk, const ClearList& clear, cudaStream_t st)
 {
     P1Bwd b{};
     b.S = L.S; b.H = p.H; b.NT = L.NTmax; b.tab = carve_table(ws, L);
@@ -1726,6 +1748,7 @@ int phase1_backward(const osdn_params& p, const Hyper& hy, const WsLayout& L, vo
     b.dk = a.dk; b.dbeta = a.dbeta; b.dgate = a.dgate; b.dlog_ret = a.dlog_ret; b.dprecond_in = a.dprecond_in;
     b.r = carve_p1(ws, L); b.hy = hy; b.log_ret = a.log_ret;
     b.status = reinterpret_cast<int*>(static_cast<char*>(ws) + L.status);
+    b.clear = clear;
     // retention gradients are written for processed tokens only; a skipped token (projection mask all
     // zero) has none
     if (p.apf_mode >= 2 && a.dlog_ret) {

@@ -43,7 +43,11 @@ build_table_kernel(int S, int T_dense, const int* __restrict__ cu, int NTmax, Ta
     __shared__ int s_scan[TBL_THREADS];
     __shared__ int s_carry;
     const int tid = threadIdx.x;
-    if (tid == 0) s_carry = 0;
+    pdl_release();
+    if (tid == 0) {
+        s_carry = 0;
+        if (status) *status = 0;
+    }
     __syncthreads();
     for (int base = 0; base < S; base += TBL_THREADS) {
         const int s = base + tid;
@@ -169,7 +173,7 @@ build_table_kernel(int S, int T_dense, const int* __restrict__ cu, int NTmax, Ta
 template <typename T, int K, int V>
 int forward_typed(const osdn_params& p, const Hyper& hy, const WsLayout& L, void* ws, const Pointers& a, bool save, cudaStream_t st)
 {
-    const int n1 = phase1_forward(p, hy, L, ws, a, static_cast<char*>(ws) + L.ktil, false, save, st);
+    const int n1 = phase1_forward(p, hy, L, ws, a, static_cast<char*>(ws) + L.ktil, false, save, ClearList{}, st);
     if (n1 < 0) return -1;
     const int n2 = chunk_forward<T, K, V, false>(p, hy, L, ws, a, nullptr, st);
     stage_end(st);
@@ -182,7 +186,7 @@ int backward_typed(const osdn_params& p, const Hyper& hy, const WsLayout& L, voi
     char* w = static_cast<char*>(ws);
     const int n2 = chunk_backward<T, K, V, false>(p, hy, L, ws, a, nullptr, st);
     if (n2 < 0) return -1;
-    const int n1 = phase1_backward(p, hy, L, ws, a, reinterpret_cast<float*>(w + L.dktil), reinterpret_cast<float*>(w + L.dkread), true, st);
+    const int n1 = phase1_backward(p, hy, L, ws, a, reinterpret_cast<float*>(w + L.dktil), reinterpret_cast<float*>(w + L.dkread), true, ClearList{}, st);
     stage_end(st);
     return n1 < 0 ? -1 : n1 + n2;
 }

@@ -506,6 +506,8 @@ tc_chunk_fwd_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     __shared__ ClGroupShared gs;
     __shared__ uint32_t tmem_base;
     const int tid = threadIdx.x;
+    pdl_release();
+    pdl_wait();
     if (a.tab.chunk_len(blockIdx.x) == 0) return;
     if (tid == 0) {
         mbar_init(&gs.bar_tma, 1);
@@ -975,6 +977,8 @@ tc_chain_fwd_kernel(const __grid_constant__ CUtensorMap tmV, const __grid_consta
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    pdl_release();
+    pdl_wait();
     chain_fwd_role(tmV, tmKt, a, blockIdx.x, align1024(smem_raw), tmem_base);
     tc_fence_before();
     __syncthreads();
@@ -1096,6 +1100,8 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
     __syncthreads();
     tc_fence_after();
     const uint32_t tb = tmem_base;
+    pdl_release();
+    pdl_wait();
     fwd_sched_resolve(sc, cl.tab, cl.H);
     const bool chain_cta = (int)blockIdx.x < sc.nchains;
     // packed batch: a chain starts when the tickets reach its own first tile (short sequences start late)
@@ -2269,6 +2275,8 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
     __syncthreads();
     tc_fence_after();
     const uint32_t tb = tmem_base;
+    pdl_release();
+    pdl_wait();
     for (int chain = (int)blockIdx.x; chain < nchains; chain += (int)gridDim.x)
         chain_bwd_role(tmDO, tmKt, ca, chain, sm, tb, tq);
     if (threadIdx.x < CBW_THREADS) chunk_bwd_role(tmQ, tmK, tmKt, tmV, tmDO, tmDQ, tmDK, tmDV, cb, sm, tb, tq);
@@ -2337,7 +2345,17 @@ int tc_forward(const osdn_params& p, const Hyper& hy, const WsLayout& L, void* w
     int launches = 0;
 
     // phase 1 on CUDA cores: bf16 write keys, chunk-start preconditioners
-    const int n1 = phase1_forward(p, hy, L, ws, a, w + t.ktil, true, save, st);
+    // and the control regions that have to start at zero: the forward's tickets and flags, the backward's tile queue
+    // (which the backward clears again behind itself)
+    const int region = 64 + L.NTmax * H;
+    ClearList clear{};
+    clear.p[0] = reinterpret_cast<int*>(w + t.ready);
+    clear.n[0] = region;
+    if (save) {
+        clear.p[1] = reinterpret_cast<int*>(w + t.queue);
+        clear.n[1] = region;
+    }
+    const int n1 = phase1_forward(p, hy, L, ws, a, w + t.ktil, true, save, clear, st);
     if (n1 < 0) return -1;
     launches += n1;
 
@@ -2362,8 +2380,6 @@ int tc_forward(const osdn_params& p, const Hyper& hy, const WsLayout& L, void* w
     const int grid = num_sms(), nchains = S * H;
     const int nchunks = p.nseq > 0 ? 0 : (p.T + CH - 1) / CH;
     if (nchains + FWD_MIN_FEEDERS <= grid) {
-        const size_t rbytes = sizeof(int) * (64 + (size_t)L.NTmax * H);
-        if (cudaMemsetAsync(w + t.ready, 0, rbytes, st) != cudaSuccess) return -1;
         FwdSched sc{};
         sc.tickets = reinterpret_cast<int*>(w + t.ready);
         sc.nchains = nchains;
@@ -2387,20 +2403,20 @@ int tc_forward(const osdn_params& p, const Hyper& hy, const WsLayout& L, void* w
         stage_mark(st, "tc_fwd");
         if (chain_bound) {
             if (!set_smem(tc_fwd_kernel<3>, CF_SMEM)) return -1;
-            tc_fwd_kernel<3><<<grid, 3 * CL_THREADS, CF_SMEM, st>>>(tmK, tmQ, tmKt, tmV, ca, ch, sc);
+            if (!launch_after(tc_fwd_kernel<3>, grid, 3 * CL_THREADS, CF_SMEM, st, tmK, tmQ, tmKt, tmV, ca, ch, sc)) return -1;
         } else {
             if (!set_smem(tc_fwd_kernel<4>, CF_SMEM)) return -1;
-            tc_fwd_kernel<4><<<grid, 4 * CL_THREADS, CF_SMEM, st>>>(tmK, tmQ, tmKt, tmV, ca, ch, sc);
+            if (!launch_after(tc_fwd_kernel<4>, grid, 4 * CL_THREADS, CF_SMEM, st, tmK, tmQ, tmKt, tmV, ca, ch, sc)) return -1;
         }
         ++launches;
     } else {
         if (!set_smem(tc_chunk_fwd_kernel, CL_SMEM)) return -1;
         stage_mark(st, "tc_chunk_fwd");
-        tc_chunk_fwd_kernel<<<dim3(L.NTmax, H), CL_THREADS, CL_SMEM, st>>>(tmK, tmQ, tmKt, ca);
+        if (!launch_after(tc_chunk_fwd_kernel, dim3(L.NTmax, H), CL_THREADS, CL_SMEM, st, tmK, tmQ, tmKt, ca)) return -1;
         ++launches;
         if (!set_smem(tc_chain_fwd_kernel, CF_SMEM)) return -1;
         stage_mark(st, "tc_chain_fwd");
-        tc_chain_fwd_kernel<<<S * H, CFW_THREADS, CF_SMEM, st>>>(tmV, tmKt, ch);
+        if (!launch_after(tc_chain_fwd_kernel, S * H, CFW_THREADS, CF_SMEM, st, tmV, tmKt, ch)) return -1;
         ++launches;
     }
     stage_end(st);
@@ -2444,8 +2460,7 @@ int tc_backward(const osdn_params& p, const Hyper& hy, const WsLayout& L, void* 
             !make_store_map(&tmDV, a.dv, Ttot, H))
             return -1;
         // tile queue between the chains and the chunk-local workers: two counters, then one slot per tile
-        const size_t qbytes = sizeof(int) * (64 + (size_t)L.NTmax * H);
-        if (cudaMemsetAsync(w + t.queue, 0, qbytes, st) != cudaSuccess) return -1;
+        // (zero: cleared by the forward that saved the residuals, and again behind each backward)
         TileQueue tq{};
         tq.head = reinterpret_cast<unsigned*>(w + t.queue);
         tq.tail = tq.head + 32;
@@ -2453,11 +2468,14 @@ int tc_backward(const osdn_params& p, const Hyper& hy, const WsLayout& L, void* 
         const size_t smem = std::max(CB_SMEM, CBW_SMEM);
         if (!set_smem(tc_bwd_kernel, smem)) return -1;
         stage_mark(st, "tc_bwd");
-        tc_bwd_kernel<<<num_sms(), CBK_THREADS, smem, st>>>(tmQ, tmK, tmKt, tmV, tmDO, tmDQ, tmDK, tmDV, ch, cb, tq, S * H);
+        if (!launch_after(tc_bwd_kernel, num_sms(), CBK_THREADS, smem, st, tmQ, tmK, tmKt, tmV, tmDO, tmDQ, tmDK, tmDV, ch, cb, tq, S * H)) return -1;
         ++launches;
     }
+    ClearList clear{};
+    clear.p[0] = reinterpret_cast<int*>(w + t.queue);
+    clear.n[0] = 64 + L.NTmax * H;
     const int n1 = phase1_backward(p, hy, L, ws, a, reinterpret_cast<float*>(w + t.dktil),
-                                   reinterpret_cast<float*>(w + t.dkread), false, st);
+                                   reinterpret_cast<float*>(w + t.dkread), false, clear, st);
     if (n1 < 0) return -1;
     launches += n1;
     stage_end(st);
