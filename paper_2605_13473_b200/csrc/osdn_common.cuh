@@ -178,8 +178,10 @@ inline P1Regions carve_p1(void* ws, const WsLayout& L)
 
 // Programmatic dependent launch: a kernel launched by launch_after may become resident while the kernel before it in the
 // stream still runs, and waits in pdl_wait, before its first access to anything that kernel or an earlier one writes,
-// until that kernel is complete (launch latency and prologue then run under its tail).  Every kernel of a call
-// does both, so that completeness carries over from kernel to kernel.
+// until that kernel is complete (launch latency and prologue then run under its tail).  Every kernel of a call waits, so
+// that completeness carries over from kernel to kernel.  pdl_release lets the next kernel's CTAs in while this one runs;
+// the kernels before tc_fwd and tc_bwd do without it: let in early, their CTAs fill the idle SMs first and the chains land
+// on neighbouring SMs, which share an instruction path (forward at 8 x 2048 tokens, 8 heads: 146 -> 153 us).
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 template <typename... P, typename... A>

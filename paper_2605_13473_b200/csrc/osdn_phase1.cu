@@ -1014,8 +1014,7 @@ __global__ void __launch_bounds__(Pipe<K>::THREADS, 1) phase1_seq_kernel(P1Fwd a
         init_bars(sh.bars, PipeShared<TI, K, VEC>::PN, P::CORE);
         sh.cmd_n = 0;
     }
-    pdl_release();
-    pdl_wait();
+    pdl_wait();   // no early release: see pdl_release
     float d_in = 1.0f, guess = 0.f;
     if (warp < P::CORE) {
         if (a.d0) d_in = a.d0[((size_t)s * H + h) * K + coord];

@@ -506,7 +506,6 @@ tc_chunk_fwd_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     __shared__ ClGroupShared gs;
     __shared__ uint32_t tmem_base;
     const int tid = threadIdx.x;
-    pdl_release();
     pdl_wait();
     if (a.tab.chunk_len(blockIdx.x) == 0) return;
     if (tid == 0) {
@@ -977,7 +976,6 @@ tc_chain_fwd_kernel(const __grid_constant__ CUtensorMap tmV, const __grid_consta
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    pdl_release();
     pdl_wait();
     chain_fwd_role(tmV, tmKt, a, blockIdx.x, align1024(smem_raw), tmem_base);
     tc_fence_before();
@@ -1100,7 +1098,6 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
     __syncthreads();
     tc_fence_after();
     const uint32_t tb = tmem_base;
-    pdl_release();
     pdl_wait();
     fwd_sched_resolve(sc, cl.tab, cl.H);
     const bool chain_cta = (int)blockIdx.x < sc.nchains;
