@@ -1,0 +1,94 @@
+"""The kernels' dispatch rules and block edges: sizes on both sides of every line, against the oracle.
+
+Tolerances are the suite's: 1e-4 of the largest value for fp32 arithmetic (parity.TOL for bf16 results)."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import parity
+from paper_2605_13473_b200 import binding, run_inputs_bwd
+from paper_2605_13473_b200.synth import OsdnHyper, draw
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+@pytest.mark.parametrize("K", [64, 128])
+@pytest.mark.parametrize("eta,keys,apf,clamp", [(0.3, "sparse", 2, 1), (0.003, "gauss", 2, 1), (0.05, "gauss", 1, 0), (0.3, "sparse", 3, 1)])
+@pytest.mark.parametrize("L", [1, 31, 32, 33, 300])
+def test_standalone_update_at_block_edges(L, eta, keys, apf, clamp, K):
+    """Blocks of 32 tokens: the smallest sequence, one short of, at and past a block, more blocks than the ring holds."""
+    hy = OsdnHyper(eta=eta, apf_mode=apf, clamp=clamp)
+    inp = draw(f"edge_{L}", 7000 + L, [L, L], 2, K, K, "fp32", dense_B=2, hyper=hy, key_kind=keys,
+               with_log_ret=apf >= 2, with_state=True)
+    b = binding.DeviceBundle(inp, DEV, need_bwd=False)
+    kt, d = torch.empty_like(b.k), torch.empty(2, 2, K, device=DEV)
+    binding.osdn_precond_update(b.params, b.k, b.beta, b.log_ret if apf >= 2 else b.gate, b.precond_in, kt, d)
+    ref = oracle.precond_update(hy, inp.seq_lens, inp.k, inp.beta, inp.gate, inp.log_ret, inp.precond_in)
+    assert parity.err(d.cpu().numpy(), ref["precond_out"]) <= 1e-4
+
+
+def _all_outputs(inp, label, **kw):
+    got = run_inputs_bwd(inp, **kw)
+    ref = parity.oracle_all(inp, True, got["projection_masks"])
+    parity.compare(got, ref, inp.io_dtype, parity.FWD_KEYS + parity.BWD_KEYS, label,
+                   tensor_core=inp.io_dtype == "bf16" and inp.K == 128)
+
+
+@pytest.mark.parametrize("shift", [3.0, 7.0])
+@pytest.mark.parametrize("lens", [[2300], [700, 64, 0, 33, 1, 1500]])
+def test_lists_of_processed_tokens(lens, shift):
+    """Retention near one without a gate: runs off the face, then tokens that leave it one at a time, so that the passes
+    work on dense runs, on lists with jumps and on short lists; more than one group of 2048 tokens, ragged packing."""
+    hy = OsdnHyper(eta=0.003, apf_mode=2, beta_aware=0)
+    inp = draw("lists", 7100 + int(shift), lens, 1, 64, 64, "fp32", dense_B=len(lens) == 1, hyper=hy, gate_kind="zero",
+               with_dout=True, with_log_ret=True, log_ret_shift=shift, with_state_cotangents=True)
+    _all_outputs(inp, f"lists_{len(lens)}_{shift}")
+
+
+@pytest.mark.parametrize("io,K", [("fp32", 64), ("fp32", 128), ("bf16", 64)])
+def test_chains_in_wide_slices(io, K):
+    """Enough chains for the wide slices of the CUDA-core state chains (the other cases have few and take the narrow ones)."""
+    hy = OsdnHyper(eta=0.003, apf_mode=1)
+    inp = draw("wide", 7200 + K, [70] * 50, 6, K, 64, io, dense_B=50, hyper=hy, with_dout=True, with_state=True,
+               with_state_cotangents=True)
+    _all_outputs(inp, f"wide_{io}_{K}")
+
+
+def test_backward_twice_on_the_same_residuals():
+    """The backward leaves its tile queue as it found it."""
+    hy = OsdnHyper(eta=0.003, apf_mode=1)
+    inp = draw("twice", 7300, [200, 200], 2, 128, 128, "bf16", dense_B=2, hyper=hy, with_dout=True)
+    b = binding.DeviceBundle(inp, DEV, need_bwd=True)
+    b.fwd(save=True)
+    seen = []
+    for _ in range(2):
+        for x in (b.dq, b.dk, b.dv):
+            x.fill_(float("nan"))
+        b.bwd(residuals_valid=True)
+        torch.cuda.synchronize()
+        assert b.device_status() == 0
+        seen.append([x.clone() for x in (b.dq, b.dk, b.dv)])
+    for x, y in zip(*seen):
+        assert not torch.isnan(x.float()).any() and torch.equal(x, y)
+
+
+@pytest.mark.parametrize("B,H,L", [(49, 3, 8), (37, 4, 9), (191, 1, 1), (192, 1, 1), (50, 3, 17)])
+@pytest.mark.parametrize("io,K,V,apf", [("bf16", 128, 128, 1), ("fp32", 64, 128, 2), ("fp32", 128, 64, 3)])
+def test_decode_on_both_sides_of_its_dispatch(B, H, L, io, K, V, apf):
+    """147 / 148 chains with several tokens, 191 / 192 with one; blocks of eight tokens: at, one past, two and one past."""
+    hy = OsdnHyper(eta=0.3, apf_mode=apf)
+    inp = draw(f"dec_{B}_{L}", 7400 + B + L, [L] * B, H, K, V, io, dense_B=B, hyper=hy, with_log_ret=apf >= 2, with_state=True)
+    p = binding.make_params(B=B, T=L, H=H, K=K, V=V, io_dtype=io, hyper=hy)
+    dt = torch.bfloat16 if io == "bf16" else torch.float32
+    q, k, v = (x.to(DEV, dt).contiguous() for x in (inp.q, inp.k, inp.v))
+    beta, gate = inp.beta.float().to(DEV), inp.gate.float().to(DEV)
+    lr = None if inp.log_ret is None else inp.log_ret.float().to(DEV)
+    S, d = inp.init_state.float().to(DEV).clone(), inp.precond_in.float().to(DEV).clone()
+    out = torch.empty(B * L, H, V, device=DEV, dtype=dt)
+    binding.osdn_decode_step(p, q, k, v, beta, gate, lr, S, d, out)
+    ref = oracle.fwd_inputs(inp)
+    assert parity.err(S.cpu().numpy(), ref["final_state"]) <= 1e-4
+    assert parity.err(d.cpu().numpy(), ref["precond_out"]) <= 1e-4
+    assert parity.err(out.float().cpu().numpy(), ref["out"]) <= parity.TOL[io]
