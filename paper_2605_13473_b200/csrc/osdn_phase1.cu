@@ -639,9 +639,9 @@ struct P1Rec {
     unsigned bits;               // forward: jumps; reverse: restarts
     uint32_t th[PB];
     float c[PB], rho[PB], off[PB];   // reverse: c holds u
-    alignas(16) float v0[128];   // y, or lambda, on entry (read and written four floats at a time)
+    float v0[128];               // y, or lambda, on entry
 };
-static_assert(sizeof(P1Rec) <= P1_REC_BYTES && P1_REC_BYTES % alignof(P1Rec) == 0, "record size");
+static_assert(sizeof(P1Rec) <= P1_REC_BYTES, "record size");
 constexpr int REC_END = 1 << 30;
 struct RecChain {   // a chain's records
     char* base;
