@@ -61,8 +61,6 @@ struct WsLayout {
     size_t p1sumk;      // [T,H]          f32   |k|^2
     size_t p1kmax;      // [T,H]          f32   largest k_r^2
     size_t p1rho;       // [T,H]          f32   retention of the preconditioner
-    size_t p1rec;       // records of solved blocks for the finishing CTAs, P1_REC_BYTES each (see P1Rec)
-    size_t p1cnt;       // [2,S,H]        i32   records published per chain, forward and reverse (zero between calls)
     size_t p1al;        // [T,H]          f32   <d_t, k_t^2> of processed tokens                (save only)
     size_t p1flags;     // [NT,H,2]       u32   per token: the step maps d_min*1 to d_min*1, mask all zero
     size_t p1skip;      // [NT,H,2]       u32   tokens the sequential pass skipped           (save only)
@@ -92,11 +90,6 @@ struct WsLayout {
     int dense_T;        // > 0 for a dense batch (see Table)
 };
 
-// Room for records: one per P1_REC_TOKENS tokens of a chain and P1_REC_MORE beside (a block that finds none left is
-// finished where it was solved).
-constexpr size_t P1_REC_BYTES = 1152;   // whole 128-byte lines: a reader of one record must not cache a part of the next
-constexpr int P1_REC_TOKENS = 16, P1_REC_MORE = 32;
-
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 inline WsLayout make_layout(const osdn_params& p, bool need_bwd)
@@ -117,8 +110,6 @@ inline WsLayout make_layout(const osdn_params& p, bool need_bwd)
     L.p1kmax = take(4 * Ttot * H);
     L.p1rho = take(4 * Ttot * H);
     L.p1flags = take(4 * NT * H * 2);
-    L.p1rec = take(P1_REC_BYTES * (Ttot / P1_REC_TOKENS + (size_t)P1_REC_MORE * S) * H);
-    L.p1cnt = take(4 * 2 * (size_t)S * H);
     if (need_bwd) {
         L.p1skip = take(4 * NT * H * 2);
         L.p1al = take(4 * Ttot * H);
@@ -168,8 +159,6 @@ inline Table carve_table(void* ws, const WsLayout& L)
 struct P1Regions {
     float *sumk, *kmax, *rho, *dtraj, *al;
     unsigned *flags, *skipw, *pmask;
-    char* rec;
-    int* cnt;
 };
 
 inline P1Regions carve_p1(void* ws, const WsLayout& L)
@@ -179,8 +168,6 @@ inline P1Regions carve_p1(void* ws, const WsLayout& L)
     r.sumk = reinterpret_cast<float*>(w + L.p1sumk);
     r.kmax = reinterpret_cast<float*>(w + L.p1kmax);
     r.rho = reinterpret_cast<float*>(w + L.p1rho);
-    r.rec = w + L.p1rec;
-    r.cnt = reinterpret_cast<int*>(w + L.p1cnt);
     r.al = reinterpret_cast<float*>(w + L.p1al);
     r.flags = reinterpret_cast<unsigned*>(w + L.p1flags);
     r.skipw = reinterpret_cast<unsigned*>(w + L.p1skip);
@@ -216,8 +203,8 @@ inline bool launch_after(void (*kernel)(P...), dim3 grid, dim3 block, size_t sme
 // Control regions that have to start at zero; cleared by the parallel preconditioner pass, the first kernel of a dense
 // call (a memset of its own costs the stream about two microseconds).
 struct ClearList {
-    int* p[4];
-    int n[4];   // ints
+    int* p[3];
+    int n[3];   // ints
 };
 
 template <typename T> __device__ __forceinline__ float ldf(const T* p);

@@ -119,7 +119,6 @@ struct P1Fwd {
     int save;
     Hyper hy;
     int* status;         // device status word (bounded waits of the rings report here)
-    int offload;         // the grid has a finishing CTA per chain behind the chains' own
     ClearList clear;
 };
 
@@ -127,7 +126,7 @@ __device__ __forceinline__ void clear_regions(const ClearList& c)
 {
     const int at = blockIdx.x * blockDim.x + threadIdx.x, step = gridDim.x * blockDim.x;
 #pragma unroll
-    for (int r = 0; r < 4; ++r)
+    for (int r = 0; r < 3; ++r)
         for (int i = at; i < c.n[r]; i += step) c.p[r][i] = 0;
 }
 
@@ -627,139 +626,10 @@ __device__ __forceinline__ void finish_block(const PipeBuf<TI, K, VEC>& B, int n
     else finish_block<TI, K, VEC, P1_CLIP>(B, n, hy, q, lane, out);
 }
 
-// ---------------------------------------------------------------------------------------------
-// Finishing CTAs.  The finishing warps issue more than the core does and slow it down by their share of the SM's issue
-// slots and shared-memory pipe (a block of 32 at a step size of 0.3: 2900 cycles alone, 4700 beside four finishing
-// warps).  When the chains leave half of the SMs idle, a second CTA per chain does that work: one warp of the chain's CTA
-// writes what the core leaves of a block (its tokens, their step scalars, the vector on entry) into a record in global
-// memory and counts it; the warps of the finishing CTA take the records in turn.  The chain never waits for them.
-// ---------------------------------------------------------------------------------------------
-struct P1Rec {
-    int n;
-    unsigned bits;               // forward: jumps; reverse: restarts
-    uint32_t th[PB];
-    float c[PB], rho[PB], off[PB];   // reverse: c holds u
-    float v0[128];               // y, or lambda, on entry
-};
-static_assert(sizeof(P1Rec) <= P1_REC_BYTES, "record size");
-constexpr int REC_END = 1 << 30;
-struct RecChain {   // a chain's records
-    char* base;
-    int* cnt;
-    int cap;
-    __device__ __forceinline__ P1Rec& at(int i) const { return *reinterpret_cast<P1Rec*>(base + (size_t)i * P1_REC_BYTES); }
-};
-__device__ __forceinline__ RecChain rec_chain(const P1Regions& r, const Table& tab, int s, int h, int H, int chain, int chains, bool reverse)
-{
-    const int len = tab.seq_len(s), cap = len / P1_REC_TOKENS + P1_REC_MORE;
-    const size_t first = (size_t)(tab.seq_tok0(s) / P1_REC_TOKENS + P1_REC_MORE * s) * H + (size_t)cap * h;
-    return {r.rec + first * P1_REC_BYTES, r.cnt + (reverse ? chains : 0) + chain, cap};
-}
-// The warp's stores to the record are out before the count says so.
-__device__ __forceinline__ void publish(int* cnt, int v, int lane)
-{
-    __threadfence();
-    __syncwarp();
-    if (lane == 0) asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(cnt), "r"(v) : "memory");
-}
-// Waits (bounded) until record i is there; false: there is none any more.
-__device__ __forceinline__ bool await_record(const int* cnt, int i, int* status, int lane)
-{
-    int v = 0;
-    const long long t0 = clock64();
-    while (true) {
-        asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(cnt) : "memory");
-        v = __shfl_sync(0xffffffffu, v, 0);
-        if ((v & ~REC_END) > i) return true;
-        if (v & REC_END) return false;
-        const bool late = clock64() - t0 > P1_WAIT_LIMIT;
-        if (__any_sync(0xffffffffu, late)) {
-            if (lane == 0 && status) atomicCAS(status, 0, P1_ERR_PIPE);
-            return false;
-        }
-        __nanosleep(200);
-    }
-}
-
-template <typename TI, typename TO, int K, bool VEC, P1Mode M>
-__device__ __forceinline__ void finish_record(const P1Fwd& a, const P1Rec& rec, const P1Coord& q, int lane)
-{
-    constexpr int R = K / 32, G = VEC ? 4 : 8;
-    const Hyper hy = a.hy;
-    const int n = rec.n;
-    const unsigned jump = rec.bits;
-    const uint32_t mine = rec.th[min(lane, n - 1)];
-    const float c_l = rec.c[lane], rho_l = rec.rho[lane], off_l = rec.off[lane];
-    float y[R];
-    load_row<R>(rec.v0, lane, y);
-    struct Rows {
-        float k[G][R], rv[VEC ? G : 1][R];
-    } even, odd;
-    auto load = [&](int j0, Rows& x) {
-#pragma unroll
-        for (int u = 0; u < G; ++u) {
-            const size_t th = __shfl_sync(0xffffffffu, mine, min(j0 + u, n - 1));
-            load_row<R>(static_cast<const TI*>(a.k) + th * K, lane, x.k[u]);
-            if constexpr (VEC) load_row<R>(a.retsrc + th * K, lane, x.rv[VEC ? u : 0]);
-        }
-    };
-    auto work = [&](int j0, const Rows& x) {
-#pragma unroll
-        for (int u = 0; u < G; ++u) {
-            const int j = j0 + u;
-            const size_t th = __shfl_sync(0xffffffffu, mine, j & (PB - 1));
-            const float c = __shfl_sync(0xffffffffu, c_l, j & (PB - 1)), rho1 = __shfl_sync(0xffffffffu, rho_l, j & (PB - 1));
-            const float off1 = __shfl_sync(0xffffffffu, off_l, j & (PB - 1));
-            if (j < n) {
-                const float keep = bit_of(jump, j) ? 0.f : 1.f;
-                float d[R], wk[R];
-                unsigned bits = 0;
-#pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    const float v = y[r] * keep, kk = x.k[u][r];
-                    const float rho = VEC ? expf(x.rv[VEC ? u : 0][r]) : rho1, off = VEC ? p1_off(rho, q) : off1;
-                    d[r] = p1_d(v, q);
-                    wk[r] = d[r] * kk;
-                    const float z = p1_raw(v, __fmul_rn(kk, kk), c, rho, off);
-                    y[r] = p1_project<M>(z, hy);
-                    bits |= y[r] == z ? (1u << r) : 0u;
-                }
-                store_row<R>(static_cast<TO*>(a.ktil) + th * K, lane, wk);
-                if (a.save) {
-                    store_row<R>(a.r.dtraj + th * K, lane, d);
-                    a.r.pmask[th * 32 + lane] = bits;
-                }
-            }
-        }
-    };
-    load(0, even);
-#pragma unroll 1
-    for (int j0 = 0; j0 < n; j0 += 2 * G) {
-        load(j0 + G, odd);
-        work(j0, even);
-        load(j0 + 2 * G, even);
-        if (j0 + G < n) work(j0 + G, odd);
-    }
-}
-template <typename TI, typename TO, int K, bool VEC>
-__device__ __forceinline__ void finish_records(const P1Fwd& a, const RecChain& rc, int warp, int lane)
-{
-    const P1Coord q = p1_coord(a.hy);
-    const P1Mode mode = p1_mode(a.hy);
-    for (int i = warp; await_record(rc.cnt, i, a.status, lane); i += Pipe<K>::WARPS) {
-        const P1Rec& rec = rc.at(i);
-        if (mode == P1_SAT) finish_record<TI, TO, K, VEC, P1_SAT>(a, rec, q, lane);
-        else if (mode == P1_FREE) finish_record<TI, TO, K, VEC, P1_FREE>(a, rec, q, lane);
-        else finish_record<TI, TO, K, VEC, P1_CLIP>(a, rec, q, lane);
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) *rc.cnt = 0;
-}
-
 // The list in sh through the ring, all roles.  y travels through sh.y; guess and rounds belong to the core warps.
 template <typename TI, typename TO, int K, bool VEC>
 __device__ __forceinline__ bool run_list(const P1Fwd& a, int h, PipeShared<TI, K, VEC>& sh, float& guess, uint32_t& rounds, uint32_t& uses,
-                                         const RecChain& rc, int& recs, int warp, int lane)
+                                         int warp, int lane)
 {
     constexpr int R = K / 32;
     using P = Pipe<K>;
@@ -849,37 +719,13 @@ __device__ __forceinline__ bool run_list(const P1Fwd& a, int h, PipeShared<TI, K
         cp_async_wait<0>();
     } else {
         TO* kt = static_cast<TO*>(a.ktil);
-        // with a finishing CTA: the first of these warps takes all blocks, as records
-        const bool record = a.offload != 0;
-        const int first = record ? (warp == P::FINISH0 ? 0 : nblk) : (int)((warp - P::FINISH0 - base) & (P::FINISH - 1));
-        for (int b = first; b < nblk; b += record ? 1 : P::FINISH) {
+        for (int b = (int)((warp - P::FINISH0 - base) & (P::FINISH - 1)); b < nblk; b += P::FINISH) {
             const int bi = (base + b) % PN;
             ok = p1_mbar_wait(&sh.bars.done[bi], ((base + b) / PN) & 1, a.status);
             if (!ok) break;
             const PipeBuf<TI, K, VEC>& B = sh.buf[bi];
             const int n = B.n;
             const uint32_t mine = th_of(b);
-            if (a.save && lane < n) a.r.al[mine] = fmaf(q.w, B.res[lane].y, q.lo * B.scal[lane].w);
-            if (record && recs < rc.cap) {
-                if (n > 0) {
-                    P1Rec& rec = rc.at(recs);
-                    if (lane == 0) {
-                        rec.n = n;
-                        rec.bits = B.jump;
-                    }
-                    rec.th[lane] = mine;
-                    rec.c[lane] = B.res[lane].x;
-                    rec.rho[lane] = B.rho[lane];
-                    rec.off[lane] = B.off[lane];
-                    float y[R];
-                    load_row<R>(B.y0, lane, y);
-                    store_row<R>(rec.v0, lane, y);
-                }
-                __syncwarp();
-                if (lane == 0) p1_mbar_arrive(&sh.bars.free_[bi]);
-                if (n > 0) publish(rc.cnt, ++recs, lane);
-                continue;
-            }
             finish_block<TI, K, VEC>(B, n, hy, q, lane, [&](int j, const float (&d)[R], const float (&kk)[R], unsigned bits) {
                 const size_t th = __shfl_sync(0xffffffffu, mine, j);
                 float wk[R];
@@ -891,6 +737,7 @@ __device__ __forceinline__ bool run_list(const P1Fwd& a, int h, PipeShared<TI, K
                     a.r.pmask[th * 32 + lane] = bits;
                 }
             });
+            if (a.save && lane < n) a.r.al[mine] = fmaf(q.w, B.res[lane].y, q.lo * B.scal[lane].w);
             __syncwarp();
             if (lane == 0) p1_mbar_arrive(&sh.bars.free_[bi]);
         }
@@ -1159,7 +1006,7 @@ __global__ void __launch_bounds__(Pipe<K>::THREADS, 1) phase1_seq_kernel(P1Fwd a
     extern __shared__ __align__(16) uint8_t p1_dyn[];
     PipeShared<TI, K, VEC>& sh = *reinterpret_cast<PipeShared<TI, K, VEC>*>(p1_dyn);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int chains = a.S * a.H, chain = blockIdx.x % chains;
+    const int chain = blockIdx.x;
     const int s = chain / a.H, h = chain % a.H, H = a.H;
     const P1Coord q = p1_coord(a.hy);
     const int coord = warp * 32 + lane;   // core warps
@@ -1168,12 +1015,6 @@ __global__ void __launch_bounds__(Pipe<K>::THREADS, 1) phase1_seq_kernel(P1Fwd a
         sh.cmd_n = 0;
     }
     pdl_wait();   // no early release: see pdl_release
-    const RecChain rc = rec_chain(a.r, a.tab, s, h, H, chain, chains, false);
-    if ((int)blockIdx.x >= chains) {
-        finish_records<TI, TO, K, VEC>(a, rc, warp, lane);
-        return;
-    }
-    int recs = 0;   // the recording warp's
     float d_in = 1.0f, guess = 0.f;
     if (warp < P::CORE) {
         if (a.d0) d_in = a.d0[((size_t)s * H + h) * K + coord];
@@ -1186,10 +1027,9 @@ __global__ void __launch_bounds__(Pipe<K>::THREADS, 1) phase1_seq_kernel(P1Fwd a
         if (warp == 0) plan.next();
         bar_sync<P::THREADS>(1);
         if (sh.cmd_n == 0) break;
-        run_list<TI, TO, K, VEC>(a, h, sh, guess, rounds, uses, rc, recs, warp, lane);
+        run_list<TI, TO, K, VEC>(a, h, sh, guess, rounds, uses, warp, lane);
         bar_sync<P::THREADS>(2);
     }
-    if (a.offload && warp == P::FINISH0) publish(rc.cnt, recs | REC_END, lane);
     if (a.d_final && warp < P::CORE) a.d_final[((size_t)s * H + h) * K + coord] = sh.cmd_dense ? p1_d(sh.y[coord], q) : d_in;
 }
 
@@ -1339,7 +1179,6 @@ struct P1Bwd {
     Hyper hy;
     int* status;
     ClearList clear;
-    int offload;            // as in P1Fwd
 };
 
 // skipped tokens: dk = dk_read + d_min dL/dktil (one warp per (chunk, head, 32-token half))
@@ -1520,75 +1359,8 @@ __device__ __forceinline__ void rev_scalar_grads(const P1Bwd& a, size_t th, cons
     if (a.hy.apf_mode == 2 && a.dlog_ret) a.dlog_ret[th] = rho * dr;
 }
 
-// A record (see P1Rec; c holds u) by one warp of a finishing CTA.
-template <typename T, int K, bool VEC> __device__ __forceinline__ void finish_rev_record(const P1Bwd& a, const P1Rec& rec, int lane)
-{
-    constexpr int R = K / 32, G = VEC ? 2 : 4;
-    const int n = rec.n;
-    const unsigned restart = rec.bits;
-    const uint32_t mine = rec.th[min(lane, n - 1)];
-    const float u_l = rec.c[lane];
-    float4 sc, gr;
-    rev_scalars(a.r.sumk[mine], a.r.kmax[mine], a.r.rho[mine], a.beta[mine], a.r.al[mine], a.hy, sc, gr);
-    if (bit_of(restart, lane)) sc.x = 0.f;
-    float lam[R];
-    load_row<R>(rec.v0, lane, lam);
-    struct Rows {
-        float k[G][R], dkt[G][R], dt[G][R], dkr[G][R], rv[VEC ? G : 1][R];
-        unsigned mask[G];
-    } even, odd;
-    auto load = [&](int j0, Rows& x) {
-#pragma unroll
-        for (int g = 0; g < G; ++g) {
-            const int j = min(j0 + g, n - 1);
-            const size_t th = __shfl_sync(0xffffffffu, mine, j);
-            load_row<R>(static_cast<const T*>(a.k) + th * K, lane, x.k[g]);
-            load_row<R>(a.dktil + th * K, lane, x.dkt[g]);
-            load_row<R>(a.r.dtraj + th * K, lane, x.dt[g]);
-            load_row<R>(a.dkread + th * K, lane, x.dkr[g]);
-            if constexpr (VEC) load_row<R>(a.log_ret + th * K, lane, x.rv[VEC ? g : 0]);
-            x.mask[g] = bit_of(restart, j) ? 0u : a.r.pmask[th * 32 + lane];
-        }
-    };
-    auto work = [&](int j0, const Rows& x) {
-        float drv[G];
-#pragma unroll
-        for (int g = 0; g < G; ++g) {
-            const int j = j0 + g, jj = j & (PB - 1);
-            const float a2 = __shfl_sync(0xffffffffu, sc.x, jj), rho = __shfl_sync(0xffffffffu, sc.y, jj);
-            const float4 gg = make_float4(__shfl_sync(0xffffffffu, gr.x, jj), 0.f, __shfl_sync(0xffffffffu, gr.z, jj), __shfl_sync(0xffffffffu, u_l, jj));
-            const size_t th = __shfl_sync(0xffffffffu, mine, jj);
-            const float au = -a2 * gg.w;
-            float lm[R], rv[R];
-            drv[g] = 0.f;
-#pragma unroll
-            for (int r = 0; r < R; ++r) {
-                rv[r] = VEC ? expf(x.rv[VEC ? g : 0][r]) : rho;
-                lm[r] = bit_of(x.mask[g], r) ? lam[r] : 0.f;
-                drv[g] = fmaf(lm[r], x.dt[g][r], drv[g]);
-                lam[r] = rev_step(lm[r], __fmul_rn(x.k[g][r], x.k[g][r]), __fmul_rn(x.k[g][r], x.dkt[g][r]), au, rv[r]);
-            }
-            if (j < n && !bit_of(restart, j)) rev_outputs<T, K, VEC>(a, th, lane, gg, a2, x.k[g], x.dt[g], x.dkt[g], x.dkr[g], lm, rv);
-        }
-        const float dr = transpose_sum(drv, lane);   // lane j: token j0 + j
-        const int j = (j0 + lane) & (PB - 1);
-        const size_t th = __shfl_sync(0xffffffffu, mine, j);
-        const float g1 = __shfl_sync(0xffffffffu, gr.y, j), u = __shfl_sync(0xffffffffu, u_l, j), rho = __shfl_sync(0xffffffffu, sc.y, j);
-        if (lane < G && j < n && !bit_of(restart, j)) rev_scalar_grads(a, th, make_float4(0.f, g1, 0.f, u), rho, dr);
-    };
-    load(0, even);
-#pragma unroll 1
-    for (int j0 = 0; j0 < n; j0 += 2 * G) {
-        load(j0 + G, odd);
-        work(j0, even);
-        load(j0 + 2 * G, even);
-        if (j0 + G < n) work(j0 + G, odd);
-    }
-}
-
 template <typename T, int K, bool VEC>
-__device__ __forceinline__ bool run_rev_list(const P1Bwd& a, int h, RevShared<T, K, VEC>& sh, uint32_t& rounds, uint32_t& uses,
-                                             const RecChain& rc, int& recs, int warp, int lane)
+__device__ __forceinline__ bool run_rev_list(const P1Bwd& a, int h, RevShared<T, K, VEC>& sh, uint32_t& rounds, uint32_t& uses, int warp, int lane)
 {
     constexpr int R = K / 32;
     using P = Pipe<K>;
@@ -1632,7 +1404,7 @@ __device__ __forceinline__ bool run_rev_list(const P1Bwd& a, int h, RevShared<T,
                 cp_async4(&B.raw[2][lane], a.r.rho + th);
                 cp_async4(&B.raw[3][lane], a.beta + th);
                 cp_async4(&B.raw[4][lane], a.r.al + th);
-                if (!a.offload) for (int o = 0; o < K * 4; o += 128) {   // what the finishing warps will read
+                for (int o = 0; o < K * 4; o += 128) {   // what the finishing warps will read
                     prefetch_l2(reinterpret_cast<const char*>(a.r.dtraj + (size_t)th * K) + o);
                     prefetch_l2(reinterpret_cast<const char*>(a.dkread + (size_t)th * K) + o);
                 }
@@ -1669,31 +1441,11 @@ __device__ __forceinline__ bool run_rev_list(const P1Bwd& a, int h, RevShared<T,
         }
         cp_async_wait<0>();
     } else {
-        const bool record = a.offload != 0;
-        const int first = record ? (warp == P::FINISH0 ? 0 : nblk) : (int)((warp - P::FINISH0 - base) & (P::FINISH - 1));
-        for (int b = first; b < nblk; b += record ? 1 : P::FINISH) {
+        for (int b = (int)((warp - P::FINISH0 - base) & (P::FINISH - 1)); b < nblk; b += P::FINISH) {
             const int bi = (base + b) % QN;
             const RevBuf<T, K, VEC>& B = sh.buf[bi];
             const int n = len_of(b);
             const uint32_t mine = th_of(b);
-            if (record && recs < rc.cap) {
-                ok = p1_mbar_wait(&sh.bars.done[bi], ((base + b) / QN) & 1, a.status);
-                if (!ok) break;
-                P1Rec& rec = rc.at(recs);
-                if (lane == 0) {
-                    rec.n = n;
-                    rec.bits = B.restart;
-                }
-                rec.th[lane] = mine;
-                rec.c[lane] = B.grad[lane].w;
-                float v[R];
-                load_row<R>(B.lam0, lane, v);
-                store_row<R>(rec.v0, lane, v);
-                __syncwarp();
-                if (lane == 0) p1_mbar_arrive(&sh.bars.free_[bi]);
-                publish(rc.cnt, ++recs, lane);
-                continue;
-            }
             struct Ahead {
                 float dt[4][R], dkr[4][R];
             } even, odd;
@@ -1889,7 +1641,7 @@ __global__ void __launch_bounds__(Pipe<K>::THREADS, 1) phase1_bwd_seq_kernel(P1B
     extern __shared__ __align__(16) uint8_t p1_dyn[];
     RevShared<T, K, VEC>& sh = *reinterpret_cast<RevShared<T, K, VEC>*>(p1_dyn);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int chains = a.S * a.H, chain = blockIdx.x % chains;
+    const int chain = blockIdx.x;
     const int s = chain / a.H, h = chain % a.H, H = a.H;
     const int coord = warp * 32 + lane;   // core warps
     const size_t mine = ((size_t)s * H + h) * K + coord;
@@ -1897,14 +1649,6 @@ __global__ void __launch_bounds__(Pipe<K>::THREADS, 1) phase1_bwd_seq_kernel(P1B
     pdl_release();
     pdl_wait();
     clear_regions(a.clear);
-    const RecChain rc = rec_chain(a.r, a.tab, s, h, H, chain, chains, true);
-    if ((int)blockIdx.x >= chains) {
-        for (int i = warp; await_record(rc.cnt, i, a.status, lane); i += P::WARPS) finish_rev_record<T, K, VEC>(a, rc.at(i), lane);
-        __syncthreads();
-        if (threadIdx.x == 0) *rc.cnt = 0;
-        return;
-    }
-    int recs = 0;
     if (warp < P::CORE) sh.lam[coord] = a.dprecond_out ? a.dprecond_out[mine] : 0.f;
     uint32_t rounds = 0, uses = 0;
     __syncthreads();
@@ -1913,10 +1657,9 @@ __global__ void __launch_bounds__(Pipe<K>::THREADS, 1) phase1_bwd_seq_kernel(P1B
         if (warp == 0) plan.next();
         bar_sync<P::THREADS>(1);
         if (sh.cmd_n == 0) break;
-        if (!run_rev_list<T, K, VEC>(a, h, sh, rounds, uses, rc, recs, warp, lane)) plan.g = -1;
+        if (!run_rev_list<T, K, VEC>(a, h, sh, rounds, uses, warp, lane)) plan.g = -1;
         bar_sync<P::THREADS>(2);
     }
-    if (a.offload && warp == P::FINISH0) publish(rc.cnt, recs | REC_END, lane);
     if (a.dprecond_in && warp < P::CORE) {
         float lam = sh.lam[coord];
         if (!sh.live) {   // the first token was skipped: lambda restarts there
@@ -1926,9 +1669,6 @@ __global__ void __launch_bounds__(Pipe<K>::THREADS, 1) phase1_bwd_seq_kernel(P1B
         a.dprecond_in[mine] = lam;
     }
 }
-
-// A finishing CTA per chain where the chains leave that many SMs idle (one of these CTAs takes an SM).
-bool finishing_ctas(int chains) { return 2 * chains <= 148; }
 
 template <typename TI, typename TO, int K>
 int fwd_launch(const P1Fwd& a, cudaStream_t st)
@@ -1942,7 +1682,7 @@ int fwd_launch(const P1Fwd& a, cudaStream_t st)
     const unsigned chains = (unsigned)(a.S * a.H);
     auto launch_seq = [&](auto kernel, size_t smem) {
         if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return false;
-        return launch_after(kernel, chains * (a.offload ? 2 : 1), Pipe<K>::THREADS, smem, st, a);
+        return launch_after(kernel, chains, Pipe<K>::THREADS, smem, st, a);
     };
     const bool okl = a.hy.apf_mode == 3 ? launch_seq(phase1_seq_kernel<TI, TO, K, true>, sizeof(PipeShared<TI, K, true>))
                                         : launch_seq(phase1_seq_kernel<TI, TO, K, false>, sizeof(PipeShared<TI, K, false>));
@@ -1964,7 +1704,7 @@ int bwd_launch(const P1Bwd& a, bool bulk, cudaStream_t st)
     const unsigned chains = (unsigned)(a.S * a.H);
     auto launch_seq = [&](auto kernel, size_t smem) {
         if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return false;
-        return launch_after(kernel, chains * (a.offload ? 2 : 1), Pipe<K>::THREADS, smem, st, a);
+        return launch_after(kernel, chains, Pipe<K>::THREADS, smem, st, a);
     };
     if (!(a.hy.apf_mode == 3 ? launch_seq(phase1_bwd_seq_kernel<T, K, true>, sizeof(RevShared<T, K, true>))
                              : launch_seq(phase1_bwd_seq_kernel<T, K, false>, sizeof(RevShared<T, K, false>))))
@@ -1988,9 +1728,6 @@ int phase1_forward(const osdn_params& p, const Hyper& hy, const WsLayout& L, voi
         f.clear.p[2] = f.status;
         f.clear.n[2] = 1;
     }
-    f.offload = finishing_ctas(L.S * p.H);
-    f.clear.p[3] = f.r.cnt;
-    f.clear.n[3] = 2 * L.S * p.H;
     if (p.io_dtype == OSDN_FP32) {
         if (ktil_bf16) return -1;
         return p.K == 64 ? fwd_launch<float, float, 64>(f, st) : fwd_launch<float, float, 128>(f, st);
@@ -2011,7 +1748,6 @@ int phase1_backward(const osdn_params& p, const Hyper& hy, const WsLayout& L, vo
     b.r = carve_p1(ws, L); b.hy = hy; b.log_ret = a.log_ret;
     b.status = reinterpret_cast<int*>(static_cast<char*>(ws) + L.status);
     b.clear = clear;
-    b.offload = finishing_ctas(L.S * p.H);
     // retention gradients are written for processed tokens only; a skipped token (projection mask all
     // zero) has none
     if (p.apf_mode >= 2 && a.dlog_ret) {
