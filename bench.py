@@ -94,10 +94,6 @@ def method_bytes(name, inp, with_bwd):
         "tc_fwd": 2 * K * es + 8 + V * es + V * es + (state if with_bwd else 0),   # both passes in one launch
         # q, k, v, dout, beta, gate, the saved state in; dq, dk, dv, dbeta, dgate out
         "tc_bwd": (2 * K + 2 * V) * es + 8 + state + (2 * K + V) * es + 8,
-        # channel-gate extension: q, k, v, beta, K gates in, out; the backward reads them again with dout and
-        # writes dq, dk, dv, dbeta and K gate gradients
-        "kda_fwd": (2 * K + 2 * V) * es + 4 + 4 * K,
-        "kda_bwd": (2 * K + 2 * V) * es + 4 + 4 * K + (2 * K + V) * es + 4 + 4 * K,
     }
     return None if name not in per else per[name] * tokh
 
@@ -114,16 +110,14 @@ def kernel_model(name, inp, NT):
     m = {}
     # CUDA-core (fp32 workspace) family
     m["phase1_fwd"] = (tokh * (K * es + 8 + K * 4) + tiles * K * 4, tokh * 9.0 * K, "hbm")
-    m["simt_chunk_local_fwd"] = (tokh * (2 * K * es + K * 4 + V * es + 8) + tiles * 4 * (2 * C * C + C * K + C * V),
-                                 tiles * (2 * f(C, C, K) + f(C, K, C) + f(C, V, C)), "alu")
-    m["simt_chain_fwd"] = (tokh * (K * es + K * 4 + V * es + 8) + tiles * 4 * (C * K + 2 * C * V + C * C + V * K),
-                           tiles * (2 * f(C, V, K) + f(C, V, C) + f(V, K, C)), "alu")
-    m["simt_chain_bwd"] = (tokh * (K * es + K * 4 + V * es + 8) + tiles * 4 * (C * K + C * V + C * C + V * K),
-                           tiles * (f(C, V, C) + f(C, V, K) + 2 * f(V, K, C)), "alu")
-    m["simt_chunk_local_bwd"] = (tokh * (3 * K * es + K * 4 + 3 * V * es + 2 * K * 4 + 16)
-                                 + tiles * 4 * (2 * C * C + 2 * C * V + 2 * V * K + 10 * C * K),
-                                 tiles * (f(C, C, V) + 5 * f(C, K, V) + f(C, C, K) * 2 + f(C, C, V)
-                                          + f(C, K, C) * 5 + f(C, V, C) + 2 * f(C, C, C)), "alu")
+    m["chunk_local_fwd"] = (tokh * (2 * K * es + K * 4 + V * es + 8) + tiles * 4 * (3 * C * C + 3 * C * K + C * V + K),
+                            tiles * (2 * f(C, C, K) + f(C, K, C) + f(C, V, C)), "alu")
+    m["chain_fwd"] = (tiles * 4 * (2 * C * K + 2 * C * V + V * K), tiles * (f(C, V, K) + f(V, K, C)), "alu")
+    m["chunk_output"] = (tokh * V * es + tiles * 4 * (C * K + C * C + C * V + V * K), tiles * (f(C, V, K) + f(C, V, C)), "alu")
+    m["chunk_pre_bwd"] = (tokh * V * es + tiles * 4 * (C * C + C * K + C * V + V * K), tiles * (f(C, V, C) + f(V, K, C)), "alu")
+    m["chain_bwd"] = (tiles * 4 * (2 * C * K + 2 * C * V + 2 * V * K), tiles * (f(C, V, K) + f(V, K, C)), "alu")
+    m["chunk_local_bwd"] = (tokh * (3 * K * es + K * 4 + 3 * V * es + 2 * K * 4 + 16) + tiles * 4 * (2 * C * C + 2 * C * V + 2 * V * K),
+                            tiles * (f(C, C, V) * 2 + 3 * f(C, K, V) + f(C, C, K) + 4 * f(C, K, C) + f(C, V, C) + 2 * f(C, C, C)), "alu")
     m["build_table"] = (NT * 12, 0.0, "hbm")
     # phase 1 (both families)
     m["phase1_spec"] = (tokh * (2 * K * es + 16), tokh * 12.0 * K, "hbm")
@@ -144,11 +138,6 @@ def kernel_model(name, inp, NT):
                    tiles * (f(128, 64, C) + f(128, 64, K) + 2 * f(128, 128, C))
                    + tiles * (2 * f(64, 64, K) + 3 * f(128, 64, K) + 2 * f(64, 64, K) + 2 * f(128, 64, C)
                               + 2 * f(64, 64, C) + 4 * f(128, 64, C)), "hbm")
-    # channel-gate extension, token-recurrent on CUDA cores: per token and state row K decays, K + K + K fused
-    # multiply-adds forward (read, write, output); the backward replays the forward's two and takes about
-    # seven more per element for the adjoint
-    m["kda_fwd"] = (tokh * ((2 * K + 2 * V) * es + 4 + 8 * K) + tiles * 4 * V * K, tokh * V * K * 8.0, "alu")
-    m["kda_bwd"] = (tokh * ((4 * K + 3 * V) * es + 8 + 24 * K) + tiles * 4 * V * K, tokh * V * K * 20.0, "alu")
     return m.get(name)
 
 

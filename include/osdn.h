@@ -59,9 +59,9 @@ typedef enum osdn_status {
 } osdn_status;
 
 /* Values found in the device status word (first 4 bytes of a workspace) after a call whose kernels
- * met an error on the device.  101..113, 121, 122, 131: a bounded wait inside a kernel ran out (an
+ * met an error on the device.  101..113, 121, 122, 131, 141: a bounded wait inside a kernel ran out (an
  * mbarrier of the tensor-core kernels, the backward's tile queue, a ready flag of the merged forward
- * launch, a ring barrier of the pipelined preconditioner pass); the kernel then skipped the dependent
+ * launch, a ring barrier of the sequential preconditioner passes, a stage copy of the fp32 state chains); the kernel then skipped the dependent
  * work and returned, and the outputs of that call are undefined. */
 enum {
     OSDN_DEVICE_OK = 0,
@@ -203,11 +203,9 @@ int osdn_decode_step(const osdn_params* p, const void* q, const void* k, const v
  *            the flags, the alignment rules, ownership and the error codes are those of osdn_fwd / osdn_bwd.
  *   dgate_k  [T,H,K] fp32, written in full.
  *   workspace: osdn_kda_workspace_bytes(p, need_bwd) bytes (0 is returned for rejected parameters); for
- *            the backward it includes, beside the regions of osdn_workspace_bytes, one row history of 16
- *            tokens and four row checkpoints per state row (S * H * V * 20 * K floats) and an fp32
- *            accumulator for dq.
- * This path runs on CUDA cores in fp32 for both io_dtypes (one warp per state row, sequential over the
- * tokens of a sequence): it is the extension's reference implementation on the device, not a tuned one.
+ *            the backward it includes, beside the regions of osdn_workspace_bytes, the in-chunk prefix of the
+ *            channel gates (fp32, [T,H,K] rounded up to whole chunks).
+ * This path computes in fp32 on CUDA cores for both io_dtypes, chunk by chunk.
  */
 size_t osdn_kda_workspace_bytes(const osdn_params* p, int need_bwd);
 int osdn_kda_fwd(const osdn_params* p, const void* q, const void* k, const void* v, const float* beta,
