@@ -313,6 +313,18 @@ constexpr int SCAN_CHUNKS = 128;                    // chunks whose words warp 0
 
 // A block's way round the ring (fetch, core, finish) takes about six times what the core needs for it, hence that many
 // helpers and a deep ring: with four buffers and two finishing warps the core waited for half of the time.
+// The forward's core warps own two coordinates a lane and have a scheduler each, 0 and 1; the helpers sit on schedulers
+// 2 and 3 (warp numbers modulo four), the warps in between leave at once.  Beside helpers on its own scheduler a core of
+// four warps took 4700 cycles for a block instead of 2900.
+template <int K> struct FwdPipe {
+    static constexpr int CORE = K / 64, FETCH0 = 2, FETCH = 2, FINISH0 = 4, FINISH = 4, THREADS = 384, ACTIVE = (CORE + FETCH + FINISH) * 32;
+    // the role number of a hardware warp: core 0 .., fetch 2, 3, finish 4 .. 7; -1: idle
+    __device__ static __forceinline__ int role(int warp)
+    {
+        const int sched = warp & 3, row = warp >> 2;
+        return sched < 2 ? (row == 0 && warp < CORE ? warp : -1) : row * 2 + sched;
+    }
+};
 template <int K> struct Pipe {
     static constexpr int CORE = K / 32, FETCH0 = CORE, FETCH = 2, FINISH0 = CORE + FETCH, FINISH = 4, WARPS = FINISH0 + FINISH, THREADS = WARPS * 32;
 };
@@ -384,7 +396,7 @@ template <typename TI, int K, bool VEC> struct PipeBuf {
     alignas(16) float rv[VEC ? PB : 1][VEC ? K : 1];   // vector retention: l_t, then (core) exp(l_t)
 };
 template <typename TI, int K, bool VEC> struct PipeShared {
-    static constexpr int CW = K / 32, PN = ring_depth(sizeof(PipeBuf<TI, K, VEC>));
+    static constexpr int CW = K / 64, PN = ring_depth(sizeof(PipeBuf<TI, K, VEC>));
     PipeBuf<TI, K, VEC> buf[PN];
     float y[K];                             // between two lists
     float c[CW][PB];                        // a core warp's c' of the round
@@ -450,34 +462,52 @@ template <int N> __device__ __forceinline__ float transpose_sum(float (&x)[N], i
     return v;
 }
 
-// One block by the core warps: y of this lane's coordinate goes through it (slots beyond its n tokens leave y alone).
+__device__ __forceinline__ float2 load2(const float* p) { return *reinterpret_cast<const float2*>(p); }
+__device__ __forceinline__ float2 load2(const __nv_bfloat16* p) { return __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(p)); }
+
+// One block by the core warps: y of this lane's coordinates goes through it (slots beyond its n tokens leave y alone).
 // r: <y, k^2> / sum k^2 of the latest token, the start of the next guess; rounds: all rounds so far.  Returns the tokens
 // that stand: n, or those before the first jump that d enters off the face (y is then its value there).
 template <typename TI, int K, bool VEC, P1Mode M>
-__device__ __forceinline__ int core_block(PipeShared<TI, K, VEC>& sh, PipeBuf<TI, K, VEC>& B, int n, float& y, float& r, uint32_t& rounds,
+__device__ __forceinline__ int core_block(PipeShared<TI, K, VEC>& sh, PipeBuf<TI, K, VEC>& B, int n, float2& y, float& r, uint32_t& rounds,
                                           const Hyper& hy, const P1Coord& q, int warp, int lane)
 {
-    constexpr int CW = Pipe<K>::CORE;
-    const int i = warp * 32 + lane;
-    float kap[PB];
+    constexpr int CW = FwdPipe<K>::CORE;
+    const int i = warp * 64 + lane * 2;   // this lane's coordinates: i, i + 1
+    float ka[PB], kb[PB];
 #pragma unroll
     for (int j = 0; j < PB; ++j) {
-        const float k = ldf(&B.k[j][i]);
-        kap[j] = __fmul_rn(k, k);
+        const float2 k = load2(&B.k[j][i]);
+        ka[j] = __fmul_rn(k.x, k.x);
+        kb[j] = __fmul_rn(k.y, k.y);
     }
+    auto retention = [&](int j) -> float2& { return *reinterpret_cast<float2*>(&B.rv[VEC ? j : 0][VEC ? i : 0]); };
     if constexpr (VEC) {
 #pragma unroll 4
         for (int j = 0; j < PB; ++j) {
-            float& v = B.rv[VEC ? j : 0][VEC ? i : 0];
-            v = j < n ? expf(v) : 1.0f;
+            float2& v = retention(j);
+            v = j < n ? make_float2(expf(v.x), expf(v.y)) : make_float2(1.f, 1.f);
         }
     }
-    B.y0[i] = y;
+    *reinterpret_cast<float2*>(B.y0 + i) = y;
     const unsigned jump = B.jump;
     const float4 sc = B.scal[lane];   // lane j: token j
     const bool jumped = bit_of(jump, lane);
     const float tol = M == P1_FREE ? 0.f : 1.4901161e-8f * fmaxf(hy.d_min, 0.f) * q.iw;
-    float c = jumped ? sc.x : fmaf(-sc.y, sc.w * r, sc.x), sum = 0.f, z = y;
+    float c = jumped ? sc.x : fmaf(-sc.y, sc.w * r, sc.x), sum = 0.f;
+    float2 z = y;
+    // a step of both coordinates; keep: 0 behind a jump (then the scalar retention is 0 already)
+    auto step = [&](float2 v, float kx, float ky, float cj, float rho, float off, int j) {
+        float rx = rho, ry = rho, ox = off, oy = off;
+        if constexpr (VEC) {   // (rho: 0 behind a jump, else 1)
+            const float2 x = retention(j);
+            ox = p1_off(x.x, q);
+            oy = p1_off(x.y, q);
+            rx *= x.x;
+            ry *= x.y;
+        }
+        return make_float2(p1_project<M>(p1_raw(v.x, kx, cj, rx, ox), hy), p1_project<M>(p1_raw(v.y, ky, cj, ry, oy), hy));
+    };
     for (int round = 0; round <= PB; ++round) {   // (round PB + 1 could change nothing)
         const uint32_t par = rounds++ & 1;
         sh.c[warp][lane] = c;
@@ -491,23 +521,19 @@ __device__ __forceinline__ int core_block(PipeShared<TI, K, VEC>& sh, PipeBuf<TI
             const float cv[4] = {c4.x, c4.y, c4.z, c4.w}, rv[4] = {r4.x, r4.y, r4.z, r4.w}, ov[4] = {o4.x, o4.y, o4.z, o4.w};
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
-                float rho = rv[u], off = ov[u];
-                if constexpr (VEC) {   // (rv[u]: 0 behind a jump, else 1)
-                    rho = B.rv[VEC ? j + u : 0][VEC ? i : 0];
-                    off = p1_off(rho, q);
-                    rho *= rv[u];
-                }
-                p[j + u] = z * kap[j + u];
-                z = p1_project<M>(p1_raw(z, kap[j + u], cv[u], rho, off), hy);
+                p[j + u] = fmaf(z.x, ka[j + u], z.y * kb[j + u]);
+                z = step(z, ka[j + u], kb[j + u], cv[u], rv[u], ov[u], j + u);
             }
         }
-        const float mine = transpose_sum(p, lane);
-        float(*part)[PB] = sh.part[par];
-        part[warp][lane] = mine;
-        bar_sync<CW * 32>(3);
-        sum = part[0][lane];
+        sum = transpose_sum(p, lane);
+        if constexpr (CW > 1) {
+            float(*part)[PB] = sh.part[par];
+            part[warp][lane] = sum;
+            bar_sync<CW * 32>(3);
+            sum = part[0][lane];
 #pragma unroll
-        for (int x = 1; x < CW; ++x) sum += part[x][lane];
+            for (int x = 1; x < CW; ++x) sum += part[x][lane];
+        }
         if (jumped) sum = 0.f;
         const float cn = fmaf(-sc.y, sum, sc.x);
         const float dc = fabsf(cn - c);
@@ -518,28 +544,24 @@ __device__ __forceinline__ int core_block(PipeShared<TI, K, VEC>& sh, PipeBuf<TI
     int stand = n;
     if (jump) {   // was d on the face at the jumps?
         auto to = [&](int end, unsigned& off_face) {
-            float v = y;
+            float2 v = y;
 #pragma unroll 4
             for (int j = 0; j < end; ++j) {
-                if (bit_of(jump, j) && v != 0.f) off_face |= 1u << j;
-                float rho = B.rho[j], off = B.off[j];
-                if constexpr (VEC) {
-                    const float x = B.rv[VEC ? j : 0][VEC ? i : 0];
-                    off = p1_off(x, q);
-                    rho *= x;
-                }
-                const float k = ldf(&B.k[j][i]);
-                v = p1_project<M>(p1_raw(v, __fmul_rn(k, k), sh.c[warp][j], rho, off), hy);
+                if (bit_of(jump, j) && (v.x != 0.f || v.y != 0.f)) off_face |= 1u << j;
+                const float2 k = load2(&B.k[j][i]);
+                v = step(v, __fmul_rn(k.x, k.x), __fmul_rn(k.y, k.y), sh.c[warp][j], B.rho[j], B.off[j], j);
             }
             return v;
         };
         unsigned bad = 0;
         to(n, bad);
         bad = __reduce_or_sync(0xffffffffu, bad);
-        if (lane == 0) sh.bad[warp] = bad;
-        bar_sync<CW * 32>(3);
+        if constexpr (CW > 1) {
+            if (lane == 0) sh.bad[warp] = bad;
+            bar_sync<CW * 32>(3);
 #pragma unroll
-        for (int x = 0; x < CW; ++x) bad |= sh.bad[x];
+            for (int x = 0; x < CW; ++x) bad |= sh.bad[x];
+        }
         if (bad) {
             stand = __ffs((int)bad) - 1;
             unsigned none = 0;
@@ -555,7 +577,7 @@ __device__ __forceinline__ int core_block(PipeShared<TI, K, VEC>& sh, PipeBuf<TI
     return stand;
 }
 template <typename TI, int K, bool VEC>
-__device__ __forceinline__ int core_block(PipeShared<TI, K, VEC>& sh, PipeBuf<TI, K, VEC>& B, int n, float& y, float& r, uint32_t& rounds,
+__device__ __forceinline__ int core_block(PipeShared<TI, K, VEC>& sh, PipeBuf<TI, K, VEC>& B, int n, float2& y, float& r, uint32_t& rounds,
                                           const Hyper& hy, const P1Coord& q, int warp, int lane)
 {
     const P1Mode mode = p1_mode(hy);
@@ -632,7 +654,7 @@ __device__ __forceinline__ bool run_list(const P1Fwd& a, int h, PipeShared<TI, K
                                          int warp, int lane)
 {
     constexpr int R = K / 32;
-    using P = Pipe<K>;
+    using P = FwdPipe<K>;
     constexpr int PN = PipeShared<TI, K, VEC>::PN;
     const int H = a.H;
     const Hyper hy = a.hy;
@@ -647,7 +669,7 @@ __device__ __forceinline__ bool run_list(const P1Fwd& a, int h, PipeShared<TI, K
     auto len_of = [&](int b) { return min(PB, total - b * PB); };
     auto th_of = [&](int b) { return lane < len_of(b) ? (uint32_t)(tok_of(b * PB + lane) * H + h) : NO_ROW; };   // lane j: token j
     if (warp < P::CORE) {
-        float y = sh.y[warp * 32 + lane];
+        float2 y = load2(sh.y + warp * 64 + lane * 2);
         int stop = total;
         bool dead = false;   // d left the list: what follows in it is dropped
         for (int b = 0; b < nblk; ++b) {
@@ -667,7 +689,7 @@ __device__ __forceinline__ bool run_list(const P1Fwd& a, int h, PipeShared<TI, K
             __syncwarp();
             if (lane == 0) p1_mbar_arrive(&sh.bars.done[bi]);
         }
-        sh.y[warp * 32 + lane] = y;
+        *reinterpret_cast<float2*>(sh.y + warp * 64 + lane * 2) = y;
         if (warp == 0 && lane == 0) sh.stop = ok ? stop : 0;
     } else if (warp < P::FINISH0) {
         // the warps take the blocks in turn
@@ -1000,52 +1022,55 @@ template <typename TI, typename TO, int K, bool VEC> struct ListPlan {
 
 // One chain per CTA.
 template <typename TI, typename TO, int K, bool VEC>
-__global__ void __launch_bounds__(Pipe<K>::THREADS, 1) phase1_seq_kernel(P1Fwd a)
+__global__ void __launch_bounds__(FwdPipe<K>::THREADS, 1) phase1_seq_kernel(P1Fwd a)
 {
-    using P = Pipe<K>;
+    using P = FwdPipe<K>;
     extern __shared__ __align__(16) uint8_t p1_dyn[];
     PipeShared<TI, K, VEC>& sh = *reinterpret_cast<PipeShared<TI, K, VEC>*>(p1_dyn);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31, warp = P::role(threadIdx.x >> 5);
     const int chain = blockIdx.x;
     const int s = chain / a.H, h = chain % a.H, H = a.H;
     const P1Coord q = p1_coord(a.hy);
-    const int coord = warp * 32 + lane;   // core warps
+    const int coord = threadIdx.x;   // (the first K threads)
     if (threadIdx.x == 0) {
         init_bars(sh.bars, PipeShared<TI, K, VEC>::PN, P::CORE);
         sh.cmd_n = 0;
     }
     pdl_wait();   // no early release: see pdl_release
     float d_in = 1.0f, guess = 0.f;
-    if (warp < P::CORE) {
+    if (coord < K) {
         if (a.d0) d_in = a.d0[((size_t)s * H + h) * K + coord];
         sh.y[coord] = p1_y(d_in, q);
     }
     uint32_t rounds = 0, uses = 0;
     __syncthreads();
+    if (warp >= 0) {
     ListPlan<TI, TO, K, VEC> plan(a, sh, s, h, lane);
     while (true) {   // warp 0 announces a list, all work it off (one call site: the warps share the code)
         if (warp == 0) plan.next();
-        bar_sync<P::THREADS>(1);
+        bar_sync<P::ACTIVE>(1);
         if (sh.cmd_n == 0) break;
         run_list<TI, TO, K, VEC>(a, h, sh, guess, rounds, uses, warp, lane);
-        bar_sync<P::THREADS>(2);
+        bar_sync<P::ACTIVE>(2);
     }
-    if (a.d_final && warp < P::CORE) a.d_final[((size_t)s * H + h) * K + coord] = sh.cmd_dense ? p1_d(sh.y[coord], q) : d_in;
+    }
+    __syncthreads();
+    if (a.d_final && coord < K) a.d_final[((size_t)s * H + h) * K + coord] = sh.cmd_dense ? p1_d(sh.y[coord], q) : d_in;
 }
 
 // The stand-alone sweep processes every token: the whole sequence is one list (see above).  The fetching warps also
 // form the normalisers here (there is no parallel pass before this kernel; max k^2, which only the rounds' tolerance
 // needs, is taken as sum k^2); the finishing ones form the write keys and the residual ratios.
 template <typename TI, typename TO, int K, bool VEC>
-__global__ void __launch_bounds__(Pipe<K>::THREADS, 1) phase1_stream_kernel(P1Args a)
+__global__ void __launch_bounds__(FwdPipe<K>::THREADS, 1) phase1_stream_kernel(P1Args a)
 {
     constexpr int R = K / 32;
-    using P = Pipe<K>;
+    using P = FwdPipe<K>;
     constexpr int PN = PipeShared<TI, K, VEC>::PN;
     extern __shared__ __align__(16) uint8_t p1_dyn[];
     PipeShared<TI, K, VEC>& sh = *reinterpret_cast<PipeShared<TI, K, VEC>*>(p1_dyn);
     __shared__ float log_part[P::FINISH];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31, warp = P::role(threadIdx.x >> 5);
     const int chain = blockIdx.x;
     const int s = chain / a.H, h = chain % a.H, H = a.H;
     // packed batch: T_dense is the packed token count; a malformed offset pair is clamped into it
@@ -1061,10 +1086,13 @@ __global__ void __launch_bounds__(Pipe<K>::THREADS, 1) phase1_stream_kernel(P1Ar
     float lsum = 0.f;
     auto len_of = [&](int b) { return min(PB, len - b * PB); };
     auto th_of = [&](int b) { return lane < len_of(b) ? (uint32_t)((t0 + b * PB + lane) * H + h) : NO_ROW; };   // lane j: token j
-    if (warp < P::CORE) {
-        const size_t at = ((size_t)s * H + h) * K + warp * 32 + lane;
-        const float d0 = a.d0 ? a.d0[at] : 1.0f;
-        float y = p1_y(d0, q), guess = 0.f;
+    if (warp < 0) {
+        // idle
+    } else if (warp < P::CORE) {
+        const size_t at = ((size_t)s * H + h) * K + warp * 64 + lane * 2;
+        const float2 d0 = a.d0 ? load2(a.d0 + at) : make_float2(1.0f, 1.0f);
+        float2 y = make_float2(p1_y(d0.x, q), p1_y(d0.y, q));
+        float guess = 0.f;
         uint32_t rounds = 0;
         for (int b = 0; b < nblk; ++b) {
             ok = bar_sync_and<P::CORE * 32>(3, p1_mbar_wait(&sh.bars.full[b % PN], (b / PN) & 1, nullptr));
@@ -1073,7 +1101,7 @@ __global__ void __launch_bounds__(Pipe<K>::THREADS, 1) phase1_stream_kernel(P1Ar
             __syncwarp();
             if (lane == 0) p1_mbar_arrive(&sh.bars.done[b % PN]);
         }
-        if (a.d_final && ok) a.d_final[at] = nblk > 0 ? p1_d(y, q) : d0;
+        if (a.d_final && ok) *reinterpret_cast<float2*>(a.d_final + at) = nblk > 0 ? make_float2(p1_d(y.x, q), p1_d(y.y, q)) : d0;
     } else if (warp < P::FINISH0) {
         auto start = [&](int b) {
             if (b >= PN) ok = p1_mbar_wait(&sh.bars.free_[b % PN], ((b / PN) - 1) & 1, nullptr);
@@ -1682,7 +1710,7 @@ int fwd_launch(const P1Fwd& a, cudaStream_t st)
     const unsigned chains = (unsigned)(a.S * a.H);
     auto launch_seq = [&](auto kernel, size_t smem) {
         if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return false;
-        return launch_after(kernel, chains, Pipe<K>::THREADS, smem, st, a);
+        return launch_after(kernel, chains, FwdPipe<K>::THREADS, smem, st, a);
     };
     const bool okl = a.hy.apf_mode == 3 ? launch_seq(phase1_seq_kernel<TI, TO, K, true>, sizeof(PipeShared<TI, K, true>))
                                         : launch_seq(phase1_seq_kernel<TI, TO, K, false>, sizeof(PipeShared<TI, K, false>));
@@ -1780,8 +1808,8 @@ int phase1_update(const osdn_params& p, const Hyper& hy, const void* k, const fl
     auto typed = [&](auto t, auto kk) {
         using T = decltype(t);
         constexpr int K = decltype(kk)::value;
-        return vec ? launch(phase1_stream_kernel<T, T, K, true>, sizeof(PipeShared<T, K, true>), Pipe<K>::THREADS)
-                   : launch(phase1_stream_kernel<T, T, K, false>, sizeof(PipeShared<T, K, false>), Pipe<K>::THREADS);
+        return vec ? launch(phase1_stream_kernel<T, T, K, true>, sizeof(PipeShared<T, K, true>), FwdPipe<K>::THREADS)
+                   : launch(phase1_stream_kernel<T, T, K, false>, sizeof(PipeShared<T, K, false>), FwdPipe<K>::THREADS);
     };
     using K64 = std::integral_constant<int, 64>;
     using K128 = std::integral_constant<int, 128>;
