@@ -502,6 +502,10 @@ def main():
     sampler = ClockSampler(local)
     sampler.start()
     time.sleep(0.3)
+    for _ in range(50):   # nvidia-smi can take longer than that to report for the first time
+        if sampler.rows or sampler.proc is None:
+            break
+        time.sleep(0.1)
     ms_total, launches = timed(step, graph, per_step, steps)
     stages = per_kernel(step, steps)
     clocks = sampler.stop()
