@@ -17,7 +17,8 @@
 //   few chains     V / 16 CTAs of 4 warps x 4 rows per chain: a call of a few sequences is bound by latency and is spread
 //                  over the chip.  They form one thread-block cluster: the preconditioner is updated in place, so the
 //                  CTA that stores the advanced vector may do so only once every CTA of the chain has read the old one;
-//                  a cluster barrier (arrive after the read, wait before the store) gives exactly that order.
+//                  a cluster barrier (releasing arrival after the read, acquiring wait before the store) gives exactly
+//                  that order.
 //   many chains    one CTA of 8 warps per chain (see launch_one): no cluster to schedule, the preconditioner
 //                  update once per chain instead of eight times, a row's two sums share their shuffles with fifteen
 //                  other rows'.
@@ -165,16 +166,6 @@ template <typename T, int K, int V, bool VEC, int RW, int WARPS, bool MULTI> __d
 #pragma unroll
         for (int j = 0; j < R / 2; ++j) S[r][j] = pack2(x[2 * j], x[2 * j + 1]);
     }
-    if constexpr (SLICES > 1) {
-        // This slice has read the chain's preconditioner: the arrival takes the loaded values as an operand, so
-        // it cannot issue before they have come back, and a load that has returned cannot see a later store.
-        // (A releasing arrival would also wait for the state rows, which are still in flight here.)
-        float seen = d[0];
-#pragma unroll
-        for (int j = 1; j < R; ++j) seen += d[j];
-        asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::"f"(seen) : "memory");
-    }
-
     // v: of this lane's row; lrv: the log-retention vector (VEC)
     auto step = [&](int t, const float (&k1)[R], const float (&q1)[R], float v, float beta, float gate, float lr, const float (&lrv)[VEC ? R : 1]) {
         const float alpha = expf(gate);
@@ -231,6 +222,10 @@ template <typename T, int K, int V, bool VEC, int RW, int WARPS, bool MULTI> __d
             for (int j = 0; j < R / 2; ++j) S[r][j] = fma2(alpha2, S[r][j], mul2(x2, t2[j]));
         }
         const float o = dots(q2);
+        // The chain's preconditioner has been read (the sums above hold it): this slice's arrival releases that read to
+        // the slice that overwrites it behind the wait.  The state rows have come back by now too and nothing has been stored yet.
+        if constexpr (SLICES > 1)
+            if (t == 0) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
         if (lane < RW) stf(op + th_of(t) * V + vb0 + vw + lane, hy.scale * o);
     };
 

@@ -87,6 +87,26 @@ def test_decode_in_place_preconditioner_over_many_waves(L):
     assert parity.err(got_out, ref["out"]) <= parity.TOL["bf16"]
 
 
+@pytest.mark.parametrize("K,V", [(128, 128), (64, 64), (128, 64)])
+@pytest.mark.parametrize("L", [1, 9])
+def test_decode_sliced_chains_read_the_preconditioner_before_it_is_overwritten(K, V, L):
+    """Few chains are cut into slices that all read the preconditioner one of them overwrites: call after call in
+    place it is, bit for bit, what a chain in one piece (many chains: the same inputs repeated) computes."""
+    hy = OsdnHyper(eta=0.3, apf_mode=1, clamp=0)
+    H, rep, steps = 8, 24, 40
+    inp = draw("decode_slices", 4300 + L, [L * steps], H, K, V, "fp32", dense_B=1, hyper=hy, with_state=True)
+    few = [inp.init_state.float().to(DEV).contiguous().clone(), inp.precond_in.float().to(DEV).contiguous().clone()]
+    many = [x.repeat(rep, *[1] * (x.dim() - 1)).contiguous() for x in few]
+    for t in range(steps):
+        tok = [x[t * L:(t + 1) * L].float().to(DEV).contiguous() for x in (inp.q, inp.k, inp.v, inp.beta, inp.gate)]
+        for B, (S, d) in ((1, few), (rep, many)):
+            p = binding.make_params(B=B, T=L, H=H, K=K, V=V, io_dtype="fp32", hyper=hy)
+            x = [y.repeat(B, *[1] * (y.dim() - 1)).contiguous() for y in tok]
+            binding.osdn_decode_step(p, *x, None, S, d, torch.empty(B * L, H, V, device=DEV))
+        assert torch.equal(many[1], few[1].expand_as(many[1])), f"step {t}"
+    assert torch.allclose(many[0], few[0].expand_as(many[0]), rtol=1e-4, atol=1e-5)
+
+
 def test_decode_continues_in_place_across_calls():
     """Two calls of 3 and 4 tokens equal one call of 7: the cache carries everything."""
     hy = OsdnHyper(eta=0.3, apf_mode=1)
