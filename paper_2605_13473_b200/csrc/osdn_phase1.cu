@@ -409,20 +409,29 @@ template <typename TI, int K, bool VEC> struct PipeShared {
     PipeBars bars;
 };
 
-// The coordinate the recurrence runs in.  With the projection on, y = (d - d_min) / w, w = d_max - d_min: with
-// c' = c / w a step is one saturating multiply-add, y' = sat(rho y + (c' k^2 + (rho - 1) d_min / w)), and
-// c' = e' - a2 <y, k^2>, e' = (e - a2 d_min sum k^2) / w.  With it off, or for a box without width, y = d (w = 1, d_min
-// taken as 0).  Core, finishing warps and the walk use the same functions, hence the same values.
-enum P1Mode { P1_SAT, P1_FREE, P1_CLIP };
+// The coordinate the recurrence runs in, y = (d - lo) / w.  With c' = c / w a step is
+//   y' = project(rho y + (c' k^2 + (rho - 1) lo / w)),   c' = e' - a2 <y, k^2>,   e' = (e - a2 lo sum k^2) / w.
+//   P1_SAT    a box of ordinary width above zero: lo = d_min, w = d_max - d_min; the projection is the saturation of a
+//             multiply-add.  d - d_min is at most d there, so that a rounding of y is none larger than one of d.
+//   P1_PLAIN  everything else: no projection; a box that is open, without width, or of a width that 1 / w could not take
+//             (w = 1); a negative lower edge, below which d - d_min would be larger than d and cost its last bits (lo = 0).
+// Where lo = d_min the lower face is y = 0.  Core, finishing warps and the walk use the same functions, hence the same
+// values.
+enum P1Mode { P1_SAT, P1_PLAIN };
 struct P1Coord {
-    float lo, w, iw, k0;   // d = lo + w y; k0 = lo / w
+    float lo, w, iw, k0;   // k0 = lo / w
 };
-__device__ __forceinline__ P1Mode p1_mode(const Hyper& hy) { return !hy.clamp ? P1_FREE : hy.d_max > hy.d_min ? P1_SAT : P1_CLIP; }
+// Whether y = 0 is the lower face, so that tokens may be skipped there.
+__device__ __forceinline__ bool p1_face(const Hyper& hy) { return hy.clamp && hy.d_min >= 0.f && hy.d_min <= 1e30f; }
+__device__ __forceinline__ P1Mode p1_mode(const Hyper& hy)
+{
+    const float w = hy.d_max - hy.d_min;
+    return p1_face(hy) && w >= 1e-12f && w <= 1e12f ? P1_SAT : P1_PLAIN;
+}
 __device__ __forceinline__ P1Coord p1_coord(const Hyper& hy)
 {
-    if (p1_mode(hy) != P1_SAT) return {0.f, 1.f, 1.f, 0.f};
-    const float w = hy.d_max - hy.d_min, iw = 1.0f / w;
-    return {hy.d_min, w, iw, hy.d_min * iw};
+    const float lo = p1_face(hy) ? hy.d_min : 0.f, w = p1_mode(hy) == P1_SAT ? hy.d_max - hy.d_min : 1.0f, iw = 1.0f / w;
+    return {lo, w, iw, lo * iw};
 }
 __device__ __forceinline__ float p1_y(float d, const P1Coord& q) { return __fmul_rn(d - q.lo, q.iw); }
 __device__ __forceinline__ float p1_d(float y, const P1Coord& q) { return fmaf(q.w, y, q.lo); }
@@ -430,11 +439,13 @@ __device__ __forceinline__ float p1_off(float rho, const P1Coord& q) { return fm
 __device__ __forceinline__ float p1_raw(float y, float kap, float c, float rho, float off) { return fmaf(rho, y, fmaf(c, kap, off)); }
 template <P1Mode M> __device__ __forceinline__ float p1_project(float x, const Hyper& hy)
 {
-    return M == P1_SAT ? __saturatef(x) : M == P1_CLIP ? fminf(fmaxf(x, hy.d_min), hy.d_max) : x;
+    if (M == P1_SAT) return __saturatef(x);
+    if (!hy.clamp) return x;
+    return p1_face(hy) ? fminf(fmaxf(x, 0.f), hy.d_max - hy.d_min) : fminf(fmaxf(x, hy.d_min), hy.d_max);
 }
 __device__ __forceinline__ float p1_project(float x, P1Mode m, const Hyper& hy)
 {
-    return m == P1_SAT ? p1_project<P1_SAT>(x, hy) : m == P1_CLIP ? p1_project<P1_CLIP>(x, hy) : x;
+    return m == P1_SAT ? p1_project<P1_SAT>(x, hy) : p1_project<P1_PLAIN>(x, hy);
 }
 // e', a2, max k^2, sum k^2 of a token
 __device__ __forceinline__ float4 p1_scalars(float sumk, float kmax, float beta, const Hyper& hy, const P1Coord& q)
@@ -493,7 +504,7 @@ __device__ __forceinline__ int core_block(PipeShared<TI, K, VEC>& sh, PipeBuf<TI
     const unsigned jump = B.jump;
     const float4 sc = B.scal[lane];   // lane j: token j
     const bool jumped = bit_of(jump, lane);
-    const float tol = M == P1_FREE ? 0.f : 1.4901161e-8f * fmaxf(hy.d_min, 0.f) * q.iw;
+    const float tol = hy.clamp ? 1.4901161e-8f * fmaxf(hy.d_min, 0.f) * q.iw : 0.f;
     float c = jumped ? sc.x : fmaf(-sc.y, sc.w * r, sc.x), sum = 0.f;
     float2 z = y;
     // a step of both coordinates; keep: 0 behind a jump (then the scalar retention is 0 already)
@@ -580,10 +591,8 @@ template <typename TI, int K, bool VEC>
 __device__ __forceinline__ int core_block(PipeShared<TI, K, VEC>& sh, PipeBuf<TI, K, VEC>& B, int n, float2& y, float& r, uint32_t& rounds,
                                           const Hyper& hy, const P1Coord& q, int warp, int lane)
 {
-    const P1Mode mode = p1_mode(hy);
-    if (mode == P1_SAT) return core_block<TI, K, VEC, P1_SAT>(sh, B, n, y, r, rounds, hy, q, warp, lane);
-    if (mode == P1_FREE) return core_block<TI, K, VEC, P1_FREE>(sh, B, n, y, r, rounds, hy, q, warp, lane);
-    return core_block<TI, K, VEC, P1_CLIP>(sh, B, n, y, r, rounds, hy, q, warp, lane);
+    if (p1_mode(hy) == P1_SAT) return core_block<TI, K, VEC, P1_SAT>(sh, B, n, y, r, rounds, hy, q, warp, lane);
+    return core_block<TI, K, VEC, P1_PLAIN>(sh, B, n, y, r, rounds, hy, q, warp, lane);
 }
 
 // Rows of D elements on their way into a buffer; lane j of the warp holds the number of row j in the source (NO_ROW: the
@@ -642,10 +651,8 @@ __device__ __forceinline__ void finish_block(const PipeBuf<TI, K, VEC>& B, int n
 template <typename TI, int K, bool VEC, typename OUT>
 __device__ __forceinline__ void finish_block(const PipeBuf<TI, K, VEC>& B, int n, const Hyper& hy, const P1Coord& q, int lane, OUT out)
 {
-    const P1Mode mode = p1_mode(hy);
-    if (mode == P1_SAT) finish_block<TI, K, VEC, P1_SAT>(B, n, hy, q, lane, out);
-    else if (mode == P1_FREE) finish_block<TI, K, VEC, P1_FREE>(B, n, hy, q, lane, out);
-    else finish_block<TI, K, VEC, P1_CLIP>(B, n, hy, q, lane, out);
+    if (p1_mode(hy) == P1_SAT) finish_block<TI, K, VEC, P1_SAT>(B, n, hy, q, lane, out);
+    else finish_block<TI, K, VEC, P1_PLAIN>(B, n, hy, q, lane, out);
 }
 
 // The list in sh through the ring, all roles.  y travels through sh.y; guess and rounds belong to the core warps.
@@ -824,7 +831,7 @@ __device__ __forceinline__ int walk_list(const P1Fwd& a, int h, PipeShared<TI, K
         s = warp_sum(s);
         const float c = fmaf(-sc.y, s, sc.x);
         unsigned bits = 0;
-        bool on = mode == P1_SAT;
+        bool on = p1_face(hy);
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             d[r] = p1_d(y[r], q);
@@ -904,7 +911,7 @@ template <typename TI, typename TO, int K, bool VEC> struct ListPlan {
     const P1Fwd& a;
     PipeShared<TI, K, VEC>& sh;
     const int h, lane, c0, c1, seq_t0, seq_len;
-    const bool sat;
+    const bool has_face;
     // the group of 32 chunks in hand: unflagged and processed tokens (a chunk per lane), tokens, first token, next one
     int cbase, base = 0, glen = 0, pos = 0;
     unsigned long long unf = 0ull, proc = 0ull, cand = 0ull;
@@ -913,7 +920,7 @@ template <typename TI, typename TO, int K, bool VEC> struct ListPlan {
 
     __device__ __forceinline__ ListPlan(const P1Fwd& a_, PipeShared<TI, K, VEC>& sh_, int s, int h_, int lane_)
         : a(a_), sh(sh_), h(h_), lane(lane_), c0(a_.tab.seq_chunk0(s)), c1(a_.tab.seq_chunk0(s + 1)), seq_t0(a_.tab.seq_tok0(s)),
-          seq_len(a_.tab.seq_len(s)), sat(p1_mode(a_.hy) == P1_SAT), cbase(c0 - 32)
+          seq_len(a_.tab.seq_len(s)), has_face(p1_face(a_.hy)), cbase(c0 - 32)
     {
         face = on_face();
     }
@@ -922,7 +929,7 @@ template <typename TI, typename TO, int K, bool VEC> struct ListPlan {
         constexpr int R = K / 32;
         float y[R];
         load_row<R>(sh.y, lane, y);
-        bool on = sat;
+        bool on = has_face;
 #pragma unroll
         for (int r = 0; r < R; ++r) on = on && y[r] == 0.f;
         return __all_sync(0xffffffffu, on) != 0;

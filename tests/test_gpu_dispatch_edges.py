@@ -36,6 +36,27 @@ def _all_outputs(inp, label, **kw):
                    tensor_core=inp.io_dtype == "bf16" and inp.K == 128)
 
 
+INF = float("inf")
+
+
+@pytest.mark.parametrize("box", [(0.5, INF), (-INF, 2.0), (-INF, INF), (0.5, 3e38), (-1e4, 1e4), (-1.0, 2.0), (0.0, 2.0), (0.7, 0.7), (0.5, 0.5 + 2.0 ** -24)],
+                         ids=lambda b: f"{b[0]:g}_{b[1]:g}")
+@pytest.mark.parametrize("L,eta,apf", [(20, 0.3, 2), (300, 0.3, 2), (300, 0.3, 3), (300, 0.003, 1)])
+def test_boxes_of_any_shape(box, L, eta, apf):
+    """Open, wide, negative and empty boxes: the sums are taken in d itself there, and no bits are lost to d - d_min.
+    Short sequences are walked, long ones go through the blocks; with the small step d rests on the lower face."""
+    hy = OsdnHyper(eta=eta, apf_mode=apf, d_min=box[0], d_max=box[1])
+    inp = draw(f"box_{L}", 7500 + L + apf, [L], 2, 64, 64, "fp32", dense_B=1, hyper=hy, key_kind="sparse" if eta > 0.1 else "gauss",
+               with_dout=True, with_log_ret=apf >= 2, with_state_cotangents=True)
+    _all_outputs(inp, f"box_{box}_{L}")
+    b = binding.DeviceBundle(inp, DEV, need_bwd=False)
+    kt, d = torch.empty_like(b.k), torch.empty(1, 2, 64, device=DEV)
+    binding.osdn_precond_update(b.params, b.k, b.beta, b.log_ret if apf >= 2 else b.gate, None, kt, d)
+    ref = oracle.precond_update(hy, inp.seq_lens, inp.k, inp.beta, inp.gate, inp.log_ret, None)
+    assert parity.err(d.cpu().numpy(), ref["precond_out"]) <= 1e-5
+    assert parity.err(kt.cpu().numpy(), ref["ktil"]) <= 1e-5
+
+
 @pytest.mark.parametrize("shift", [3.0, 7.0])
 @pytest.mark.parametrize("lens", [[2300], [700, 64, 0, 33, 1, 1500]])
 def test_lists_of_processed_tokens(lens, shift):
