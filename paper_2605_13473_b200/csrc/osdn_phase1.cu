@@ -1326,7 +1326,7 @@ __device__ __forceinline__ void rev_core_block(RevShared<T, K, VEC>& sh, RevBuf<
     }
     B.lam0[i] = lam;
     const float4 sc = B.scal[lane];   // lane j: token j
-    float u = 0.f, l = lam;
+    float u = 0.f, un = 0.f, l = lam;   // un: the sums of the latest lambda
     for (int round = 0; round <= PB; ++round) {
         const uint32_t par = rounds++ & 1;
         sh.au[warp][lane] = -sc.x * u;
@@ -1349,7 +1349,7 @@ __device__ __forceinline__ void rev_core_block(RevShared<T, K, VEC>& sh, RevBuf<
         float(*part)[PB] = sh.part[par];
         part[warp][lane] = mine;
         bar_sync<CW * 32>(3);
-        float un = part[0][lane];
+        un = part[0][lane];
 #pragma unroll
         for (int x = 1; x < CW; ++x) un += part[x][lane];
         const float du = fabsf(un - u);
@@ -1358,7 +1358,7 @@ __device__ __forceinline__ void rev_core_block(RevShared<T, K, VEC>& sh, RevBuf<
         u = un;
     }
     lam = l;
-    if (warp == 0) B.grad[lane].w = u;
+    if (warp == 0) B.grad[lane].w = un;   // (a small a2 lets lambda stand before u does: the gradients need u itself)
 }
 
 // What a processed token leaves: dk and, where one per coordinate is asked for, the retention gradient.

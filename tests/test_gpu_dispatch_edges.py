@@ -57,6 +57,20 @@ def test_boxes_of_any_shape(box, L, eta, apf):
     assert parity.err(kt.cpu().numpy(), ref["ktil"]) <= 1e-5
 
 
+@pytest.mark.parametrize("beta", [1e-2, 1e-3, 1e-4, 1e-6])
+def test_small_write_strengths_in_the_reverse_blocks(beta):
+    """beta so small that the coupling of a block's tokens vanishes: lambda stands after one round, but the gradients of
+    the write strengths and keys need the sums <lambda, k^2> of that lambda.  Bound: about ten fp32 roundings (2e-6)."""
+    hy = OsdnHyper(eta=0.3, apf_mode=2)
+    inp = draw("small_beta", 7600, [300], 2, 64, 64, "fp32", dense_B=1, hyper=hy, key_kind="sparse", with_dout=True,
+               with_log_ret=True, with_state_cotangents=True)
+    inp.beta = torch.full_like(inp.beta, beta)
+    got = run_inputs_bwd(inp)
+    ref = parity.oracle_all(inp, True, got["projection_masks"])
+    for key in ("dbeta", "dk", "dlog_ret"):
+        assert parity.err(got[key], ref[key], norm="l2") <= 2e-6, key
+
+
 @pytest.mark.parametrize("shift", [3.0, 7.0])
 @pytest.mark.parametrize("lens", [[2300], [700, 64, 0, 33, 1, 1500]])
 def test_lists_of_processed_tokens(lens, shift):
