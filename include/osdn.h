@@ -204,7 +204,8 @@ int osdn_decode_step(const osdn_params* p, const void* q, const void* k, const v
  *   dgate_k  [T,H,K] fp32, written in full.
  *   workspace: osdn_kda_workspace_bytes(p, need_bwd) bytes (0 is returned for rejected parameters); for
  *            the backward it includes, beside the regions of osdn_workspace_bytes, the in-chunk prefix of the
- *            channel gates (fp32, [T,H,K] rounded up to whole chunks).
+ *            channel gates (two fp32 parts, [T,H,K] each, rounded up to whole chunks).  A gate below -104, -inf
+ *            included, is a factor of zero.
  * This path computes in fp32 on CUDA cores for both io_dtypes, chunk by chunk.
  */
 size_t osdn_kda_workspace_bytes(const osdn_params* p, int need_bwd);

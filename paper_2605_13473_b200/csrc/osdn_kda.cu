@@ -11,10 +11,10 @@
 
 namespace osdn {
 
-// The in-chunk gate prefix of every tile, which the backward reads again.
+// The in-chunk gate prefix of every tile (high and low parts), which the backward reads again.
 size_t kda_extra_bytes(const osdn_params& p, const WsLayout& L, bool need_bwd)
 {
-    return need_bwd ? align_up((size_t)L.NTmax * p.H * CH * p.K * 4, 256) : 0;
+    return need_bwd ? align_up((size_t)L.NTmax * p.H * 2 * CH * p.K * 4, 256) : 0;
 }
 
 namespace {

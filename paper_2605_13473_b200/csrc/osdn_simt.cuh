@@ -8,9 +8,10 @@
 // G is the inclusive prefix of the log-gates inside the chunk.
 //
 // With a channel gate the factors exp(G_ic - G_jc) sit inside the contraction.  Where every |G_C| of the chunk is at
-// most SAFE_RANGE they are split over the operands, exp(G_ic) and exp(-G_jc), both far inside the fp32 range
-// (relative error of a product of the two: that of the prefix, as for the difference), and the scores are plain
-// products.  A chunk with stronger gates forms the differences pair by pair.
+// most SAFE_RANGE they are split over the operands, exp(G_ic) and exp(-G_jc), both far inside the fp32 range, and the
+// scores are plain products.  A chunk with stronger gates forms the differences pair by pair.  A factor's relative error
+// is the absolute error of its exponent, and a prefix of -30 in one float is off by 1e-6 (one of -10000, behind a gate
+// that forgets everything, by 5e-4): the prefix is kept as a sum of two floats.
 #pragma once
 
 #include "osdn_common.cuh"
@@ -249,7 +250,7 @@ struct ChunkArgs {
     const float *beta, *gate;        // gate: [T,H], channel gate [T,H,K]
     const float* ktil;
     float *Tm, *P, *R, *W, *U;       // R: the Gram with its gate factors, A without beta
-    float *Ktr, *Qg, *gC, *G;        // G: channel gate only, [tile][64][K]
+    float *Ktr, *Qg, *gC, *G;        // G: channel gate only, [tile][2][64][K], the prefix's high and low parts
     // output pass, backward
     void* out;
     const void* dout;
@@ -260,37 +261,102 @@ struct ChunkArgs {
     Hyper hy;
 };
 
-__device__ __forceinline__ float4 exp4(const float4& v) { return make_float4(__expf(v.x), __expf(v.y), __expf(v.z), __expf(v.w)); }
+__device__ __forceinline__ float4 exp4(const float4& v) { return make_float4(expf(v.x), expf(v.y), expf(v.z), expf(v.w)); }
+// exp of a sum h + l with |l| a rounding of h
+__device__ __forceinline__ float exp_sum(float h, float l)
+{
+    const float e = expf(h);
+    return fmaf(e, l, e);
+}
+__device__ __forceinline__ float4 exp_sum(const float4& h, const float4& l) { return make_float4(exp_sum(h.x, l.x), exp_sum(h.y, l.y), exp_sum(h.z, l.z), exp_sum(h.w, l.w)); }
+// x + y into x, the rounding of the sum into e
+__device__ __forceinline__ void add_exact(float& x, float& e, float y)
+{
+    const float s = x + y, b = s - x;
+    e += (x - (s - b)) + (y - b);
+    x = s;
+}
+// exp((ah + al) - (bh + bl))
+__device__ __forceinline__ float exp_diff(float ah, float al, float bh, float bl)
+{
+    float e = al - bl;
+    add_exact(ah, e, -bh);
+    return exp_sum(ah, e);
+}
+__device__ __forceinline__ float4 exp_diff(const float4& ah, const float4& al, const float4& bh, const float4& bl)
+{
+    return make_float4(exp_diff(ah.x, al.x, bh.x, bl.x), exp_diff(ah.y, al.y, bh.y, bl.y), exp_diff(ah.z, al.z, bh.z, bl.z), exp_diff(ah.w, al.w, bh.w, bl.w));
+}
 __device__ __forceinline__ float4 operator*(const float4& a, const float4& b) { return make_float4(a.x * b.x, a.y * b.y, a.z * b.z, a.w * b.w); }
 __device__ __forceinline__ float4 operator-(const float4& a, const float4& b) { return make_float4(a.x - b.x, a.y - b.y, a.z - b.z, a.w - b.w); }
+__device__ __forceinline__ float4 operator+(const float4& a, const float4& b) { return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w); }
 __device__ __forceinline__ float4 neg_part(const float4& v) { return make_float4(fminf(v.x, 0.f), fminf(v.y, 0.f), fminf(v.z, 0.f), fminf(v.w, 0.f)); }
 template <int TN> __device__ __forceinline__ float4 quad(const float (&x)[TN], int c) { return make_float4(x[c], x[c + 1], x[c + 2], x[c + 3]); }
 template <int TN> __device__ __forceinline__ void set_quad(float (&x)[TN], int c, const float4& v) { x[c] = v.x; x[c + 1] = v.y; x[c + 2] = v.z; x[c + 3] = v.w; }
 
 // Strong channel gates: acc[i][n] += sum_j c(m, j) b(j, n) exp(G_mn - G_jn) over j <= m, or with REV exp(G_jn - G_mn)
-// over j >= m.  c is zero on the other side of the diagonal, where the exponent is clamped.
-template <bool REV, int TN, class C, class B, class GG>
-__device__ __forceinline__ void pair_mm(float (&acc)[4][TN], int j0, int j1, const Lane& l, C c, B b, GG g)
+// over j >= m.  c is zero on the other side of the diagonal, where the exponent is clamped.  g, gl: the prefix's parts.
+template <bool REV, int TN, class C, class B, class GG, class GL>
+__device__ __forceinline__ void pair_mm(float (&acc)[4][TN], int j0, int j1, const Lane& l, C c, B b, GG g, GL gl)
 {
 #pragma unroll
     for (int cc = 0; cc < TN; cc += 4) {
         const int n = col_of<false>(l, cc);
-        float4 gm[4];
+        float4 gm[4], lm[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) gm[i] = g(row_of(l, i), n);
+        for (int i = 0; i < 4; ++i) {
+            gm[i] = g(row_of(l, i), n);
+            lm[i] = gl(row_of(l, i), n);
+        }
         for (int j = j0; j < j1; ++j) {
-            const float4 bj = b(j, n), gj = g(j, n);
+            const float4 bj = b(j, n), gj = g(j, n), lj = gl(j, n);
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-                const float4 e = c(row_of(l, i), j) * (bj * exp4(neg_part(REV ? gj - gm[i] : gm[i] - gj)));
+                const float4 e = c(row_of(l, i), j) * (bj * exp4(neg_part(REV ? (gj - gm[i]) + (lj - lm[i]) : (gm[i] - gj) + (lm[i] - lj))));
                 set_quad(acc[i], cc, make_float4(acc[i][cc] + e.x, acc[i][cc + 1] + e.y, acc[i][cc + 2] + e.z, acc[i][cc + 3] + e.w));
             }
         }
     }
 }
 
-// In-chunk prefix of the channel gates in shared memory, [64][LD], over the rows; the threads cut the rows into
-// segments.  With REV the suffix instead.  tot: [CL_NT / K][K] scratch.
+// A gate below this is a factor of zero in fp32 whatever its value (exp(-104) is less than half of the smallest number),
+// and taken as this the prefix stays finite.
+constexpr float GATE_FLOOR = -104.f;
+
+// In-chunk prefix of the channel gates in shared memory, [64][LD], over the rows, as high parts in x and low parts in lo;
+// the threads cut the rows into segments.  tot: [2][CL_NT / K][K] scratch.
+template <int K, int LD> __device__ __forceinline__ void gate_prefix(float* x, float* lo, float* tot)
+{
+    constexpr int SEG = CL_NT / K, ROWS = CH / SEG;
+    const int c = threadIdx.x % K, s = threadIdx.x / K;
+    auto gate = [&](int r) {
+        const float g = x[(s * ROWS + r) * LD + c];
+        return g < GATE_FLOOR ? GATE_FLOOR : g;
+    };
+    float h = 0.f, l = 0.f;
+#pragma unroll
+    for (int r = 0; r < ROWS; ++r) add_exact(h, l, gate(r));
+    tot[s * K + c] = h;
+    tot[(SEG + s) * K + c] = l;
+    __syncthreads();
+    h = l = 0.f;
+#pragma unroll
+    for (int o = 0; o < SEG; ++o)
+        if (o < s) {
+            add_exact(h, l, tot[o * K + c]);
+            l += tot[(SEG + o) * K + c];
+        }
+#pragma unroll
+    for (int r = 0; r < ROWS; ++r) {
+        add_exact(h, l, gate(r));
+        const float g = h + l;
+        x[(s * ROWS + r) * LD + c] = g;
+        lo[(s * ROWS + r) * LD + c] = (h - g) + l;
+    }
+    __syncthreads();
+}
+
+// Inclusive sums of the columns of x, [64][LD], down the rows (REV: up), in place.  tot: [CL_NT / K][K] scratch.
 template <int K, int LD, bool REV> __device__ __forceinline__ void column_scan(float* x, float* tot)
 {
     constexpr int SEG = CL_NT / K, ROWS = CH / SEG;
@@ -315,7 +381,7 @@ template <int K, int LD, bool REV> __device__ __forceinline__ void column_scan(f
 
 template <typename T, int K, int V, bool CG> struct LocalFwd {
     static constexpr int LD = K + 4;
-    static constexpr size_t SMEM = sizeof(float) * ((CG ? 4 : 3) * CH * LD + 2 * CH * LC);
+    static constexpr size_t SMEM = sizeof(float) * ((CG ? 5 : 3) * CH * LD + 2 * CH * LC);
     // scalar gate at K = V = 64: two CTAs per SM
     static constexpr int MIN_CTAS = !CG && K + V == 128 ? 2 : 1;
 };
@@ -331,7 +397,8 @@ __global__ void __launch_bounds__(CL_NT, LocalFwd<T, K, V, CG>::MIN_CTAS) chunk_
     float* sQ = sKt + CH * LD;        // q; channel gate: gamma (.) q
     float* sT = sQ + CH * LD;
     float* sA = sT + CH * LC;
-    float* sG = sA + CH * LC;         // channel gate only
+    float* sG = sA + CH * LC;         // channel gate only: the prefix's high and low parts
+    float* sL = sG + CH * LD;
     __shared__ GateVecs gv;
     __shared__ float tmp[32 * 32];
 
@@ -351,9 +418,9 @@ __global__ void __launch_bounds__(CL_NT, LocalFwd<T, K, V, CG>::MIN_CTAS) chunk_
         load_tile<float, K, CL_NT>(sG, LD, a.gate, tok0, len, H, h);
         if (threadIdx.x < CH) gv.beta[threadIdx.x] = threadIdx.x < len ? a.beta[(size_t)(tok0 + threadIdx.x) * H + h] : 0.f;
         __syncthreads();
-        column_scan<K, LD, false>(sG, tmp);
+        gate_prefix<K, LD>(sG, sL, tmp);
         safe = __syncthreads_and(threadIdx.x >= K || fabsf(sG[(CH - 1) * LD + (threadIdx.x & (K - 1))]) <= SAFE_RANGE);
-        if (threadIdx.x < K) a.gC[tile * K + threadIdx.x] = __expf(sG[(CH - 1) * LD + threadIdx.x]);
+        if (threadIdx.x < K) a.gC[tile * K + threadIdx.x] = exp_sum(sG[(CH - 1) * LD + threadIdx.x], sL[(CH - 1) * LD + threadIdx.x]);
     } else {
         load_gates(gv, a.gate, a.beta, tok0, len, H, h);
         __syncthreads();
@@ -364,13 +431,16 @@ __global__ void __launch_bounds__(CL_NT, LocalFwd<T, K, V, CG>::MIN_CTAS) chunk_
         const size_t g = tile * CH * K + e * 4;
         const float4 q = ld4(sQ + i * LD + n), kt = ld4(sKt + i * LD + n);
         if constexpr (CG) {
-            const float4 G = ld4(sG + i * LD + n), eg = exp4(G), qg = eg * q;
-            if (a.G) st4(a.G + g, G);
+            const float4 G = ld4(sG + i * LD + n), gl = ld4(sL + i * LD + n), eg = exp_sum(G, gl), qg = eg * q;
+            if (a.G) {
+                st4(a.G + tile * 2 * CH * K + e * 4, G);
+                st4(a.G + (tile * 2 + 1) * CH * K + e * 4, gl);
+            }
             st4(a.Qg + g, qg);
-            st4(a.Ktr + g, exp4(ld4(sG + (CH - 1) * LD + n) - G) * kt);
+            st4(a.Ktr + g, exp_diff(ld4(sG + (CH - 1) * LD + n), ld4(sL + (CH - 1) * LD + n), G, gl) * kt);
             st4(sQ + i * LD + n, qg);
             st4(sK + i * LD + n, eg * ld4(sK + i * LD + n));
-            if (safe) st4(sKt + i * LD + n, exp4(-1.f * G) * kt);
+            if (safe) st4(sKt + i * LD + n, exp_sum(-1.f * G, -1.f * gl) * kt);
         } else {
             st4(a.Qg + g, gv.gam[i] * q);
             st4(a.Ktr + g, gv.rho[i] * kt);
@@ -389,18 +459,19 @@ __global__ void __launch_bounds__(CL_NT, LocalFwd<T, K, V, CG>::MIN_CTAS) chunk_
         } else {
             const Rows<T, K> x = rows_of<T, K>(grp == 0 ? a.k : a.q, tok0, len, H, h);
             for (int k = 0; k < K; k += 4) {
-                float4 kt[4], gn[4];
+                float4 kt[4], gn[4], ln[4];
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     kt[j] = ld4(sKt + col_of<true>(l, j) * LD + k);
                     gn[j] = ld4(sG + col_of<true>(l, j) * LD + k);
+                    ln[j] = ld4(sL + col_of<true>(l, j) * LD + k);
                 }
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
-                    const float4 xm = x(row_of(l, i), k), gm = ld4(sG + row_of(l, i) * LD + k);
+                    const float4 xm = x(row_of(l, i), k), gm = ld4(sG + row_of(l, i) * LD + k), lm = ld4(sL + row_of(l, i) * LD + k);
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
-                        const float4 p = (xm * kt[j]) * exp4(neg_part(gm - gn[j]));
+                        const float4 p = (xm * kt[j]) * exp4(neg_part((gm - gn[j]) + (lm - ln[j])));
                         acc[i][j] += (p.x + p.y) + (p.z + p.w);
                     }
                 }
@@ -903,8 +974,11 @@ __global__ void __launch_bounds__(CL_NT) chunk_local_bwd_kernel(ChunkArgs a)
     const float* dSg = a.dSn + tile * V * K;
     const float* dUg = a.dU + tile * CH * V;
     const float* ddUg = a.ddU + tile * CH * V;
-    const float* Gg = CG ? a.G + tile * CH * K : nullptr;
+    const float* Gg = CG ? a.G + tile * 2 * CH * K : nullptr;
     auto G4 = [&](int i, int n) { return ld4(Gg + i * K + n); };
+    auto L4 = [&](int i, int n) { return ld4(Gg + (CH + i) * K + n); };
+    auto expG = [&](int i, int n) { return exp_sum(G4(i, n), L4(i, n)); };
+    auto expmG = [&](int i, int n) { return exp_sum(-1.f * G4(i, n), -1.f * L4(i, n)); };
     float* sU = sX;                                  // dU [64][LU], until X is written
     float* sV = V == 64 ? sY : sX;                   // v  [64][LU]
 
@@ -915,9 +989,8 @@ __global__ void __launch_bounds__(CL_NT) chunk_local_bwd_kernel(ChunkArgs a)
         const Rows<float, K> ktr = rows_of<float, K>(a.ktil, tok0, len, H, h);
         float4 k = kr(i, n), kt = ktr(i, n);
         if constexpr (CG) {
-            const float4 G = G4(i, n);
-            k = exp4(G) * k;
-            if (safe) kt = exp4(-1.f * G) * kt;
+            k = expG(i, n) * k;
+            if (safe) kt = expmG(i, n) * kt;
             st4(sQ + i * LD + n, ld4(a.Qg + tile * CH * K + e * 4));
         } else {
             st4(sQ + i * LD + n, qr(i, n));
@@ -1002,7 +1075,6 @@ __global__ void __launch_bounds__(CL_NT) chunk_local_bwd_kernel(ChunkArgs a)
             for (int cc = 0; cc < TN; cc += 4) set_quad(acc[i], cc, f(row_of(l, i), col_of<false>(l, cc)) * quad(acc[i], cc));
     };
     auto splat = [](float x) { return make_float4(x, x, x, x); };
-    auto expG = [&](int m, int n) { return exp4(G4(m, n)); };
     // channel gate: x (.) y of a tile, plus z, into dst [64][LD]
     auto put_products = [&](auto& acc, auto ld, float* dst, auto z) {
         constexpr int TN = sizeof(acc[0]) / 4;
@@ -1045,7 +1117,7 @@ __global__ void __launch_bounds__(CL_NT) chunk_local_bwd_kernel(ChunkArgs a)
                 scale_rows(acc, expG);
             } else {
                 scale_rows(acc, expG);
-                pair_mm<false, TK>(acc, 0, m_hi, l, [&](int m, int j) { return sDP[m * LC + j]; }, ldKt, G4);
+                pair_mm<false, TK>(acc, 0, m_hi, l, [&](int m, int j) { return sDP[m * LC + j]; }, ldKt, G4, L4);
                 products(qr);
             }
         }
@@ -1106,7 +1178,7 @@ __global__ void __launch_bounds__(CL_NT) chunk_local_bwd_kernel(ChunkArgs a)
         // towards dktil: rho (.) dKtr; channel gate, safe: gC (.) dKtr, the common factor exp(-G) follows at the end
         if constexpr (!CG) scale_rows(keep, [&](int m, int) { return splat(gv.rho[m]); });
         else if (safe) scale_rows(keep, [&](int, int n) { return expG(CH - 1, n); });
-        else scale_rows(keep, [&](int m, int n) { return exp4(G4(CH - 1, n) - G4(m, n)); });
+        else scale_rows(keep, [&](int m, int n) { return exp_diff(G4(CH - 1, n), L4(CH - 1, n), G4(m, n), L4(m, n)); });
         float col[TK];
 #pragma unroll
         for (int j = 0; j < TK; ++j) col[j] = 0.f;
@@ -1174,7 +1246,7 @@ __global__ void __launch_bounds__(CL_NT) chunk_local_bwd_kernel(ChunkArgs a)
                 scale_rows(keep, expG);
             } else {
                 scale_rows(keep, expG);
-                pair_mm<false, TK>(keep, 0, m_hi, l, [&](int m, int j) { return sX[m * LC + j]; }, ldKt, G4);
+                pair_mm<false, TK>(keep, 0, m_hi, l, [&](int m, int j) { return sX[m * LC + j]; }, ldKt, G4, L4);
                 put(kr);
             }
         }
@@ -1186,14 +1258,14 @@ __global__ void __launch_bounds__(CL_NT) chunk_local_bwd_kernel(ChunkArgs a)
             tile_mm<true, false, TK>(keep, m_lo, CH, l, dPt, ldQ);
             tile_mm<true, false, TK>(keep, m_lo, CH, l, Xt, ldK);
         } else {
-            pair_mm<true, TK>(keep, m_lo, CH, l, [&](int m, int j) { return sDP[j * LC + m]; }, qr, G4);
-            pair_mm<true, TK>(keep, m_lo, CH, l, [&](int m, int j) { return sX[j * LC + m]; }, kr, G4);
+            pair_mm<true, TK>(keep, m_lo, CH, l, [&](int m, int j) { return sDP[j * LC + m]; }, qr, G4, L4);
+            pair_mm<true, TK>(keep, m_lo, CH, l, [&](int m, int j) { return sX[j * LC + m]; }, kr, G4, L4);
         }
         if constexpr (!CG) {
             row_dots(keep, ldKt, sE[2]);
         } else {
             put_products(keep, ldKt, sE2, [](int, int) { return make_float4(0.f, 0.f, 0.f, 0.f); });
-            if (safe) scale_rows(keep, [&](int m, int n) { return exp4(-1.f * G4(m, n)); });
+            if (safe) scale_rows(keep, expmG);
         }
         store_rows(keep, a.dktil, K);
     }

@@ -47,6 +47,21 @@ def test_forward_and_backward_match_the_oracle(name):
     parity.compare(got, ref, inp.io_dtype, BWD, label="oskda/" + name)
 
 
+@pytest.mark.parametrize("gate", [-20.0, -200.0, -1e4, -np.inf])
+@pytest.mark.parametrize("K,V", [(64, 64), (128, 128)])
+def test_gates_that_forget_everything(gate, K, V):
+    """Now and then a token whose gate wipes the state: the decays between the tokens behind it are as exact as without
+    it (bound: about ten fp32 roundings), and a factor of zero may be written as minus infinity."""
+    inp = _case(68, [200], 2, K, V, "fp32", 2, dense_B=1, eta=0.003)
+    inp.gate[5::40] = float(gate)
+    inp.gate[23::40, :, ::2] = float(gate)
+    got = binding.run_inputs_bwd(inp)
+    ref = parity.oracle_all(inp, bwd=True, gpu_masks=got["projection_masks"])
+    parity.compare(got, ref, "fp32", BWD, label=f"oskda/gate_{gate}")
+    for key in FWD + ("dq", "dk", "dv", "dbeta", "dgate"):
+        assert parity.err(got[key], ref[key], norm="l2") <= 2e-6, key
+
+
 def test_forward_alone_and_recomputed_residuals():
     inp = _case(71, [100, 100], 2, 128, 128, "fp32", 2, dense_B=2)
     f = binding.run_inputs_fwd(inp)
