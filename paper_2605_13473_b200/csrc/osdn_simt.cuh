@@ -937,8 +937,12 @@ __global__ void __launch_bounds__(K / 64 * 256) chain_wide_kernel(ChainArgs a)
 //
 // The gate gradient needs no sums of its own over the score matrices: with
 //   E_i = dq_i (.) q_i + dk_read_i (.) k_i - dktil_i (.) ktil_i     (phase-2 gradients)
-// dG_i = E_i + 1[i = last] (sum_j dKtr_j (.) Ktr_j + gC (.) sum_v dS (.) S), summed over the channels when the gate
-// is a scalar, and the gate's gradient is its suffix sum inside the chunk.
+// dG_i = E_i + 1[i = last] (sum_j dKtr_j (.) Ktr_j + gC (.) sum_v dS (.) S), summed over the channels, and the gate's
+// gradient is its suffix sum inside the chunk.
+// With a gate per channel that sum is taken apart, since behind strong gates it is small against terms that cancel in it: a
+// token's product with itself (the diagonal of P), which is in dq (.) q and in dktil (.) ktil, is left out of both; and what
+// the chunk's end takes from the writes, sum over j < i of dKtr_j (.) Ktr_j, is a prefix sum instead of the total less a
+// suffix.
 // ---------------------------------------------------------------------------------------
 template <int K> constexpr size_t local_bwd_smem() { return sizeof(float) * (4 * CH * (K + 4) + 4 * CH * LC); }
 template <typename T, int K, int V, bool CG>
@@ -955,8 +959,8 @@ __global__ void __launch_bounds__(CL_NT) chunk_local_bwd_kernel(ChunkArgs a)
     float* sY = sDP + CH * LC;      // T^T dT
     float* sT = sY + CH * LC;       // T.  sY and sT together: channel gate, at the end: dktil (.) ktil
     __shared__ GateVecs gv;
-    __shared__ float sB[3][CH], sE[3][CH];
-    __shared__ float sRed[PARTS][K], sR[8][K];   // column sums of dS (.) S and of dKtr (.) Ktr
+    __shared__ float sB[3][CH], sE[3][CH];   // channel gate: sE[0] the diagonal of dP
+    __shared__ __align__(16) float sRed[PARTS][K], sR[8][K];   // column sums of dS (.) S and of dKtr (.) Ktr
 
     const int c = blockIdx.x, h = blockIdx.y, H = a.H;
     const int len = a.tab.chunk_len(c);
@@ -1030,6 +1034,10 @@ __global__ void __launch_bounds__(CL_NT) chunk_local_bwd_kernel(ChunkArgs a)
                 const int m = row_of(l, i), n = col_of<true>(l, j);
                 float x = n <= m ? scale * acc[i][j] : 0.f;
                 if constexpr (!CG) x *= expf(fminf(gv.G[m] - gv.G[n], 0.f));
+                else if (n == m) {
+                    sE[0][m] = x;
+                    x = 0.f;
+                }
                 sDP[m * LC + n] = x;
             }
     } else {
@@ -1087,6 +1095,14 @@ __global__ void __launch_bounds__(CL_NT) chunk_local_bwd_kernel(ChunkArgs a)
                 st4(dst + m * LD + n, make_float4(p.x + o.x, p.y + o.y, p.z + o.z, p.w + o.w));
             }
     };
+    // channel gate: the diagonal of dP times x
+    auto add_diag = [&](auto& acc, auto ld) {
+        constexpr int TN = sizeof(acc[0]) / 4;
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int cc = 0; cc < TN; cc += 4) set_quad(acc[i], cc, quad(acc[i], cc) + sE[0][row_of(l, i)] * ld(row_of(l, i), col_of<false>(l, cc)));
+    };
     auto ldK = [&](int m, int n) { return ld4(sK + m * LD + n); };
     auto ldKt = [&](int m, int n) { return ld4(sKt + m * LD + n); };
     auto ldQ = [&](int m, int n) { return ld4(sQ + m * LD + n); };
@@ -1114,11 +1130,13 @@ __global__ void __launch_bounds__(CL_NT) chunk_local_bwd_kernel(ChunkArgs a)
             if (safe) {
                 tile_mm<false, false, TK>(acc, 0, m_hi, l, dP, ldKt);
                 products(ldQ);
+                add_diag(acc, ldKt);
                 scale_rows(acc, expG);
             } else {
                 scale_rows(acc, expG);
                 pair_mm<false, TK>(acc, 0, m_hi, l, [&](int m, int j) { return sDP[m * LC + j]; }, ldKt, G4, L4);
                 products(qr);
+                add_diag(acc, ldKt);
             }
         }
         store_rows(acc, static_cast<T*>(a.dq), K);
@@ -1179,21 +1197,26 @@ __global__ void __launch_bounds__(CL_NT) chunk_local_bwd_kernel(ChunkArgs a)
         if constexpr (!CG) scale_rows(keep, [&](int m, int) { return splat(gv.rho[m]); });
         else if (safe) scale_rows(keep, [&](int, int n) { return expG(CH - 1, n); });
         else scale_rows(keep, [&](int m, int n) { return exp_diff(G4(CH - 1, n), L4(CH - 1, n), G4(m, n), L4(m, n)); });
-        float col[TK];
+        if constexpr (!CG) {
+            float col[TK];
 #pragma unroll
-        for (int j = 0; j < TK; ++j) col[j] = 0.f;
+            for (int j = 0; j < TK; ++j) col[j] = 0.f;
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+            for (int i = 0; i < 4; ++i)
 #pragma unroll
-            for (int cc = 0; cc < TK; cc += 4) {
-                const float4 p = quad(keep[i], cc) * ldKt(row_of(l, i), col_of<false>(l, cc));
-                col[cc] += p.x; col[cc + 1] += p.y; col[cc + 2] += p.z; col[cc + 3] += p.w;
-            }
+                for (int cc = 0; cc < TK; cc += 4) {
+                    const float4 p = quad(keep[i], cc) * ldKt(row_of(l, i), col_of<false>(l, cc));
+                    col[cc] += p.x; col[cc + 1] += p.y; col[cc + 2] += p.z; col[cc + 3] += p.w;
+                }
 #pragma unroll
-        for (int j = 0; j < TK; ++j) col[j] += __shfl_xor_sync(0xffffffffu, col[j], 16);
-        if (!(threadIdx.x & 16))
+            for (int j = 0; j < TK; ++j) col[j] += __shfl_xor_sync(0xffffffffu, col[j], 16);
+            if (!(threadIdx.x & 16))
 #pragma unroll
-            for (int cc = 0; cc < TK; cc += 4) st4(&sR[(threadIdx.x >> 5) & 7][col_of<false>(l, cc)], quad(col, cc));
+                for (int cc = 0; cc < TK; cc += 4) st4(&sR[(threadIdx.x >> 5) & 7][col_of<false>(l, cc)], quad(col, cc));
+        } else {   // waits in dktil, for the same thread
+            store_rows(keep, a.dktil, K);
+            zero(keep);
+        }
     }
     __syncthreads();
 
@@ -1264,7 +1287,20 @@ __global__ void __launch_bounds__(CL_NT) chunk_local_bwd_kernel(ChunkArgs a)
         if constexpr (!CG) {
             row_dots(keep, ldKt, sE[2]);
         } else {
+            const Rows<float, K> part = rows_of<float, K>(a.dktil, tok0, len, H, h);   // (rows beyond len: dU is zero there)
             put_products(keep, ldKt, sE2, [](int, int) { return make_float4(0.f, 0.f, 0.f, 0.f); });
+            if (safe) add_diag(keep, ldQ);
+            else add_diag(keep, qr);
+            asm volatile("bar.sync 1, 256;" ::: "memory");   // gamma (.) q has been read: its place takes dKtr (.) Ktr
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int cc = 0; cc < TK; cc += 4) {
+                    const int m = row_of(l, i), n = col_of<false>(l, cc);
+                    const float4 x = part(m, n);
+                    st4(sQ + m * LD + n, x * ldKt(m, n));
+                    set_quad(keep[i], cc, quad(keep[i], cc) + x);
+                }
             if (safe) scale_rows(keep, expmG);
         }
         store_rows(keep, a.dktil, K);
@@ -1297,24 +1333,20 @@ __global__ void __launch_bounds__(CL_NT) chunk_local_bwd_kernel(ChunkArgs a)
             if (i + 32 < len) a.dgate[th + (size_t)32 * H] = y;
         }
     } else {
-        for (int e = threadIdx.x; e < CH * K; e += CL_NT) {
-            const int i = e / K, n = e % K;
-            float x = sW[i * LD + n] - sE2[i * LD + n];
-            if (i == CH - 1) {
-                float tot = 0.f;
-#pragma unroll
-                for (int p = 0; p < 8; ++p) x += sR[p][n];
-#pragma unroll
-                for (int p = 0; p < PARTS; ++p) tot += sRed[p][n];
-                x = fmaf(a.gC[tile * K + n], tot, x);
-            }
-            sW[i * LD + n] = x;
+        for (int e = threadIdx.x; e < CH * K / 4; e += CL_NT) {
+            const int i = e / (K / 4), n = e % (K / 4) * 4;
+            st4(sW + i * LD + n, ld4(sW + i * LD + n) - ld4(sE2 + i * LD + n));
         }
         __syncthreads();
         column_scan<K, LD, true>(sW, sK);
+        column_scan<K, LD, false>(sQ, sK);
         for (int e = threadIdx.x; e < len * (K / 4); e += CL_NT) {
             const int i = e / (K / 4), n = e % (K / 4) * 4;
-            st4(a.dgate + ((size_t)(tok0 + i) * H + h) * K + n, ld4(sW + i * LD + n));
+            float4 tot = make_float4(0.f, 0.f, 0.f, 0.f), x = ld4(sW + i * LD + n);
+#pragma unroll
+            for (int p = 0; p < PARTS; ++p) tot = tot + ld4(&sRed[p][n]);
+            if (i > 0) x = x + ld4(sQ + (i - 1) * LD + n);
+            st4(a.dgate + ((size_t)(tok0 + i) * H + h) * K + n, x + ld4(a.gC + tile * K + n) * tot);
         }
     }
     if (threadIdx.x >= 64 && threadIdx.x < 64 + CH) {

@@ -62,6 +62,16 @@ def test_gates_that_forget_everything(gate, K, V):
         assert parity.err(got[key], ref[key], norm="l2") <= 2e-6, key
 
 
+def test_gate_gradients_behind_strong_gates():
+    """Strong gates on every token: their gradients are small against the terms that meet in them, and as exact as the
+    other gradients (bound: five fp32 roundings)."""
+    inp = _case(69, [700, 200], 2, 128, 128, "fp32", 2, gate_kind="strong", eta=0.003)
+    got = binding.run_inputs_bwd(inp)
+    ref = parity.oracle_all(inp, bwd=True, gpu_masks=got["projection_masks"])
+    for key in ("dq", "dk", "dv", "dbeta", "dgate"):
+        assert parity.err(got[key], ref[key], norm="l2") <= 6e-7, key
+
+
 def test_forward_alone_and_recomputed_residuals():
     inp = _case(71, [100, 100], 2, 128, 128, "fp32", 2, dense_B=2)
     f = binding.run_inputs_fwd(inp)
