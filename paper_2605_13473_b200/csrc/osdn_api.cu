@@ -206,7 +206,7 @@ int osdn_bwd(const osdn_params* p, const void* q, const void* k, const void* v, 
 size_t osdn_kda_workspace_bytes(const osdn_params* p, int need_bwd)
 {
     if (validate(p) != OSDN_OK || p->apf_mode == OSDN_APF_ALIAS_GATE) return 0;
-    const WsLayout L = make_layout(*p, need_bwd != 0);
+    const WsLayout L = make_layout(*p, need_bwd != 0, true);
     return align_up(L.total, 256) + kda_extra_bytes(*p, L, need_bwd != 0);
 }
 
@@ -226,7 +226,7 @@ int osdn_kda_fwd(const osdn_params* p, const void* q, const void* k, const void*
         if (x && !aligned16(x)) return OSDN_MISALIGNED;
     if (reinterpret_cast<uintptr_t>(workspace) & 255u) return OSDN_MISALIGNED;
     const bool save = (p->flags & OSDN_FLAG_SAVE_RESIDUALS) != 0;
-    const WsLayout L = make_layout(*p, save);
+    const WsLayout L = make_layout(*p, save, true);
     if (workspace_bytes < align_up(L.total, 256) + kda_extra_bytes(*p, L, save)) return OSDN_WORKSPACE_TOO_SMALL;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     Pointers a{};
@@ -257,7 +257,7 @@ int osdn_kda_bwd(const osdn_params* p, const void* q, const void* k, const void*
     for (const void* x : ptrs)
         if (x && !aligned16(x)) return OSDN_MISALIGNED;
     if (reinterpret_cast<uintptr_t>(workspace) & 255u) return OSDN_MISALIGNED;
-    const WsLayout L = make_layout(*p, true);
+    const WsLayout L = make_layout(*p, true, true);
     if (workspace_bytes < align_up(L.total, 256) + kda_extra_bytes(*p, L, true)) return OSDN_WORKSPACE_TOO_SMALL;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     const Hyper hy = make_hyper(*p);

@@ -67,19 +67,19 @@ struct WsLayout {
     size_t pmask;       // [T,H,32]       u32   projection pass masks of processed tokens: word of lane l,
                         //                      bit r = coordinate (K/32) l + r passes gradient    (save only)
     size_t dtraj;       // [T,H,K]        f32   d_t of processed tokens                      (save only)
+    // CUDA-core family.  The tensor-core family lays its own regions over these, from ktil on, and needs less.
     size_t ktil;        // [T,H,K]        f32   write keys
-    size_t Tm;          // [NT,H,64,64]   f32   UT inverse
+    size_t Sn;          // [NT,H,V,K]     f32   state at chunk start (in ktil's place where no backward will ask for that)
     size_t P;           // [NT,H,64,64]   f32   masked, decayed q.ktil scores
     size_t W;           // [NT,H,64,K]    f32
-    size_t U;           // [NT,H,64,V]    f32
-    size_t dU;          // [NT,H,64,V]    f32   chunk update (new values)
-    size_t Sn;          // [NT,H,V,K]     f32   state at chunk start
-    // CUDA-core family only
-    size_t R;           // [NT,H,64,64]   f32   masked, decayed k.ktil scores (A without beta)
+    size_t dU;          // [NT,H,64,V]    f32   U, then the chunk update (new values) in its place
     size_t Ktr;         // [NT,H,64,K]    f32   write keys decayed to the chunk's end
-    size_t Qg;          // [NT,H,64,K]    f32   queries decayed from the chunk's start
-    size_t gC;          // [NT,H,K]       f32   decay of the whole chunk
+    size_t gam;         // [NT,H,64]      f32   scalar gate: decay from the chunk's start to each token
+    size_t Qg;          // [NT,H,64,K]    f32   channel gate: queries decayed from the chunk's start
+    size_t gC;          // [NT,H,K]       f32   channel gate: decay of the whole chunk
     // backward only
+    size_t Tm;          // [NT,H,64,64]   f32   UT inverse
+    size_t R;           // [NT,H,64,64]   f32   masked, decayed k.ktil scores (A without beta)
     size_t ddU;         // [NT,H,64,V]    f32
     size_t dSn;         // [NT,H,V,K]     f32   state cotangent at chunk end
     size_t dktil;       // [T,H,K]        f32
@@ -92,7 +92,10 @@ struct WsLayout {
 
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
-inline WsLayout make_layout(const osdn_params& p, bool need_bwd)
+// channel_gate: the layout of the osdn_kda calls.  The scalar-gate forward's is no larger than two 64 x 64 tiles, W, U, dU, ktil
+// and Sn side by side, whatever the shape: osdn_fwd_static has to take 8192 token-heads at K = V = 128, and every caller
+// holds these bytes.
+inline WsLayout make_layout(const osdn_params& p, bool need_bwd, bool channel_gate = false)
 {
     WsLayout L{};
     const int S = p.nseq > 0 ? p.nseq : p.B;
@@ -116,18 +119,25 @@ inline WsLayout make_layout(const osdn_params& p, bool need_bwd)
         L.pmask = take(4 * Ttot * H * 32);
         L.dtraj = take(4 * Ttot * H * K);
     }
-    L.ktil = take(4 * Ttot * H * K);
-    L.Tm = take(4 * NT * H * CH * CH);
+    if (need_bwd) {
+        L.ktil = take(4 * Ttot * H * K);
+        L.Sn = take(4 * NT * H * V * K);
+    } else {   // (a chunk is 64 tokens and V at least 64: Sn is the larger one)
+        L.ktil = L.Sn = take(4 * NT * H * V * K);
+    }
     L.P = take(4 * NT * H * CH * CH);
     L.W = take(4 * NT * H * CH * K);
-    L.U = take(4 * NT * H * CH * V);
     L.dU = take(4 * NT * H * CH * V);
-    L.Sn = take(4 * NT * H * V * K);
-    L.R = take(4 * NT * H * CH * CH);
     L.Ktr = take(4 * NT * H * CH * K);
-    L.Qg = take(4 * NT * H * CH * K);
-    L.gC = take(4 * NT * H * K);
+    if (channel_gate) {
+        L.Qg = take(4 * NT * H * CH * K);
+        L.gC = take(4 * NT * H * K);
+    } else {
+        L.gam = take(4 * NT * H * CH);
+    }
     if (need_bwd) {
+        L.Tm = take(4 * NT * H * CH * CH);
+        L.R = take(4 * NT * H * CH * CH);
         L.ddU = take(4 * NT * H * CH * V);
         L.dSn = take(4 * NT * H * V * K);
         L.dktil = take(4 * Ttot * H * K);

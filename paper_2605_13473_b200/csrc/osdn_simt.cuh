@@ -3,6 +3,7 @@
 // that the chains and the output do not know which gate it is:
 //   Ktr = rho (.) ktil   (rho_i = exp(G_C - G_i), what a write still counts for at the chunk's end)
 //   Qg  = gamma (.) q    (gamma_i = exp(G_i));   gC = exp(G_C), one value per key channel
+// (with a scalar gate Qg is not written: its readers scale q by gamma, and gC is gamma's last value)
 //   W = T diag(beta) (gamma (.) K),  U = T diag(beta) V,  P_ij = sum_c q_ic ktil_jc exp(G_ic - G_jc)
 //   dU = U - W S^T,  S+ = S diag(gC) + dU^T Ktr,  O = scale (Qg S^T + P dU)
 // G is the inclusive prefix of the log-gates inside the chunk.
@@ -249,8 +250,9 @@ struct ChunkArgs {
     const void *q, *k, *v;
     const float *beta, *gate;        // gate: [T,H], channel gate [T,H,K]
     const float* ktil;
-    float *Tm, *P, *R, *W, *U;       // R: the Gram with its gate factors, A without beta
-    float *Ktr, *Qg, *gC, *G;        // G: channel gate only, [tile][2][64][K], the prefix's high and low parts
+    float *Tm, *P, *R, *W, *U;       // R: the Gram with its gate factors, A without beta.  Tm, R: null without a backward
+    float *gam;                      // scalar gate only
+    float *Ktr, *Qg, *gC, *G;        // Qg, gC: channel gate only.  G: channel gate only, [tile][2][64][K], the prefix's high and low parts
     // output pass, backward
     void* out;
     const void* dout;
@@ -424,13 +426,14 @@ __global__ void __launch_bounds__(CL_NT, LocalFwd<T, K, V, CG>::MIN_CTAS) chunk_
     } else {
         load_gates(gv, a.gate, a.beta, tok0, len, H, h);
         __syncthreads();
-        if (threadIdx.x < K) a.gC[tile * K + threadIdx.x] = gv.gam[CH - 1];
+        if (threadIdx.x < CH) a.gam[tile * CH + threadIdx.x] = gv.gam[threadIdx.x];
     }
     for (int e = threadIdx.x; e < CH * K / 4; e += CL_NT) {
         const int i = e / (K / 4), n = e % (K / 4) * 4;
         const size_t g = tile * CH * K + e * 4;
-        const float4 q = ld4(sQ + i * LD + n), kt = ld4(sKt + i * LD + n);
+        const float4 kt = ld4(sKt + i * LD + n);
         if constexpr (CG) {
+            const float4 q = ld4(sQ + i * LD + n);
             const float4 G = ld4(sG + i * LD + n), gl = ld4(sL + i * LD + n), eg = exp_sum(G, gl), qg = eg * q;
             if (a.G) {
                 st4(a.G + tile * 2 * CH * K + e * 4, G);
@@ -442,7 +445,6 @@ __global__ void __launch_bounds__(CL_NT, LocalFwd<T, K, V, CG>::MIN_CTAS) chunk_
             st4(sK + i * LD + n, eg * ld4(sK + i * LD + n));
             if (safe) st4(sKt + i * LD + n, exp_sum(-1.f * G, -1.f * gl) * kt);
         } else {
-            st4(a.Qg + g, gv.gam[i] * q);
             st4(a.Ktr + g, gv.rho[i] * kt);
         }
     }
@@ -485,14 +487,16 @@ __global__ void __launch_bounds__(CL_NT, LocalFwd<T, K, V, CG>::MIN_CTAS) chunk_
                 const int m = row_of(l, i), n = col_of<true>(l, j);
                 float g = n < m || (n == m && grp == 1) ? acc[i][j] : 0.f;
                 if constexpr (!CG) g *= expf(fminf(gv.G[m] - gv.G[n], 0.f));
-                out[m * CH + n] = g;
+                if (grp == 1 || a.R) out[m * CH + n] = g;
                 if (grp == 0) sA[m * LC + n] = gv.beta[m] * g;
             }
     }
     __syncthreads();
     ut_inverse_64(sA, sT, tmp);
-    float* Tg = a.Tm + tile * CH * CH;
-    for (int e = threadIdx.x; e < CH * CH / 4; e += CL_NT) st4(Tg + e * 4, ld4(sT + (e / 16) * LC + (e % 16) * 4));
+    if (a.Tm) {
+        float* Tg = a.Tm + tile * CH * CH;
+        for (int e = threadIdx.x; e < CH * CH / 4; e += CL_NT) st4(Tg + e * 4, ld4(sT + (e / 16) * LC + (e % 16) * 4));
+    }
 
     // W = T diag(beta) (gamma K) ; U = T diag(beta) V.  T is lower triangular: rows of a warp end at 8 w + 8.
     const int jend = (l.tm & ~1) * 4 + 8;
@@ -523,7 +527,19 @@ __global__ void __launch_bounds__(CL_NT, LocalFwd<T, K, V, CG>::MIN_CTAS) chunk_
 // O = scale (Qg S_n^T + P dU), one tile per CTA once the chain has left S_n and dU: the output is off the
 // sequential path.
 template <int K, int V> constexpr size_t output_smem() { return sizeof(float) * ((CH + V) * (K + 4) + CH * LC); }
-template <typename T, int K, int V>
+// gamma (.) q of a tile into shared memory.
+template <typename T, int K, bool CG, int LD, int NT> __device__ __forceinline__ void load_gated_q(float* dst, const ChunkArgs& a, size_t tile, int tok0, int len, int h)
+{
+    const Rows<T, K> q = rows_of<T, K>(a.q, tok0, len, a.H, h);
+#pragma unroll 4
+    for (int e = threadIdx.x; e < CH * K / 4; e += NT) {
+        const int i = e / (K / 4), n = e % (K / 4) * 4;
+        if constexpr (CG) st4(dst + i * LD + n, ld4(a.Qg + tile * CH * K + e * 4));
+        else st4(dst + i * LD + n, a.gam[tile * CH + i] * q(i, n));
+    }
+}
+
+template <typename T, int K, int V, bool CG>
 __global__ void __launch_bounds__(256) output_kernel(ChunkArgs a)
 {
     extern __shared__ __align__(16) float sm[];
@@ -538,13 +554,11 @@ __global__ void __launch_bounds__(256) output_kernel(ChunkArgs a)
     const size_t tile = (size_t)c * H + h;
     const Lane l{(int)threadIdx.x >> 4, (int)threadIdx.x & 15};
     const float* S = a.Sn + tile * V * K;
-    const float* Q = a.Qg + tile * CH * K;
     const float* P = a.P + tile * CH * CH;
     const float* dU = a.dU + tile * CH * V;
 #pragma unroll 8
     for (int e = threadIdx.x; e < V * K / 4; e += NT) st4(sS + e / (K / 4) * LD + e % (K / 4) * 4, ld4(S + e * 4));
-#pragma unroll 4
-    for (int e = threadIdx.x; e < CH * K / 4; e += NT) st4(sQ + e / (K / 4) * LD + e % (K / 4) * 4, ld4(Q + e * 4));
+    load_gated_q<T, K, CG, LD, NT>(sQ, a, tile, tok0, len, h);
 #pragma unroll 4
     for (int e = threadIdx.x; e < CH * CH / 4; e += NT) st4(sP + e / 16 * LC + e % 16 * 4, ld4(P + e * 4));
     float4 u[CH * V / 4 / NT];
@@ -586,7 +600,7 @@ __global__ void __launch_bounds__(256) output_kernel(ChunkArgs a)
 // What the reverse chain's step does not need the state cotangent for, tile-parallel:
 //   ddU0 = scale P^T dO  (into ddU)   and   G0 = scale dO^T Qg  (into dSn, which the chain then overwrites)
 template <int K, int V> constexpr size_t pre_bwd_smem() { return sizeof(float) * (CH * CH + CH * V + CH * K); }
-template <typename T, int K, int V>
+template <typename T, int K, int V, bool CG>
 __global__ void __launch_bounds__(256) pre_bwd_kernel(ChunkArgs a)
 {
     extern __shared__ __align__(16) float sm[];
@@ -601,12 +615,10 @@ __global__ void __launch_bounds__(256) pre_bwd_kernel(ChunkArgs a)
     const size_t tile = (size_t)c * H + h;
     const Lane l{(int)threadIdx.x >> 4, (int)threadIdx.x & 15};
     const float* P = a.P + tile * CH * CH;
-    const float* Q = a.Qg + tile * CH * K;
     const float s = a.hy.scale;
 #pragma unroll 4
     for (int e = threadIdx.x; e < CH * CH / 4; e += NT) st4(sP + e * 4, ld4(P + e * 4));
-#pragma unroll 4
-    for (int e = threadIdx.x; e < CH * K / 4; e += NT) st4(sQ + e * 4, ld4(Q + e * 4));
+    load_gated_q<T, K, CG, K, NT>(sQ, a, tile, tok0, len, h);
     load_tile<T, V, NT>(sO, V, static_cast<const T*>(a.dout), tok0, len, H, h);
     __syncthreads();
     {
@@ -646,7 +658,8 @@ __global__ void __launch_bounds__(256) pre_bwd_kernel(ChunkArgs a)
 struct ChainArgs {
     int H;
     Table tab;
-    const float *X, *Y, *D0, *G0, *gC, *S0;   // G0, S0 nullable
+    const float *X, *Y, *D0, *G0, *S0;        // G0, S0 nullable
+    const float *gC, *gam;                    // decay of a chunk: per channel (channel gate), or gam's last value
     float *D, *Sall, *Sfin;                   // Sall: S before every chunk of the walk; Sfin nullable
     int* status;
 };
@@ -740,7 +753,7 @@ template <int K> struct NarrowShared {
     uint64_t full[2];
 };
 
-template <int K, int V, bool BWD>
+template <int K, int V, bool BWD, bool CG>
 __global__ void __launch_bounds__(CNT) chain_narrow_kernel(ChainArgs a)
 {
     extern __shared__ __align__(16) float sm[];
@@ -773,7 +786,12 @@ __global__ void __launch_bounds__(CNT) chain_narrow_kernel(ChainArgs a)
         const Stage<K>& g = s.stage[j & 1];
         float g0[PER] = {}, gc[PER];
         if constexpr (BWD) ldn(g0, a.G0 + (tile * V + v0) * K + t * PER);
-        ldn(gc, a.gC + tile * K + sk);
+        if constexpr (CG) ldn(gc, a.gC + tile * K + sk);
+        else {
+            const float g1 = a.gam[tile * CH + CH - 1];
+#pragma unroll
+            for (int x = 0; x < PER; ++x) gc[x] = g1;
+        }
         stn(s.S + sv * LD + sk, S);
         if (j + 1 < w.n) fetch_stage<K>(s.stage[(j + 1) & 1], a, tile_of(j + 1), &s.full[(j + 1) & 1]);
         const bool ok = umma::mbar_wait(&s.full[j & 1], (j >> 1) & 1, a.status, CODE_SIMT_RING);
@@ -835,7 +853,7 @@ template <int K> struct WideShared {
     uint64_t full[2];
 };
 
-template <int K, int V, bool BWD>
+template <int K, int V, bool BWD, bool CG>
 __global__ void __launch_bounds__(K / 64 * 256) chain_wide_kernel(ChainArgs a)
 {
     extern __shared__ __align__(16) float sm[];
@@ -867,7 +885,9 @@ __global__ void __launch_bounds__(K / 64 * 256) chain_wide_kernel(ChainArgs a)
         float* sn = a.Sall + (tile * V + v0) * K;
         if (j + 1 < w.n) fetch_stage<K>(s.stage[(j + 1) & 1], a, tile_of(j + 1), &s.full[(j + 1) & 1]);
         float4 g0[4], d0[CH * WS / 4 / NT];
-        const float4 gc = ld4(a.gC + tile * K + k_own);
+        float4 gc;
+        if constexpr (CG) gc = ld4(a.gC + tile * K + k_own);
+        else gc.x = gc.y = gc.z = gc.w = a.gam[tile * CH + CH - 1];
         if constexpr (BWD)
 #pragma unroll
             for (int i = 0; i < 4; ++i) g0[i] = ld4(a.G0 + (tile * V + v0 + l.tm * 4 + i) * K + k_own);
@@ -1366,17 +1386,17 @@ template <typename F> bool set_smem(F* kernel, size_t bytes)
 // Narrow or wide slices: whichever walk is expected to end first.  A step of a wide slice (eight times the rows)
 // takes about WIDE_STEP times a narrow one's; what decides is how many waves of CTAs each cut makes.
 constexpr int WIDE_STEP_TENTHS = 25;
-template <int K, int V, bool BWD> int launch_chain(const ChainArgs& ch, int chains, cudaStream_t st)
+template <int K, int V, bool BWD, bool CG> int launch_chain(const ChainArgs& ch, int chains, cudaStream_t st)
 {
     constexpr int PER_SM = K == 64 ? 2 : 1, SLOTS = 148 * PER_SM;
     const long narrow = ((long)chains * (V / VS) + SLOTS - 1) / SLOTS, wide = ((long)chains * (V / WS) + SLOTS - 1) / SLOTS;
     stage_mark(st, BWD ? "chain_bwd" : "chain_fwd");
     if (narrow * 10 <= wide * WIDE_STEP_TENTHS) {
-        if (!set_smem(chain_narrow_kernel<K, V, BWD>, sizeof(NarrowShared<K>))) return -1;
-        chain_narrow_kernel<K, V, BWD><<<dim3(chains, V / VS), CNT, sizeof(NarrowShared<K>), st>>>(ch);
+        if (!set_smem(chain_narrow_kernel<K, V, BWD, CG>, sizeof(NarrowShared<K>))) return -1;
+        chain_narrow_kernel<K, V, BWD, CG><<<dim3(chains, V / VS), CNT, sizeof(NarrowShared<K>), st>>>(ch);
     } else {
-        if (!set_smem(chain_wide_kernel<K, V, BWD>, sizeof(WideShared<K>))) return -1;
-        chain_wide_kernel<K, V, BWD><<<dim3(chains, V / WS), K / 64 * 256, sizeof(WideShared<K>), st>>>(ch);
+        if (!set_smem(chain_wide_kernel<K, V, BWD, CG>, sizeof(WideShared<K>))) return -1;
+        chain_wide_kernel<K, V, BWD, CG><<<dim3(chains, V / WS), K / 64 * 256, sizeof(WideShared<K>), st>>>(ch);
     }
     return 1;
 }
@@ -1384,11 +1404,11 @@ template <int K, int V, bool BWD> int launch_chain(const ChainArgs& ch, int chai
 inline ChunkArgs chunk_args(const osdn_params& p, const Hyper& hy, const WsLayout& L, void* ws, const Pointers& a, float* G)
 {
     char* w = static_cast<char*>(ws);
-    auto F = [&](size_t off) { return reinterpret_cast<float*>(w + off); };
+    auto F = [&](size_t off) { return off ? reinterpret_cast<float*>(w + off) : nullptr; };   // (none of these regions is the first)
     ChunkArgs c{};
     c.H = p.H; c.tab = carve_table(ws, L); c.q = a.q; c.k = a.k; c.v = a.v; c.beta = a.beta; c.gate = a.gate;
-    c.ktil = F(L.ktil); c.Tm = F(L.Tm); c.P = F(L.P); c.R = F(L.R); c.W = F(L.W); c.U = F(L.U);
-    c.Ktr = F(L.Ktr); c.Qg = F(L.Qg); c.gC = F(L.gC); c.G = G; c.Sn = F(L.Sn); c.dU = F(L.dU); c.hy = hy;
+    c.ktil = F(L.ktil); c.Tm = F(L.Tm); c.P = F(L.P); c.R = F(L.R); c.W = F(L.W); c.U = F(L.dU);
+    c.Ktr = F(L.Ktr); c.Qg = F(L.Qg); c.gC = F(L.gC); c.gam = F(L.gam); c.G = G; c.Sn = F(L.Sn); c.dU = F(L.dU); c.hy = hy;
     return c;
 }
 
@@ -1404,13 +1424,13 @@ int chunk_forward(const osdn_params& p, const Hyper& hy, const WsLayout& L, void
     stage_mark(st, "chunk_local_fwd");
     chunk_local_fwd_kernel<T, K, V, CG><<<tiles, CL_NT, LF::SMEM, st>>>(c);
     ChainArgs ch{};
-    ch.H = p.H; ch.tab = c.tab; ch.X = c.W; ch.Y = c.Ktr; ch.D0 = c.U; ch.gC = c.gC; ch.S0 = a.init_state;
+    ch.H = p.H; ch.tab = c.tab; ch.X = c.W; ch.Y = c.Ktr; ch.D0 = c.U; ch.gC = c.gC; ch.gam = c.gam; ch.S0 = a.init_state;
     ch.D = const_cast<float*>(c.dU); ch.Sall = const_cast<float*>(c.Sn); ch.Sfin = a.final_state;
     ch.status = reinterpret_cast<int*>(static_cast<char*>(ws) + L.status);
-    if (launch_chain<K, V, false>(ch, L.S * p.H, st) < 0) return -1;
-    if (!set_smem(output_kernel<T, K, V>, output_smem<K, V>())) return -1;
+    if (launch_chain<K, V, false, CG>(ch, L.S * p.H, st) < 0) return -1;
+    if (!set_smem(output_kernel<T, K, V, CG>, output_smem<K, V>())) return -1;
     stage_mark(st, "chunk_output");
-    output_kernel<T, K, V><<<tiles, 256, output_smem<K, V>(), st>>>(c);
+    output_kernel<T, K, V, CG><<<tiles, 256, output_smem<K, V>(), st>>>(c);
     return cudaGetLastError() == cudaSuccess ? 3 : -1;
 }
 
@@ -1424,14 +1444,14 @@ int chunk_backward(const osdn_params& p, const Hyper& hy, const WsLayout& L, voi
     c.dout = a.dout; c.ddU = F(L.ddU); c.dSn = F(L.dSn); c.dktil = F(L.dktil); c.dkread = F(L.dkread);
     c.dq = a.dq; c.dv = a.dv; c.dbeta = a.dbeta; c.dgate = a.dgate;
     const dim3 tiles(L.NTmax, p.H);
-    if (!set_smem(pre_bwd_kernel<T, K, V>, pre_bwd_smem<K, V>())) return -1;
+    if (!set_smem(pre_bwd_kernel<T, K, V, CG>, pre_bwd_smem<K, V>())) return -1;
     stage_mark(st, "chunk_pre_bwd");
-    pre_bwd_kernel<T, K, V><<<tiles, 256, pre_bwd_smem<K, V>(), st>>>(c);
+    pre_bwd_kernel<T, K, V, CG><<<tiles, 256, pre_bwd_smem<K, V>(), st>>>(c);
     ChainArgs ch{};
-    ch.H = p.H; ch.tab = c.tab; ch.X = c.Ktr; ch.Y = c.W; ch.D0 = c.ddU; ch.G0 = c.dSn; ch.gC = c.gC; ch.S0 = a.dfinal_state;
+    ch.H = p.H; ch.tab = c.tab; ch.X = c.Ktr; ch.Y = c.W; ch.D0 = c.ddU; ch.G0 = c.dSn; ch.gC = c.gC; ch.gam = c.gam; ch.S0 = a.dfinal_state;
     ch.D = c.ddU; ch.Sall = c.dSn; ch.Sfin = a.dinit_state;
     ch.status = reinterpret_cast<int*>(w + L.status);
-    if (launch_chain<K, V, true>(ch, L.S * p.H, st) < 0) return -1;
+    if (launch_chain<K, V, true, CG>(ch, L.S * p.H, st) < 0) return -1;
     if (!set_smem(chunk_local_bwd_kernel<T, K, V, CG>, local_bwd_smem<K>())) return -1;
     stage_mark(st, "chunk_local_bwd");
     chunk_local_bwd_kernel<T, K, V, CG><<<tiles, CL_NT, local_bwd_smem<K>(), st>>>(c);

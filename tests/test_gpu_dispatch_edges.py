@@ -82,6 +82,22 @@ def test_lists_of_processed_tokens(lens, shift):
     _all_outputs(inp, f"lists_{len(lens)}_{shift}")
 
 
+@pytest.mark.parametrize("io,flags", [("bf16", 0), ("fp32", 0), ("bf16", binding.FLAG_FORCE_SIMT)])
+def test_built_in_scratch_takes_8192_token_heads(io, flags):
+    """osdn_fwd_static at 1024 tokens, 8 heads of 128, in every kernel family: the results of osdn_fwd, bit for bit."""
+    inp = draw("static", 7700, [1024], 8, 128, 128, io, dense_B=1, with_state=True)
+    b = binding.DeviceBundle(inp, DEV, need_bwd=False, flags=flags)
+    b.fwd()
+    want = [b.out.clone(), b.final_state.clone(), b.precond_out.clone()]
+    for x in (b.out, b.final_state, b.precond_out):
+        x.zero_()
+    rc = binding.osdn_fwd_static(b.params, b.q, b.k, b.v, b.beta, b.gate, None, b.init_state, b.precond_in, b.out, b.final_state, b.precond_out)
+    torch.cuda.synchronize()
+    assert rc == 0 and binding.osdn_read_static_status() == 0
+    for x, y in zip(want, (b.out, b.final_state, b.precond_out)):
+        assert torch.equal(x, y)
+
+
 @pytest.mark.parametrize("io,K", [("fp32", 64), ("fp32", 128), ("bf16", 64)])
 def test_chains_in_wide_slices(io, K):
     """Enough chains for the wide slices of the CUDA-core state chains (the other cases have few and take the narrow ones)."""

@@ -46,6 +46,27 @@ def test_workspace_sizes_and_validation(lib):
     assert osdn.osdn_workspace_bytes(q, False) == 0
 
 
+@pytest.mark.parametrize("K", [64, 128])
+@pytest.mark.parametrize("V", [64, 128])
+def test_forward_workspace_has_a_ceiling(lib, K, V):
+    """The forward's scratch is at most the write keys, two 64 x 64 tiles, W, U, dU and the chunk states side by side (with
+    two scalars per token-head, the flags and the table), whatever the shape: what fits the built-in scratch stays accepted."""
+    up = lambda n: -(-n // 256) * 256
+    for B, T, nseq in ((1, 1, 0), (1, 64, 0), (3, 65, 0), (25, 1, 0), (1, 1024, 0), (8, 2048, 0), (1, 1024, 9)):
+        for H in (1, 3, 8):
+            for io in ("fp32", "bf16"):
+                p = osdn.make_params(B=B, T=T, H=H, K=K, V=V, io_dtype=io, hyper=OsdnHyper())
+                if nseq:
+                    p.nseq, p.cu_seqlens = nseq, 0x1000   # never dereferenced
+                S, n = nseq or B, B * T
+                nt = n // 64 + S if nseq else B * (-(-T // 64))
+                regions = [256, 4 * (4 * S + 1 + 6 * nt + 4), 4 * n * H, 4 * n * H, 8 * nt * H, 4 * n * H * K] + [4 * nt * H * 4096] * 2
+                regions += [4 * nt * H * 64 * K] + [4 * nt * H * 64 * V] * 2 + [4 * nt * H * K * V]
+                assert osdn.osdn_workspace_bytes(p, False) <= sum(map(up, regions)), (B, T, H, io, nseq)
+    p = osdn.make_params(B=1, T=1024, H=8, K=128, V=128, io_dtype="bf16", hyper=OsdnHyper())
+    assert osdn.osdn_workspace_bytes(p, False) <= binding.STATIC_SCRATCH_BYTES
+
+
 def test_calls_reject_bad_arguments_before_any_launch(lib):
     hy = OsdnHyper()
     p = osdn.make_params(B=1, T=64, H=1, K=64, V=64, io_dtype="fp32", hyper=hy)
