@@ -186,6 +186,17 @@ inline P1Regions carve_p1(void* ws, const WsLayout& L)
     return r;
 }
 
+inline int num_sms()
+{
+    static int n = 0;
+    if (!n) {
+        int dev = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0)
+            n = 148;
+    }
+    return n;
+}
+
 // Programmatic dependent launch: a kernel launched by launch_after may become resident while the kernel before it in the
 // stream still runs, and waits in pdl_wait, before its first access to anything that kernel or an earlier one writes,
 // until that kernel is complete (launch latency and prologue then run under its tail).  Every kernel of a call waits, so

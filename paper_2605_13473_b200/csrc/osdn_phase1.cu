@@ -93,6 +93,29 @@ template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile(
 // ---------------------------------------------------------------------------------------------
 // plain streaming sweep (the stand-alone preconditioner update; no workspace)
 // ---------------------------------------------------------------------------------------------
+// The coordinate the recurrence runs in, y = (d - lo) / w.  With c' = c / w a step is
+//   y' = project(rho y + (c' k^2 + (rho - 1) lo / w)),   c' = e' - a2 <y, k^2>,   e' = (e - a2 lo sum k^2) / w.
+//   P1_SAT    a box of ordinary width above zero: lo = d_min, w = d_max - d_min; the projection is the saturation of a
+//             multiply-add.  d - d_min is at most d there, so that a rounding of y is none larger than one of d.
+//   P1_PLAIN  everything else: no projection; a box that is open, without width, or of a width that 1 / w could not take
+//             (w = 1); a negative lower edge, below which d - d_min would be larger than d and cost its last bits (lo = 0).
+// Where lo = d_min the lower face is y = 0.  Core, finishing warps and the walk use the same functions, hence the same
+// values.
+enum P1Mode { P1_SAT, P1_PLAIN };
+struct P1Coord {           // made by the host: in the kernels these are constants, not registers and a division
+    float lo, w, iw, k0;   // k0 = lo / w
+    P1Mode mode;
+    bool face;             // y = 0 is the lower face, tokens may be skipped there
+};
+inline P1Coord p1_coord(const Hyper& hy)
+{
+    const bool face = hy.clamp && hy.d_min >= 0.f && hy.d_min <= 1e30f;
+    const float width = hy.d_max - hy.d_min;
+    const P1Mode mode = face && width >= 1e-12f && width <= 1e12f ? P1_SAT : P1_PLAIN;
+    const float lo = face ? hy.d_min : 0.f, w = mode == P1_SAT ? width : 1.0f, iw = 1.0f / w;
+    return {lo, w, iw, lo * iw, mode, face};
+}
+
 struct P1Args {
     int S, H, T_dense;
     const int* cu;
@@ -103,6 +126,7 @@ struct P1Args {
     float* ratio;      // nullable: residual ratio q_t per token-head
     float* log_sum;    // nullable: sum_t log q_t per chain
     Hyper hy;
+    P1Coord q;
 };
 
 // ---------------------------------------------------------------------------------------------
@@ -118,6 +142,7 @@ struct P1Fwd {
     P1Regions r;
     int save;
     Hyper hy;
+    P1Coord q;
     int* status;         // device status word (bounded waits of the rings report here)
     ClearList clear;
 };
@@ -316,8 +341,9 @@ constexpr int SCAN_CHUNKS = 128;                    // chunks whose words warp 0
 // The forward's core warps own two coordinates a lane and have a scheduler each, 0 and 1; the helpers sit on schedulers
 // 2 and 3 (warp numbers modulo four), the warps in between leave at once.  Beside helpers on its own scheduler a core of
 // four warps took 4700 cycles for a block instead of 2900.
-template <int K> struct FwdPipe {
+template <int K, bool MANY> struct FwdPipe {
     static constexpr int CORE = K / 64, FETCH0 = 2, FETCH = 2, FINISH0 = 4, FINISH = 4, THREADS = 384, ACTIVE = (CORE + FETCH + FINISH) * 32;
+    static constexpr int CTAS = 1, RING_BYTES = 216 * 1024;
     // the role number of a hardware warp: core 0 .., fetch 2, 3, finish 4 .. 7; -1: idle
     __device__ static __forceinline__ int role(int warp)
     {
@@ -325,15 +351,26 @@ template <int K> struct FwdPipe {
         return sched < 2 ? (row == 0 && warp < CORE ? warp : -1) : row * 2 + sched;
     }
 };
+// More chains than SMs: one fetching and one finishing warp and a short ring, so that three chains share an SM (one to an
+// SM, they queue for it: the moving stand-alone update of 1024 tokens, 74 us for 64 chains, took 203 us for 300 and now
+// takes 118; the forward's pass 265 -> 160 us).
+template <int K> struct FwdPipe<K, true> {
+    static constexpr int CORE = K / 64, FETCH0 = CORE, FETCH = 1, FINISH0 = CORE + 1, FINISH = 1, THREADS = (CORE + 2) * 32, ACTIVE = THREADS;
+    static constexpr int CTAS = 3, RING_BYTES = 72 * 1024;
+    __device__ static __forceinline__ int role(int warp) { return warp; }
+};
 template <int K> struct Pipe {
     static constexpr int CORE = K / 32, FETCH0 = CORE, FETCH = 2, FINISH0 = CORE + FETCH, FINISH = 4, WARPS = FINISH0 + FINISH, THREADS = WARPS * 32;
 };
 constexpr int RING_MAX = 8;
-static_assert(RING_MAX / 2 % Pipe<128>::FETCH == 0 && RING_MAX / 2 % Pipe<128>::FINISH == 0, "a buffer belongs to one fetching and one finishing warp");
-// Buffers of the given size that fit the CTA's shared memory beside the rest: RING_MAX or half of it.  Both are multiples
-// of the numbers of fetching and of finishing warps, so that all uses of a buffer are the same warps' and follow one
-// another in order (a wait tells a barrier's phases apart by their parity only).
-constexpr int ring_depth(size_t bytes) { return bytes * RING_MAX <= 216 * 1024 ? RING_MAX : RING_MAX / 2; }
+// Buffers of the given size that fit `room` bytes: RING_MAX or half of it, or any number with one helper of each kind.  The
+// depth is a multiple of the numbers of fetching and of finishing warps, so that all uses of a buffer are the same warps'
+// and follow one another in order (a wait tells a barrier's phases apart by their parity only).
+constexpr int ring_depth(size_t bytes, size_t room, int helpers)
+{
+    if (helpers == 1) return bytes * 4 <= room ? 4 : (int)(room / bytes);
+    return bytes * RING_MAX <= room ? RING_MAX : RING_MAX / 2;
+}
 
 __device__ __forceinline__ void p1_mbar_init(uint64_t* b, int count)
 {
@@ -395,8 +432,10 @@ template <typename TI, int K, bool VEC> struct PipeBuf {
     int n;                                  // core: tokens of the block that stand
     alignas(16) float rv[VEC ? PB : 1][VEC ? K : 1];   // vector retention: l_t, then (core) exp(l_t)
 };
-template <typename TI, int K, bool VEC> struct PipeShared {
-    static constexpr int CW = K / 64, PN = ring_depth(sizeof(PipeBuf<TI, K, VEC>));
+template <typename TI, int K, bool VEC, bool MANY> struct PipeShared {
+    using P = FwdPipe<K, MANY>;
+    static constexpr int CW = P::CORE, PN = ring_depth(sizeof(PipeBuf<TI, K, VEC>), P::RING_BYTES, P::FINISH);
+    static_assert(PN >= 2 && PN % P::FETCH == 0 && PN % P::FINISH == 0, "a buffer belongs to one fetching and one finishing warp");
     PipeBuf<TI, K, VEC> buf[PN];
     float y[K];                             // between two lists
     float c[CW][PB];                        // a core warp's c' of the round
@@ -409,43 +448,15 @@ template <typename TI, int K, bool VEC> struct PipeShared {
     PipeBars bars;
 };
 
-// The coordinate the recurrence runs in, y = (d - lo) / w.  With c' = c / w a step is
-//   y' = project(rho y + (c' k^2 + (rho - 1) lo / w)),   c' = e' - a2 <y, k^2>,   e' = (e - a2 lo sum k^2) / w.
-//   P1_SAT    a box of ordinary width above zero: lo = d_min, w = d_max - d_min; the projection is the saturation of a
-//             multiply-add.  d - d_min is at most d there, so that a rounding of y is none larger than one of d.
-//   P1_PLAIN  everything else: no projection; a box that is open, without width, or of a width that 1 / w could not take
-//             (w = 1); a negative lower edge, below which d - d_min would be larger than d and cost its last bits (lo = 0).
-// Where lo = d_min the lower face is y = 0.  Core, finishing warps and the walk use the same functions, hence the same
-// values.
-enum P1Mode { P1_SAT, P1_PLAIN };
-struct P1Coord {
-    float lo, w, iw, k0;   // k0 = lo / w
-};
-// Whether y = 0 is the lower face, so that tokens may be skipped there.
-__device__ __forceinline__ bool p1_face(const Hyper& hy) { return hy.clamp && hy.d_min >= 0.f && hy.d_min <= 1e30f; }
-__device__ __forceinline__ P1Mode p1_mode(const Hyper& hy)
-{
-    const float w = hy.d_max - hy.d_min;
-    return p1_face(hy) && w >= 1e-12f && w <= 1e12f ? P1_SAT : P1_PLAIN;
-}
-__device__ __forceinline__ P1Coord p1_coord(const Hyper& hy)
-{
-    const float lo = p1_face(hy) ? hy.d_min : 0.f, w = p1_mode(hy) == P1_SAT ? hy.d_max - hy.d_min : 1.0f, iw = 1.0f / w;
-    return {lo, w, iw, lo * iw};
-}
 __device__ __forceinline__ float p1_y(float d, const P1Coord& q) { return __fmul_rn(d - q.lo, q.iw); }
 __device__ __forceinline__ float p1_d(float y, const P1Coord& q) { return fmaf(q.w, y, q.lo); }
 __device__ __forceinline__ float p1_off(float rho, const P1Coord& q) { return fmaf(rho, q.k0, -q.k0); }
 __device__ __forceinline__ float p1_raw(float y, float kap, float c, float rho, float off) { return fmaf(rho, y, fmaf(c, kap, off)); }
-template <P1Mode M> __device__ __forceinline__ float p1_project(float x, const Hyper& hy)
+template <P1Mode M> __device__ __forceinline__ float p1_project(float x, const Hyper& hy, const P1Coord& q)
 {
     if (M == P1_SAT) return __saturatef(x);
     if (!hy.clamp) return x;
-    return p1_face(hy) ? fminf(fmaxf(x, 0.f), hy.d_max - hy.d_min) : fminf(fmaxf(x, hy.d_min), hy.d_max);
-}
-__device__ __forceinline__ float p1_project(float x, P1Mode m, const Hyper& hy)
-{
-    return m == P1_SAT ? p1_project<P1_SAT>(x, hy) : p1_project<P1_PLAIN>(x, hy);
+    return q.face ? fminf(fmaxf(x, 0.f), hy.d_max - hy.d_min) : fminf(fmaxf(x, hy.d_min), hy.d_max);
 }
 // e', a2, max k^2, sum k^2 of a token
 __device__ __forceinline__ float4 p1_scalars(float sumk, float kmax, float beta, const Hyper& hy, const P1Coord& q)
@@ -479,11 +490,11 @@ __device__ __forceinline__ float2 load2(const __nv_bfloat16* p) { return __bfloa
 // One block by the core warps: y of this lane's coordinates goes through it (slots beyond its n tokens leave y alone).
 // r: <y, k^2> / sum k^2 of the latest token, the start of the next guess; rounds: all rounds so far.  Returns the tokens
 // that stand: n, or those before the first jump that d enters off the face (y is then its value there).
-template <typename TI, int K, bool VEC, P1Mode M>
-__device__ __forceinline__ int core_block(PipeShared<TI, K, VEC>& sh, PipeBuf<TI, K, VEC>& B, int n, float2& y, float& r, uint32_t& rounds,
+template <typename TI, int K, bool VEC, bool MANY, P1Mode M>
+__device__ __forceinline__ int core_block(PipeShared<TI, K, VEC, MANY>& sh, PipeBuf<TI, K, VEC>& B, int n, float2& y, float& r, uint32_t& rounds,
                                           const Hyper& hy, const P1Coord& q, int warp, int lane)
 {
-    constexpr int CW = FwdPipe<K>::CORE;
+    constexpr int CW = FwdPipe<K, MANY>::CORE;
     const int i = warp * 64 + lane * 2;   // this lane's coordinates: i, i + 1
     float ka[PB], kb[PB];
 #pragma unroll
@@ -517,7 +528,7 @@ __device__ __forceinline__ int core_block(PipeShared<TI, K, VEC>& sh, PipeBuf<TI
             rx *= x.x;
             ry *= x.y;
         }
-        return make_float2(p1_project<M>(p1_raw(v.x, kx, cj, rx, ox), hy), p1_project<M>(p1_raw(v.y, ky, cj, ry, oy), hy));
+        return make_float2(p1_project<M>(p1_raw(v.x, kx, cj, rx, ox), hy, q), p1_project<M>(p1_raw(v.y, ky, cj, ry, oy), hy, q));
     };
     for (int round = 0; round <= PB; ++round) {   // (round PB + 1 could change nothing)
         const uint32_t par = rounds++ & 1;
@@ -587,12 +598,12 @@ __device__ __forceinline__ int core_block(PipeShared<TI, K, VEC>& sh, PipeBuf<TI
     r = __shfl_sync(0xffffffffu, sum / fmaxf(sc.w, 1e-30f), n - 1);
     return stand;
 }
-template <typename TI, int K, bool VEC>
-__device__ __forceinline__ int core_block(PipeShared<TI, K, VEC>& sh, PipeBuf<TI, K, VEC>& B, int n, float2& y, float& r, uint32_t& rounds,
+template <typename TI, int K, bool VEC, bool MANY>
+__device__ __forceinline__ int core_block(PipeShared<TI, K, VEC, MANY>& sh, PipeBuf<TI, K, VEC>& B, int n, float2& y, float& r, uint32_t& rounds,
                                           const Hyper& hy, const P1Coord& q, int warp, int lane)
 {
-    if (p1_mode(hy) == P1_SAT) return core_block<TI, K, VEC, P1_SAT>(sh, B, n, y, r, rounds, hy, q, warp, lane);
-    return core_block<TI, K, VEC, P1_PLAIN>(sh, B, n, y, r, rounds, hy, q, warp, lane);
+    if (q.mode == P1_SAT) return core_block<TI, K, VEC, MANY, P1_SAT>(sh, B, n, y, r, rounds, hy, q, warp, lane);
+    return core_block<TI, K, VEC, MANY, P1_PLAIN>(sh, B, n, y, r, rounds, hy, q, warp, lane);
 }
 
 // Rows of D elements on their way into a buffer; lane j of the warp holds the number of row j in the source (NO_ROW: the
@@ -642,7 +653,7 @@ __device__ __forceinline__ void finish_block(const PipeBuf<TI, K, VEC>& B, int n
             const float v = y[r] * keep;
             d[r] = p1_d(v, q);
             const float x = p1_raw(v, __fmul_rn(kk[r], kk[r]), c, rho[r], off[r]);
-            y[r] = p1_project<M>(x, hy);
+            y[r] = p1_project<M>(x, hy, q);
             bits |= y[r] == x ? (1u << r) : 0u;
         }
         out(j, d, kk, bits);
@@ -651,21 +662,21 @@ __device__ __forceinline__ void finish_block(const PipeBuf<TI, K, VEC>& B, int n
 template <typename TI, int K, bool VEC, typename OUT>
 __device__ __forceinline__ void finish_block(const PipeBuf<TI, K, VEC>& B, int n, const Hyper& hy, const P1Coord& q, int lane, OUT out)
 {
-    if (p1_mode(hy) == P1_SAT) finish_block<TI, K, VEC, P1_SAT>(B, n, hy, q, lane, out);
+    if (q.mode == P1_SAT) finish_block<TI, K, VEC, P1_SAT>(B, n, hy, q, lane, out);
     else finish_block<TI, K, VEC, P1_PLAIN>(B, n, hy, q, lane, out);
 }
 
 // The list in sh through the ring, all roles.  y travels through sh.y; guess and rounds belong to the core warps.
-template <typename TI, typename TO, int K, bool VEC>
-__device__ __forceinline__ bool run_list(const P1Fwd& a, int h, PipeShared<TI, K, VEC>& sh, float& guess, uint32_t& rounds, uint32_t& uses,
+template <typename TI, typename TO, int K, bool VEC, bool MANY>
+__device__ __forceinline__ bool run_list(const P1Fwd& a, int h, PipeShared<TI, K, VEC, MANY>& sh, float& guess, uint32_t& rounds, uint32_t& uses,
                                          int warp, int lane)
 {
     constexpr int R = K / 32;
-    using P = FwdPipe<K>;
-    constexpr int PN = PipeShared<TI, K, VEC>::PN;
+    using P = FwdPipe<K, MANY>;
+    constexpr int PN = PipeShared<TI, K, VEC, MANY>::PN;
     const int H = a.H;
     const Hyper hy = a.hy;
-    const P1Coord q = p1_coord(hy);
+    const P1Coord& q = a.q;
     const int tok0 = sh.cmd_tok, total = sh.cmd_n;
     const bool dense = sh.cmd_dense != 0;
     const int nblk = (total + PB - 1) / PB;
@@ -685,7 +696,7 @@ __device__ __forceinline__ bool run_list(const P1Fwd& a, int h, PipeShared<TI, K
             if (!ok) break;
             PipeBuf<TI, K, VEC>& B = sh.buf[bi];
             if (!dead) {
-                const int n = len_of(b), stand = core_block<TI, K, VEC>(sh, B, n, y, guess, rounds, hy, q, warp, lane);
+                const int n = len_of(b), stand = core_block<TI, K, VEC, MANY>(sh, B, n, y, guess, rounds, hy, q, warp, lane);
                 if (stand < n) {
                     dead = true;
                     stop = b * PB + stand;
@@ -737,13 +748,13 @@ __device__ __forceinline__ bool run_list(const P1Fwd& a, int h, PipeShared<TI, K
             __syncwarp();
             if (lane == 0) p1_mbar_arrive(&sh.bars.full[bi]);
         };
-        int b = (int)((warp - P::FETCH0 + base) & 1);
+        int b = (int)((warp - P::FETCH0 - base) & (P::FETCH - 1));
         if (b < nblk) start(b);
-        for (; b < nblk && ok; b += 2) {
+        for (; b < nblk && ok; b += P::FETCH) {
             cp_async_wait<0>();
             __syncwarp();
             complete(b);
-            if (b + 2 < nblk) start(b + 2);
+            if (b + P::FETCH < nblk) start(b + P::FETCH);
         }
         cp_async_wait<0>();
     } else {
@@ -778,14 +789,16 @@ __device__ __forceinline__ bool run_list(const P1Fwd& a, int h, PipeShared<TI, K
 // A list of at most PB entries by warp 0 alone, token by token (a few tokens are done before a ring would be full, and
 // the code is short).  An entry marked with bit 15 is skipped when d enters it on the face.  Returns the entries
 // that stand (fewer than n where d is off the face at a jump); sets the bits of the processed tokens in `proc`.
-template <typename TI, typename TO, int K, bool VEC>
-__device__ __forceinline__ int walk_list(const P1Fwd& a, int h, PipeShared<TI, K, VEC>& sh, int tok0, int n, bool& face, unsigned long long& proc, int lane)
+template <typename TI, typename TO, int K, bool VEC, bool MANY>
+__device__ __forceinline__ int walk_list(const P1Fwd& a, int h, PipeShared<TI, K, VEC, MANY>& sh, int tok0, int n, bool& face, unsigned long long& proc, int lane)
 {
     constexpr int R = K / 32;
     const int H = a.H;
     const Hyper hy = a.hy;
-    const P1Coord q = p1_coord(hy);
-    const P1Mode mode = p1_mode(hy);
+    const P1Coord& q = a.q;
+    // the projection as minimum and maximum in every mode: the same values, and no choice per token on the walk's path
+    const bool clip = hy.clamp;
+    const float bottom = q.face ? 0.f : hy.d_min, top = q.mode == P1_SAT ? 1.0f : q.face ? hy.d_max - hy.d_min : hy.d_max;
     PipeBuf<TI, K, VEC>& B = sh.buf[0];
     const uint32_t mine = lane < n ? (uint32_t)((tok0 + ((int)sh.list[lane] & 0x7fff)) * H + h) : NO_ROW;
     fetch_rows<TI, K>(&B.k[0][0], static_cast<const TI*>(a.k), mine, n, lane);
@@ -831,13 +844,13 @@ __device__ __forceinline__ int walk_list(const P1Fwd& a, int h, PipeShared<TI, K
         s = warp_sum(s);
         const float c = fmaf(-sc.y, s, sc.x);
         unsigned bits = 0;
-        bool on = p1_face(hy);
+        bool on = q.face;
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             d[r] = p1_d(y[r], q);
             wk[r] = d[r] * kk[r];
             const float x = p1_raw(y[r], __fmul_rn(kk[r], kk[r]), c, rho[r], off[r]);
-            y[r] = p1_project(x, mode, hy);
+            y[r] = clip ? fminf(fmaxf(x, bottom), top) : x;
             bits |= y[r] == x ? (1u << r) : 0u;
             on = on && y[r] == 0.f;
         }
@@ -907,20 +920,19 @@ __device__ __forceinline__ void scan_words(unsigned long long* words, const unsi
 //   off the face  every token, WALK at first, then 128 and twice as many each time d is still off at the end
 // What is not listed is skipped: its write key d_min k is there already and its projection mask is all zero.
 // Lists of up to PB entries are walked, unless they are dense and mostly unflagged (d will not be back soon).
-template <typename TI, typename TO, int K, bool VEC> struct ListPlan {
+template <typename TI, typename TO, int K, bool VEC, bool MANY> struct ListPlan {
     const P1Fwd& a;
-    PipeShared<TI, K, VEC>& sh;
+    PipeShared<TI, K, VEC, MANY>& sh;
     const int h, lane, c0, c1, seq_t0, seq_len;
-    const bool has_face;
     // the group of 32 chunks in hand: unflagged and processed tokens (a chunk per lane), tokens, first token, next one
     int cbase, base = 0, glen = 0, pos = 0;
     unsigned long long unf = 0ull, proc = 0ull, cand = 0ull;
     int follow = 3, run = WALK;
     bool face, listed = false, touched = false;
 
-    __device__ __forceinline__ ListPlan(const P1Fwd& a_, PipeShared<TI, K, VEC>& sh_, int s, int h_, int lane_)
+    __device__ __forceinline__ ListPlan(const P1Fwd& a_, PipeShared<TI, K, VEC, MANY>& sh_, int s, int h_, int lane_)
         : a(a_), sh(sh_), h(h_), lane(lane_), c0(a_.tab.seq_chunk0(s)), c1(a_.tab.seq_chunk0(s + 1)), seq_t0(a_.tab.seq_tok0(s)),
-          seq_len(a_.tab.seq_len(s)), has_face(p1_face(a_.hy)), cbase(c0 - 32)
+          seq_len(a_.tab.seq_len(s)), cbase(c0 - 32)
     {
         face = on_face();
     }
@@ -929,7 +941,7 @@ template <typename TI, typename TO, int K, bool VEC> struct ListPlan {
         constexpr int R = K / 32;
         float y[R];
         load_row<R>(sh.y, lane, y);
-        bool on = has_face;
+        bool on = a.q.face;
 #pragma unroll
         for (int r = 0; r < R; ++r) on = on && y[r] == 0.f;
         return __all_sync(0xffffffffu, on) != 0;
@@ -1011,7 +1023,7 @@ template <typename TI, typename TO, int K, bool VEC> struct ListPlan {
             }
             touched = true;
             if (walk) {
-                const int stop = walk_list<TI, TO, K, VEC>(a, h, sh, seq_t0 + base, n, face, proc, lane);
+                const int stop = walk_list<TI, TO, K, VEC, MANY>(a, h, sh, seq_t0 + base, n, face, proc, lane);
                 pos = ((int)sh.list[stop - 1] & 0x7fff) + 1;
                 run = face || listed ? WALK : 4 * PB;
                 continue;
@@ -1028,19 +1040,19 @@ template <typename TI, typename TO, int K, bool VEC> struct ListPlan {
 };
 
 // One chain per CTA.
-template <typename TI, typename TO, int K, bool VEC>
-__global__ void __launch_bounds__(FwdPipe<K>::THREADS, 1) phase1_seq_kernel(P1Fwd a)
+template <typename TI, typename TO, int K, bool VEC, bool MANY>
+__global__ void __launch_bounds__(FwdPipe<K, MANY>::THREADS, FwdPipe<K, MANY>::CTAS) phase1_seq_kernel(P1Fwd a)
 {
-    using P = FwdPipe<K>;
+    using P = FwdPipe<K, MANY>;
     extern __shared__ __align__(16) uint8_t p1_dyn[];
-    PipeShared<TI, K, VEC>& sh = *reinterpret_cast<PipeShared<TI, K, VEC>*>(p1_dyn);
+    PipeShared<TI, K, VEC, MANY>& sh = *reinterpret_cast<PipeShared<TI, K, VEC, MANY>*>(p1_dyn);
     const int lane = threadIdx.x & 31, warp = P::role(threadIdx.x >> 5);
     const int chain = blockIdx.x;
     const int s = chain / a.H, h = chain % a.H, H = a.H;
-    const P1Coord q = p1_coord(a.hy);
+    const P1Coord& q = a.q;
     const int coord = threadIdx.x;   // (the first K threads)
     if (threadIdx.x == 0) {
-        init_bars(sh.bars, PipeShared<TI, K, VEC>::PN, P::CORE);
+        init_bars(sh.bars, PipeShared<TI, K, VEC, MANY>::PN, P::CORE);
         sh.cmd_n = 0;
     }
     pdl_wait();   // no early release: see pdl_release
@@ -1052,12 +1064,12 @@ __global__ void __launch_bounds__(FwdPipe<K>::THREADS, 1) phase1_seq_kernel(P1Fw
     uint32_t rounds = 0, uses = 0;
     __syncthreads();
     if (warp >= 0) {
-    ListPlan<TI, TO, K, VEC> plan(a, sh, s, h, lane);
+    ListPlan<TI, TO, K, VEC, MANY> plan(a, sh, s, h, lane);
     while (true) {   // warp 0 announces a list, all work it off (one call site: the warps share the code)
         if (warp == 0) plan.next();
         bar_sync<P::ACTIVE>(1);
         if (sh.cmd_n == 0) break;
-        run_list<TI, TO, K, VEC>(a, h, sh, guess, rounds, uses, warp, lane);
+        run_list<TI, TO, K, VEC, MANY>(a, h, sh, guess, rounds, uses, warp, lane);
         bar_sync<P::ACTIVE>(2);
     }
     }
@@ -1068,14 +1080,14 @@ __global__ void __launch_bounds__(FwdPipe<K>::THREADS, 1) phase1_seq_kernel(P1Fw
 // The stand-alone sweep processes every token: the whole sequence is one list (see above).  The fetching warps also
 // form the normalisers here (there is no parallel pass before this kernel; max k^2, which only the rounds' tolerance
 // needs, is taken as sum k^2); the finishing ones form the write keys and the residual ratios.
-template <typename TI, typename TO, int K, bool VEC>
-__global__ void __launch_bounds__(FwdPipe<K>::THREADS, 1) phase1_stream_kernel(P1Args a)
+template <typename TI, typename TO, int K, bool VEC, bool MANY>
+__global__ void __launch_bounds__(FwdPipe<K, MANY>::THREADS, FwdPipe<K, MANY>::CTAS) phase1_stream_kernel(P1Args a)
 {
     constexpr int R = K / 32;
-    using P = FwdPipe<K>;
-    constexpr int PN = PipeShared<TI, K, VEC>::PN;
+    using P = FwdPipe<K, MANY>;
+    constexpr int PN = PipeShared<TI, K, VEC, MANY>::PN;
     extern __shared__ __align__(16) uint8_t p1_dyn[];
-    PipeShared<TI, K, VEC>& sh = *reinterpret_cast<PipeShared<TI, K, VEC>*>(p1_dyn);
+    PipeShared<TI, K, VEC, MANY>& sh = *reinterpret_cast<PipeShared<TI, K, VEC, MANY>*>(p1_dyn);
     __shared__ float log_part[P::FINISH];
     const int lane = threadIdx.x & 31, warp = P::role(threadIdx.x >> 5);
     const int chain = blockIdx.x;
@@ -1084,7 +1096,7 @@ __global__ void __launch_bounds__(FwdPipe<K>::THREADS, 1) phase1_stream_kernel(P
     const int t0 = a.cu ? min(max(a.cu[s], 0), a.T_dense) : s * a.T_dense;
     const int len = a.cu ? min(max(a.cu[s + 1], t0), a.T_dense) - t0 : a.T_dense;
     const Hyper hy = a.hy;
-    const P1Coord q = p1_coord(hy);
+    const P1Coord& q = a.q;
     if (threadIdx.x == 0) init_bars(sh.bars, PN, P::CORE);
     __syncthreads();
     const int nblk = (len + PB - 1) / PB;
@@ -1104,7 +1116,7 @@ __global__ void __launch_bounds__(FwdPipe<K>::THREADS, 1) phase1_stream_kernel(P
         for (int b = 0; b < nblk; ++b) {
             ok = bar_sync_and<P::CORE * 32>(3, p1_mbar_wait(&sh.bars.full[b % PN], (b / PN) & 1, nullptr));
             if (!ok) break;
-            core_block<TI, K, VEC>(sh, sh.buf[b % PN], len_of(b), y, guess, rounds, hy, q, warp, lane);
+            core_block<TI, K, VEC, MANY>(sh, sh.buf[b % PN], len_of(b), y, guess, rounds, hy, q, warp, lane);
             __syncwarp();
             if (lane == 0) p1_mbar_arrive(&sh.bars.done[b % PN]);
         }
@@ -1125,7 +1137,7 @@ __global__ void __launch_bounds__(FwdPipe<K>::THREADS, 1) phase1_stream_kernel(P
         };
         int b = warp - P::FETCH0;
         if (b < nblk) start(b);
-        for (; b < nblk && ok; b += 2) {
+        for (; b < nblk && ok; b += P::FETCH) {
             cp_async_wait<0>();
             __syncwarp();
             PipeBuf<TI, K, VEC>& B = sh.buf[b % PN];
@@ -1151,7 +1163,7 @@ __global__ void __launch_bounds__(FwdPipe<K>::THREADS, 1) phase1_stream_kernel(P
             if (lane == 0) B.jump = 0u;
             __syncwarp();
             if (lane == 0) p1_mbar_arrive(&sh.bars.full[b % PN]);
-            if (b + 2 < nblk) start(b + 2);
+            if (b + P::FETCH < nblk) start(b + P::FETCH);
         }
         cp_async_wait<0>();
     } else {
@@ -1281,7 +1293,8 @@ template <typename T, int K, bool VEC> struct RevBuf {
     alignas(16) float rv[VEC ? PB : 1][VEC ? K : 1];   // vector retention: l_t, then (core) exp(l_t)
 };
 template <typename T, int K, bool VEC> struct RevShared {
-    static constexpr int CW = K / 32, QN = ring_depth(sizeof(RevBuf<T, K, VEC>));
+    static constexpr int CW = K / 32, QN = ring_depth(sizeof(RevBuf<T, K, VEC>), 216 * 1024, Pipe<K>::FINISH);
+    static_assert(QN >= 3 && QN % Pipe<K>::FETCH == 0 && QN % Pipe<K>::FINISH == 0, "a buffer belongs to one fetching and one finishing warp");
     RevBuf<T, K, VEC> buf[QN];
     float lam[K];                           // between two lists
     float au[CW][PB];                       // a core warp's -a2 u of the round
@@ -1705,6 +1718,16 @@ __global__ void __launch_bounds__(Pipe<K>::THREADS, 1) phase1_bwd_seq_kernel(P1B
     }
 }
 
+// The kernel variant for a number of chains; launch(VEC, MANY) gets the two as types.  The line is where the chains no longer
+// have an SM each (stand-alone update, 1024 moving tokens: 144 chains 74 us one to an SM; 160 chains 136 us that way, 95 us
+// sharing).
+template <typename F> bool p1_variant(bool vec, unsigned chains, F launch)
+{
+    const bool many = chains > (unsigned)num_sms();
+    if (vec) return many ? launch(std::true_type(), std::true_type()) : launch(std::true_type(), std::false_type());
+    return many ? launch(std::false_type(), std::true_type()) : launch(std::false_type(), std::false_type());
+}
+
 template <typename TI, typename TO, int K>
 int fwd_launch(const P1Fwd& a, cudaStream_t st)
 {
@@ -1715,12 +1738,13 @@ int fwd_launch(const P1Fwd& a, cudaStream_t st)
     else phase1_spec_kernel<TI, TO, K, false><<<gspec, 128, 0, st>>>(a);
     stage_mark(st, "phase1_seq");
     const unsigned chains = (unsigned)(a.S * a.H);
-    auto launch_seq = [&](auto kernel, size_t smem) {
+    const bool okl = p1_variant(a.hy.apf_mode == 3, chains, [&](auto vec, auto many) {
+        constexpr bool VEC = decltype(vec)::value, MANY = decltype(many)::value;
+        constexpr size_t smem = sizeof(PipeShared<TI, K, VEC, MANY>);
+        const auto kernel = phase1_seq_kernel<TI, TO, K, VEC, MANY>;
         if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return false;
-        return launch_after(kernel, chains, FwdPipe<K>::THREADS, smem, st, a);
-    };
-    const bool okl = a.hy.apf_mode == 3 ? launch_seq(phase1_seq_kernel<TI, TO, K, true>, sizeof(PipeShared<TI, K, true>))
-                                        : launch_seq(phase1_seq_kernel<TI, TO, K, false>, sizeof(PipeShared<TI, K, false>));
+        return launch_after(kernel, chains, FwdPipe<K, MANY>::THREADS, smem, st, a);
+    });
     if (!okl) return -1;
     return cudaGetLastError() == cudaSuccess ? 2 : -1;
 }
@@ -1756,7 +1780,7 @@ int phase1_forward(const osdn_params& p, const Hyper& hy, const WsLayout& L, voi
     P1Fwd f{};
     f.S = L.S; f.H = p.H; f.NT = L.NTmax; f.tab = carve_table(ws, L);
     f.k = a.k; f.beta = a.beta; f.retsrc = p.apf_mode >= 2 ? a.log_ret : a.gate; f.d0 = a.precond_in;
-    f.ktil = ktil; f.d_final = a.precond_out; f.r = carve_p1(ws, L); f.save = save ? 1 : 0; f.hy = hy;
+    f.ktil = ktil; f.d_final = a.precond_out; f.r = carve_p1(ws, L); f.save = save ? 1 : 0; f.hy = hy; f.q = p1_coord(hy);
     f.status = reinterpret_cast<int*>(static_cast<char*>(ws) + L.status);
     f.clear = clear;
     if (L.dense_T) {   // (a packed batch's table kernel has cleared it)
@@ -1767,9 +1791,7 @@ int phase1_forward(const osdn_params& p, const Hyper& hy, const WsLayout& L, voi
         if (ktil_bf16) return -1;
         return p.K == 64 ? fwd_launch<float, float, 64>(f, st) : fwd_launch<float, float, 128>(f, st);
     }
-    if (ktil_bf16)
-        return p.K == 64 ? fwd_launch<__nv_bfloat16, __nv_bfloat16, 64>(f, st)
-                         : fwd_launch<__nv_bfloat16, __nv_bfloat16, 128>(f, st);
+    if (ktil_bf16) return p.K == 128 ? fwd_launch<__nv_bfloat16, __nv_bfloat16, 128>(f, st) : -1;   // (the tensor-core family)
     return p.K == 64 ? fwd_launch<__nv_bfloat16, float, 64>(f, st) : fwd_launch<__nv_bfloat16, float, 128>(f, st);
 }
 
@@ -1803,20 +1825,20 @@ int phase1_update(const osdn_params& p, const Hyper& hy, const void* k, const fl
     pa.S = p.nseq > 0 ? p.nseq : p.B;
     pa.H = p.H; pa.T_dense = p.T; pa.cu = p.nseq > 0 ? p.cu_seqlens : nullptr;
     pa.k = k; pa.beta = beta; pa.retsrc = retsrc; pa.d0 = precond_in; pa.ktil = ktil_out;
-    pa.d_final = precond_out; pa.ratio = ratio_out; pa.log_sum = log_sum_out; pa.hy = hy;
+    pa.d_final = precond_out; pa.ratio = ratio_out; pa.log_sum = log_sum_out; pa.hy = hy; pa.q = p1_coord(hy);
     const unsigned chains = (unsigned)(pa.S * pa.H);
     stage_mark(st, "phase1_stream");
-    const bool vec = hy.apf_mode == 3;
-    auto launch = [&](auto kernel, size_t smem, int threads) {
-        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return false;
-        kernel<<<chains, threads, smem, st>>>(pa);
-        return true;
-    };
     auto typed = [&](auto t, auto kk) {
         using T = decltype(t);
         constexpr int K = decltype(kk)::value;
-        return vec ? launch(phase1_stream_kernel<T, T, K, true>, sizeof(PipeShared<T, K, true>), FwdPipe<K>::THREADS)
-                   : launch(phase1_stream_kernel<T, T, K, false>, sizeof(PipeShared<T, K, false>), FwdPipe<K>::THREADS);
+        return p1_variant(hy.apf_mode == 3, chains, [&](auto vec, auto many) {
+            constexpr bool VEC = decltype(vec)::value, MANY = decltype(many)::value;
+            constexpr size_t smem = sizeof(PipeShared<T, K, VEC, MANY>);
+            const auto kernel = phase1_stream_kernel<T, T, K, VEC, MANY>;
+            if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return false;
+            kernel<<<chains, FwdPipe<K, MANY>::THREADS, smem, st>>>(pa);
+            return true;
+        });
     };
     using K64 = std::integral_constant<int, 64>;
     using K128 = std::integral_constant<int, 128>;

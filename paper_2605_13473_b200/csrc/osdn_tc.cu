@@ -2295,17 +2295,6 @@ __global__ void wait_timeout_selftest_kernel(int* status, long long limit_cycles
     mbar_wait(&bar, 0, status, code, limit_cycles);
 }
 
-int num_sms()
-{
-    static int n = 0;
-    if (!n) {
-        int dev = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0)
-            n = 148;
-    }
-    return n;
-}
-
 template <typename F> bool set_smem(F* kernel, size_t bytes)
 {
     return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) == cudaSuccess;

@@ -1,6 +1,8 @@
 """The kernels' dispatch rules and block edges: sizes on both sides of every line, against the oracle.
 
 Tolerances are the suite's: 1e-4 of the largest value for fp32 arithmetic (parity.TOL for bf16 results)."""
+import copy
+
 import numpy as np
 import pytest
 import torch
@@ -80,6 +82,37 @@ def test_lists_of_processed_tokens(lens, shift):
     inp = draw("lists", 7100 + int(shift), lens, 1, 64, 64, "fp32", dense_B=len(lens) == 1, hyper=hy, gate_kind="zero",
                with_dout=True, with_log_ret=True, log_ret_shift=shift, with_state_cotangents=True)
     _all_outputs(inp, f"lists_{len(lens)}_{shift}")
+
+
+@pytest.mark.parametrize("io,K", [("bf16", 128), ("fp32", 128), ("fp32", 64)])
+@pytest.mark.parametrize("apf,eta,shift", [(2, 0.3, 5.0), (2, 0.003, 7.0), (3, 0.3, 3.0), (1, 0.003, 5.0)])
+def test_more_chains_than_sms(io, K, apf, eta, shift):
+    """Beyond one chain per SM the preconditioner passes share SMs: bit for bit what the few chains compute, and the
+    oracle's write keys.  300 tokens: walked lists, blocks, more blocks than the short ring holds, a ragged last one."""
+    hy = OsdnHyper(eta=eta, apf_mode=apf, beta_aware=int(shift != 7.0))
+    few = draw("many", 7800 + apf, [300, 300], 4, K, K, io, dense_B=2, hyper=hy, key_kind="sparse" if eta > 0.1 else "gauss",
+               gate_kind="zero" if shift == 7.0 else "softplus", with_log_ret=apf >= 2, log_ret_shift=shift, with_state=True)
+    results = {}
+    for rep in (1, 20):   # 8 and 160 chains
+        more = lambda x: None if x is None else x.repeat(rep, *[1] * (x.dim() - 1)).contiguous()
+        big = copy.copy(few)
+        big.seq_lens, big.dense_B = few.seq_lens * rep, 2 * rep
+        for name in ("q", "k", "v", "beta", "gate", "log_ret", "init_state", "precond_in"):
+            setattr(big, name, more(getattr(few, name)))
+        b = binding.DeviceBundle(big, DEV, need_bwd=True)
+        b.fwd(save=True)
+        kt, d, ratio = torch.empty_like(b.k), torch.empty_like(b.precond_out), torch.empty_like(b.beta)
+        ret = b.log_ret if apf >= 2 else b.gate
+        binding.osdn_precond_update(b.params, b.k, b.beta, ret, b.precond_in, kt, d)
+        binding.osdn_residual_ratio(b.params, b.k, b.beta, ret, b.precond_in, ratio, None)
+        torch.cuda.synchronize()
+        assert b.device_status() == 0
+        results[rep] = [kt, d, ratio, b.precond_out, b.projection_masks()]
+    for x, y in zip(results[1], results[20]):
+        assert torch.equal(y, x.repeat(20, *[1] * (x.dim() - 1)))
+    ref = oracle.precond_update(hy, few.seq_lens, few.k, few.beta, few.gate, few.log_ret, few.precond_in)
+    assert parity.err(results[1][1].cpu().numpy(), ref["precond_out"]) <= 1e-5
+    assert parity.err(results[1][0].float().cpu().numpy(), ref["ktil"]) <= (1e-5 if io == "fp32" else 2.0 ** -8)
 
 
 @pytest.mark.parametrize("io,flags", [("bf16", 0), ("fp32", 0), ("bf16", binding.FLAG_FORCE_SIMT)])
