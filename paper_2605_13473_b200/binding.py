@@ -102,10 +102,11 @@ def _call(*args) -> int:
     global _call
     load_library()
     try:
-        from ._osdn_call import call
+        from ._osdn_call import call, register
     except ImportError as e:
         raise RuntimeError("the extension module _osdn_call is missing or does not load: build it first "
                            "(python paper_2605_13473_b200/build.py); there is no fallback path") from e
+    register(OsdnParams)
     _call = call
     return call(*args)
 

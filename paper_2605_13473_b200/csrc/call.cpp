@@ -52,6 +52,21 @@ template <> int with_workspace<Bwd>(Bwd fn, const osdn_params* p, void** x, size
               f(16), f(17), f(18), x[19], bytes, st);
 }
 
+struct GilReleased {   // taken back on every way out
+    PyThreadState* state = PyEval_SaveThread();
+    ~GilReleased() { PyEval_RestoreThread(state); }
+};
+
+PyObject* g_params_type = nullptr;   // binding.OsdnParams
+
+// register(type): the class of call's params
+PyObject* register_params(PyObject*, PyObject* type)
+{
+    Py_INCREF(type);
+    Py_XSETREF(g_params_type, type);
+    Py_RETURN_NONE;
+}
+
 // call(which, params, *tensors) -> status code of the library
 PyObject* call(PyObject*, PyObject* const* args, Py_ssize_t n)
 {
@@ -65,38 +80,51 @@ PyObject* call(PyObject*, PyObject* const* args, Py_ssize_t n)
         PyErr_SetString(PyExc_TypeError, "unknown call, or a wrong number of tensors");
         return nullptr;
     }
+    const int known = g_params_type ? PyObject_IsInstance(args[1], g_params_type) : 0;
+    if (known < 0) return nullptr;
+    if (!known) {
+        PyErr_SetString(PyExc_TypeError, "params: not an OsdnParams");
+        return nullptr;
+    }
     Py_buffer view;   // the ctypes structure's own memory
     if (PyObject_GetBuffer(args[1], &view, PyBUF_SIMPLE) != 0) return nullptr;
     PyObject* result = nullptr;
     void* x[20];
     size_t bytes = 0;
-    bool ok = view.len == (Py_ssize_t)sizeof(osdn_params);
+    bool ok = view.len >= (Py_ssize_t)sizeof(osdn_params);
     if (!ok) PyErr_SetString(PyExc_TypeError, "params: not an OsdnParams");
-    for (Py_ssize_t i = 0; ok && i < n - 2; ++i) ok = pointer_of(args[2 + i], &x[i], &bytes);   // the workspace is the last
-    if (ok) {
-        try {
+    // torch throws where a tensor has no memory of its own (under vmap or grad) or there is no device: nothing may leave
+    // through the C entry, it would end the process
+    try {
+        for (Py_ssize_t i = 0; ok && i < n - 2; ++i) ok = pointer_of(args[2 + i], &x[i], &bytes);   // the workspace is the last
+        if (ok) {
             void* st = c10::cuda::getCurrentCUDAStream().stream();
             const osdn_params* p = static_cast<const osdn_params*>(view.buf);
             auto f = [&](int i) { return static_cast<float*>(x[i]); };
             int rc = 0;
-            PyThreadState* released = PyEval_SaveThread();   // a launch may wait for room in the stream
-            switch (which) {
-                case FWD: rc = with_workspace<Fwd>(&osdn_fwd, p, x, bytes, st); break;
-                case KDA_FWD: rc = with_workspace<Fwd>(&osdn_kda_fwd, p, x, bytes, st); break;
-                case BWD: rc = with_workspace<Bwd>(&osdn_bwd, p, x, bytes, st); break;
-                case KDA_BWD: rc = with_workspace<Bwd>(&osdn_kda_bwd, p, x, bytes, st); break;
-                case PRECOND: rc = osdn_precond_update(p, x[0], f(1), f(2), f(3), x[4], f(5), st); break;
-                case RATIO: rc = osdn_residual_ratio(p, x[0], f(1), f(2), f(3), f(4), f(5), f(6), st); break;
-                case DECODE: rc = osdn_decode_step(p, x[0], x[1], x[2], f(3), f(4), f(5), f(6), f(7), x[8], st); break;
-                case FWD_STATIC:
-                    rc = osdn_fwd_static(p, x[0], x[1], x[2], f(3), f(4), f(5), f(6), f(7), x[8], f(9), f(10), st);
-                    break;
+            {
+                const GilReleased released;   // a launch may wait for room in the stream
+                switch (which) {
+                    case FWD: rc = with_workspace<Fwd>(&osdn_fwd, p, x, bytes, st); break;
+                    case KDA_FWD: rc = with_workspace<Fwd>(&osdn_kda_fwd, p, x, bytes, st); break;
+                    case BWD: rc = with_workspace<Bwd>(&osdn_bwd, p, x, bytes, st); break;
+                    case KDA_BWD: rc = with_workspace<Bwd>(&osdn_kda_bwd, p, x, bytes, st); break;
+                    case PRECOND: rc = osdn_precond_update(p, x[0], f(1), f(2), f(3), x[4], f(5), st); break;
+                    case RATIO: rc = osdn_residual_ratio(p, x[0], f(1), f(2), f(3), f(4), f(5), f(6), st); break;
+                    case DECODE: rc = osdn_decode_step(p, x[0], x[1], x[2], f(3), f(4), f(5), f(6), f(7), x[8], st); break;
+                    case FWD_STATIC:
+                        rc = osdn_fwd_static(p, x[0], x[1], x[2], f(3), f(4), f(5), f(6), f(7), x[8], f(9), f(10), st);
+                        break;
+                }
             }
-            PyEval_RestoreThread(released);
             result = PyLong_FromLong(rc);
-        } catch (const std::exception& e) {
-            PyErr_SetString(PyExc_RuntimeError, e.what());
         }
+    } catch (const c10::Error& e) {
+        PyErr_SetString(PyExc_RuntimeError, e.what_without_backtrace());
+    } catch (const std::exception& e) {
+        PyErr_SetString(PyExc_RuntimeError, e.what());
+    } catch (...) {
+        PyErr_SetString(PyExc_RuntimeError, "unknown C++ exception");
     }
     PyBuffer_Release(&view);
     return result;
@@ -104,6 +132,7 @@ PyObject* call(PyObject*, PyObject* const* args, Py_ssize_t n)
 
 PyMethodDef methods[] = {{"call", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(call)), METH_FASTCALL,
                           "call(which, params, *tensors) -> status code"},
+                         {"register", register_params, METH_O, "register(type): the class of call's params"},
                          {nullptr, nullptr, 0, nullptr}};
 PyModuleDef module = {PyModuleDef_HEAD_INIT, "_osdn_call", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
 

@@ -117,6 +117,37 @@ def test_calls_reject_bad_arguments_before_any_launch(lib):
     assert rc == -2
 
 
+def test_calls_refuse_what_is_no_params_or_no_memory(lib):
+    """Through the marshalled entry: an exception, and never the end of the process (hence the child)."""
+    import subprocess
+    import sys
+    code = """
+import ctypes, torch, paper_2605_13473_b200 as osdn
+from paper_2605_13473_b200 import binding
+p = osdn.make_params(B=1, T=1, H=1, K=64, V=64, io_dtype="fp32")
+def refused(kind, *args):
+    try:
+        binding.osdn_decode_step(*args)
+    except kind as e:
+        print("refused", type(e).__name__, flush=True)
+x = torch.empty(64)
+refused(TypeError, bytes(p), x, x, x, x, x, None, x, x, x)     # the right number of bytes
+refused(TypeError, None, x, x, x, x, x, None, x, x, x)
+refused(TypeError, p, 5, x, x, x, x, None, x, x, x)
+refused(ValueError, p, torch.empty(64, 2).t(), x, x, x, x, None, x, x, x)
+class Sub(binding.OsdnParams):
+    _fields_ = [("more", ctypes.c_int)]
+refused(RuntimeError, Sub(), None, x, x, x, x, None, x, x, x)  # taken as params (all zero): refused further down
+def inside(t):
+    refused(RuntimeError, p, t, x, x, x, x, None, x, x, x)     # a wrapped tensor has no memory of its own
+    return t.sum()
+torch.func.vmap(inside)(torch.empty(3, 64))
+torch.func.grad(inside)(torch.empty(64))
+"""
+    r = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0 and r.stdout.count("refused") == 7, (r.returncode, r.stdout, r.stderr[-2000:])
+
+
 def test_missing_library_fails_loudly(tmp_path):
     with pytest.raises(RuntimeError, match="no fallback"):
         osdn.load_library(str(tmp_path / "libosdn.so"))
