@@ -10,7 +10,9 @@ import sysconfig
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libosdn.so")
-CALL_LIB = os.path.join(HERE, "_osdn_call.so")   # python module: argument marshalling of the hot calls
+# python module: argument marshalling of the hot calls.  Its name carries the interpreter's ABI, so that another one does
+# not load it.
+CALL_LIB = os.path.join(HERE, "_osdn_call" + sysconfig.get_config_var("EXT_SUFFIX"))
 SOURCES = ["osdn_api.cu", "osdn_phase1.cu", "osdn_simt.cu", "osdn_tc.cu", "osdn_decode.cu", "osdn_kda.cu"]
 
 
@@ -18,12 +20,20 @@ def _newest(paths):
     return max(os.path.getmtime(p) for p in paths)
 
 
+def _torch_dir() -> str:
+    return os.path.dirname(importlib.util.find_spec("torch").origin)
+
+
+def call_inputs() -> list:
+    """What the extension module is built from; torch's C++ interface changes with its version."""
+    return [os.path.join(CSRC, "call.cpp"), os.path.join(os.path.dirname(HERE), "include", "osdn.h"),
+            os.path.join(_torch_dir(), "version.py")]
+
+
 def _build_call(force: bool) -> None:
-    src = os.path.join(CSRC, "call.cpp")
-    header = os.path.join(os.path.dirname(HERE), "include", "osdn.h")
-    if not force and os.path.exists(CALL_LIB) and os.path.getmtime(CALL_LIB) >= _newest([src, header]):
+    if not force and os.path.exists(CALL_LIB) and os.path.getmtime(CALL_LIB) >= _newest(call_inputs()):
         return
-    torch_dir = os.path.dirname(importlib.util.find_spec("torch").origin)
+    src, torch_dir = call_inputs()[0], _torch_dir()
     inc = os.path.join(torch_dir, "include")
     subprocess.run(["g++", "-std=c++17", "-O2", "-fPIC", "-shared", "-fvisibility=hidden", "-I" + inc,
                     "-I" + os.path.join(inc, "torch", "csrc", "api", "include"), "-I/usr/local/cuda/include",

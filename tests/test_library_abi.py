@@ -148,6 +148,19 @@ torch.func.grad(inside)(torch.empty(64))
     assert r.returncode == 0 and r.stdout.count("refused") == 7, (r.returncode, r.stdout, r.stderr[-2000:])
 
 
+def test_extension_belongs_to_this_interpreter_and_torch(lib):
+    """Another interpreter does not find it, another torch has it built again."""
+    import importlib
+    import sysconfig
+
+    import torch
+    from paper_2605_13473_b200 import build as b
+    module = importlib.import_module("paper_2605_13473_b200._osdn_call")
+    assert module.__file__ == b.CALL_LIB and b.CALL_LIB.endswith(sysconfig.get_config_var("EXT_SUFFIX"))
+    assert os.path.join(os.path.dirname(torch.__file__), "version.py") in b.call_inputs()
+    assert os.path.getmtime(b.CALL_LIB) >= max(map(os.path.getmtime, b.call_inputs()))
+
+
 def test_missing_library_fails_loudly(tmp_path):
     with pytest.raises(RuntimeError, match="no fallback"):
         osdn.load_library(str(tmp_path / "libosdn.so"))
