@@ -241,6 +241,11 @@ __device__ __forceinline__ void ut_inverse_64(const float* sA, float* sT, float*
 // ---------------------------------------------------------------------------------------
 // arguments of the tile-parallel passes
 // ---------------------------------------------------------------------------------------
+// One CTA per (chunk, head): chunks along x, heads along y and, beyond what a grid's y takes, z.
+constexpr int GRID_Y = 65535;
+inline dim3 tile_grid(int chunks, int H) { return dim3(chunks, H < GRID_Y ? H : GRID_Y, (H + GRID_Y - 1) / GRID_Y); }
+__device__ __forceinline__ int tile_head() { return blockIdx.z * GRID_Y + blockIdx.y; }
+
 constexpr float SAFE_RANGE = 30.f;
 constexpr int CL_NT = 512;   // two groups of 256 threads, each with its own product between two barriers
 
@@ -404,7 +409,8 @@ __global__ void __launch_bounds__(CL_NT, LocalFwd<T, K, V, CG>::MIN_CTAS) chunk_
     __shared__ GateVecs gv;
     __shared__ float tmp[32 * 32];
 
-    const int c = blockIdx.x, h = blockIdx.y, H = a.H;
+    const int c = blockIdx.x, h = tile_head(), H = a.H;
+    if (h >= H) return;
     const int len = a.tab.chunk_len(c);
     if (len == 0) return;
     const int tok0 = a.tab.chunk_tok0(c);
@@ -547,7 +553,8 @@ __global__ void __launch_bounds__(256) output_kernel(ChunkArgs a)
     float* sQ = sm;                  // [64][LD]
     float* sS = sQ + CH * LD;        // [V][LD], S_n; then dU [64][V]
     float* sP = sS + V * LD;         // [64][LC]
-    const int c = blockIdx.x, h = blockIdx.y, H = a.H;
+    const int c = blockIdx.x, h = tile_head(), H = a.H;
+    if (h >= H) return;
     const int len = a.tab.chunk_len(c);
     if (len == 0) return;
     const int tok0 = a.tab.chunk_tok0(c);
@@ -608,7 +615,8 @@ __global__ void __launch_bounds__(256) pre_bwd_kernel(ChunkArgs a)
     float* sP = sm;
     float* sO = sP + CH * CH;   // [64][V]
     float* sQ = sO + CH * V;    // [64][K]
-    const int c = blockIdx.x, h = blockIdx.y, H = a.H;
+    const int c = blockIdx.x, h = tile_head(), H = a.H;
+    if (h >= H) return;
     const int len = a.tab.chunk_len(c);
     if (len == 0) return;
     const int tok0 = a.tab.chunk_tok0(c);
@@ -982,7 +990,8 @@ __global__ void __launch_bounds__(CL_NT) chunk_local_bwd_kernel(ChunkArgs a)
     __shared__ float sB[3][CH], sE[3][CH];   // channel gate: sE[0] the diagonal of dP
     __shared__ __align__(16) float sRed[PARTS][K], sR[8][K];   // column sums of dS (.) S and of dKtr (.) Ktr
 
-    const int c = blockIdx.x, h = blockIdx.y, H = a.H;
+    const int c = blockIdx.x, h = tile_head(), H = a.H;
+    if (h >= H) return;
     const int len = a.tab.chunk_len(c);
     if (len == 0) return;
     const int tok0 = a.tab.chunk_tok0(c);
@@ -1418,7 +1427,7 @@ int chunk_forward(const osdn_params& p, const Hyper& hy, const WsLayout& L, void
 {
     ChunkArgs c = chunk_args(p, hy, L, ws, a, G);
     c.out = a.out;
-    const dim3 tiles(L.NTmax, p.H);
+    const dim3 tiles = tile_grid(L.NTmax, p.H);
     using LF = LocalFwd<T, K, V, CG>;
     if (!set_smem(chunk_local_fwd_kernel<T, K, V, CG>, LF::SMEM)) return -1;
     stage_mark(st, "chunk_local_fwd");
@@ -1443,7 +1452,7 @@ int chunk_backward(const osdn_params& p, const Hyper& hy, const WsLayout& L, voi
     ChunkArgs c = chunk_args(p, hy, L, ws, a, G);
     c.dout = a.dout; c.ddU = F(L.ddU); c.dSn = F(L.dSn); c.dktil = F(L.dktil); c.dkread = F(L.dkread);
     c.dq = a.dq; c.dv = a.dv; c.dbeta = a.dbeta; c.dgate = a.dgate;
-    const dim3 tiles(L.NTmax, p.H);
+    const dim3 tiles = tile_grid(L.NTmax, p.H);
     if (!set_smem(pre_bwd_kernel<T, K, V, CG>, pre_bwd_smem<K, V>())) return -1;
     stage_mark(st, "chunk_pre_bwd");
     pre_bwd_kernel<T, K, V, CG><<<tiles, 256, pre_bwd_smem<K, V>(), st>>>(c);

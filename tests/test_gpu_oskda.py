@@ -72,6 +72,35 @@ def test_gate_gradients_behind_strong_gates():
         assert parity.err(got[key], ref[key], norm="l2") <= 6e-7, key
 
 
+def test_more_heads_than_a_grid_has_rows():
+    """65600 heads: the last ones equal the same heads on their own (up to the order of sums of the two chain cuts)."""
+    H, K, tail = 65600, 64, 65
+    gen = torch.Generator(device="cuda:0").manual_seed(72)
+    rnd = lambda *s: torch.randn(*s, generator=gen, device="cuda:0")
+    full = dict(q=rnd(1, H, K), k=torch.nn.functional.normalize(rnd(1, H, K), dim=-1), v=rnd(1, H, K), beta=torch.sigmoid(rnd(1, H)),
+                gate=-0.1 * rnd(1, H, K).abs(), log_ret=-0.01 * rnd(1, H).abs(), dout=rnd(1, H, K))
+    hy = OsdnHyper(eta=0.3, apf_mode=2, channel_gate=1)
+    res = []
+    for heads in (slice(0, H), slice(H - tail, H)):
+        x = {k: v[:, heads].clone() for k, v in full.items()}
+        n = x["beta"].shape[1]
+        p = binding.make_params(B=1, T=1, H=n, K=K, V=K, io_dtype="fp32", hyper=hy)
+        ws = torch.empty(binding.osdn_kda_workspace_bytes(p, True), device="cuda:0", dtype=torch.uint8)
+        out, dq, dk, dv, dgate = (torch.full((1, n, K), float("nan"), device="cuda:0") for _ in range(5))
+        dbeta, dlr = torch.empty(1, n, device="cuda:0"), torch.empty(1, n, device="cuda:0")
+        ins = [x[k] for k in ("q", "k", "v", "beta", "gate", "log_ret")] + [None, None]
+        p.flags = binding.FLAG_SAVE_RESIDUALS
+        binding.osdn_kda_fwd(p, *ins, out, None, None, ws)
+        p.flags = binding.FLAG_RESIDUALS_VALID
+        binding.osdn_kda_bwd(p, *ins, x["dout"], None, None, dq, dk, dv, dbeta, dgate, dlr, None, None, ws)
+        torch.cuda.synchronize()
+        assert binding.osdn_read_device_status(ws) == 0
+        res.append([y[:, -tail:].clone() for y in (out, dq, dk, dv, dgate, dbeta)])
+        del ws
+    for a, b in zip(*res):
+        assert torch.allclose(a, b, rtol=1e-4, atol=1e-6)
+
+
 def test_forward_alone_and_recomputed_residuals():
     inp = _case(71, [100, 100], 2, 128, 128, "fp32", 2, dense_B=2)
     f = binding.run_inputs_fwd(inp)
