@@ -1392,15 +1392,17 @@ template <typename F> bool set_smem(F* kernel, size_t bytes)
     return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) == cudaSuccess;
 }
 
-// Narrow or wide slices: whichever walk is expected to end first.  A step of a wide slice (eight times the rows)
-// takes about WIDE_STEP times a narrow one's; what decides is how many waves of CTAs each cut makes.
-constexpr int WIDE_STEP_TENTHS = 25;
+// Narrow or wide slices: whichever walk is expected to end first.  What decides is how many waves of CTAs each cut makes; a
+// wave of wide slices (eight times the rows) takes as long as WIDE_STEP waves of narrow ones.  Measured, 512 tokens, forward
+// chain, microseconds for 1, 2, 3, 4, 5 waves of narrow slices against one of wide ones: K = 64 29, 48, 64 against 53;
+// K = 128 27, 46, 66, 86, 106 against 86.
+template <int K> constexpr int WIDE_STEP_TENTHS = K == 64 ? 25 : 35;
 template <int K, int V, bool BWD, bool CG> int launch_chain(const ChainArgs& ch, int chains, cudaStream_t st)
 {
-    constexpr int PER_SM = K == 64 ? 2 : 1, SLOTS = 148 * PER_SM;
+    const int SLOTS = num_sms() * (K == 64 ? 2 : 1);   // CTAs of either kind that fit an SM: by their shared memory
     const long narrow = ((long)chains * (V / VS) + SLOTS - 1) / SLOTS, wide = ((long)chains * (V / WS) + SLOTS - 1) / SLOTS;
     stage_mark(st, BWD ? "chain_bwd" : "chain_fwd");
-    if (narrow * 10 <= wide * WIDE_STEP_TENTHS) {
+    if (narrow * 10 <= wide * WIDE_STEP_TENTHS<K>) {
         if (!set_smem(chain_narrow_kernel<K, V, BWD, CG>, sizeof(NarrowShared<K>))) return -1;
         chain_narrow_kernel<K, V, BWD, CG><<<dim3(chains, V / VS), CNT, sizeof(NarrowShared<K>), st>>>(ch);
     } else {
