@@ -28,7 +28,8 @@ def test_standalone_update_at_block_edges(L, eta, keys, apf, clamp, K):
     kt, d = torch.empty_like(b.k), torch.empty(2, 2, K, device=DEV)
     binding.osdn_precond_update(b.params, b.k, b.beta, b.log_ret if apf >= 2 else b.gate, b.precond_in, kt, d)
     ref = oracle.precond_update(hy, inp.seq_lens, inp.k, inp.beta, inp.gate, inp.log_ret, inp.precond_in)
-    assert parity.err(d.cpu().numpy(), ref["precond_out"]) <= 1e-4
+    assert parity.err(d.cpu().numpy(), ref["precond_out"]) <= 1e-5
+    assert parity.err(kt.cpu().numpy(), ref["ktil"]) <= 1e-5
 
 
 def _all_outputs(inp, label, **kw):
@@ -138,6 +139,17 @@ def test_chains_in_wide_slices(io, K):
     inp = draw("wide", 7200 + K, [70] * 50, 6, K, 64, io, dense_B=50, hyper=hy, with_dout=True, with_state=True,
                with_state_cotangents=True)
     _all_outputs(inp, f"wide_{io}_{K}")
+
+
+@pytest.mark.parametrize("io,cg,gates", [("fp32", 0, "softplus"), ("bf16", 0, "softplus"), ("fp32", 1, "softplus"), ("fp32", 1, "strong"), ("bf16", 1, "mixture")])
+def test_chains_in_wide_slices_of_128_rows(io, cg, gates):
+    """K = V = 128 in wide slices, two to a chain (from 28 chains on): scalar and channel gates, weak and strong."""
+    hy = OsdnHyper(eta=0.003, apf_mode=2, channel_gate=cg)
+    inp = draw("wide128", 7250 + cg, [150] * 8, 5, 128, 128, io, dense_B=8, hyper=hy, gate_kind=gates, with_dout=True,
+               with_log_ret=True, with_state=True, with_state_cotangents=True)
+    got = run_inputs_bwd(inp, flags=binding.FLAG_FORCE_SIMT)
+    ref = parity.oracle_all(inp, True, got["projection_masks"])
+    parity.compare(got, ref, io, parity.FWD_KEYS + parity.BWD_KEYS, f"wide128_{io}_{cg}_{gates}")
 
 
 def test_backward_twice_on_the_same_residuals():
