@@ -109,7 +109,6 @@ def kernel_model(name, inp, NT):
     f = lambda m, n, k: 2.0 * m * n * k
     m = {}
     # CUDA-core (fp32 workspace) family
-    m["phase1_fwd"] = (tokh * (K * es + 8 + K * 4) + tiles * K * 4, tokh * 9.0 * K, "hbm")
     m["chunk_local_fwd"] = (tokh * (2 * K * es + K * 4 + V * es + 8) + tiles * 4 * (3 * C * C + 3 * C * K + C * V + K),
                             tiles * (2 * f(C, C, K) + f(C, K, C) + f(C, V, C)), "alu")
     m["chain_fwd"] = (tiles * 4 * (2 * C * K + 2 * C * V + V * K), tiles * (f(C, V, K) + f(V, K, C)), "alu")

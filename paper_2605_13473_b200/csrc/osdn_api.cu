@@ -269,7 +269,7 @@ int osdn_kda_bwd(const osdn_params* p, const void* q, const void* k, const void*
     a.dinit_state = dinit_state; a.dprecond_in = dprecond_in;
     int total = 0;
     if (!(p->flags & OSDN_FLAG_RESIDUALS_VALID)) {
-            Pointers f = a;
+        Pointers f = a;
         f.out = static_cast<char*>(workspace) + L.out_scratch;
         f.final_state = nullptr;
         f.precond_out = nullptr;
@@ -544,7 +544,6 @@ int osdn_fwd_static(const osdn_params* p, const void* q, const void* k, const vo
     void* scratch = static_scratch_address();
     if (!scratch) return OSDN_CUDA_ERROR;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-    // the device status word is the only part that must start at zero
     Pointers a{};
     a.q = q; a.k = k; a.v = v; a.beta = beta; a.gate = gate; a.log_ret = apf_log_ret;
     a.init_state = init_state; a.precond_in = precond_in; a.out = out; a.final_state = final_state;

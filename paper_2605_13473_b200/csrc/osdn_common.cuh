@@ -241,6 +241,75 @@ template <> __device__ __forceinline__ void stf<__nv_bfloat16>(__nv_bfloat16* p,
     *p = __float2bfloat16_rn(x);
 }
 
+__device__ __forceinline__ float warp_sum(float x)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    return x;
+}
+
+// Lane l of a warp owns the R = K / 32 consecutive coordinates R l .. R l + R - 1, so that a
+// row of K values is one vector access per lane.
+template <int R> __device__ __forceinline__ void load_row(const float* p, int lane, float (&x)[R])
+{
+    if constexpr (R == 4) {
+        const float4 v = *reinterpret_cast<const float4*>(p + 4 * lane);
+        x[0] = v.x; x[1] = v.y; x[2] = v.z; x[3] = v.w;
+    } else {
+        const float2 v = *reinterpret_cast<const float2*>(p + 2 * lane);
+        x[0] = v.x; x[1] = v.y;
+    }
+}
+template <int R> __device__ __forceinline__ void load_row(const __nv_bfloat16* p, int lane, float (&x)[R])
+{
+    if constexpr (R == 4) {
+        const uint2 v = *reinterpret_cast<const uint2*>(p + 4 * lane);
+        const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&v.x));
+        const float2 b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&v.y));
+        x[0] = a.x; x[1] = a.y; x[2] = b.x; x[3] = b.y;
+    } else {
+        const uint32_t v = *reinterpret_cast<const uint32_t*>(p + 2 * lane);
+        const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&v));
+        x[0] = a.x; x[1] = a.y;
+    }
+}
+template <int R> __device__ __forceinline__ void store_row(float* p, int lane, const float (&x)[R])
+{
+    if constexpr (R == 4) *reinterpret_cast<float4*>(p + 4 * lane) = make_float4(x[0], x[1], x[2], x[3]);
+    else *reinterpret_cast<float2*>(p + 2 * lane) = make_float2(x[0], x[1]);
+}
+template <int R> __device__ __forceinline__ void store_row(__nv_bfloat16* p, int lane, const float (&x)[R])
+{
+    if constexpr (R == 4) {
+        __nv_bfloat162 a = __floats2bfloat162_rn(x[0], x[1]), b = __floats2bfloat162_rn(x[2], x[3]);
+        uint2 v;
+        v.x = *reinterpret_cast<uint32_t*>(&a);
+        v.y = *reinterpret_cast<uint32_t*>(&b);
+        *reinterpret_cast<uint2*>(p + 4 * lane) = v;
+    } else {
+        __nv_bfloat162 a = __floats2bfloat162_rn(x[0], x[1]);
+        *reinterpret_cast<uint32_t*>(p + 2 * lane) = *reinterpret_cast<uint32_t*>(&a);
+    }
+}
+
+// Lane l gets the warp's sum of x[l % N]: the N sums share their shuffles.
+template <int N> __device__ __forceinline__ float transpose_sum(float (&x)[N], int lane)
+{
+#pragma unroll
+    for (int s = N / 2; s > 0; s >>= 1) {
+        const bool up = (lane & s) != 0;
+#pragma unroll
+        for (int i = 0; i < s; ++i) {
+            const float send = up ? x[i] : x[i + s], keep = up ? x[i + s] : x[i];
+            x[i] = keep + __shfl_xor_sync(0xffffffffu, send, s);
+        }
+    }
+    float v = x[0];
+#pragma unroll
+    for (int s = N; s < 32; s <<= 1) v += __shfl_xor_sync(0xffffffffu, v, s);
+    return v;
+}
+
 // Everything a forward / backward launch sequence needs.
 struct Pointers {
     const void *q, *k, *v;

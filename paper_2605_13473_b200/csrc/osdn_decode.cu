@@ -41,42 +41,6 @@ struct DecArgs {
     Hyper hy;
 };
 
-__device__ __forceinline__ float dec_warp_sum(float x)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-    return x;
-}
-
-template <int R> __device__ __forceinline__ void dec_load(const float* p, int lane, float (&x)[R])
-{
-    if constexpr (R == 4) {
-        const float4 t = *reinterpret_cast<const float4*>(p + 4 * lane);
-        x[0] = t.x; x[1] = t.y; x[2] = t.z; x[3] = t.w;
-    } else {
-        const float2 t = *reinterpret_cast<const float2*>(p + 2 * lane);
-        x[0] = t.x; x[1] = t.y;
-    }
-}
-template <int R> __device__ __forceinline__ void dec_load(const __nv_bfloat16* p, int lane, float (&x)[R])
-{
-    if constexpr (R == 4) {
-        const uint2 t = *reinterpret_cast<const uint2*>(p + 4 * lane);
-        const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&t.x));
-        const float2 b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&t.y));
-        x[0] = a.x; x[1] = a.y; x[2] = b.x; x[3] = b.y;
-    } else {
-        const uint32_t t = *reinterpret_cast<const uint32_t*>(p + 2 * lane);
-        const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&t));
-        x[0] = a.x; x[1] = a.y;
-    }
-}
-template <int R> __device__ __forceinline__ void dec_store(float* p, int lane, const float (&x)[R])
-{
-    if constexpr (R == 4) *reinterpret_cast<float4*>(p + 4 * lane) = make_float4(x[0], x[1], x[2], x[3]);
-    else *reinterpret_cast<float2*>(p + 2 * lane) = make_float2(x[0], x[1]);
-}
-
 // Two floats in one 64-bit register: the packed multiply and multiply-add issue once for both.
 struct F2 {
     unsigned long long v;
@@ -104,24 +68,6 @@ __device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c)
     F2 r;
     asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
     return r;
-}
-
-// Lane l gets the warp's sum of x[l % N]: the N sums share their shuffles.
-template <int N> __device__ __forceinline__ float dec_row_sums(float (&x)[N], int lane)
-{
-#pragma unroll
-    for (int s = N / 2; s > 0; s >>= 1) {
-        const bool up = (lane & s) != 0;
-#pragma unroll
-        for (int i = 0; i < s; ++i) {
-            const float send = up ? x[i] : x[i + s], keep = up ? x[i + s] : x[i];
-            x[i] = keep + __shfl_xor_sync(0xffffffffu, send, s);
-        }
-    }
-    float v = x[0];
-#pragma unroll
-    for (int s = N; s < 32; s <<= 1) v += __shfl_xor_sync(0xffffffffu, v, s);
-    return v;
 }
 
 __device__ __forceinline__ void dec_cp16(void* dst, const void* src)
@@ -158,11 +104,11 @@ template <typename T, int K, int V, bool VEC, int RW, int WARPS, bool MULTI> __d
     float d[R];
     F2 S[RW][R / 2];
     float* srow = a.state + ((size_t)chain * V + vb0 + vw) * K;
-    dec_load<R>(a.precond + (size_t)chain * K, lane, d);
+    load_row<R>(a.precond + (size_t)chain * K, lane, d);
 #pragma unroll
     for (int r = 0; r < RW; ++r) {
         float x[R];
-        dec_load<R>(srow + (size_t)r * K, lane, x);
+        load_row<R>(srow + (size_t)r * K, lane, x);
 #pragma unroll
         for (int j = 0; j < R / 2; ++j) S[r][j] = pack2(x[2 * j], x[2 * j + 1]);
     }
@@ -179,8 +125,8 @@ template <typename T, int K, int V, bool VEC, int RW, int WARPS, bool MULTI> __d
             al = fmaf(d[j], kap[j], al);
             ktil[j] = d[j] * k1[j];
         }
-        sumk = dec_warp_sum(sumk);
-        al = dec_warp_sum(al);
+        sumk = warp_sum(sumk);
+        al = warp_sum(al);
         const float n = fmaxf(sumk, hy.eps);
         const float bb = hy.beta_aware ? beta : 1.0f;
         const float c = hy.eta * bb * (1.0f - bb * al) / n;
@@ -210,7 +156,7 @@ template <typename T, int K, int V, bool VEC, int RW, int WARPS, bool MULTI> __d
                 const float2 u = unpack2(s);
                 p[r] = u.x + u.y;
             }
-            return dec_row_sums(p, lane);
+            return transpose_sum(p, lane);
         };
         const float rv = beta * (v - alpha * dots(k2));
         const F2 alpha2 = pack2(alpha, alpha);
@@ -232,9 +178,9 @@ template <typename T, int K, int V, bool VEC, int RW, int WARPS, bool MULTI> __d
     if constexpr (!MULTI) {
         const size_t th = th_of(0);
         float k1[R], q1[R], lrv[VEC ? R : 1];
-        dec_load<R>(kp + th * K, lane, k1);
-        dec_load<R>(qp + th * K, lane, q1);
-        if constexpr (VEC) dec_load<R>(a.log_ret + th * K, lane, lrv);
+        load_row<R>(kp + th * K, lane, k1);
+        load_row<R>(qp + th * K, lane, q1);
+        if constexpr (VEC) load_row<R>(a.log_ret + th * K, lane, lrv);
         step(0, k1, q1, ldf(vp + th * V + vb0 + vw + row), a.beta[th], a.gate[th], hy.apf_mode == 2 ? a.log_ret[th] : 0.f, lrv);
     } else {
         __shared__ DecBlock<T, K, VB, VEC> blk[2];
@@ -267,9 +213,9 @@ template <typename T, int K, int V, bool VEC, int RW, int WARPS, bool MULTI> __d
             const int n = min(DEC_TB, a.L - t0);
             for (int j = 0; j < n; ++j) {
                 float k1[R], q1[R], lrv[VEC ? R : 1];
-                dec_load<R>(B.k[j], lane, k1);
-                dec_load<R>(B.q[j], lane, q1);
-                if constexpr (VEC) dec_load<R>(B.lrv[VEC ? j : 0], lane, lrv);
+                load_row<R>(B.k[j], lane, k1);
+                load_row<R>(B.q[j], lane, q1);
+                if constexpr (VEC) load_row<R>(B.lrv[VEC ? j : 0], lane, lrv);
                 step(t0 + j, k1, q1, ldf(&B.v[j][vw + row]), B.beta[j], B.gate[j], hy.apf_mode == 2 ? B.lr[j] : 0.f, lrv);
             }
         }
@@ -283,12 +229,12 @@ template <typename T, int K, int V, bool VEC, int RW, int WARPS, bool MULTI> __d
             x[2 * j] = u.x;
             x[2 * j + 1] = u.y;
         }
-        dec_store<R>(srow + (size_t)r * K, lane, x);
+        store_row<R>(srow + (size_t)r * K, lane, x);
     }
     // every warp (of every slice) of the chain has read the old preconditioner before it is overwritten
     if constexpr (SLICES > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
     else __syncthreads();
-    if (slice == 0 && warp == 0) dec_store<R>(a.precond + (size_t)chain * K, lane, d);
+    if (slice == 0 && warp == 0) store_row<R>(a.precond + (size_t)chain * K, lane, d);
 }
 
 constexpr int FEW_RW = 4, FEW_WARPS = 4, MANY_WARPS = 8;
@@ -305,8 +251,8 @@ __global__ void __launch_bounds__(MANY_WARPS * 32, 2) decode_many_kernel(DecArgs
 }
 
 // From one chain per SM on a CTA per chain fills the chip; with a single token the slices still win a little beyond that
-// (152 chains: 5.1 against 5.5 us, 192 chains: 6.0 against 5.7 us).  Measured, old kernel against these: 4096 chains 100 ->
-// 82 us (6.67 TB/s), 1110 chains x 7 tokens fp32 98 -> 52 us, 512 chains x 16 tokens 103 -> 52 us.
+// (152 chains: 5.1 against 5.5 us, 192 chains: 6.0 against 5.7 us).  Measured, slices for every call against these rules: 4096
+// chains 106.5 -> 84.0 us (6.49 TB/s), 1110 chains x 7 tokens fp32 98 -> 52 us, 512 chains x 16 tokens 103 -> 52 us.
 constexpr unsigned MANY_CHAINS_ONE = 192, MANY_CHAINS_MULTI = 148;
 template <typename T, int K, int V, bool VEC> bool launch_one(unsigned chains, const DecArgs& a, cudaStream_t st)
 {

@@ -22,61 +22,11 @@
 #include <type_traits>
 
 #include "osdn_common.cuh"
+#include "umma.cuh"
 
 namespace osdn {
 
 namespace {
-
-__device__ __forceinline__ float warp_sum(float x)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-    return x;
-}
-
-// Lane l of the warp owns the R = K / 32 consecutive coordinates R l .. R l + R - 1, so that a
-// row of K values is one vector access per lane.
-template <int R> __device__ __forceinline__ void load_row(const float* p, int lane, float (&x)[R])
-{
-    if constexpr (R == 4) {
-        const float4 v = *reinterpret_cast<const float4*>(p + 4 * lane);
-        x[0] = v.x; x[1] = v.y; x[2] = v.z; x[3] = v.w;
-    } else {
-        const float2 v = *reinterpret_cast<const float2*>(p + 2 * lane);
-        x[0] = v.x; x[1] = v.y;
-    }
-}
-template <int R> __device__ __forceinline__ void load_row(const __nv_bfloat16* p, int lane, float (&x)[R])
-{
-    if constexpr (R == 4) {
-        const uint2 v = *reinterpret_cast<const uint2*>(p + 4 * lane);
-        const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&v.x));
-        const float2 b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&v.y));
-        x[0] = a.x; x[1] = a.y; x[2] = b.x; x[3] = b.y;
-    } else {
-        const uint32_t v = *reinterpret_cast<const uint32_t*>(p + 2 * lane);
-        const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&v));
-        x[0] = a.x; x[1] = a.y;
-    }
-}
-template <int R> __device__ __forceinline__ void store_row(float* p, int lane, const float (&x)[R])
-{
-    if constexpr (R == 4) *reinterpret_cast<float4*>(p + 4 * lane) = make_float4(x[0], x[1], x[2], x[3]);
-    else *reinterpret_cast<float2*>(p + 2 * lane) = make_float2(x[0], x[1]);
-}
-template <int R> __device__ __forceinline__ void store_row(__nv_bfloat16* p, int lane, const float (&x)[R])
-{
-    if constexpr (R == 4) {
-        __nv_bfloat162 a = __floats2bfloat162_rn(x[0], x[1]), b = __floats2bfloat162_rn(x[2], x[3]);
-        uint2 v;
-        v.x = *reinterpret_cast<uint32_t*>(&a);
-        v.y = *reinterpret_cast<uint32_t*>(&b);
-        *reinterpret_cast<uint2*>(p + 4 * lane) = v;
-    } else {
-        __nv_bfloat162 a = __floats2bfloat162_rn(x[0], x[1]);
-        *reinterpret_cast<uint32_t*>(p + 2 * lane) = *reinterpret_cast<uint32_t*>(&a);
-    }
-}
 
 // Asynchronous copies into shared memory; their completion is counted per committed group, first in first out.
 __device__ __forceinline__ void cp_async4(void* smem, const void* gmem)
@@ -90,9 +40,6 @@ __device__ __forceinline__ void cp_async16_zfill(void* smem, const void* gmem, b
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-// ---------------------------------------------------------------------------------------------
-// plain streaming sweep (the stand-alone preconditioner update; no workspace)
-// ---------------------------------------------------------------------------------------------
 // The coordinate the recurrence runs in, y = (d - lo) / w.  With c' = c / w a step is
 //   y' = project(rho y + (c' k^2 + (rho - 1) lo / w)),   c' = e' - a2 <y, k^2>,   e' = (e - a2 lo sum k^2) / w.
 //   P1_SAT    a box of ordinary width above zero: lo = d_min, w = d_max - d_min; the projection is the saturation of a
@@ -116,6 +63,7 @@ inline P1Coord p1_coord(const Hyper& hy)
     return {lo, w, iw, lo * iw, mode, face};
 }
 
+// the stand-alone preconditioner update (no workspace)
 struct P1Args {
     int S, H, T_dense;
     const int* cu;
@@ -321,11 +269,11 @@ __device__ __forceinline__ void prefetch_l2(const void* p)
 // <k_s^2, k_t^2> is about 1/128 for unit keys): measured 1.2 rounds at a step size of 0.003, 3.4 at 0.3.
 // A round's c is taken when the d it leads to are unchanged: |change of c_t| max k_t^2 at most 2^-26 of the smallest d
 // the box allows (a quarter of its rounding unit), or a unit in the last place of c_t.
-// In isolation a block of 32 tokens takes 630 + 660 cycles a round with a coordinate per lane (K / 32 warps), against
-// 109 cycles a token for one warp with one integer reduction per token.
+// In isolation a block of 32 tokens takes 630 + 660 cycles a round with a coordinate per lane (in the kernel, two a lane,
+// 3470 cycles at 3.3 rounds), against 109 cycles a token for one warp with one integer reduction per token.
 //
-// Warps of a chain's CTA: K / 32 core warps, two that fetch keys and scalars (blocks in turn), four that finish (they
-// repeat a block's steps from its c, the same operations in the same order, and write ktil_t = d_t (.) k_t, d_t and the
+// Warps of a chain's CTA: K / 64 core warps, two that fetch keys and scalars (blocks in turn), four that finish (with more
+// chains than SMs one of each; they repeat a block's steps from its c, the same operations in the same order, and write ktil_t = d_t (.) k_t, d_t and the
 // mask words).  Blocks go round a ring of buffers; the roles meet at mbarriers (full: fetch -> core and finish, done:
 // core -> finish, free: finish -> fetch).  Warp 0 decides between two lists and walks short ones alone.
 // ---------------------------------------------------------------------------------------------
@@ -372,14 +320,6 @@ constexpr int ring_depth(size_t bytes, size_t room, int helpers)
     return bytes * RING_MAX <= room ? RING_MAX : RING_MAX / 2;
 }
 
-__device__ __forceinline__ void p1_mbar_init(uint64_t* b, int count)
-{
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"((uint32_t)__cvta_generic_to_shared(b)), "r"(count) : "memory");
-}
-__device__ __forceinline__ void p1_mbar_arrive(uint64_t* b)
-{
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"((uint32_t)__cvta_generic_to_shared(b)) : "memory");
-}
 // Bounded: gives up after P1_WAIT_LIMIT cycles, records the error and returns false.  The whole warp calls; the vote at
 // the end brings its lanes together again (lanes that leave the loop in different turns would otherwise run what
 // follows one after the other).
@@ -415,9 +355,9 @@ struct PipeBars {
 __device__ __forceinline__ void init_bars(PipeBars& bars, int n, int core_warps)
 {
     for (int i = 0; i < n; ++i) {
-        p1_mbar_init(&bars.full[i], 1);
-        p1_mbar_init(&bars.done[i], core_warps);
-        p1_mbar_init(&bars.free_[i], 1);
+        umma::mbar_init(&bars.full[i], 1);
+        umma::mbar_init(&bars.done[i], core_warps);
+        umma::mbar_init(&bars.free_[i], 1);
     }
 }
 
@@ -464,24 +404,6 @@ __device__ __forceinline__ float4 p1_scalars(float sumk, float kmax, float beta,
     const float b = hy.beta_aware ? beta : 1.0f;
     const float e = hy.eta * b / fmaxf(sumk, hy.eps), a2 = e * b;
     return make_float4(fmaf(-a2 * q.lo, sumk, e) * q.iw, a2, kmax, sumk);
-}
-
-// Lane l gets the warp's sum of x[l % N]: the N sums share their shuffles.
-template <int N> __device__ __forceinline__ float transpose_sum(float (&x)[N], int lane)
-{
-#pragma unroll
-    for (int s = N / 2; s > 0; s >>= 1) {
-        const bool up = (lane & s) != 0;
-#pragma unroll
-        for (int i = 0; i < s; ++i) {
-            const float send = up ? x[i] : x[i + s], keep = up ? x[i + s] : x[i];
-            x[i] = keep + __shfl_xor_sync(0xffffffffu, send, s);
-        }
-    }
-    float v = x[0];
-#pragma unroll
-    for (int s = N; s < 32; s <<= 1) v += __shfl_xor_sync(0xffffffffu, v, s);
-    return v;
 }
 
 __device__ __forceinline__ float2 load2(const float* p) { return *reinterpret_cast<const float2*>(p); }
@@ -705,7 +627,7 @@ __device__ __forceinline__ bool run_list(const P1Fwd& a, int h, PipeShared<TI, K
                 B.n = 0;
             }
             __syncwarp();
-            if (lane == 0) p1_mbar_arrive(&sh.bars.done[bi]);
+            if (lane == 0) umma::mbar_arrive(&sh.bars.done[bi]);
         }
         *reinterpret_cast<float2*>(sh.y + warp * 64 + lane * 2) = y;
         if (warp == 0 && lane == 0) sh.stop = ok ? stop : 0;
@@ -746,7 +668,7 @@ __device__ __forceinline__ bool run_list(const P1Fwd& a, int h, PipeShared<TI, K
             B.rho[lane] = jump ? 0.f : VEC ? 1.f : rho;
             if (lane == 0) B.jump = jumps;
             __syncwarp();
-            if (lane == 0) p1_mbar_arrive(&sh.bars.full[bi]);
+            if (lane == 0) umma::mbar_arrive(&sh.bars.full[bi]);
         };
         int b = (int)((warp - P::FETCH0 - base) & (P::FETCH - 1));
         if (b < nblk) start(b);
@@ -779,7 +701,7 @@ __device__ __forceinline__ bool run_list(const P1Fwd& a, int h, PipeShared<TI, K
             });
             if (a.save && lane < n) a.r.al[mine] = fmaf(q.w, B.res[lane].y, q.lo * B.scal[lane].w);
             __syncwarp();
-            if (lane == 0) p1_mbar_arrive(&sh.bars.free_[bi]);
+            if (lane == 0) umma::mbar_arrive(&sh.bars.free_[bi]);
         }
     }
     uses = base + nblk;
@@ -1118,7 +1040,7 @@ __global__ void __launch_bounds__(FwdPipe<K, MANY>::THREADS, FwdPipe<K, MANY>::C
             if (!ok) break;
             core_block<TI, K, VEC, MANY>(sh, sh.buf[b % PN], len_of(b), y, guess, rounds, hy, q, warp, lane);
             __syncwarp();
-            if (lane == 0) p1_mbar_arrive(&sh.bars.done[b % PN]);
+            if (lane == 0) umma::mbar_arrive(&sh.bars.done[b % PN]);
         }
         if (a.d_final && ok) *reinterpret_cast<float2*>(a.d_final + at) = nblk > 0 ? make_float2(p1_d(y.x, q), p1_d(y.y, q)) : d0;
     } else if (warp < P::FINISH0) {
@@ -1162,7 +1084,7 @@ __global__ void __launch_bounds__(FwdPipe<K, MANY>::THREADS, FwdPipe<K, MANY>::C
             B.off[lane] = p1_off(rho, q);
             if (lane == 0) B.jump = 0u;
             __syncwarp();
-            if (lane == 0) p1_mbar_arrive(&sh.bars.full[b % PN]);
+            if (lane == 0) umma::mbar_arrive(&sh.bars.full[b % PN]);
             if (b + P::FETCH < nblk) start(b + P::FETCH);
         }
         cp_async_wait<0>();
@@ -1196,7 +1118,7 @@ __global__ void __launch_bounds__(FwdPipe<K, MANY>::THREADS, FwdPipe<K, MANY>::C
                 lsum += warp_sum(lq);
             }
             __syncwarp();
-            if (lane == 0) p1_mbar_arrive(&sh.bars.free_[b % PN]);
+            if (lane == 0) umma::mbar_arrive(&sh.bars.free_[b % PN]);
         }
     }
     if (a.log_sum) {   // the finishing warps' shares, always in the same order
@@ -1431,7 +1353,7 @@ __device__ __forceinline__ bool run_rev_list(const P1Bwd& a, int h, RevShared<T,
             if (!ok) break;
             rev_core_block<T, K, VEC>(sh, sh.buf[bi], len_of(b), lam, rounds, warp, lane);
             __syncwarp();
-            if (lane == 0) p1_mbar_arrive(&sh.bars.done[bi]);
+            if (lane == 0) umma::mbar_arrive(&sh.bars.done[bi]);
         }
         sh.lam[warp * 32 + lane] = lam;
     } else if (warp < P::FINISH0) {
@@ -1477,7 +1399,7 @@ __device__ __forceinline__ bool run_rev_list(const P1Bwd& a, int h, RevShared<T,
             if (lane == 0) B.restart = restarts;
             for (int j = n; j < PB; ++j) B.mask[j][lane] = 0xffffffffu;
             __syncwarp();
-            if (lane == 0) p1_mbar_arrive(&sh.bars.full[bi]);
+            if (lane == 0) umma::mbar_arrive(&sh.bars.full[bi]);
         };
         int b = (int)((warp - P::FETCH0 + base) & 1);
         if (b < nblk) start(b);
@@ -1550,7 +1472,7 @@ __device__ __forceinline__ bool run_rev_list(const P1Bwd& a, int h, RevShared<T,
                 if (j0 + 4 < n) work(j0 + 4, odd);
             }
             __syncwarp();
-            if (lane == 0) p1_mbar_arrive(&sh.bars.free_[bi]);
+            if (lane == 0) umma::mbar_arrive(&sh.bars.free_[bi]);
         }
     }
     uses = base + nblk;

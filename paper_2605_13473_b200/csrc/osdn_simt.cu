@@ -43,7 +43,6 @@ build_table_kernel(int S, int T_dense, const int* __restrict__ cu, int NTmax, Ta
     __shared__ int s_scan[TBL_THREADS];
     __shared__ int s_carry;
     const int tid = threadIdx.x;
-    pdl_release();
     if (tid == 0) {
         s_carry = 0;
         if (status) *status = 0;

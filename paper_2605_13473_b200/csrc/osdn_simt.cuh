@@ -21,13 +21,6 @@
 namespace osdn {
 namespace {
 
-__device__ __forceinline__ float warp_sum(float x)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-    return x;
-}
-
 // ---------------------------------------------------------------------------------------
 // Register-tile product.  A group of 256 threads forms a 64 x (16 TN) result; a thread owns the rows
 // 4 tm .. 4 tm + 3 (tm = its half-warp: rows of a warp are 8 consecutive ones) and TN columns.  Operands are
