@@ -250,14 +250,16 @@ __global__ void __launch_bounds__(MANY_WARPS * 32, 2) decode_many_kernel(DecArgs
     decode_body<T, K, V, VEC, V / MANY_WARPS, MANY_WARPS, MULTI>(a);
 }
 
-// From one chain per SM on a CTA per chain fills the chip; with a single token the slices still win a little beyond that
-// (152 chains: 5.1 against 5.5 us, 192 chains: 6.0 against 5.7 us).  Measured, slices for every call against these rules: 4096
-// chains 106.5 -> 84.0 us (6.49 TB/s), 1110 chains x 7 tokens fp32 98 -> 52 us, 512 chains x 16 tokens 103 -> 52 us.
-constexpr unsigned MANY_CHAINS_ONE = 192, MANY_CHAINS_MULTI = 148;
+// From about two chains to three SMs on a CTA per chain is the faster one: it has no slices to wait for one another.  Measured
+// in a graph, K = V = 128, slices against a CTA per chain, us: one token 64 chains 2.96 / 3.40, 96 chains 3.35 / 3.42, 112
+// chains 3.92 / 3.68, 144 chains 5.09 / 3.92; 7 tokens 64 chains 7.6 / 9.3, 96 chains 9.6 / 9.4, 128 chains 13.4 / 9.5.  Slices
+// for every call against these rules: 4096 chains 106.5 -> 84.0 us (6.49 TB/s), 1110 chains x 7 tokens fp32 98 -> 52 us, 512
+// chains x 16 tokens 103 -> 52 us.
+constexpr unsigned MANY_CHAINS = 104;
 template <typename T, int K, int V, bool VEC> bool launch_one(unsigned chains, const DecArgs& a, cudaStream_t st)
 {
     constexpr unsigned SLICES = V / (FEW_RW * FEW_WARPS);
-    if (chains >= (a.L > 1 ? MANY_CHAINS_MULTI : MANY_CHAINS_ONE)) {
+    if (chains >= MANY_CHAINS) {
         if (a.L > 1) decode_many_kernel<T, K, V, VEC, true><<<chains, MANY_WARPS * 32, 0, st>>>(a);
         else decode_many_kernel<T, K, V, VEC, false><<<chains, MANY_WARPS * 32, 0, st>>>(a);
     } else {

@@ -170,10 +170,10 @@ def test_backward_twice_on_the_same_residuals():
         assert not torch.isnan(x.float()).any() and torch.equal(x, y)
 
 
-@pytest.mark.parametrize("B,H,L", [(49, 3, 8), (37, 4, 9), (191, 1, 1), (192, 1, 1), (50, 3, 17)])
+@pytest.mark.parametrize("B,H,L", [(49, 3, 8), (37, 4, 9), (191, 1, 1), (192, 1, 1), (50, 3, 17), (103, 1, 1), (104, 1, 1), (103, 1, 9), (52, 2, 9)])
 @pytest.mark.parametrize("io,K,V,apf", [("bf16", 128, 128, 1), ("fp32", 64, 128, 2), ("fp32", 128, 64, 3)])
 def test_decode_on_both_sides_of_its_dispatch(B, H, L, io, K, V, apf):
-    """147 / 148 chains with several tokens, 191 / 192 with one; blocks of eight tokens: at, one past, two and one past."""
+    """103 / 104 chains, with one token and several (and well beyond); blocks of eight tokens: at, one past, two and one past."""
     hy = OsdnHyper(eta=0.3, apf_mode=apf)
     inp = draw(f"dec_{B}_{L}", 7400 + B + L, [L] * B, H, K, V, io, dense_B=B, hyper=hy, with_log_ret=apf >= 2, with_state=True)
     p = binding.make_params(B=B, T=L, H=H, K=K, V=V, io_dtype=io, hyper=hy)
