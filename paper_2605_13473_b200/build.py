@@ -50,7 +50,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
         _build_call(False)
         return LIB
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
-    cmd = [nvcc, "-std=c++17", "-O3", "-lineinfo", "-gencode", "arch=compute_100a,code=sm_100a",
+    cmd = [nvcc, "--threads", "0", "-std=c++17", "-O3", "-lineinfo", "-gencode", "arch=compute_100a,code=sm_100a",
            "-Xcompiler", "-fPIC", "-shared", "-o", LIB] + srcs
     if verbose:
         cmd.insert(1, "-Xptxas")
