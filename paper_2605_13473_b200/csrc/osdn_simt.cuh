@@ -950,11 +950,14 @@ __global__ void __launch_bounds__(K / 64 * 256) chain_wide_kernel(ChainArgs a)
 }
 
 // ---------------------------------------------------------------------------------------
-// chunk-local backward: gradients through P, the state-advance factors, W, U, T, A, gates.
+// chunk-local backward: gradients through P, the state-advance factors, the solve, A, gates.
 //
-// Fourteen products per tile in five phases; in each the two groups of 256 threads form different products.
-// Bound by the FMAs.  k, ktil, q (gated as in the forward), T and the 64 x 64 intermediates sit in shared memory;
-// S, dS, ddU, v and dO are read where they are, by rows that a half-warp shares or by whole lines.
+// With dU = T R, R = diag(beta) (V - gamma (.) K S^T):  dVb = T^T ddU is R's gradient, dA = -strictLower(dVb dU^T) the
+// scores', and dKb = -dVb S the read keys' share of R.  (Gradients of W, U and T, and T^T dT T^T, are never formed: a fifth
+// fewer FMAs than that way, and one phase fewer.)  Ten products per tile in three phases; in each the two groups of 256
+// threads form different ones.  Bound by the FMAs and the shared-memory pipe.  k, ktil, q (gated as in the forward), dU, dVb, T
+// and the 64 x 64 intermediates sit in shared memory; S, dS, ddU, v and dO are read where they are, by rows that a half-warp
+// shares or by whole lines.
 //
 // The gate gradient needs no sums of its own over the score matrices: with
 //   E_i = dq_i (.) q_i + dk_read_i (.) k_i - dktil_i (.) ktil_i     (phase-2 gradients)
@@ -965,7 +968,7 @@ __global__ void __launch_bounds__(K / 64 * 256) chain_wide_kernel(ChainArgs a)
 // the chunk's end takes from the writes, sum over j < i of dKtr_j (.) Ktr_j, is a prefix sum instead of the total less a
 // suffix.
 // ---------------------------------------------------------------------------------------
-template <int K> constexpr size_t local_bwd_smem() { return sizeof(float) * (4 * CH * (K + 4) + 4 * CH * LC); }
+template <int K, int V> constexpr size_t local_bwd_smem() { return sizeof(float) * (3 * CH * (K + 4) + CH * ((K > V ? K : V) + 4) + 4 * CH * LC); }
 template <typename T, int K, int V, bool CG>
 __global__ void __launch_bounds__(CL_NT) chunk_local_bwd_kernel(ChunkArgs a)
 {
@@ -974,11 +977,11 @@ __global__ void __launch_bounds__(CL_NT) chunk_local_bwd_kernel(ChunkArgs a)
     float* sK = sm;                 // as in the forward: channel gate gamma (.) k
     float* sKt = sK + CH * LD;      //                    safe: ktil exp(-G)
     float* sQ = sKt + CH * LD;      //                    gamma (.) q
-    float* sW = sQ + CH * LD;       // dW; channel gate, at the end: dq (.) q + dk (.) k
-    float* sX = sW + CH * LD;       // [64][LC] dU and v (with sDP or sY), dT, then dA * beta_i * gates
-    float* sDP = sX + CH * LC;      // dP * gates
-    float* sY = sDP + CH * LC;      // T^T dT
-    float* sT = sY + CH * LC;       // T.  sY and sT together: channel gate, at the end: dktil (.) ktil
+    float* sW = sQ + CH * LD;       // dVb [64][LU]; channel gate, at the end: dq (.) q + dk (.) k [64][LD]
+    float* sX = sW + CH * (K > V ? LD : LU);   // [64][LC] dA * beta_i * gates; before that, and the space behind it, dU [64][LU]
+    float* sT = sX + 2 * CH * LC;   // T.  Channel gate, at the end, with the space before it: dktil (.) ktil
+    float* sDP = sT + CH * LC;      // dP * gates
+    float* sU = sX;
     __shared__ GateVecs gv;
     __shared__ float sB[3][CH], sE[3][CH];   // channel gate: sE[0] the diagonal of dP
     __shared__ __align__(16) float sRed[PARTS][K], sR[8][K];   // column sums of dS (.) S and of dKtr (.) Ktr
@@ -1005,8 +1008,6 @@ __global__ void __launch_bounds__(CL_NT) chunk_local_bwd_kernel(ChunkArgs a)
     auto L4 = [&](int i, int n) { return ld4(Gg + (CH + i) * K + n); };
     auto expG = [&](int i, int n) { return exp_sum(G4(i, n), L4(i, n)); };
     auto expmG = [&](int i, int n) { return exp_sum(-1.f * G4(i, n), -1.f * L4(i, n)); };
-    float* sU = sX;                                  // dU [64][LU], until X is written
-    float* sV = V == 64 ? sY : sX;                   // v  [64][LU]
 
     bool safe = true;
     if constexpr (CG) safe = __syncthreads_and(threadIdx.x >= K || fabsf(Gg[(CH - 1) * K + (threadIdx.x & (K - 1))]) <= SAFE_RANGE);
@@ -1028,7 +1029,6 @@ __global__ void __launch_bounds__(CL_NT) chunk_local_bwd_kernel(ChunkArgs a)
     for (int e = threadIdx.x; e < CH * CH / 4; e += CL_NT) st4(sT + (e / 16) * LC + (e % 16) * 4, ld4(a.Tm + tile * CH * CH + e * 4));
 #pragma unroll 4
     for (int e = threadIdx.x; e < CH * V / 4; e += CL_NT) st4(sU + e / (V / 4) * LU + e % (V / 4) * 4, ld4(dUg + e * 4));
-    if (V == 64) load_tile<T, V, CL_NT>(sV, LU, static_cast<const T*>(a.v), tok0, len, H, h);
     if constexpr (CG) {
         if (threadIdx.x < CH) gv.beta[threadIdx.x] = threadIdx.x < len ? a.beta[(size_t)(tok0 + threadIdx.x) * H + h] : 0.f;
     } else {
@@ -1040,36 +1040,6 @@ __global__ void __launch_bounds__(CL_NT) chunk_local_bwd_kernel(ChunkArgs a)
 #pragma unroll 8
         for (int v = part; v < V; v += PARTS) s = fmaf(Sg[v * K + n], dSg[v * K + n], s);
         sRed[part][n] = s;
-    }
-    __syncthreads();
-
-    // (1) dP * gates = 1[j<=i] scale dO dU^T               |  dW = -ddU S
-    if (grp == 0) {
-        float acc[4][4];
-        zero(acc);
-        tile_mm<false, true, 4>(acc, 0, V, l, [&](int m, int k) { return dor(m, k); }, [&](int n, int k) { return ld4(sU + n * LU + k); });
-        if constexpr (V == 128) asm volatile("bar.sync 2, 256;" ::: "memory");   // dU reaches into sDP: all of it has been read
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int m = row_of(l, i), n = col_of<true>(l, j);
-                float x = n <= m ? scale * acc[i][j] : 0.f;
-                if constexpr (!CG) x *= expf(fminf(gv.G[m] - gv.G[n], 0.f));
-                else if (n == m) {
-                    sE[0][m] = x;
-                    x = 0.f;
-                }
-                sDP[m * LC + n] = x;
-            }
-    } else {
-        float acc[4][TK];
-        zero(acc);
-        tile_mm<false, false, TK>(acc, 0, V, l, [&](int m, int k) { return ld4(ddUg + m * V + k); }, [&](int k, int n) { return ld4(Sg + k * K + n); });
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int cc = 0; cc < TK; cc += 4) st4(sW + row_of(l, i) * LD + col_of<false>(l, cc), -1.f * quad(acc[i], cc));
     }
     __syncthreads();
 
@@ -1129,7 +1099,41 @@ __global__ void __launch_bounds__(CL_NT) chunk_local_bwd_kernel(ChunkArgs a)
     auto ldKt = [&](int m, int n) { return ld4(sKt + m * LD + n); };
     auto ldQ = [&](int m, int n) { return ld4(sQ + m * LD + n); };
 
-    // (2) dq = gamma (scale dO S) + dP ktil (gated)         |  dT = dW (beta gamma K)^T + ddU (beta V)^T
+    // (1) dVb = T^T ddU ; dv = beta dVb                     |  dP * gates = 1[j<=i] scale dO dU^T
+    if (grp == 0) {
+        float acc[4][TV];
+        zero(acc);
+        tile_mm<true, false, TV>(acc, m_lo, CH, l, [&](int k, int m) { return ld4(sT + k * LC + m); }, [&](int k, int n) { return ld4(ddUg + k * V + n); });
+        row_dots(acc, vr, sB[1]);
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int cc = 0; cc < TV; cc += 4) st4(sW + row_of(l, i) * LU + col_of<false>(l, cc), quad(acc[i], cc));
+        scale_rows(acc, [&](int m, int) { return splat(gv.beta[m]); });
+        store_rows(acc, static_cast<T*>(a.dv), V);
+    } else {
+        float acc[4][4];
+        zero(acc);
+        tile_mm<false, true, 4>(acc, 0, V, l, [&](int m, int k) { return dor(m, k); }, [&](int n, int k) { return ld4(sU + n * LU + k); });
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int m = row_of(l, i), n = col_of<true>(l, j);
+                float x = n <= m ? scale * acc[i][j] : 0.f;
+                if constexpr (!CG) x *= expf(fminf(gv.G[m] - gv.G[n], 0.f));
+                else if (n == m) {
+                    sE[0][m] = x;
+                    x = 0.f;
+                }
+                sDP[m * LC + n] = x;
+            }
+    }
+    __syncthreads();
+
+    float keep[4][TK];   // group 0: dk of the read key; group 1: dktil
+    zero(keep);
+    // (2) dq = gamma (scale dO S) + dP ktil (gated)         |  dA = -strictLower(dVb dU^T), dbeta_i += dA_ij R_ij
     if (grp == 0) {
         float acc[4][TK];
         zero(acc);
@@ -1162,58 +1166,34 @@ __global__ void __launch_bounds__(CL_NT) chunk_local_bwd_kernel(ChunkArgs a)
             }
         }
         store_rows(acc, static_cast<T*>(a.dq), K);
-    } else {
-        float acc[4][4];
-        zero(acc);
-        tile_mm<false, true, 4>(acc, 0, K, l, [&](int m, int k) { return ld4(sW + m * LD + k); }, [&](int n, int k) { return ld4(sK + n * LD + k); });
-        if constexpr (!CG) {
-#pragma unroll
-            for (int j = 0; j < 4; ++j)
-#pragma unroll
-                for (int i = 0; i < 4; ++i) acc[i][j] *= gv.gam[col_of<true>(l, j)];
-        }
-        if constexpr (V == 64) {
-            tile_mm<false, true, 4>(acc, 0, V, l, [&](int m, int k) { return ld4(ddUg + m * V + k); }, [&](int n, int k) { return ld4(sV + n * LU + k); });
-        } else {   // v through sX and sY, 64 columns each
-            const int t = threadIdx.x & 255;
-#pragma unroll 4
-            for (int e = t; e < CH * V / 4; e += 256) {
-                const int i = e / (V / 4), n = e % (V / 4) * 4;
-                st4((n < 64 ? sX : sY) + i * LC + (n & 63), vr(i, n));
-            }
-            asm volatile("bar.sync 1, 256;" ::: "memory");
-            tile_mm<false, true, 4>(acc, 0, V, l, [&](int m, int k) { return ld4(ddUg + m * V + k); },
-                                    [&](int n, int k) { return ld4((k < 64 ? sX : sY) + n * LC + (k & 63)); });
-            asm volatile("bar.sync 1, 256;" ::: "memory");   // v has been read
-        }
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int j = 0; j < 4; ++j) sX[row_of(l, i) * LC + col_of<true>(l, j)] = gv.beta[col_of<true>(l, j)] * acc[i][j];
-    }
-    __syncthreads();
-
-    // (3) dKb = T^T dW (kept by group 0: dk grows from it), dVb = T^T ddU   |  T^T dT ; dKtr = dU dS (kept by group 1)
-    float keep[4][TK];   // group 0: dk of the read key; group 1: dktil
-    zero(keep);
-    if (grp == 0) {
-        auto Tt = [&](int k, int m) { return ld4(sT + k * LC + m); };
-        tile_mm<true, false, TK>(keep, m_lo, CH, l, Tt, [&](int k, int n) { return ld4(sW + k * LD + n); });
-        if constexpr (!CG) scale_rows(keep, [&](int m, int) { return splat(gv.gam[m]); });
+        // dKb = -dVb S (dk grows from it)                   |  dKtr = dU dS (dktil grows from it)
+        tile_mm<false, false, TK>(keep, 0, V, l, [&](int m, int k) { return ld4(sW + m * LU + k); }, [&](int k, int n) { return ld4(Sg + k * K + n); });
+        scale_rows(keep, [&](int m, int) { return splat(CG ? -1.f : -gv.gam[m]); });
         row_dots(keep, ldK, sB[0]);
         scale_rows(keep, [&](int m, int) { return splat(gv.beta[m]); });
-        float acc[4][TV];
-        zero(acc);
-        tile_mm<true, false, TV>(acc, m_lo, CH, l, Tt, [&](int k, int n) { return ld4(ddUg + k * V + n); });
-        row_dots(acc, vr, sB[1]);
-        scale_rows(acc, [&](int m, int) { return splat(gv.beta[m]); });
-        store_rows(acc, static_cast<T*>(a.dv), V);
     } else {
-        float acc[4][4];
-        zero(acc);
-        tile_mm<true, false, 4>(acc, m_lo, CH, l, [&](int k, int m) { return ld4(sT + k * LC + m); }, [&](int k, int n) { return ld4(sX + k * LC + n); });
+        {
+            float acc[4][4];
+            zero(acc);
+            tile_mm<false, true, 4>(acc, 0, V, l, [&](int m, int k) { return ld4(sW + m * LU + k); }, [&](int n, int k) { return ld4(sU + n * LU + k); });
+            asm volatile("bar.sync 1, 256;" ::: "memory");   // dU, whose space X takes, has been read
+            const float* Rg = a.R + tile * CH * CH;
 #pragma unroll
-        for (int i = 0; i < 4; ++i) st4(sY + row_of(l, i) * LC + col_of<false>(l, 0), quad(acc[i], 0));
+            for (int i = 0; i < 4; ++i) {
+                const int m = row_of(l, i);
+                float s = 0.f;
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const int n = col_of<true>(l, j);
+                    float da = n < m ? -acc[i][j] : 0.f;
+                    s = fmaf(da, Rg[m * CH + n], s);
+                    if constexpr (!CG) da *= expf(fminf(gv.G[m] - gv.G[n], 0.f));
+                    sX[m * LC + n] = da * gv.beta[m];
+                }
+                s = half_sum(s);
+                if (l.tn == 0) sB[2][m] = s;
+            }
+        }
         tile_mm<false, false, TK>(keep, 0, V, l, [&](int m, int k) { return ld4(dUg + m * V + k); }, [&](int k, int n) { return ld4(dSg + k * K + n); });
         // towards dktil: rho (.) dKtr; channel gate, safe: gC (.) dKtr, the common factor exp(-G) follows at the end
         if constexpr (!CG) scale_rows(keep, [&](int m, int) { return splat(gv.rho[m]); });
@@ -1239,44 +1219,14 @@ __global__ void __launch_bounds__(CL_NT) chunk_local_bwd_kernel(ChunkArgs a)
             store_rows(keep, a.dktil, K);
             zero(keep);
         }
+        auto dPt = [&](int k, int m) { return ld4(sDP + k * LC + m); };
+        if (!CG || safe) tile_mm<true, false, TK>(keep, m_lo, CH, l, dPt, ldQ);
+        else pair_mm<true, TK>(keep, m_lo, CH, l, [&](int m, int j) { return sDP[j * LC + m]; }, qr, G4, L4);
     }
     __syncthreads();
 
-    // (4) dA = -strictLower(T^T dT T^T), the contraction halved between the groups; dbeta_i += dA_ij R_ij
-    {
-        float acc[4][4];
-        zero(acc);
-        tile_mm<false, true, 4>(acc, grp * 32, grp * 32 + 32, l, [&](int m, int k) { return ld4(sY + m * LC + k); }, [&](int n, int k) { return ld4(sT + n * LC + k); });
-        if (grp == 1)
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) sX[row_of(l, i) * LC + col_of<true>(l, j)] = acc[i][j];
-        __syncthreads();
-        if (grp == 0) {
-            const float* Rg = a.R + tile * CH * CH;
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int m = row_of(l, i);
-                float s = 0.f;
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const int n = col_of<true>(l, j);
-                    float* x = sX + m * LC + n;
-                    float da = n < m ? -(acc[i][j] + *x) : 0.f;
-                    s = fmaf(da, Rg[m * CH + n], s);
-                    if constexpr (!CG) da *= expf(fminf(gv.G[m] - gv.G[n], 0.f));
-                    *x = da * gv.beta[m];
-                }
-                s = half_sum(s);
-                if (l.tn == 0) sB[2][m] = s;
-            }
-        }
-    }
-    __syncthreads();
-
-    // (5) dk (read side) = beta gamma dKb + X ktil (gated)   |  dktil = dKtr part + dP^T q + X^T k (gated)
-    float* sE2 = sY;   // channel gate: dktil (.) ktil, over sY and sT
+    // (3) dk (read side) = beta gamma dKb + X ktil (gated)   |  dktil = dKtr part + dP^T q + X^T k (gated)
+    float* sE2 = sT - CH * LC;   // channel gate: dktil (.) ktil, over the rest of dU and T
     if (grp == 0) {
         auto X = [&](int m, int k) { return ld4(sX + m * LC + k); };
         if constexpr (!CG) {
@@ -1297,15 +1247,8 @@ __global__ void __launch_bounds__(CL_NT) chunk_local_bwd_kernel(ChunkArgs a)
         }
         store_rows(keep, a.dkread, K);
     } else {
-        auto dPt = [&](int k, int m) { return ld4(sDP + k * LC + m); };
-        auto Xt = [&](int k, int m) { return ld4(sX + k * LC + m); };
-        if (!CG || safe) {
-            tile_mm<true, false, TK>(keep, m_lo, CH, l, dPt, ldQ);
-            tile_mm<true, false, TK>(keep, m_lo, CH, l, Xt, ldK);
-        } else {
-            pair_mm<true, TK>(keep, m_lo, CH, l, [&](int m, int j) { return sDP[j * LC + m]; }, qr, G4, L4);
-            pair_mm<true, TK>(keep, m_lo, CH, l, [&](int m, int j) { return sX[j * LC + m]; }, kr, G4, L4);
-        }
+        if (!CG || safe) tile_mm<true, false, TK>(keep, m_lo, CH, l, [&](int k, int m) { return ld4(sX + k * LC + m); }, ldK);
+        else pair_mm<true, TK>(keep, m_lo, CH, l, [&](int m, int j) { return sX[j * LC + m]; }, kr, G4, L4);
         if constexpr (!CG) {
             row_dots(keep, ldKt, sE[2]);
         } else {
@@ -1456,9 +1399,9 @@ int chunk_backward(const osdn_params& p, const Hyper& hy, const WsLayout& L, voi
     ch.D = c.ddU; ch.Sall = c.dSn; ch.Sfin = a.dinit_state;
     ch.status = reinterpret_cast<int*>(w + L.status);
     if (launch_chain<K, V, true, CG>(ch, L.S * p.H, st) < 0) return -1;
-    if (!set_smem(chunk_local_bwd_kernel<T, K, V, CG>, local_bwd_smem<K>())) return -1;
+    if (!set_smem(chunk_local_bwd_kernel<T, K, V, CG>, local_bwd_smem<K, V>())) return -1;
     stage_mark(st, "chunk_local_bwd");
-    chunk_local_bwd_kernel<T, K, V, CG><<<tiles, CL_NT, local_bwd_smem<K>(), st>>>(c);
+    chunk_local_bwd_kernel<T, K, V, CG><<<tiles, CL_NT, local_bwd_smem<K, V>(), st>>>(c);
     return cudaGetLastError() == cudaSuccess ? 3 : -1;
 }
 
