@@ -107,20 +107,6 @@ bool make_token_map(CUtensorMap* m, const void* base, size_t rows, int H)
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// Map over the same kind of tensor for storing dense [64 tokens x 128 features] tiles (no swizzle).
-bool make_store_map(CUtensorMap* m, void* base, size_t rows, int H)
-{
-    PFN_cuTensorMapEncodeTiled enc = get_encoder();
-    if (!enc) return false;
-    cuuint64_t dims[2] = {(cuuint64_t)H * KD, (cuuint64_t)rows};
-    cuuint64_t strides[1] = {(cuuint64_t)H * KD * 2};
-    cuuint32_t box[2] = {KD, 64};
-    cuuint32_t estr[2] = {1, 1};
-    return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-               CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) ==
-           CUDA_SUCCESS;
-}
-
 __device__ __forceinline__ uint8_t* align1024(uint8_t* p)
 {
     return reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(p) + 1023) & ~uintptr_t(1023));
@@ -1452,19 +1438,17 @@ __device__ __forceinline__ void chain_bwd_role(const CUtensorMap& tmDO, const CU
 
 // ---------------------------------------------------------------------------------------------
 // chunk-local backward.  Feature-major ("transposed") accumulators: lane = feature, column = token.
-//   phase A : dP' = dO dU^T ; dQ1^T = S^T dO^T ; dKtr^T = dS^T dU ; dW^T = -S^T ddU
-//             (reads only what the chain kernels and the caller wrote: issued a tile ahead)
-//   phase B : dT = (dW K^T) beta gamma + (ddU V^T) beta ; dKb^T = dW^T T ; dVb^T = ddU^T T ;
-//             dq2^T = Ktil^T M1^T ; dktil^T = Q^T M1            (M1 = scale Gamma (.) lower(dP'))
-//             dbeta_j += sum_i T_ij (gamma_j dW K^T + ddU V^T)_ij
-//   phase C : Y = T^T dT ; rawkk = K Ktil^T
-//   phase D : Z = Y T^T, dA = -strictLower(Z), M2 = dA beta_i Gamma_ij, dbeta_i += sum_j dA_ij Gamma_ij rawkk_ij
-//   phase E : dktil^T += K^T M2 ; dkr^T = Ktil^T M2^T
-//   final   : dq = scale gamma dQ1 + dq2 ; dktil += rho dKtr ; dk_read = dkr + beta gamma dKb ;
-//             dv = beta dVb ; dgate from the products of the gradients with their inputs
+// With dU = T R, R = diag(beta) (V - gamma K S^T):  dL/dR = T^T ddU =: dVb, dL/dA = -strictLower(dVb dU^T).
+//   phase A : dVb^T = ddU^T T ; dP' = dO dU^T ; dQ1^T = S^T dO^T ; dKtr^T = dS^T dU
+//             (reads only what the chain kernels and the caller wrote: issued ahead)
+//   phase B : dA = -strictLower(dVb dU^T) ; dKb^T = -S^T dVb^T ; dq2^T = Ktil^T M1^T ; dktil^T = Q^T M1
+//             (M1 = scale Gamma (.) lower(dP'))
+//   phase C : dktil^T += K^T M2 ; dkr^T = Ktil^T M2'^T      (M2' = dA (.) Gamma, M2 = diag(beta) M2')
+//   final   : dq = scale gamma dQ1 + dq2 ; dv = beta dVb ; dktil += rho dKtr ; dk_read = beta (gamma dKb + dkr) ;
+//             dbeta = <dVb, v> + <gamma dKb + dkr, k> ; dgate from the products of the gradients with their inputs
 // ---------------------------------------------------------------------------------------------
 struct TcChunkBwdArgs {
-    int H, ntiles, nseq;
+    int H, nseq;
     Table tab;
     const float *beta, *gate;
     float scale, d_min;
@@ -1475,779 +1459,656 @@ struct TcChunkBwdArgs {
     int* status;
 };
 
-constexpr int CBW_THREADS = 512;   // 16 warps = 4 lane quadrants x 4 column groups
+constexpr int CBW_WARPS = 16, CBW_THREADS = CBW_WARPS * 32, CBW_MMA_WARP = 16, CBW_PROD_WARP = 17;
+static_assert((CBW_PROD_WARP + 1) * 32 == CBK_THREADS, "the chunk-local role takes every warp of the CTA");
 constexpr uint32_t R_Q = 0, R_K = 16384, R_KT = 32768, R_V = 49152, R_DO = 65536, R_DU = 81920, R_DDU = 98304,
-                   R_T = 114688, R_S = 122880, R_DS = 155648, R_RAW = 188416;
-constexpr uint32_t R_DWT = R_DO;                 // dW^T image replaces dO after phase A
-// M1, dT, Y and M2 are live one after the other (each is written once the product that read its
-// predecessor has finished), so they share one 8 KB image behind the fp32 scratch.
-constexpr uint32_t R_IMG = R_RAW + 24576;
-// Output staging ([token][feature] tiles over dead space): dq over V (dead after phase B; dq is complete
-// then and is formed while phase C runs), dv over Q (dead once dq is formed; dv is formed while phase E
-// runs), dk after the last product in a region of its own; the fp32 copies of dk_read and dL/dktil,
-// needed only when some token's preconditioner step was really taken, over T, S and dS.  When every token of a full chunk was
-// skipped, the space of dO, dU, ddU, T, S and dS is therefore never reused inside a tile and the next
-// tile's copies of them start as soon as the last product reading the current ones has finished.
-constexpr uint32_t ST_DQ = R_V, ST_DV = R_Q, ST_DK = R_RAW, ST_DKR = 114688, ST_DKT = 147456;
-constexpr int CBW_STORE_TID = 256;   // the thread that sends the output tiles off (and owns their bulk group)
-constexpr int CBW_QUEUE_TID = 480;   // the thread that talks to the tile queue (a warp that issues no products)
-static_assert(ST_DKT + 32768 <= R_RAW, "fp32 staging tiles must fit below the fp32 scratch");
-constexpr size_t CBW_SMEM = R_RAW + 32768 + 1024;
+                   R_T = 114688, R_S = 122880, R_DS = 155648, R_M2 = 188416, R_M1 = 204800;
+constexpr uint32_t R_DVB = R_DDU;   // the dVb^T image replaces ddU, which only the first product reads
+// Output tiles over dead space: dq over v, dv over dO, dk over the images of phase C.
+constexpr uint32_t ST_DQ = R_V, ST_DV = R_DO, ST_DK = R_M2;
+constexpr size_t CBW_SMEM = R_M1 + 8192 + 1024;
 
-// The chunk-local backward of the tiles drawn from the queue, by the first CBW_THREADS threads of the CTA
-// (their barrier is hardware barrier 1).  `tb`: 512 tensor-memory columns.
+// The chunk-local backward of the tiles drawn from the queue, by all CBK_THREADS threads of the CTA: sixteen epilogue warps
+// (4 lane quadrants x 4 groups of 16 columns), one warp that issues the products, one that talks to the tile queue, copies
+// tiles in and out and finishes the per-token sums.  `tb`: 512 tensor-memory columns.  The roles meet at mbarriers only, each
+// completed once per tile (vec: one of the two):
+//   vec[2] per-token scalars and the tile's coordinates are in shared memory               producer -> all
+//   c, s, tok, v   copies: ddU T dO dU | S dS | q k ktil | v                               producer -> issuer, epilogue
+//   mma[0..3]      dVb, dP' | dA (and dQ1, dKtr) | dKb, dq2, first half of dktil | phase C  tensor core -> epilogue
+//   e_a    images of M1 and dVb written                                                    epilogue -> issuer
+//   e_d    images of M2 written, dv staged, <dS, S> formed                                 epilogue -> issuer, producer
+//   e_f    everything of the tile is read; dq, dk staged, partial sums written             epilogue -> issuer, producer
+// A copy of the next tile is requested as soon as the space that it lands in is dead, the next tile's first products run
+// under this tile's last epilogue.
+// What bounds it: with three dependent phases (five when dL/dT was formed from dW K^T and ddU V^T and carried through
+// T^T . T^T) the tile's copies, 184 KB in and 48 KB out.  Epilogues read the accumulators in the fragment layout of ldmatrix:
+// two packed instructions move what sixteen 2-byte accesses of a lane-per-feature layout did, and a token's sum over
+// the features is three shuffles.
 __device__ __forceinline__ void chunk_bwd_role(const CUtensorMap& tmQ, const CUtensorMap& tmK, const CUtensorMap& tmKt,
                                                const CUtensorMap& tmV, const CUtensorMap& tmDO, const CUtensorMap& tmDQ,
                                                const CUtensorMap& tmDK, const CUtensorMap& tmDV, const TcChunkBwdArgs& a,
                                                uint8_t* sm, uint32_t tb, const TileQueue& tq)
 {
-    // bar_ct: dO and the tiles written by the chain kernels (everything phase A reads);
-    // bar_tok: q, k, ktil, v
-    __shared__ uint64_t bar_ct, bar_tok, bar_mma[5];
-    __shared__ int sNext[4];   // next tile of this CTA: {tile, head, first token, length}; tile -1: not published yet, -2: none left
-    // per-token sums of a tile (two buffers: the sums of a tile are finished while the next tile's phase B runs)
-    __shared__ __align__(16) float sdBv[2][CH], sdGv[2][CH], sRedv[2][CBW_THREADS / 32];
-    // in-chunk gate prefix G_i, gamma_i = exp(G_i), rho_i = exp(G_C - G_i): two buffers, the next tile's
-    // vectors are formed during this tile's last stretch
-    __shared__ __align__(16) float sGv[2][3][CH];
-    // per-token gate and beta and the two skip words of a tile, copied asynchronously one tile ahead
-    // (two buffers; values fetched into registers that early would be spilled, and the spill would wait
-    // for the load)
-    __shared__ __align__(16) float sScal[2][2][CH];
+    __shared__ uint64_t bar_vec[2], bar_c, bar_s, bar_tok, bar_v, bar_zero, bar_mma[4], bar_ea, bar_ed, bar_ef;
+    __shared__ int sInfo[2][4];                            // tile (-1: no more), first token, length, head
     __shared__ unsigned sSkipW[2][2];
-    __shared__ float sRsumv[2];
-    __shared__ __align__(16) float sFirstKt[KD];
+    __shared__ __align__(16) float sVec[2][4][CH];         // G_i, gamma_i = exp(G_i), rho_i = exp(G_C - G_i), beta_i
+    __shared__ float sSum[2][4][2][CH];                    // per quadrant of features: gate and beta terms of every token
+    __shared__ float sRed[2][CBW_WARPS];
 
     const int H = a.H;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int quad = warp & 3, colq = warp >> 2;   // lane quadrant, column group (16 columns each)
-    const int f = quad * 32 + lane;                 // feature (k or v) owned in 128-lane accumulators
-    // 64-row accumulators keep their rows in lanes 0-15 of each quadrant: thread t reads row
-    // quad * 16 + (t & 15), eight columns (threads 16-31 the second eight of the warp's sixteen)
-    const int row64 = quad * 16 + (lane & 15);
-    const int jb = colq * 16 + (lane >> 4) * 8;     // first of the eight columns
-    const uint32_t addr64 = ((uint32_t)(quad * 32) << 16) + colq * 16;
-
     if (tid == 0) {
-        mbar_init(&bar_ct, 1);
-        mbar_init(&bar_tok, 1);
-        // the independent products of a phase are issued by different warps (the issue rate of one
-        // thread, not the tensor pipe, limits these small shapes); each issuer commits for itself
-        const uint32_t issuers[5] = {4, 6, 2, 1, 2};
-        for (int i = 0; i < 5; ++i) mbar_init(&bar_mma[i], issuers[i]);
+        for (uint64_t* b : {&bar_vec[0], &bar_vec[1], &bar_c, &bar_s, &bar_tok, &bar_v, &bar_mma[0], &bar_mma[1], &bar_mma[2], &bar_mma[3]}) mbar_init(b, 1);
+        for (uint64_t* b : {&bar_zero, &bar_ea, &bar_ed, &bar_ef}) mbar_init(b, CBW_WARPS);
         fence_mbar_init();
     }
     tc_fence_before();
-    named_sync(1, CBW_THREADS);
+    __syncthreads();
     tc_fence_after();
-    const uint32_t lane_addr = (uint32_t)(quad * 32) << 16;
 
-    // tensor memory columns
-    const uint32_t cDP = 64, cDQ1 = 128, cDKTR = 192, cDW = 256;                       // phase A
-    const uint32_t cDTA = 320, cDTB = 384, cDKB = 256, cDVB = 64, cDQ2 = 0, cDKT = 448;   // phase B
-    const uint32_t cY = 320, cRAW = 384, cZ = 320, cDKR = 384;                          // phases C, D, E
+    // tensor memory columns (64 each); dkr takes the place of dA
+    const uint32_t cDP = tb, cDQ1 = tb + 64, cDKTR = tb + 128, cDVB = tb + 192;
+    const uint32_t cDA = tb + 256, cDKB = tb + 320, cDQ2 = tb + 384, cDKT = tb + 448, cDKR = cDA;
 
-    // persistent: one CTA per SM walks over the (chunk, head) tiles.  The operands of the next tile
-    // are requested as soon as the shared-memory regions they land in are dead, its per-token scalars
-    // are fetched into registers one tile ahead, and its first products (phase A, which reads only what
-    // the chain kernels and the caller wrote) are issued while the current tile's sums and stores
-    // are still being formed.
-    // Tiles come from the queue the chains fill, in the order they were finished: thread 0 draws a ticket,
-    // looks the slot up (waiting, within a bound, only where nothing else is left to do) and leaves the
-    // tile's coordinates in shared memory for the others.
-    const int total = a.tab.seq_chunk0(a.nseq) * H;   // realised (chunk, head) tiles
-    auto resolve = [&](int v) {   // queue thread only: v = slot value (tile + 1) or 0 (not published)
-        if (!v) { sNext[0] = -1; return; }
-        const int t = v - 1, c = t / H;
-        sNext[0] = t;
-        sNext[1] = t - c * H;
-        sNext[2] = a.tab.chunk_tok0(c);
-        sNext[3] = a.tab.chunk_len(c);
-        fence_proxy_async_all();   // the tile's images are read through the async proxy
-    };
-    auto lookup_blocking = [&](unsigned ticket) {   // queue thread only
-        if (ticket >= (unsigned)total) { sNext[0] = -2; return; }
-        int v = ld_acquire_gpu(tq.slots + ticket);
-        if (!v) {
+    if (warp == CBW_PROD_WARP) {
+        // ------------------------------------------------------------------ producer
+        const int total = a.tab.seq_chunk0(a.nseq) * H;   // realised (chunk, head) tiles
+        struct Tile { int t, h, tok0, len; };
+        auto resolve = [&](int v) {   // v = slot value (tile + 1)
+            Tile x{v - 1, 0, 0, 0};
+            const int c = x.t / H;
+            x.h = x.t - c * H;
+            x.tok0 = a.tab.chunk_tok0(c);
+            x.len = a.tab.chunk_len(c);
+            fence_proxy_async_all();   // the tile's images are read through the async proxy
+            return x;
+        };
+        auto draw = [&]() {
+            unsigned t = 0;
+            if (lane == 0) t = atomicAdd(tq.head, 1u);
+            return t;   // lane 0 only: broadcast where it is used, long after the atomic
+        };
+        // slot of a ticket: 0 where the chains have not published it yet
+        auto look = [&](unsigned ticket) { return ld_acquire_gpu(tq.slots + ticket); };
+        auto look_blocking = [&](unsigned ticket) {
+            int v = look(ticket);
             const long long t0 = clock64();
-            while (!(v = ld_acquire_gpu(tq.slots + ticket))) {
-                if (clock64() - t0 > WAIT_LIMIT_CYCLES || *reinterpret_cast<volatile int*>(a.status) != 0) break;
+            while (!v) {
+                if (clock64() - t0 > WAIT_LIMIT_CYCLES || *reinterpret_cast<volatile int*>(a.status) != 0) {
+                    if (lane == 0) atomicCAS(a.status, 0, ERR_QUEUE);
+                    break;
+                }
                 __nanosleep(64);
+                v = look(ticket);
             }
-            if (!v) atomicCAS(a.status, 0, ERR_QUEUE);
-        }
-        if (!v) { sNext[0] = -2; return; }
-        resolve(v);
-    };
-    // The copies of a tile arrive on one phase of each barrier; the transaction count is announced with
-    // the first group that is issued, whichever that is.
-    constexpr uint32_t CT_TX = 2 * BOX + 16384 + 16384 + 8192 + 32768 + 32768, TOK_TX = 8 * BOX;
-    auto load_kkt = [&](int hh, int t0) {
-        for (int hf = 0; hf < 2; ++hf) {
-            tma_load_2d(sm + R_K + hf * BOX, &tmK, hh * KD + hf * 64, t0, &bar_tok);
-            tma_load_2d(sm + R_KT + hf * BOX, &tmKt, hh * KD + hf * 64, t0, &bar_tok);
-        }
-    };
-    auto load_qv = [&](int hh, int t0) {
-        for (int hf = 0; hf < 2; ++hf) {
-            tma_load_2d(sm + R_Q + hf * BOX, &tmQ, hh * KD + hf * 64, t0, &bar_tok);
-            tma_load_2d(sm + R_V + hf * BOX, &tmV, hh * KD + hf * 64, t0, &bar_tok);
-        }
-    };
-    auto load_dout = [&](int hh, int t0) {
-        for (int hf = 0; hf < 2; ++hf) tma_load_2d(sm + R_DO + hf * BOX, &tmDO, hh * KD + hf * 64, t0, &bar_ct);
-    };
-    auto load_du_ds_s = [&](int t) {
-        bulk_load(sm + R_DU, a.dUT + (size_t)t * 16384, 16384, &bar_ct);
-        bulk_load(sm + R_DS, a.dSn + (size_t)t * 32768, 32768, &bar_ct);
-        bulk_load(sm + R_S, a.Sn + (size_t)t * 32768, 32768, &bar_ct);
-    };
-    auto load_ddu = [&](int t) { bulk_load(sm + R_DDU, a.ddUT + (size_t)t * 16384, 16384, &bar_ct); };
-    auto load_t = [&](int t) { bulk_load(sm + R_T, a.Tm + (size_t)t * 8192, 8192, &bar_ct); };
-    auto fetch_scalars = [&](int t, int hh, int t0, int ln, int buf) {   // tokens beyond the chunk read as zero
-        if (tid < CH) {
-            const bool in = tid < ln;
-            const size_t th = (size_t)(t0 + (in ? tid : 0)) * H + hh;
-            cp_async4_zfill(&sScal[buf][0][tid], a.gate + th, in);
-            cp_async4_zfill(&sScal[buf][1][tid], a.beta + th, in);
-        } else if (tid < CH + 2) {
-            cp_async4_zfill(&sSkipW[buf][tid - CH], a.skipw + (size_t)t * 2 + (tid - CH), true);
-        }
-        cp_async_commit();
-    };
-    // phase A: dP' = dO dU^T ; dQ1^T = S^T dO^T ; dKtr^T = dS^T dU ; dW^T = -S^T ddU  (warps 0-3, one each)
-    auto issue_phase_a = [&](bool go) {
-        if (lane == 0 && warp < 4 && go) {
-            tc_fence_after();
-            if (warp == 0) {   // dP'[i][j] = sum_v dO[i][v] dU[j][v]                               (M = 64)
-                const uint64_t db0 = desc_mnmajor(sm + R_DU, 0);
-                for (int k = 0; k < 8; ++k)
-                    mma_ss(tb + cDP, desc_advance(desc_kmajor(sm + R_DO + (k >> 2) * BOX), 32 * (k & 3)),
-                           desc_advance(db0, 2048 * k), make_idesc(64, 64, IDESC_B_MN), k > 0);
+            return __shfl_sync(0xffffffffu, v, 0);
+        };
+        auto load_tok = [&](const CUtensorMap& m, uint32_t region, const Tile& x, uint64_t* bar) {
+            for (int hf = 0; hf < 2; ++hf) tma_load_2d(sm + region + hf * BOX, &m, x.h * KD + hf * 64, x.tok0, bar);
+        };
+        auto store_tok = [&](const CUtensorMap& m, uint32_t region, const Tile& x) {
+            for (int hf = 0; hf < 2; ++hf) tma_store_2d(&m, x.h * KD + hf * 64, x.tok0, sm + region + hf * BOX);
+        };
+        auto load_t_ds = [&](const Tile& x) {
+            mbar_expect_tx(&bar_c, 8192 + 3 * 16384);
+            bulk_load(sm + R_T, a.Tm + (size_t)x.t * 8192, 8192, &bar_c);
+            mbar_expect_tx(&bar_s, 65536);
+            bulk_load(sm + R_DS, a.dSn + (size_t)x.t * 32768, 32768, &bar_s);
+        };
+        auto load_u_s = [&](const Tile& x) {
+            bulk_load(sm + R_DDU, a.ddUT + (size_t)x.t * 16384, 16384, &bar_c);
+            bulk_load(sm + R_DU, a.dUT + (size_t)x.t * 16384, 16384, &bar_c);
+            bulk_load(sm + R_S, a.Sn + (size_t)x.t * 32768, 32768, &bar_s);
+        };
+        auto load_do = [&](const Tile& x) { load_tok(tmDO, R_DO, x, &bar_c); };
+        auto load_kkq = [&](const Tile& x) {
+            mbar_expect_tx(&bar_tok, 6 * BOX);
+            load_tok(tmK, R_K, x, &bar_tok);
+            load_tok(tmKt, R_KT, x, &bar_tok);
+            load_tok(tmQ, R_Q, x, &bar_tok);
+        };
+        auto load_v = [&](const Tile& x) {
+            mbar_expect_tx(&bar_v, 2 * BOX);
+            load_tok(tmV, R_V, x, &bar_v);
+        };
+        // The next tile's operands on their way into L2 while this one is worked on: most of them were written by the
+        // forward pass and come from HBM.
+        auto warm = [&](const Tile& x) {
+            bulk_prefetch(a.Tm + (size_t)x.t * 8192, 8192);
+            bulk_prefetch(a.dSn + (size_t)x.t * 32768, 32768);
+            bulk_prefetch(a.dUT + (size_t)x.t * 16384, 16384);
+            bulk_prefetch(a.Sn + (size_t)x.t * 32768, 32768);
+            bulk_prefetch(a.ddUT + (size_t)x.t * 16384, 16384);
+            for (int hf = 0; hf < 2; ++hf) {
+                const int c = x.h * KD + hf * 64;
+                tma_prefetch_2d(&tmDO, c, x.tok0);
+                tma_prefetch_2d(&tmK, c, x.tok0);
+                tma_prefetch_2d(&tmKt, c, x.tok0);
+                tma_prefetch_2d(&tmQ, c, x.tok0);
+                tma_prefetch_2d(&tmV, c, x.tok0);
             }
-            if (warp == 1) {   // dQ1^T[k][i] = sum_v S[v][k] dO[i][v]
-                const uint64_t da0 = desc_mnmajor(sm + R_S, 16384);
-                for (int k = 0; k < 8; ++k)
-                    mma_ss(tb + cDQ1, desc_advance(da0, 2048 * k),
-                           desc_advance(desc_kmajor(sm + R_DO + (k >> 2) * BOX), 32 * (k & 3)),
-                           make_idesc(128, 64, IDESC_A_MN), k > 0);
+        };
+        struct Scal { float ga, gb, ba, bb; unsigned w; };
+        auto fetch = [&](const Tile& x) {   // lane: tokens l and l + 32; tokens beyond the chunk read as zero
+            Scal y;
+            const bool in0 = lane < x.len, in1 = lane + 32 < x.len;
+            const size_t th = (size_t)(x.tok0 + lane) * H + x.h, th1 = th + (size_t)32 * H;
+            y.ga = in0 ? a.gate[th] : 0.f;
+            y.gb = in1 ? a.gate[th1] : 0.f;
+            y.ba = in0 ? a.beta[th] : 0.f;
+            y.bb = in1 ? a.beta[th1] : 0.f;
+            y.w = lane < 2 ? a.skipw[(size_t)x.t * 2 + lane] : 0u;
+            return y;
+        };
+        auto publish = [&](const Tile& x, const Scal& y, int buf) {   // x.t < 0: no more tiles
+            if (x.t >= 0) {
+                float sa = y.ga, sb = y.gb;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const float ua = __shfl_up_sync(0xffffffffu, sa, o), ub = __shfl_up_sync(0xffffffffu, sb, o);
+                    if (lane >= o) { sa += ua; sb += ub; }
+                }
+                sb += __shfl_sync(0xffffffffu, sa, 31);
+                const float tot = __shfl_sync(0xffffffffu, sb, 31);
+                float(*v)[CH] = sVec[buf];
+                v[0][lane] = sa;
+                v[0][lane + 32] = sb;
+                v[1][lane] = __expf(sa);
+                v[1][lane + 32] = __expf(sb);
+                v[2][lane] = __expf(tot - sa);
+                v[2][lane + 32] = __expf(tot - sb);
+                v[3][lane] = y.ba;
+                v[3][lane + 32] = y.bb;
+                if (lane < 2) sSkipW[buf][lane] = y.w;
             }
-            if (warp == 2) {   // dKtr^T[k][j] = sum_v dS[v][k] dU[j][v]
-                const uint64_t da0 = desc_mnmajor(sm + R_DS, 16384), db0 = desc_mnmajor(sm + R_DU, 0);
-                for (int k = 0; k < 8; ++k)
-                    mma_ss(tb + cDKTR, desc_advance(da0, 2048 * k), desc_advance(db0, 2048 * k),
-                           make_idesc(128, 64, IDESC_A_MN | IDESC_B_MN), k > 0);
+            if (lane == 0) {
+                sInfo[buf][0] = x.t;
+                sInfo[buf][1] = x.tok0;
+                sInfo[buf][2] = x.len;
+                sInfo[buf][3] = x.h;
             }
-            if (warp == 3) {   // dW^T[k][i] = -sum_v S[v][k] ddU[i][v]
-                const uint64_t da0 = desc_mnmajor(sm + R_S, 16384), db0 = desc_mnmajor(sm + R_DDU, 0);
-                for (int k = 0; k < 8; ++k)
-                    mma_ss(tb + cDW, desc_advance(da0, 2048 * k), desc_advance(db0, 2048 * k),
-                           make_idesc(128, 64, IDESC_A_MN | IDESC_B_MN | IDESC_A_NEG), k > 0);
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&bar_vec[buf]);
+        };
+        // dgate_j is the suffix sum of the per-token terms (the in-chunk prefix G_i collects every g_j with j <= i); the
+        // chunk-level term goes to the last token
+        auto finish_sums = [&](const Tile& x, int buf) {
+            float s[2], b[2];
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const int j = lane + 32 * u;
+                s[u] = (sSum[buf][0][0][j] + sSum[buf][1][0][j]) + (sSum[buf][2][0][j] + sSum[buf][3][0][j]);
+                b[u] = (sSum[buf][0][1][j] + sSum[buf][1][1][j]) + (sSum[buf][2][1][j] + sSum[buf][3][1][j]);
             }
-            mma_commit(&bar_mma[0]);
-        }
-    };
-    auto gate_vectors = [&](int buf) {   // one warp; lane: tokens l and l + 32
-        float sa = sScal[buf][0][lane], sb = sScal[buf][0][lane + 32];
+            float tot = lane < CBW_WARPS ? sRed[buf][lane] : 0.f;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const float ua = __shfl_up_sync(0xffffffffu, sa, o), ub = __shfl_up_sync(0xffffffffu, sb, o);
-            if (lane >= o) { sa += ua; sb += ub; }
-        }
-        sb += __shfl_sync(0xffffffffu, sa, 31);
-        const float tot = __shfl_sync(0xffffffffu, sb, 31);
-        sGv[buf][0][lane] = sa;
-        sGv[buf][0][lane + 32] = sb;
-        sGv[buf][1][lane] = __expf(sa);
-        sGv[buf][1][lane + 32] = __expf(sb);
-        sGv[buf][2][lane] = __expf(tot - sa);
-        sGv[buf][2][lane + 32] = __expf(tot - sb);
-    };
-    // The per-token sums of a tile (gate and beta gradients) are finished one tile later, while the tensor
-    // core works on the next tile's phase B: the partial terms stay in registers until then.
-    float gv[16];       // per column: gate contribution of this thread's feature
-    float rsum = 0.f;
-    bool pend = false;  // the previous tile's sums are still to be finished
-    int p_tok0 = 0, p_h = 0, p_len = 0;
-    auto reduce_sums = [&](int buf) {   // all warps: 32 features of each warp, 16 columns at once
+            for (int o = 16; o > 0; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
+            if (lane == 31) s[1] += tot;
 #pragma unroll
-        for (int step = 0; step < 4; ++step) {   // a lane keeps one half of its columns, hands the other half over
-            const int off = 16 >> step, n = 8 >> step;
-            const bool upper = (lane & off) != 0;
-#pragma unroll
-            for (int i = 0; i < n; ++i) {
-                const float gs = upper ? gv[i] : gv[i + n], gk = upper ? gv[i + n] : gv[i];
-                gv[i] = gk + __shfl_xor_sync(0xffffffffu, gs, off);
+            for (int o = 1; o < 32; o <<= 1) {
+                const float u0 = __shfl_down_sync(0xffffffffu, s[0], o), u1 = __shfl_down_sync(0xffffffffu, s[1], o);
+                if (lane + o < 32) { s[0] += u0; s[1] += u1; }
             }
-        }
-        gv[0] += __shfl_xor_sync(0xffffffffu, gv[0], 1);   // the two lanes that ended up with the same column
-        if ((lane & 1) == 0) atomicAdd(&sdGv[buf][colq * 16 + (lane >> 1)], gv[0]);
+            s[0] += __shfl_sync(0xffffffffu, s[1], 0);
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) rsum += __shfl_xor_sync(0xffffffffu, rsum, o);
-        if (lane == 0) atomicAdd(&sRsumv[buf], rsum);
-    };
-    // one warp: dgate_j is the suffix sum of the per-token terms (the in-chunk prefix G_i collects every
-    // g_j with j <= i); the chunk-level term goes to the last token
-    auto finish_sums = [&](int buf, int t0, int hh, int ln) {
-        float s0 = sdGv[buf][lane], s1 = sdGv[buf][lane + 32];
-        float gl = sScal[buf][0][lane] + sScal[buf][0][lane + 32], tot = lane < CBW_THREADS / 32 ? sRedv[buf][lane] : 0.f;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            gl += __shfl_xor_sync(0xffffffffu, gl, o);
-            tot += __shfl_xor_sync(0xffffffffu, tot, o);
-        }
-        if (lane == 31) s1 += sRsumv[buf] + __expf(gl) * tot;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const float u0 = __shfl_down_sync(0xffffffffu, s0, o), u1 = __shfl_down_sync(0xffffffffu, s1, o);
-            if (lane + o < 32) { s0 += u0; s1 += u1; }
-        }
-        s0 += __shfl_sync(0xffffffffu, s1, 0);
-        if (lane < ln) {
-            const size_t th = (size_t)(t0 + lane) * H + hh;
-            a.dgate[th] = s0;
-            a.dbeta[th] = sdBv[buf][lane];
-        }
-        if (lane + 32 < ln) {
-            const size_t th = (size_t)(t0 + lane + 32) * H + hh;
-            a.dgate[th] = s1;
-            a.dbeta[th] = sdBv[buf][lane + 32];
-        }
-    };
-    uint32_t ph = 0;   // barrier phase parity: number of tiles processed so far, mod 2
-    // queue thread: the ticket of the next tile is drawn a tile ahead and its slot is read at the top of
-    // the tile, long before the value is looked at, so that neither round trip to memory is waited for
-    unsigned ticket_next = 0, ticket_after = 0;
-    int slot_next = 0;
-    if (tid == CBW_QUEUE_TID) {
-        lookup_blocking(atomicAdd(tq.head, 1u));
-        ticket_next = atomicAdd(tq.head, 1u);
-    }
-    named_sync(1, CBW_THREADS);
-    int tile_l = sNext[0], h = sNext[1], tok0 = sNext[2], len = sNext[3];
-    bool a_issued = false;   // phase A of the current tile was issued at the end of the previous one
-    if (tile_l >= 0) {
-        if (tid == 0) {
-            mbar_expect_tx(&bar_ct, CT_TX);
-            load_dout(h, tok0);
-            load_du_ds_s(tile_l);
-            load_ddu(tile_l);
-            load_t(tile_l);
-            mbar_expect_tx(&bar_tok, TOK_TX);
-            load_kkt(h, tok0);
-            load_qv(h, tok0);
-        }
-        fetch_scalars(tile_l, h, tok0, len, 0);
-    }
-    while (tile_l >= 0) {
-    const float* sg = sScal[ph][0];      // log-gates of the chunk's tokens
-    const float* sBeta = sScal[ph][1];
-    float* sdB = sdBv[ph];
-    float* sdG = sdGv[ph];
-    float* sRed = sRedv[ph];
-    const float* sG = sGv[ph][0];
-    const float* sGam = sGv[ph][1];
-    const float* sRho = sGv[ph][2];
-    if (tid < CH) {
-        sdB[tid] = 0.f;
-        sdG[tid] = 0.f;
-    }
-    if (tid == 0) sRsumv[ph] = 0.f;
-    cp_async_wait_all();
-    named_sync(1, CBW_THREADS);
-    // the next tile's slot and the ticket of the tile after it (both values are used much later)
-    if (tid == CBW_QUEUE_TID) {
-        ticket_after = atomicAdd(tq.head, 1u);
-        slot_next = ticket_next < (unsigned)total ? ld_acquire_gpu(tq.slots + ticket_next) : 0;
-    }
-    const unsigned long long sk = (unsigned long long)sSkipW[ph][0] | ((unsigned long long)sSkipW[ph][1] << 32);
-    // Full chunks leave through TMA tile stores (dq, dv always; dk when every token's preconditioner
-    // step was skipped); ragged or mixed chunks are copied row by row.  In the all-skipped case the
-    // space of dO and of each chain tile is not reused by the output staging, so the next tile's copy of
-    // it starts as soon as the last product reading it has finished ("early"), and when that tile is a
-    // full chunk its phase A is issued before this tile's sums are formed ("a_early").
-    const bool full = len == CH;
-    const bool dk_tile = full && sk == ~0ull;
-    if (warp == 0) gate_vectors((int)ph);
-    bool ok = mbar_wait(&bar_ct, ph, a.status, ERR_TMA);
-    if (len < CH) {   // a ragged chunk never had its phase A issued ahead
-        for (int hf = 0; hf < 2; ++hf) zero_tail_rows(sm + R_DO + hf * BOX, len, tid, CBW_THREADS);
-        fence_proxy_async();
-    }
-    tc_fence_before();
-    named_sync(1, CBW_THREADS);
+            for (int u = 0; u < 2; ++u)
+                if (lane + 32 * u < x.len) {
+                    const size_t th = (size_t)(x.tok0 + lane + 32 * u) * H + x.h;
+                    a.dgate[th] = s[u];
+                    a.dbeta[th] = b[u];
+                }
+        };
 
-    // ---- phase A -------------------------------------------------------------------------------
-    if (!a_issued) issue_phase_a(ok);
-    ok = ok && mbar_wait(&bar_mma[0], ph, a.status, ERR_MMA1);
-    tc_fence_after();
-    // epilogue A
-    float gam8[8];   // Gamma_ij = exp(G_i - G_j) for this thread's row and columns, j <= i (else 0)
-    {
-        // dP' -> M1 = scale Gamma (.) lower(dP')
-        const int i = row64;
-        const float Gi = sG[i];
-        {
-            uint32_t r2[8];
-            tmem_ld_half8(tb + cDP + addr64, r2);
-            float m1[8];
-#pragma unroll
-            for (int x = 0; x < 8; ++x) gam8[x] = jb + x <= i ? __expf(Gi - sG[jb + x]) : 0.f;
-            tmem_ld_wait();
-#pragma unroll
-            for (int x = 0; x < 8; ++x) m1[x] = a.scale * gam8[x] * __uint_as_float(r2[x]);
-            *reinterpret_cast<uint4*>(sm + R_IMG + sw128_chunk(i, jb >> 3)) =
-                make_uint4(pack_bf16(m1[0], m1[1]), pack_bf16(m1[2], m1[3]), pack_bf16(m1[4], m1[5]), pack_bf16(m1[6], m1[7]));
+        Tile cur{-1, 0, 0, 0};
+        unsigned ticket = __shfl_sync(0xffffffffu, draw(), 0), after = draw();
+        if (ticket < (unsigned)total) {
+            const int v = look_blocking(ticket);
+            if (v) cur = resolve(v);
         }
-        // dW^T -> bf16 image [rows k][cols i]
-        {
-            uint32_t r[16];
-            tmem_ld16(tb + cDW + lane_addr + colq * 16, r);
-            tmem_ld_wait();
-#pragma unroll
-            for (int c2 = 0; c2 < 2; ++c2)
-                *reinterpret_cast<uint4*>(sm + R_DWT + sw128_chunk(f, colq * 2 + c2)) = make_uint4(
-                    pack_bf16(__uint_as_float(r[c2 * 8 + 0]), __uint_as_float(r[c2 * 8 + 1])),
-                    pack_bf16(__uint_as_float(r[c2 * 8 + 2]), __uint_as_float(r[c2 * 8 + 3])),
-                    pack_bf16(__uint_as_float(r[c2 * 8 + 4]), __uint_as_float(r[c2 * 8 + 5])),
-                    pack_bf16(__uint_as_float(r[c2 * 8 + 6]), __uint_as_float(r[c2 * 8 + 7])));
-        }
-    }
-    ok = ok && mbar_wait(&bar_tok, ph, a.status, ERR_TMA);   // q, k, ktil, v have landed
-    if (len < CH) {
-        for (int hf = 0; hf < 2; ++hf) {
-            zero_tail_rows(sm + R_Q + hf * BOX, len, tid, CBW_THREADS);
-            zero_tail_rows(sm + R_K + hf * BOX, len, tid, CBW_THREADS);
-            zero_tail_rows(sm + R_KT + hf * BOX, len, tid, CBW_THREADS);
-            zero_tail_rows(sm + R_V + hf * BOX, len, tid, CBW_THREADS);
-        }
-    }
-    fence_proxy_async();
-    tc_fence_before();
-    named_sync(1, CBW_THREADS);
-
-    // ---- phase B -------------------------------------------------------------------------------
-    if (lane == 0 && warp < 6 && ok) {
-        tc_fence_after();
-        if (warp == 0) {   // dT_a[i][j] = sum_k dW[i][k] K[j][k]                               (M = 64)
-            const uint64_t da0 = desc_mnmajor(sm + R_DWT, 0);
-            for (int k = 0; k < 8; ++k)
-                mma_ss(tb + cDTA, desc_advance(da0, 2048 * k),
-                       desc_advance(desc_kmajor(sm + R_K + (k >> 2) * BOX), 32 * (k & 3)),
-                       make_idesc(64, 64, IDESC_A_MN), k > 0);
-        }
-        if (warp == 1) {   // dT_b[i][j] = sum_v ddU[i][v] V[j][v]                              (M = 64)
-            const uint64_t da0 = desc_mnmajor(sm + R_DDU, 0);
-            for (int k = 0; k < 8; ++k)
-                mma_ss(tb + cDTB, desc_advance(da0, 2048 * k),
-                       desc_advance(desc_kmajor(sm + R_V + (k >> 2) * BOX), 32 * (k & 3)),
-                       make_idesc(64, 64, IDESC_A_MN), k > 0);
-        }
-        if (warp == 2 || warp == 3) {   // dKb^T[k][j] = sum_i dW^T[k][i] T[i][j] ;  dVb^T[v][j] = sum_i ddU^T[v][i] T[i][j]
-            const uint64_t db0 = desc_mnmajor(sm + R_T, 0);
-            const uint64_t da0 = desc_kmajor(sm + R_DWT), da1 = desc_kmajor(sm + R_DDU);
-            if (warp == 2)
-                for (int k = 0; k < 4; ++k)
-                    mma_ss(tb + cDKB, desc_advance(da0, 32 * k), desc_advance(db0, 2048 * k),
-                           make_idesc(128, 64, IDESC_B_MN), k > 0);
-            else
-                for (int k = 0; k < 4; ++k)
-                    mma_ss(tb + cDVB, desc_advance(da1, 32 * k), desc_advance(db0, 2048 * k),
-                           make_idesc(128, 64, IDESC_B_MN), k > 0);
-        }
-        if (warp == 4 || warp == 5) {   // dq2^T[k][i] = sum_j Ktil[j][k] M1[i][j] ;  dktil^T[k][j] = sum_i Q[i][k] M1[i][j]
-            const uint64_t da0 = desc_mnmajor(sm + R_KT, BOX), da1 = desc_mnmajor(sm + R_Q, BOX);
-            const uint64_t dbk = desc_kmajor(sm + R_IMG), dbm = desc_mnmajor(sm + R_IMG, 0);
-            if (warp == 4)
-                for (int k = 0; k < 4; ++k)
-                    mma_ss(tb + cDQ2, desc_advance(da0, 2048 * k), desc_advance(dbk, 32 * k),
-                           make_idesc(128, 64, IDESC_A_MN), k > 0);
-            else
-                for (int k = 0; k < 4; ++k)
-                    mma_ss(tb + cDKT, desc_advance(da1, 2048 * k), desc_advance(dbm, 2048 * k),
-                           make_idesc(128, 64, IDESC_A_MN | IDESC_B_MN), k > 0);
-        }
-        mma_commit(&bar_mma[1]);
-    }
-    if (pend) reduce_sums((int)(ph ^ 1u));   // the previous tile's per-token sums
-    // <dS, S>_F while the tensor core works on phase B (both images share the same layout)
-    {
-        float p4[4] = {0.f, 0.f, 0.f, 0.f};   // independent partial sums: no chain of dependent multiply-adds
-#pragma unroll
-        for (int it = 0; it < 2048 / CBW_THREADS; ++it) {
-            const int e = tid + it * CBW_THREADS;
-            const uint4 x = *reinterpret_cast<const uint4*>(sm + R_S + e * 16);
-            const uint4 y = *reinterpret_cast<const uint4*>(sm + R_DS + e * 16);
-            const __nv_bfloat162* px = reinterpret_cast<const __nv_bfloat162*>(&x);
-            const __nv_bfloat162* py = reinterpret_cast<const __nv_bfloat162*>(&y);
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const float2 fx = __bfloat1622float2(px[q]), fy = __bfloat1622float2(py[q]);
-                p4[q] = fmaf(fx.x, fy.x, p4[q]);
-                p4[q] = fmaf(fx.y, fy.y, p4[q]);
+        Scal sc{};
+        if (cur.t >= 0) {
+            if (lane == 0) {
+                load_t_ds(cur);
+                load_u_s(cur);
+                load_do(cur);
+                load_kkq(cur);
+                load_v(cur);
             }
+            __syncwarp();
+            sc = fetch(cur);
         }
-        float part = (p4[0] + p4[1]) + (p4[2] + p4[3]);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
-        if (lane == 0) sRed[warp] = part;
-    }
-    named_sync(1, CBW_THREADS);   // every thread is done reading S / dS: phase A has finished, dU, dS and S are dead
-    if (pend && warp == 1) finish_sums((int)(ph ^ 1u), p_tok0, p_h, p_len);
-    // the next tile, if the chains have published it already (asked again at the end of this tile if not);
-    // the queue thread works this out while everybody waits for phase B, the others read it after the next barrier
-    if (tid == CBW_QUEUE_TID) {
-        if (ticket_next >= (unsigned)total) sNext[0] = -2;
-        else resolve(slot_next);
-        if (dk_tile && sNext[0] >= 0 && ok) {
-            mbar_expect_tx(&bar_ct, CT_TX);
-            load_du_ds_s(sNext[0]);
-        }
-    }
-    ok = ok && mbar_wait(&bar_mma[1], ph, a.status, ERR_MMA2);
-    tc_fence_after();
-    {   // dT = dT_a beta_j gamma_j + dT_b beta_j  -> bf16 image [rows i][cols j];
-        // dbeta_j += sum_i T_ij (gamma_j dT_a + dT_b)_ij: beta enters W = T diag(beta gamma) K and
-        // U = T diag(beta) V column by column
-        const int i = row64;
-        uint32_t r1[8], r2[8];
-        tmem_ld_half8(tb + cDTA + addr64, r1);
-        tmem_ld_half8(tb + cDTB + addr64, r2);
-        const uint4 tw = *reinterpret_cast<const uint4*>(sm + R_T + sw128_chunk(i, jb >> 3));
-        const float4 ba = *reinterpret_cast<const float4*>(&sBeta[jb]), bb = *reinterpret_cast<const float4*>(&sBeta[jb + 4]);
-        const float4 ga = *reinterpret_cast<const float4*>(&sGam[jb]), gb = *reinterpret_cast<const float4*>(&sGam[jb + 4]);
-        const float bj[8] = {ba.x, ba.y, ba.z, ba.w, bb.x, bb.y, bb.z, bb.w};
-        const float gj[8] = {ga.x, ga.y, ga.z, ga.w, gb.x, gb.y, gb.z, gb.w};
-        float tij[8];
-        {
-            const __nv_bfloat162* p0 = reinterpret_cast<const __nv_bfloat162*>(&tw);
-#pragma unroll
-            for (int x = 0; x < 4; ++x) {
-                const float2 u0 = __bfloat1622float2(p0[x]);
-                tij[2 * x] = u0.x;
-                tij[2 * x + 1] = u0.y;
+        publish(cur, sc, 0);
+        for (uint32_t it = 0; cur.t >= 0; ++it) {
+            const uint32_t ph = it & 1;
+            const bool full = cur.len == CH;
+            // the next tile, if the chains have published it already (asked again behind this tile if not)
+            ticket = __shfl_sync(0xffffffffu, after, 0);
+            const bool more = ticket < (unsigned)total;
+            if (more) after = draw();
+            Tile next{-1, 0, 0, 0};
+            int v = more ? __shfl_sync(0xffffffffu, look(ticket), 0) : 0;
+            const bool known = v != 0;
+            if (known) {
+                next = resolve(v);
+                if (lane == 0) warm(next);
+                __syncwarp();
+                sc = fetch(next);
             }
-        }
-        tmem_ld_wait();
-        float t[8], cs[8];
-#pragma unroll
-        for (int x = 0; x < 8; ++x) {
-            const float u = gj[x] * __uint_as_float(r1[x]) + __uint_as_float(r2[x]);
-            t[x] = bj[x] * u;
-            cs[x] = tij[x] * u;
-        }
-        *reinterpret_cast<uint4*>(sm + R_IMG + sw128_chunk(i, jb >> 3)) =
-            make_uint4(pack_bf16(t[0], t[1]), pack_bf16(t[2], t[3]), pack_bf16(t[4], t[5]), pack_bf16(t[6], t[7]));
-        // column sums over the 16 rows of a half warp: in each of three steps a lane keeps one half of its
-        // columns and hands the other half to its partner; a last exchange joins the two lanes that end
-        // up with the same column
-#pragma unroll
-        for (int step = 0; step < 3; ++step) {
-            const int off = 8 >> step, n = 4 >> step;
-            const bool upper = (lane & off) != 0;
-#pragma unroll
-            for (int x = 0; x < n; ++x) {
-                const float send = upper ? cs[x] : cs[x + n], keep = upper ? cs[x + n] : cs[x];
-                cs[x] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+            if (known || !more) publish(next, sc, (int)(ph ^ 1u));
+            if (!mbar_wait(&bar_ed, ph, a.status, ERR_MMA2)) break;
+            // dA is formed, hence dVb, dP', dQ1 and dKtr too: T and dS are dead
+            if (lane == 0) {
+                if (full) {
+                    store_tok(tmDV, ST_DV, cur);
+                    bulk_commit();
+                }
+                if (known) load_t_ds(next);
             }
-        }
-        cs[0] += __shfl_xor_sync(0xffffffffu, cs[0], 1);
-        if ((lane & 1) == 0) atomicAdd(&sdB[jb + ((lane & 15) >> 1)], cs[0]);
-    }
-    fence_proxy_async();
-    tc_fence_before();
-    named_sync(1, CBW_THREADS);
-
-    int tile_next = sNext[0], h_next = sNext[1], tok0_next = sNext[2], len_next = sNext[3];
-    const bool next_known = tile_next >= 0;
-    if (next_known) fetch_scalars(tile_next, h_next, tok0_next, len_next, (int)(ph ^ 1u));
-    const bool early = dk_tile && next_known;
-    const bool a_early = early && len_next == CH;
-
-    // ---- phase C: Y[a][b] = sum_i T[i][a] dT[i][b] ; rawkk[i][j] = <k_i, ktil_j> -------------------
-    if (lane == 0 && warp < 2 && ok) {
-        tc_fence_after();
-        if (warp == 0) {
-            const uint64_t da0 = desc_mnmajor(sm + R_T, 0), db0 = desc_mnmajor(sm + R_IMG, 0);
-            for (int k = 0; k < 4; ++k)
-                mma_ss(tb + cY, desc_advance(da0, 2048 * k), desc_advance(db0, 2048 * k),
-                       make_idesc(64, 64, IDESC_A_MN | IDESC_B_MN), k > 0);
-        } else {
-            for (int k = 0; k < 8; ++k)   // (M = 64)
-                mma_ss(tb + cRAW, desc_advance(desc_kmajor(sm + R_K + (k >> 2) * BOX), 32 * (k & 3)),
-                       desc_advance(desc_kmajor(sm + R_KT + (k >> 2) * BOX), 32 * (k & 3)), make_idesc(64, 64), k > 0);
-        }
-        mma_commit(&bar_mma[2]);
-        if (early && warp == 0) {   // phase B has finished: ddU and the dW^T image (in the space of dO) are dead
-            load_ddu(tile_next);
-            load_dout(h_next, tok0_next);
-        }
-    }
-    // dq = scale gamma dQ1 + dq2 (both complete since phase B) while the tensor core works on phase C
-    // (lane = feature f, columns = tokens; four token columns at a time)
-    const uint32_t boxf = (uint32_t)(f >> 6) * BOX;
-    const uint32_t fc = f & 63;
-    {
-        __nv_bfloat16* stq = reinterpret_cast<__nv_bfloat16*>(sm + ST_DQ);
-#pragma unroll
-        for (int cb = 0; cb < 4; ++cb) {
-            const int j0 = colq * 16 + cb * 4;
-            uint32_t rq1[4], rq2[4];
-            tmem_ld4(tb + cDQ1 + lane_addr + j0, rq1);
-            tmem_ld4(tb + cDQ2 + lane_addr + j0, rq2);
-            float qv[4];
-            const float4 g4 = *reinterpret_cast<const float4*>(&sGam[j0]);
-            const float gj[4] = {g4.x, g4.y, g4.z, g4.w};
-#pragma unroll
-            for (int x = 0; x < 4; ++x)
-                qv[x] = __bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(sm + R_Q + boxf + sw128_elem(j0 + x, fc)));
-            tmem_ld_wait();
-#pragma unroll
-            for (int x = 0; x < 4; ++x) {
-                const float dq = a.scale * gj[x] * __uint_as_float(rq1[x]) + __uint_as_float(rq2[x]);
-                gv[cb * 4 + x] = dq * qv[x];
-                stq[(j0 + x) * KD + f] = __float2bfloat16_rn(dq);
-            }
-        }
-    }
-    ok = ok && mbar_wait(&bar_mma[2], ph, a.status, ERR_MMA2);
-    tc_fence_after();
-    float rawg[8];   // Gamma_ij <k_i, ktil_j>, j < i (kept in registers for the beta gradient of phase D)
-    {
-        const int i = row64;
-        uint32_t r[8], r1[8];
-        tmem_ld_half8(tb + cY + addr64, r);
-        tmem_ld_half8(tb + cRAW + addr64, r1);
-        tmem_ld_wait();
-#pragma unroll
-        for (int x = 0; x < 8; ++x) rawg[x] = jb + x < i ? gam8[x] * __uint_as_float(r1[x]) : 0.f;
-        *reinterpret_cast<uint4*>(sm + R_IMG + sw128_chunk(i, jb >> 3)) = make_uint4(
-            pack_bf16(__uint_as_float(r[0]), __uint_as_float(r[1])), pack_bf16(__uint_as_float(r[2]), __uint_as_float(r[3])),
-            pack_bf16(__uint_as_float(r[4]), __uint_as_float(r[5])), pack_bf16(__uint_as_float(r[6]), __uint_as_float(r[7])));
-    }
-    fence_proxy_async();
-    tc_fence_before();
-    named_sync(1, CBW_THREADS);
-
-    if (tid == CBW_STORE_TID && ok && full) {   // the dq tile is staged (fenced before the barrier above)
-        tma_store_2d(&tmDQ, h * KD, tok0, sm + ST_DQ);
-        bulk_commit();
-    }
-    // ---- phase D: Z[a][b] = sum_c Y[a][c] T[b][c] ; dA = -strictLower(Z) --------------------------
-    if (tid == 0 && ok) {
-        tc_fence_after();
-        const uint64_t da0 = desc_kmajor(sm + R_IMG), db0 = desc_kmajor(sm + R_T);
-        for (int k = 0; k < 4; ++k)
-            mma_ss(tb + cZ, desc_advance(da0, 32 * k), desc_advance(db0, 32 * k), make_idesc(64, 64), k > 0);
-        mma_commit(&bar_mma[3]);
-    }
-    ok = ok && mbar_wait(&bar_mma[3], ph, a.status, ERR_MMA2);
-    tc_fence_after();
-    {
-        const int i = row64;
-        const float bi = sBeta[i];
-        float db = 0.f;
-        uint32_t r[8];
-        tmem_ld_half8(tb + cZ + addr64, r);
-        tmem_ld_wait();
-        float m2[8];
-#pragma unroll
-        for (int x = 0; x < 8; ++x) {
-            const float da = jb + x < i ? -__uint_as_float(r[x]) : 0.f;
-            db = fmaf(da, rawg[x], db);
-            m2[x] = da * bi * gam8[x];
-        }
-        *reinterpret_cast<uint4*>(sm + R_IMG + sw128_chunk(i, jb >> 3)) =
-            make_uint4(pack_bf16(m2[0], m2[1]), pack_bf16(m2[2], m2[3]), pack_bf16(m2[4], m2[5]), pack_bf16(m2[6], m2[7]));
-        db += __shfl_xor_sync(0xffffffffu, db, 16);   // the two halves of a row's sixteen columns
-        if (lane < 16) atomicAdd(&sdB[i], db);
-    }
-    fence_proxy_async();
-    tc_fence_before();
-    named_sync(1, CBW_THREADS);
-
-    // ---- phase E: dktil^T += K^T M2 ; dkr^T = Ktil^T M2^T -----------------------------------------
-    if (lane == 0 && warp < 2 && ok) {
-        tc_fence_after();
-        const uint64_t da0 = desc_mnmajor(sm + R_K, BOX), da1 = desc_mnmajor(sm + R_KT, BOX);
-        const uint64_t dbm = desc_mnmajor(sm + R_IMG, 0), dbk = desc_kmajor(sm + R_IMG);
-        if (warp == 0)
-            for (int k = 0; k < 4; ++k)
-                mma_ss(tb + cDKT, desc_advance(da0, 2048 * k), desc_advance(dbm, 2048 * k),
-                       make_idesc(128, 64, IDESC_A_MN | IDESC_B_MN), 1);
-        else
-            for (int k = 0; k < 4; ++k)
-                mma_ss(tb + cDKR, desc_advance(da1, 2048 * k), desc_advance(dbk, 32 * k),
-                       make_idesc(128, 64, IDESC_A_MN), k > 0);
-        mma_commit(&bar_mma[4]);
-        if (early && warp == 0) load_t(tile_next);   // phase D has finished: T is dead
-    }
-    // dv = beta dVb (complete since phase B) while the tensor core works on phase E; staged over Q (every
-    // read of q ended before the barrier that followed phase C)
-    {
-        __nv_bfloat16* stv = reinterpret_cast<__nv_bfloat16*>(sm + ST_DV);
-#pragma unroll
-        for (int cb = 0; cb < 4; ++cb) {
-            const int j0 = colq * 16 + cb * 4;
-            uint32_t rvb[4];
-            tmem_ld4(tb + cDVB + lane_addr + j0, rvb);
-            const float4 b4 = *reinterpret_cast<const float4*>(&sBeta[j0]);
-            const float bj[4] = {b4.x, b4.y, b4.z, b4.w};
-            tmem_ld_wait();
-#pragma unroll
-            for (int x = 0; x < 4; ++x) stv[(j0 + x) * KD + f] = __float2bfloat16_rn(bj[x] * __uint_as_float(rvb[x]));
-        }
-    }
-    ok = ok && mbar_wait(&bar_mma[4], ph, a.status, ERR_MMA2);
-    tc_fence_after();
-
-    // ---- final epilogue (lane = feature f, columns = tokens): dk --------------------------------------
-    rsum = 0.f;
-    if (ok) {
-        // Results are staged in shared memory as [token][feature] tiles (the operand tiles of the
-        // finished products are dead by now) and written out with 16-byte stores afterwards.
-        __nv_bfloat16* stk = reinterpret_cast<__nv_bfloat16*>(sm + ST_DK);
-        float* stkr = reinterpret_cast<float*>(sm + ST_DKR);
-        float* stkt = reinterpret_cast<float*>(sm + ST_DKT);
-        // four token columns at a time: few enough live registers for the whole loop to stay in them
-#pragma unroll
-        for (int cb = 0; cb < 4; ++cb) {
-            const int j0 = colq * 16 + cb * 4;
-            uint32_t rkt[4], rdk[4], rkb[4], rkr[4];
-            tmem_ld4(tb + cDKTR + lane_addr + j0, rkt);
-            tmem_ld4(tb + cDKT + lane_addr + j0, rdk);
-            tmem_ld4(tb + cDKB + lane_addr + j0, rkb);
-            tmem_ld4(tb + cDKR + lane_addr + j0, rkr);
-            float kv[4], ktv[4];
-            const float4 b4 = *reinterpret_cast<const float4*>(&sBeta[j0]);
-            const float4 g4 = *reinterpret_cast<const float4*>(&sGam[j0]);
-            const float4 r4 = *reinterpret_cast<const float4*>(&sRho[j0]);
-            const float bj[4] = {b4.x, b4.y, b4.z, b4.w}, gj[4] = {g4.x, g4.y, g4.z, g4.w};
-            const float rj[4] = {r4.x, r4.y, r4.z, r4.w};
-#pragma unroll
-            for (int x = 0; x < 4; ++x) {
-                const uint32_t eo = boxf + sw128_elem(j0 + x, fc);
-                kv[x] = __bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(sm + R_K + eo));
-                ktv[x] = __bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(sm + R_KT + eo));
-            }
-            tmem_ld_wait();
-#pragma unroll
-            for (int x = 0; x < 4; ++x) {
-                const int j = j0 + x;
-                const float dktr = rj[x] * __uint_as_float(rkt[x]);
-                const float dkt = dktr + __uint_as_float(rdk[x]);
-                const float dkb = __uint_as_float(rkb[x]);
-                const float dkr = bj[x] * gj[x] * dkb + __uint_as_float(rkr[x]);
-                gv[cb * 4 + x] += dkr * kv[x] - dkt * ktv[x];
-                rsum = fmaf(dktr, ktv[x], rsum);
-                stk[j * KD + f] = __float2bfloat16_rn(dkr + a.d_min * dkt);
-                if (!dk_tile) {   // fp32 copies feed the preconditioner's reverse pass only
-                    stkr[j * KD + f] = dkr;
-                    stkt[j * KD + f] = dkt;
-                } else if (j == 0) {
-                    sFirstKt[f] = dkt;   // a reverse pass may restart at the first token
+            __syncwarp();
+            if (!mbar_wait(&bar_mma[2], ph, a.status, ERR_MMA2)) break;
+            if (lane == 0) {
+                if (known) load_u_s(next);   // S, dU and the dVb image (in the space of ddU) are dead
+                if (full) {
+                    bulk_wait_read();
+                    if (known) load_do(next);
                 }
             }
+            __syncwarp();
+            if (!mbar_wait(&bar_ef, ph, a.status, ERR_MMA2)) break;
+            if (lane == 0) {
+                if (full) {
+                    store_tok(tmDQ, ST_DQ, cur);
+                    store_tok(tmDK, ST_DK, cur);
+                    bulk_commit();
+                }
+                if (known) {
+                    if (!full) load_do(next);
+                    load_kkq(next);
+                }
+            }
+            __syncwarp();
+            finish_sums(cur, (int)ph);
+            if (lane == 0 && full) bulk_wait_read();   // v lands where dq was staged, the next M2 images where dk was
+            __syncwarp();
+            if (known) {
+                if (lane == 0) load_v(next);
+            } else if (more) {
+                v = look_blocking(ticket);
+                if (!v) break;
+                next = resolve(v);
+                if (lane == 0) {
+                    load_t_ds(next);
+                    load_u_s(next);
+                    load_do(next);
+                    load_kkq(next);
+                    load_v(next);
+                }
+                __syncwarp();
+                sc = fetch(next);
+                publish(next, sc, (int)(ph ^ 1u));
+            }
+            __syncwarp();
+            cur = next;
+        }
+        if (lane == 0) bulk_wait_all();
+        __syncwarp();
+    } else if (warp == CBW_MMA_WARP) {
+        // ------------------------------------------------------------------ tensor-core issuer
+        uint32_t ragged = 0;
+        for (uint32_t it = 0;; ++it) {
+            const uint32_t ph = it & 1;
+            if (!mbar_wait(&bar_vec[ph], (it >> 1) & 1, a.status, ERR_TMA) || sInfo[ph][0] < 0) break;
+            if (!mbar_wait(&bar_c, ph, a.status, ERR_TMA)) break;
+            if (sInfo[ph][2] < CH && !mbar_wait(&bar_zero, ragged++ & 1, a.status, ERR_TMA)) break;
+            tc_fence_after();
+            if (lane == 0) {   // phase A, first part
+                {   // dVb^T[v][j] = sum_i ddU^T[v][i] T[i][j]
+                    const uint64_t da0 = desc_kmajor(sm + R_DDU), db0 = desc_mnmajor(sm + R_T, 0);
+                    for (int k = 0; k < 4; ++k)
+                        mma_ss(cDVB, desc_advance(da0, 32 * k), desc_advance(db0, 2048 * k), make_idesc(128, 64, IDESC_B_MN), k > 0);
+                }
+                {   // dP'[i][j] = sum_v dO[i][v] dU[j][v]                                      (M = 64)
+                    const uint64_t db0 = desc_mnmajor(sm + R_DU, 0);
+                    for (int k = 0; k < 8; ++k)
+                        mma_ss(cDP, desc_advance(desc_kmajor(sm + R_DO + (k >> 2) * BOX), 32 * (k & 3)),
+                               desc_advance(db0, 2048 * k), make_idesc(64, 64, IDESC_B_MN), k > 0);
+                }
+                mma_commit(&bar_mma[0]);
+            }
+            __syncwarp();
+            if (!mbar_wait(&bar_s, ph, a.status, ERR_TMA)) break;
+            if (it > 0 && !mbar_wait(&bar_ef, ph ^ 1u, a.status, ERR_MMA1)) break;   // the previous dQ1 and dKtr have been read
+            tc_fence_after();
+            if (lane == 0) {   // phase A, second part: only the later epilogues read it
+                const uint64_t das = desc_mnmajor(sm + R_S, 16384), dads = desc_mnmajor(sm + R_DS, 16384), dbu = desc_mnmajor(sm + R_DU, 0);
+                for (int k = 0; k < 8; ++k)   // dQ1^T[k][i] = sum_v S[v][k] dO[i][v]
+                    mma_ss(cDQ1, desc_advance(das, 2048 * k), desc_advance(desc_kmajor(sm + R_DO + (k >> 2) * BOX), 32 * (k & 3)),
+                           make_idesc(128, 64, IDESC_A_MN), k > 0);
+                for (int k = 0; k < 8; ++k)   // dKtr^T[k][j] = sum_v dS[v][k] dU[j][v]
+                    mma_ss(cDKTR, desc_advance(dads, 2048 * k), desc_advance(dbu, 2048 * k),
+                           make_idesc(128, 64, IDESC_A_MN | IDESC_B_MN), k > 0);
+            }
+            __syncwarp();
+            if (!mbar_wait(&bar_tok, ph, a.status, ERR_TMA) || !mbar_wait(&bar_ea, ph, a.status, ERR_MMA1)) break;
+            tc_fence_after();
+            if (lane == 0) {   // phase B
+                const uint64_t dbv = desc_mnmajor(sm + R_DVB, 0);
+                {   // dA[a][b] = sum_v dVb[a][v] dU[b][v] (its negative, its strictly lower part)     (M = 64)
+                    const uint64_t dbu = desc_mnmajor(sm + R_DU, 0);
+                    for (int k = 0; k < 8; ++k)
+                        mma_ss(cDA, desc_advance(dbv, 2048 * k), desc_advance(dbu, 2048 * k),
+                               make_idesc(64, 64, IDESC_A_MN | IDESC_B_MN), k > 0);
+                }
+                mma_commit(&bar_mma[1]);
+                {   // dKb^T[k][j] = -sum_v S[v][k] dVb[j][v]
+                    const uint64_t das = desc_mnmajor(sm + R_S, 16384);
+                    for (int k = 0; k < 8; ++k)
+                        mma_ss(cDKB, desc_advance(das, 2048 * k), desc_advance(dbv, 2048 * k),
+                               make_idesc(128, 64, IDESC_A_MN | IDESC_B_MN | IDESC_A_NEG), k > 0);
+                }
+                {   // dq2^T[k][i] = sum_j Ktil[j][k] M1[i][j] ;  dktil^T[k][j] = sum_i Q[i][k] M1[i][j]
+                    const uint64_t da0 = desc_mnmajor(sm + R_KT, BOX), da1 = desc_mnmajor(sm + R_Q, BOX);
+                    const uint64_t dbk = desc_kmajor(sm + R_M1), dbm = desc_mnmajor(sm + R_M1, 0);
+                    for (int k = 0; k < 4; ++k)
+                        mma_ss(cDQ2, desc_advance(da0, 2048 * k), desc_advance(dbk, 32 * k), make_idesc(128, 64, IDESC_A_MN), k > 0);
+                    for (int k = 0; k < 4; ++k)
+                        mma_ss(cDKT, desc_advance(da1, 2048 * k), desc_advance(dbm, 2048 * k),
+                               make_idesc(128, 64, IDESC_A_MN | IDESC_B_MN), k > 0);
+                }
+                mma_commit(&bar_mma[2]);
+            }
+            __syncwarp();
+            if (!mbar_wait(&bar_ed, ph, a.status, ERR_MMA2)) break;
+            tc_fence_after();
+            if (lane == 0) {   // phase C: dktil^T += K^T M2 ; dkr^T[k][i] = sum_j Ktil[j][k] M2'[i][j]
+                const uint64_t da0 = desc_mnmajor(sm + R_K, BOX), da1 = desc_mnmajor(sm + R_KT, BOX);
+                const uint64_t dbm = desc_mnmajor(sm + R_M2, 0), dbk = desc_kmajor(sm + R_M2 + 8192);
+                for (int k = 0; k < 4; ++k)
+                    mma_ss(cDKT, desc_advance(da0, 2048 * k), desc_advance(dbm, 2048 * k),
+                           make_idesc(128, 64, IDESC_A_MN | IDESC_B_MN), 1);
+                for (int k = 0; k < 4; ++k)
+                    mma_ss(cDKR, desc_advance(da1, 2048 * k), desc_advance(dbk, 32 * k), make_idesc(128, 64, IDESC_A_MN), k > 0);
+                mma_commit(&bar_mma[3]);
+            }
+            __syncwarp();
+        }
+    } else {
+        // ------------------------------------------------------------------ epilogue warps
+        const int quad = warp & 3, colq = warp >> 2;      // lane quadrant (32 features or 16 rows), group of 16 columns
+        const int lr = lane >> 2, lc = 2 * (lane & 3);    // fragment row and first column
+        const uint32_t lane_addr = (uint32_t)(quad * 32) << 16;
+        const uint32_t s0 = smem_u32(sm);
+        // addresses of the 8 x 8 matrices (half = lane / 16, octet of columns = lane / 8 % 2) that this lane provides:
+        const int half = lane >> 4, oct = (lane >> 3) & 1, mr = lane & 7;
+        const uint32_t offI = sw128_chunk(quad * 16 + half * 8 + mr, colq * 2 + oct);          // 64 x 64 image
+        const uint32_t offF = sw128_chunk(quad * 32 + half * 8 + mr, colq * 2 + oct);          // feature-major image
+        const uint32_t offT = (uint32_t)(quad >> 1) * BOX + sw128_chunk(colq * 16 + oct * 8 + mr, (quad & 1) * 4 + half);   // token tile; second sixteen features: ^ 32
+        const int i0 = quad * 16 + lr, j0 = colq * 16 + lc;   // row (and i0 + 8) of 64-row accumulators; columns j0, j0 + 1, j0 + 8, j0 + 9
+        uint32_t ragged = 0;
+        for (uint32_t it = 0;; ++it) {
+            const uint32_t ph = it & 1;
+            if (!mbar_wait(&bar_vec[ph], (it >> 1) & 1, a.status, ERR_TMA)) break;
+            const int tile = sInfo[ph][0], tok0 = sInfo[ph][1], len = sInfo[ph][2], h = sInfo[ph][3];
+            if (tile < 0) break;
+            const unsigned long long sk = (unsigned long long)sSkipW[ph][0] | ((unsigned long long)sSkipW[ph][1] << 32);
+            const float *sG = sVec[ph][0], *sGam = sVec[ph][1], *sRho = sVec[ph][2], *sBeta = sVec[ph][3];
+            if (len < CH) {   // rows beyond the sequence belong to another one
+                if (!mbar_wait(&bar_c, ph, a.status, ERR_TMA) || !mbar_wait(&bar_tok, ph, a.status, ERR_TMA) ||
+                    !mbar_wait(&bar_v, ph, a.status, ERR_TMA))
+                    break;
+                for (const uint32_t reg : {R_DO, R_Q, R_K, R_KT, R_V})
+                    for (int hf = 0; hf < 2; ++hf) zero_tail_rows(sm + reg + hf * BOX, len, tid, CBW_THREADS);
+                fence_proxy_async();
+                named_sync(1, CBW_THREADS);
+                if (lane == 0) mbar_arrive(&bar_zero);
+                ++ragged;
+            }
+            // ---- M1 = scale Gamma (.) lower(dP') and dVb^T as operands
+            float gam[8], dvb[2][8];   // Gamma_ij = exp(G_i - G_j), j <= i (else 0); index 4 octet + 2 (row half) + column parity
+            {
+                const float Gi[2] = {sG[i0], sG[i0 + 8]};
+                float Gj[2][2];
+#pragma unroll
+                for (int o = 0; o < 2; ++o) {
+                    const float2 g2 = *reinterpret_cast<const float2*>(sG + j0 + 8 * o);
+                    Gj[o][0] = g2.x;
+                    Gj[o][1] = g2.y;
+                }
+#pragma unroll
+                for (int o = 0; o < 2; ++o)
+#pragma unroll
+                    for (int rh = 0; rh < 2; ++rh)
+#pragma unroll
+                        for (int e = 0; e < 2; ++e)
+                            gam[4 * o + 2 * rh + e] = j0 + 8 * o + e <= i0 + 8 * rh ? __expf(Gi[rh] - Gj[o][e]) : 0.f;
+            }
+            if (!mbar_wait(&bar_mma[0], ph, a.status, ERR_MMA1)) break;
+            tc_fence_after();
+            {
+                uint32_t r[8];
+                tmem_ld_frag16(cDP + lane_addr + colq * 16, r);
+#pragma unroll
+                for (int hf = 0; hf < 2; ++hf)
+                    tmem_ld_frag16(cDVB + lane_addr + ((uint32_t)(16 * hf) << 16) + colq * 16, reinterpret_cast<uint32_t*>(dvb[hf]));
+                tmem_ld_wait();
+                uint32_t m[4];
+#pragma unroll
+                for (int x = 0; x < 4; ++x)
+                    m[x] = pack_bf16(a.scale * gam[2 * x] * __uint_as_float(r[2 * x]), a.scale * gam[2 * x + 1] * __uint_as_float(r[2 * x + 1]));
+                stmatrix_x4(s0 + R_M1 + offI, m[0], m[2], m[1], m[3]);
+#pragma unroll
+                for (int hf = 0; hf < 2; ++hf) {
+                    uint32_t p[4];
+#pragma unroll
+                    for (int x = 0; x < 4; ++x) p[x] = pack_bf16(dvb[hf][2 * x], dvb[hf][2 * x + 1]);
+                    stmatrix_x4(s0 + R_DVB + offF + hf * 2048, p[0], p[2], p[1], p[3]);
+                }
+            }
+            fence_proxy_async();
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&bar_ea);
+
+            // ---- while dA is formed: dv = beta dVb (stored once dQ1 has read dO) and dVb's share of the beta gradient, <dS, S>
+            uint32_t wv[2][4];
+            float gv[4] = {}, bv[4];   // per-token terms of this thread's features: tokens j0, j0 + 1, j0 + 8, j0 + 9
+            float bj[4];
+            {
+                const float2 b0 = *reinterpret_cast<const float2*>(sBeta + j0), b1 = *reinterpret_cast<const float2*>(sBeta + j0 + 8);
+                bj[0] = b0.x; bj[1] = b0.y; bj[2] = b1.x; bj[3] = b1.y;
+            }
+#pragma unroll
+            for (int x = 0; x < 4; ++x) bv[x] = 0.f;
+            if (!mbar_wait(&bar_v, ph, a.status, ERR_TMA)) break;
+#pragma unroll
+            for (int hf = 0; hf < 2; ++hf) {
+                uint32_t vr[4];   // matrices (half, octet): fragment index 2 octet + half <-> register 2 half + octet
+                ldmatrix_x4_trans(s0 + R_V + (offT ^ (32u * hf)), vr);
+#pragma unroll
+                for (int o = 0; o < 2; ++o)
+#pragma unroll
+                    for (int rh = 0; rh < 2; ++rh) {
+                        const float x0 = dvb[hf][4 * o + 2 * rh], x1 = dvb[hf][4 * o + 2 * rh + 1];
+                        const uint32_t vw = vr[2 * rh + o];
+                        bv[2 * o] = fmaf(x0, bf16_lo(vw), bv[2 * o]);
+                        bv[2 * o + 1] = fmaf(x1, bf16_hi(vw), bv[2 * o + 1]);
+                        wv[hf][2 * rh + o] = pack_bf16(bj[2 * o] * x0, bj[2 * o + 1] * x1);
+                    }
+            }
+            float part;
+            if (!mbar_wait(&bar_s, ph, a.status, ERR_TMA)) break;
+            {   // rows 8 warp .. of both images: the diagonals of 8 x 8 products are the rows' inner products
+                float c[4] = {};
+                const uint32_t row = (uint32_t)(warp * 8 + mr);
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const uint32_t off = (uint32_t)(q >> 1) * 16384 + sw128_chunk(row, (uint32_t)((q & 1) * 4) + (uint32_t)(lane >> 3));
+                    uint32_t x[4], y[4];
+                    ldmatrix_x4(s0 + R_DS + off, x);
+                    ldmatrix_x4(s0 + R_S + off, y);
+                    mma_bf16(c, x[0], 0u, x[1], 0u, y[0], y[1]);
+                    mma_bf16(c, x[2], 0u, x[3], 0u, y[2], y[3]);
+                }
+                part = (lr >> 1) == (lane & 3) ? ((lr & 1) ? c[1] : c[0]) : 0.f;
+            }
+
+            // ---- dA = -strictLower -> M2 = beta_i dA Gamma, M2' = dA Gamma
+            if (!mbar_wait(&bar_mma[1], ph, a.status, ERR_MMA2)) break;
+            tc_fence_after();
+            {
+                uint32_t r[8];
+                tmem_ld_frag16(cDA + lane_addr + colq * 16, r);
+                const float bi[2] = {sBeta[i0], sBeta[i0 + 8]};
+#pragma unroll
+                for (int hf = 0; hf < 2; ++hf)
+                    stmatrix_x4_trans(s0 + ST_DV + (offT ^ (32u * hf)), wv[hf][0], wv[hf][1], wv[hf][2], wv[hf][3]);
+                tmem_ld_wait();
+                uint32_t m[4], mp[4];
+#pragma unroll
+                for (int x = 0; x < 4; ++x) {   // x = 2 octet + row half
+                    const int o = x >> 1, rh = x & 1;
+                    float u[2];
+#pragma unroll
+                    for (int e = 0; e < 2; ++e)
+                        u[e] = j0 + 8 * o + e < i0 + 8 * rh ? -__uint_as_float(r[2 * x + e]) * gam[2 * x + e] : 0.f;
+                    mp[x] = pack_bf16(u[0], u[1]);
+                    m[x] = pack_bf16(bi[rh] * u[0], bi[rh] * u[1]);
+                }
+                stmatrix_x4(s0 + R_M2 + offI, m[0], m[2], m[1], m[3]);
+                stmatrix_x4(s0 + R_M2 + 8192 + offI, mp[0], mp[2], mp[1], mp[3]);
+            }
+            fence_proxy_async();
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&bar_ed);
+
+            // ---- while phase C runs: dq = scale gamma dQ1 + dq2, staged over v
+            float gj[4];
+            {
+                const float2 g0 = *reinterpret_cast<const float2*>(sGam + j0), g1 = *reinterpret_cast<const float2*>(sGam + j0 + 8);
+                gj[0] = g0.x; gj[1] = g0.y; gj[2] = g1.x; gj[3] = g1.y;
+            }
+            if (!mbar_wait(&bar_mma[2], ph, a.status, ERR_MMA2)) break;
+            tc_fence_after();
+#pragma unroll
+            for (int hf = 0; hf < 2; ++hf) {
+                const uint32_t ad = lane_addr + ((uint32_t)(16 * hf) << 16) + colq * 16;
+                uint32_t r1[8], r2[8], qr[4], w[4];
+                tmem_ld_frag16(cDQ1 + ad, r1);
+                tmem_ld_frag16(cDQ2 + ad, r2);
+                ldmatrix_x4_trans(s0 + R_Q + (offT ^ (32u * hf)), qr);
+                tmem_ld_wait();
+#pragma unroll
+                for (int o = 0; o < 2; ++o)
+#pragma unroll
+                    for (int rh = 0; rh < 2; ++rh) {
+                        const int x = 4 * o + 2 * rh;
+                        const float d0 = a.scale * gj[2 * o] * __uint_as_float(r1[x]) + __uint_as_float(r2[x]);
+                        const float d1 = a.scale * gj[2 * o + 1] * __uint_as_float(r1[x + 1]) + __uint_as_float(r2[x + 1]);
+                        gv[2 * o] = fmaf(d0, bf16_lo(qr[2 * rh + o]), gv[2 * o]);
+                        gv[2 * o + 1] = fmaf(d1, bf16_hi(qr[2 * rh + o]), gv[2 * o + 1]);
+                        w[2 * rh + o] = pack_bf16(d0, d1);
+                    }
+                stmatrix_x4_trans(s0 + ST_DQ + (offT ^ (32u * hf)), w[0], w[1], w[2], w[3]);
+            }
+
+            // ---- dk = dk_read + d_min dL/dktil; the fp32 parts only where the preconditioner's reverse pass reads them
+            float rj[4];
+            {
+                const float2 r0 = *reinterpret_cast<const float2*>(sRho + j0), r1 = *reinterpret_cast<const float2*>(sRho + j0 + 8);
+                rj[0] = r0.x; rj[1] = r0.y; rj[2] = r1.x; rj[3] = r1.y;
+            }
+            const unsigned long long in = len == CH ? ~0ull : (1ull << len) - 1;
+            const uint32_t want_kr = (uint32_t)((~sk & in) >> (colq * 16)) & 0xffffu;                       // step really taken
+            const uint32_t want_kt = (uint32_t)(((~sk | (~sk << 1) | 1ull) & in) >> (colq * 16)) & 0xffffu;   // ... or a restart behind it
+            float rsum = 0.f;
+            if (!mbar_wait(&bar_mma[3], ph, a.status, ERR_MMA2)) break;
+            tc_fence_after();
+#pragma unroll
+            for (int hf = 0; hf < 2; ++hf) {
+                const uint32_t ad = lane_addr + ((uint32_t)(16 * hf) << 16) + colq * 16;
+                uint32_t rt[8], rd[8], rb[8], rk[8], kr[4], ktr[4], w[4];
+                tmem_ld_frag16(cDKTR + ad, rt);
+                tmem_ld_frag16(cDKT + ad, rd);
+                tmem_ld_frag16(cDKB + ad, rb);
+                tmem_ld_frag16(cDKR + ad, rk);
+                ldmatrix_x4_trans(s0 + R_K + (offT ^ (32u * hf)), kr);
+                ldmatrix_x4_trans(s0 + R_KT + (offT ^ (32u * hf)), ktr);
+                tmem_ld_wait();
+                float dkr[8], dkt[8];
+#pragma unroll
+                for (int o = 0; o < 2; ++o)
+#pragma unroll
+                    for (int rh = 0; rh < 2; ++rh) {
+                        const uint32_t kw = kr[2 * rh + o], tw = ktr[2 * rh + o];
+#pragma unroll
+                        for (int e = 0; e < 2; ++e) {
+                            const int x = 4 * o + 2 * rh + e, j = 2 * o + e;
+                            const float kv = e ? bf16_hi(kw) : bf16_lo(kw), ktv = e ? bf16_hi(tw) : bf16_lo(tw);
+                            const float dktr = rj[j] * __uint_as_float(rt[x]);
+                            dkt[x] = dktr + __uint_as_float(rd[x]);
+                            const float u = fmaf(gj[j], __uint_as_float(rb[x]), __uint_as_float(rk[x]));   // dk_read / beta
+                            dkr[x] = bj[j] * u;
+                            gv[j] += dkr[x] * kv - dkt[x] * ktv;
+                            bv[j] = fmaf(u, kv, bv[j]);
+                            rsum = fmaf(dktr, ktv, rsum);
+                        }
+                        const int x = 4 * o + 2 * rh;
+                        w[2 * rh + o] = pack_bf16(fmaf(a.d_min, dkt[x], dkr[x]), fmaf(a.d_min, dkt[x + 1], dkr[x + 1]));
+                    }
+                stmatrix_x4_trans(s0 + ST_DK + (offT ^ (32u * hf)), w[0], w[1], w[2], w[3]);
+                if (want_kt) {
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const int bit = lc + 8 * (j >> 1) + (j & 1);
+                        const size_t g = ((size_t)(tok0 + colq * 16 + bit) * H + h) * KD + quad * 32 + hf * 16 + lr;
+                        const int x = 4 * (j >> 1) + (j & 1);
+                        if ((want_kt >> bit) & 1u) {
+                            a.dktil[g] = dkt[x];
+                            a.dktil[g + 8] = dkt[x + 2];
+                        }
+                        if ((want_kr >> bit) & 1u) {
+                            a.dkread[g] = dkr[x];
+                            a.dkread[g + 8] = dkr[x + 2];
+                        }
+                    }
+                }
+            }
+            {   // per-token sums over the warp's 32 features: lane bit 4 picks the set, bits 3 and 2 the token of the four
+                float x[8] = {gv[0], gv[1], gv[2], gv[3], bv[0], bv[1], bv[2], bv[3]};
+#pragma unroll
+                for (int st = 4; st > 0; st >>= 1) {
+                    const bool up = (lane & (4 * st)) != 0;
+#pragma unroll
+                    for (int y = 0; y < st; ++y) {
+                        const float send = up ? x[y] : x[y + st], keep = up ? x[y + st] : x[y];
+                        x[y] = keep + __shfl_xor_sync(0xffffffffu, send, 4 * st);
+                    }
+                }
+                sSum[ph][quad][lane >> 4][j0 + 8 * ((lane >> 3) & 1) + ((lane >> 2) & 1)] = x[0];
+                const float y = warp_sum(fmaf(sGam[CH - 1], part, rsum));   // gamma_C <dS, S> and the writes' decay to the chunk's end
+                if (lane == 0) sRed[ph][warp] = y;
+            }
+            fence_proxy_async();
+            tc_fence_before();
+            if (len < CH) {   // a ragged chunk leaves row by row
+                named_sync(1, CBW_THREADS);
+                for (int e = tid; e < len * 16; e += CBW_THREADS) {
+                    const int j = e >> 4, ch = e & 15;
+                    const size_t g = ((size_t)(tok0 + j) * H + h) * KD + ch * 8;
+                    const uint32_t off = (uint32_t)(ch >> 3) * BOX + sw128_chunk(j, ch & 7);
+                    *reinterpret_cast<uint4*>(a.dq + g) = *reinterpret_cast<const uint4*>(sm + ST_DQ + off);
+                    *reinterpret_cast<uint4*>(a.dv + g) = *reinterpret_cast<const uint4*>(sm + ST_DV + off);
+                    if ((sk >> j) & 1ull) *reinterpret_cast<uint4*>(a.dk + g) = *reinterpret_cast<const uint4*>(sm + ST_DK + off);
+                }
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&bar_ef);
         }
     }
-    fence_proxy_async();
     tc_fence_before();
-    ok = named_sync_and(1, CBW_THREADS, ok);   // block-uniform from here on; staging complete, q, k, ktil dead, accumulators read
-    if (tid == CBW_STORE_TID && early) {   // the next tile's k, ktil (q, v follow once the dv, dq tiles have left their space)
-        mbar_expect_tx(&bar_tok, TOK_TX);
-        load_kkt(h_next, tok0_next);
-    }
-    if (tid == CBW_STORE_TID && ok && full) {   // the tiles leave while the per-token sums below are formed
-        tma_store_2d(&tmDV, h * KD, tok0, sm + ST_DV);
-        if (dk_tile) tma_store_2d(&tmDK, h * KD, tok0, sm + ST_DK);
-        bulk_commit();
-    }
-    if (a_early) {
-        // phase A of the next tile: everything it reads was requested before this tile's phase C ended
-        bool okn = true;
-        if (warp < 4 && ok) okn = mbar_wait(&bar_ct, ph ^ 1u, a.status, ERR_TMA);
-        issue_phase_a(ok && okn);
-    }
-    if (ok) {
-        if (!full) {
-            for (int e = tid; e < len * 16; e += CBW_THREADS) {
-                const int j = e >> 4, ch = e & 15;
-                const size_t g = ((size_t)(tok0 + j) * H + h) * KD + ch * 8;
-                *reinterpret_cast<uint4*>(a.dq + g) = *reinterpret_cast<const uint4*>(sm + ST_DQ + j * 256 + ch * 16);
-                *reinterpret_cast<uint4*>(a.dv + g) = *reinterpret_cast<const uint4*>(sm + ST_DV + j * 256 + ch * 16);
-            }
-        }
-        if (!dk_tile) {
-            for (int e = tid; e < len * 16; e += CBW_THREADS) {
-                const int j = e >> 4, ch = e & 15;
-                const size_t g = ((size_t)(tok0 + j) * H + h) * KD + ch * 8;
-                if ((sk >> j) & 1ull)
-                    *reinterpret_cast<uint4*>(a.dk + g) =
-                        *reinterpret_cast<const uint4*>(sm + ST_DK + j * 256 + ch * 16);
-            }
-        }
-        if (dk_tile) {
-            // only the first token's dL/dktil is needed (a reverse pass may restart there)
-            for (int e = tid; e < 32; e += CBW_THREADS) {
-                const size_t g = ((size_t)tok0 * H + h) * KD + e * 4;
-                *reinterpret_cast<uint4*>(a.dktil + g) = *reinterpret_cast<const uint4*>(&sFirstKt[e * 4]);
-            }
-        } else {
-            for (int e = tid; e < len * 32; e += CBW_THREADS) {
-                const int j = e >> 5, ch = e & 31;
-                const size_t g = ((size_t)(tok0 + j) * H + h) * KD + ch * 4;
-                const bool skipped = (sk >> j) & 1ull;
-                if (!skipped)
-                    *reinterpret_cast<uint4*>(a.dkread + g) =
-                        *reinterpret_cast<const uint4*>(sm + ST_DKR + j * 512 + ch * 16);
-                if (!skipped || j == 0 || !((sk >> (j - 1)) & 1ull))
-                    *reinterpret_cast<uint4*>(a.dktil + g) =
-                        *reinterpret_cast<const uint4*>(sm + ST_DKT + j * 512 + ch * 16);
-            }
-        }
-        if (full && tid == CBW_STORE_TID) {
-            bulk_wait_read();   // the staging tiles may be overwritten by the next tile
-            if (early) load_qv(h_next, tok0_next);
-        }
-    }
-    if (tile_next == -1 && tid == CBW_QUEUE_TID) lookup_blocking(ticket_next);   // not published when this tile began: wait for it now
-    named_sync(1, CBW_THREADS);   // every copy-out read of the staging tiles is done
-    if (!next_known) {
-        tile_next = sNext[0]; h_next = sNext[1]; tok0_next = sNext[2]; len_next = sNext[3];
-        if (tile_next >= 0) fetch_scalars(tile_next, h_next, tok0_next, len_next, (int)(ph ^ 1u));
-    }
-    if (tid == 0 && tile_next >= 0) {
-        if (!early) {
-            mbar_expect_tx(&bar_ct, CT_TX);
-            load_dout(h_next, tok0_next);
-            load_du_ds_s(tile_next);
-            load_ddu(tile_next);
-            load_t(tile_next);
-            mbar_expect_tx(&bar_tok, TOK_TX);
-            load_kkt(h_next, tok0_next);
-            load_qv(h_next, tok0_next);
-        }
-    }
-    a_issued = a_early && ok;
-    pend = ok;
-    p_tok0 = tok0;
-    p_h = h;
-    p_len = len;
-    ph ^= 1u;
-    ticket_next = ticket_after;
-    tile_l = tile_next;
-    h = h_next;
-    tok0 = tok0_next;
-    len = len_next;
-    }   // tile loop
-    if (pend) {   // the last tile's sums
-        reduce_sums((int)(ph ^ 1u));
-        named_sync(1, CBW_THREADS);
-        if (warp == 1) finish_sums((int)(ph ^ 1u), p_tok0, p_h, p_len);
-    }
-    if (tid == CBW_STORE_TID) bulk_wait_all();
-    tc_fence_before();
-    named_sync(1, CBW_THREADS);
+    __syncthreads();
 }
 
 // Backward of the layer's second phase in one launch.  CTA b first walks the chains b, b + grid, ...
@@ -2276,7 +2137,7 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
     pdl_wait();
     for (int chain = (int)blockIdx.x; chain < nchains; chain += (int)gridDim.x)
         chain_bwd_role(tmDO, tmKt, ca, chain, sm, tb, tq);
-    if (threadIdx.x < CBW_THREADS) chunk_bwd_role(tmQ, tmK, tmKt, tmV, tmDO, tmDQ, tmDK, tmDV, cb, sm, tb, tq);
+    chunk_bwd_role(tmQ, tmK, tmKt, tmV, tmDO, tmDQ, tmDK, tmDV, cb, sm, tb, tq);
     tc_fence_before();
     __syncthreads();
     if (warp == 0) tmem_dealloc(tb, 512);
@@ -2434,7 +2295,7 @@ int tc_backward(const osdn_params& p, const Hyper& hy, const WsLayout& L, void* 
         ch.WT = U8(t.WT); ch.P = U8(t.P); ch.Qg = U8(t.Qg); ch.dSn = U8(t.dSn); ch.ddUT = U8(t.ddUT);
         ch.status = status;
         TcChunkBwdArgs cb{};
-        cb.H = H; cb.ntiles = L.NTmax * H; cb.nseq = S; cb.tab = tab; cb.beta = a.beta; cb.gate = a.gate; cb.scale = hy.scale; cb.d_min = hy.d_min;
+        cb.H = H; cb.nseq = S; cb.tab = tab; cb.beta = a.beta; cb.gate = a.gate; cb.scale = hy.scale; cb.d_min = hy.d_min;
         cb.Tm = U8(t.Tm); cb.Sn = U8(t.Sn); cb.dSn = U8(t.dSn); cb.dUT = U8(t.dUT); cb.ddUT = U8(t.ddUT);
         cb.skipw = carve_p1(ws, L).skipw;
         cb.dq = static_cast<__nv_bfloat16*>(a.dq); cb.dk = static_cast<__nv_bfloat16*>(a.dk);
@@ -2442,8 +2303,8 @@ int tc_backward(const osdn_params& p, const Hyper& hy, const WsLayout& L, void* 
         cb.dktil = reinterpret_cast<float*>(w + t.dktil); cb.dkread = reinterpret_cast<float*>(w + t.dkread);
         cb.status = status;
         CUtensorMap tmDQ, tmDK, tmDV;
-        if (!make_store_map(&tmDQ, a.dq, Ttot, H) || !make_store_map(&tmDK, a.dk, Ttot, H) ||
-            !make_store_map(&tmDV, a.dv, Ttot, H))
+        if (!make_token_map(&tmDQ, a.dq, Ttot, H) || !make_token_map(&tmDK, a.dk, Ttot, H) ||
+            !make_token_map(&tmDV, a.dv, Ttot, H))
             return -1;
         // tile queue between the chains and the chunk-local workers: two counters, then one slot per tile
         // (zero: cleared by the forward that saved the residuals, and again behind each backward)

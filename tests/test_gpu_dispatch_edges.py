@@ -170,6 +170,32 @@ def test_backward_twice_on_the_same_residuals():
         assert not torch.isnan(x.float()).any() and torch.equal(x, y)
 
 
+@pytest.mark.parametrize("kind", ["gated", "moving", "mixture"])
+@pytest.mark.parametrize("lens", [[1], [63, 65], [64, 64], [129, 0, 191]], ids=str)
+def test_backward_tiles_at_their_edges(lens, kind):
+    """Chunk-local backward on the tensor cores: tiles of 1, 63, 64 tokens and a remainder, every step skipped, some and none;
+    twice on the same residuals, bit for bit (the second time every counter, flag and staging area has been used)."""
+    hy = OsdnHyper(eta=0.3 if kind == "moving" else 0.003, apf_mode=2 if kind == "moving" else 1)
+    inp = draw(f"tiles_{kind}", 7900 + len(lens), lens, 2, 128, 128, "bf16", dense_B=len(lens) if len(set(lens)) == 1 else 0, hyper=hy,
+               key_kind="sparse" if kind == "moving" else "gauss", gate_kind="mixture" if kind == "mixture" else "softplus",
+               with_dout=True, with_log_ret=kind == "moving", with_state=True, with_state_cotangents=True)
+    got = run_inputs_bwd(inp)
+    ref = parity.oracle_all(inp, True, got["projection_masks"])
+    parity.compare(got, ref, "bf16", parity.BWD_KEYS, f"tiles_{kind}_{lens}", tensor_core=True)
+    b = binding.DeviceBundle(inp, DEV, need_bwd=True)
+    b.fwd(save=True)
+    seen = []
+    for _ in range(2):
+        for x in (b.dq, b.dk, b.dv):
+            x.fill_(float("nan"))
+        b.bwd(residuals_valid=True)
+        torch.cuda.synchronize()
+        assert b.device_status() == 0
+        seen.append([x.clone() for x in (b.dq, b.dk, b.dv)])
+    for x, y in zip(*seen):
+        assert not torch.isnan(x.float()).any() and torch.equal(x, y)
+
+
 @pytest.mark.parametrize("B,H,L", [(49, 3, 8), (37, 4, 9), (191, 1, 1), (192, 1, 1), (50, 3, 17), (103, 1, 1), (104, 1, 1), (103, 1, 9), (52, 2, 9)])
 @pytest.mark.parametrize("io,K,V,apf", [("bf16", 128, 128, 1), ("fp32", 64, 128, 2), ("fp32", 128, 64, 3)])
 def test_decode_on_both_sides_of_its_dispatch(B, H, L, io, K, V, apf):
