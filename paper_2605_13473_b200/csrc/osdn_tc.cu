@@ -279,7 +279,8 @@ __device__ __forceinline__ void chunk_fwd_tile(const CUtensorMap& tmK, const CUt
     if (len == 0) return;
     const int tok0 = a.tab.chunk_tok0(c);
     const size_t tile = (size_t)c * H + h;
-    const int warp = tid >> 5, lane = tid & 31;
+    const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
+    const bool lead = lane == 0;
     const int quad = warp & 3, half = warp >> 2;
 
     if (tid == 0) {
@@ -327,14 +328,14 @@ __device__ __forceinline__ void chunk_fwd_tile(const CUtensorMap& tmK, const CUt
     }
 
     // ---- D1[128 x 64] = [K;Q] Ktil^T ---------------------------------------------------------
-    if (tid == 0 && ok) {
+    if (warp == 0 && ok) {
         const uint32_t idesc = make_idesc(128, 64);
         for (int s = 0; s < 8; ++s) {
             const uint64_t da = desc_advance(desc_kmajor(sKQ + (s >> 2) * 16384), 32 * (s & 3));
             const uint64_t db = desc_advance(desc_kmajor(sKt + (s >> 2) * BOX), 32 * (s & 3));
-            mma_ss(tb, da, db, idesc, s > 0);
+            mma_ss(tb, da, db, idesc, s > 0, lead);
         }
-        mma_commit(&bar_mma1);
+        mma_commit(&bar_mma1, lead);
     }
     // gated, scaled queries for both state chains, while the product runs: Qg = scale gamma_i Q
     // (same image layout as Q)
@@ -449,13 +450,13 @@ __device__ __forceinline__ void chunk_fwd_tile(const CUtensorMap& tmK, const CUt
     sync();
 
     // ---- D2[128 x 64] = K^T Tbg^T  (W^T) -----------------------------------------------------
-    if (tid == 0 && ok) {
+    if (warp == 0 && ok) {
         tc_fence_after();
         const uint32_t idesc = make_idesc(128, 64, IDESC_A_MN);
         const uint64_t da0 = desc_mnmajor(sKQ, 16384);
         const uint64_t db0 = desc_kmajor(sTb);
-        for (int s = 0; s < 4; ++s) mma_ss(tb + 64, desc_advance(da0, 2048 * s), desc_advance(db0, 32 * s), idesc, s > 0);
-        mma_commit(&bar_mma2);
+        for (int s = 0; s < 4; ++s) mma_ss(tb + 64, desc_advance(da0, 2048 * s), desc_advance(db0, 32 * s), idesc, s > 0, lead);
+        mma_commit(&bar_mma2, lead);
     }
     ok = ok && mbar_wait(&bar_mma2, ph, a.status, ERR_MMA2);
     tc_fence_after();
@@ -585,7 +586,8 @@ __device__ __forceinline__ void chain_fwd_role(const CUtensorMap& tmV, const CUt
     const int s = chain / H, h = chain % H;
     const int c0 = a.tab.seq_chunk0(s), c1 = a.tab.seq_chunk0(s + 1);
     const int seq_t0 = a.tab.seq_tok0(s), seq_len = a.tab.seq_len(s);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
+    const bool lead = lane == 0;
     const int quad = warp & 3, colq = (warp >> 2) & 3;
     const int v = quad * 32 + lane;             // state row owned by a state-warp thread
     float* fin = a.final_state ? a.final_state + (((size_t)s * H + h) * KD + v) * KD + colq * 32 : nullptr;
@@ -683,7 +685,7 @@ __device__ __forceinline__ void chain_fwd_role(const CUtensorMap& tmV, const CUt
             const uint32_t idesc = make_idesc(128, 64, IDESC_A_MN);
             const uint64_t da0 = desc_mnmajor(d + ST_V, BOX), db0 = desc_kmajor(d + ST_TB);
             for (int k = 0; k < 4; ++k)
-                mma_ss(tDU, desc_advance(da0, 2048 * k), desc_advance(db0, 32 * k), idesc, k > 0);
+                mma_ss(tDU, desc_advance(da0, 2048 * k), desc_advance(db0, 32 * k), idesc, k > 0, lead);
         };
         for (int n = 0; n < nchunks && ok; ++n) {
             const int st = n & 1;
@@ -693,60 +695,62 @@ __device__ __forceinline__ void chain_fwd_role(const CUtensorMap& tmV, const CUt
             ok = ok && mbar_wait(&bar_s_ready, n & 1, a.status, ERR_CHAIN_MMA1);
             if (!ok) break;
             tc_fence_after();
-            if (lane == 0) {
+            if (lead && a.save) {
                 bulk_wait_read();   // saved images of the previous chunk have left shared memory
-                if (a.save) {
-                    bulk_store(a.Sn + tile * 32768, sS, 32768);
-                    bulk_commit();
-                }
+                bulk_store(a.Sn + tile * 32768, sS, 32768);
+                bulk_commit();
+            }
+            __syncwarp();
+            {
                 if (!ut_issued) issue_ut(d);
                 {   // dU^T -= S W^T
                     const uint32_t idesc = make_idesc(128, 64, IDESC_A_NEG | IDESC_B_MN);
                     const uint64_t db0 = desc_mnmajor(d + ST_WT, 0);
                     for (int k = 0; k < 8; ++k)
                         mma_ss(tDU, desc_advance(desc_kmajor(sS + (k >> 2) * 16384), 32 * (k & 3)),
-                               desc_advance(db0, 2048 * k), idesc, 1);
+                               desc_advance(db0, 2048 * k), idesc, 1, lead);
                 }
-                mma_commit(&bar_du_done);
+                mma_commit(&bar_du_done, lead);
             }
             __syncwarp();
             // the output accumulators of chunk n - 2 (same buffers) have been read
             if (n >= 2) ok = mbar_wait(&bar_o_free[st], ((n >> 1) - 1) & 1, a.status, ERR_CHAIN_MMA2);
             if (!ok) break;
             tc_fence_after();
-            if (lane == 0) {   // O^T = S Qg^T
+            {   // O^T = S Qg^T
                 const uint32_t idesc = make_idesc(128, 64);
                 for (int k = 0; k < 8; ++k)
                     mma_ss(tO + st * 64, desc_advance(desc_kmajor(sS + (k >> 2) * 16384), 32 * (k & 3)),
-                           desc_advance(desc_kmajor(d + ST_QG + (k >> 2) * BOX), 32 * (k & 3)), idesc, k > 0);
+                           desc_advance(desc_kmajor(d + ST_QG + (k >> 2) * BOX), 32 * (k & 3)), idesc, k > 0, lead);
             }
             __syncwarp();
             ok = mbar_wait(&bar_du_ready, n & 1, a.status, ERR_CHAIN_MMA2);
             if (!ok) break;
             tc_fence_after();
-            if (lane == 0) {
+            if (lead && a.save) {
                 // The image of S sent off at the start of this chunk must have left shared memory before
                 // the state update is released: its completion lets the state warps overwrite that image.
                 bulk_wait_read();
-                if (a.save) {
-                    bulk_store(a.dUT + tile * 16384, sDU1, 16384);
-                    bulk_commit();
-                }
+                bulk_store(a.dUT + tile * 16384, sDU1, 16384);
+                bulk_commit();
+            }
+            __syncwarp();
+            {
                 {   // S += (rho dU)^T Ktil
                     const uint32_t idesc = make_idesc(128, 128, IDESC_B_MN);
                     const uint64_t da0 = desc_kmajor(sDU2), db0 = desc_mnmajor(d + ST_KT, BOX);
                     for (int k = 0; k < 4; ++k)
-                        mma_ss(tS, desc_advance(da0, 32 * k), desc_advance(db0, 2048 * k), idesc, 1);
+                        mma_ss(tS, desc_advance(da0, 32 * k), desc_advance(db0, 2048 * k), idesc, 1, lead);
                 }
-                mma_commit(&bar_s_done);
+                mma_commit(&bar_s_done, lead);
                 {   // O^T += dU^T P'^T
                     const uint32_t idesc = make_idesc(128, 64);
                     const uint64_t da0 = desc_kmajor(sDU1), db0 = desc_kmajor(d + ST_P);
                     for (int k = 0; k < 4; ++k)
-                        mma_ss(tO + st * 64, desc_advance(da0, 32 * k), desc_advance(db0, 32 * k), idesc, 1);
+                        mma_ss(tO + st * 64, desc_advance(da0, 32 * k), desc_advance(db0, 32 * k), idesc, 1, lead);
                 }
-                mma_commit(&bar_o_done[st]);
-                mma_commit(&bar_empty[st]);
+                mma_commit(&bar_o_done[st], lead);
+                mma_commit(&bar_empty[st], lead);
             }
             __syncwarp();
             // The part of the next chunk's dU^T that does not depend on the state goes in now, while the
@@ -755,7 +759,7 @@ __device__ __forceinline__ void chain_fwd_role(const CUtensorMap& tmV, const CUt
             if (n + 1 < nchunks && chunk_len(n + 1) == CH) {
                 ok = mbar_wait(&bar_full[st ^ 1], ((n + 1) >> 1) & 1, a.status, ERR_CHAIN_TMA);
                 if (!ok) break;
-                if (lane == 0) issue_ut(sStage + (st ^ 1) * STAGE_BYTES);
+                issue_ut(sStage + (st ^ 1) * STAGE_BYTES);
                 __syncwarp();
                 ut_issued = true;
             }
@@ -1162,7 +1166,8 @@ __device__ __forceinline__ void chain_bwd_role(const CUtensorMap& tmDO, const CU
     const int s = chain / H, h = chain % H;
     const int c0 = a.tab.seq_chunk0(s), c1 = a.tab.seq_chunk0(s + 1);
     const int seq_t0 = a.tab.seq_tok0(s), seq_len = a.tab.seq_len(s);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
+    const bool lead = lane == 0;
     const int quad = warp & 3, colq = (warp >> 2) & 3;
     const int v = quad * 32 + lane;
     float* dini = a.dinit_state ? a.dinit_state + (((size_t)s * H + h) * KD + v) * KD + colq * 32 : nullptr;
@@ -1246,7 +1251,7 @@ __device__ __forceinline__ void chain_bwd_role(const CUtensorMap& tmDO, const CU
             const uint32_t idesc = make_idesc(128, 64, IDESC_A_MN | IDESC_B_MN);
             const uint64_t da0 = desc_mnmajor(d + BS_DO, BOX), db0 = desc_mnmajor(d + BS_P, 0);
             for (int k = 0; k < 4; ++k)
-                mma_ss(tA1, desc_advance(da0, 2048 * k), desc_advance(db0, 2048 * k), idesc, k > 0);
+                mma_ss(tA1, desc_advance(da0, 2048 * k), desc_advance(db0, 2048 * k), idesc, k > 0, lead);
         };
         for (int n = 0; n < nchunks && ok; ++n) {
             const int st = n & 1;
@@ -1256,43 +1261,49 @@ __device__ __forceinline__ void chain_bwd_role(const CUtensorMap& tmDO, const CU
             ok = ok && mbar_wait(&bar_s_ready, n & 1, a.status, ERR_CHAIN_MMA1);
             if (!ok) break;
             tc_fence_after();
-            if (lane == 0) {
+            if (lead) {
                 bulk_wait_read();   // the ddU^T image of the previous chunk has left shared memory
                 bulk_store(a.dSn + tile * 32768, sdS, 32768);   // cotangent at the end of this chunk
                 bulk_commit();
+            }
+            __syncwarp();
+            {
                 if (!a1_issued) issue_a1(d);
                 {   // acc2 = dS Ktil^T
                     const uint32_t idesc = make_idesc(128, 64);
                     for (int k = 0; k < 8; ++k)
                         mma_ss(tA2, desc_advance(desc_kmajor(sdS + (k >> 2) * 16384), 32 * (k & 3)),
-                               desc_advance(desc_kmajor(d + BS_KT + (k >> 2) * BOX), 32 * (k & 3)), idesc, k > 0);
+                               desc_advance(desc_kmajor(d + BS_KT + (k >> 2) * BOX), 32 * (k & 3)), idesc, k > 0, lead);
                 }
-                mma_commit(&bar_a_done);
+                mma_commit(&bar_a_done, lead);
                 {   // dS += dO^T Qg (the accumulator has been decayed before s_ready)
                     const uint32_t idesc = make_idesc(128, 128, IDESC_A_MN | IDESC_B_MN);
                     const uint64_t da0 = desc_mnmajor(d + BS_DO, BOX), db0 = desc_mnmajor(d + BS_QG, BOX);
                     for (int k = 0; k < 4; ++k)
-                        mma_ss(tS, desc_advance(da0, 2048 * k), desc_advance(db0, 2048 * k), idesc, 1);
+                        mma_ss(tS, desc_advance(da0, 2048 * k), desc_advance(db0, 2048 * k), idesc, 1, lead);
                 }
             }
             __syncwarp();
             ok = mbar_wait(&bar_a_ready, n & 1, a.status, ERR_CHAIN_MMA2);
             if (!ok) break;
             tc_fence_after();
-            if (lane == 0) {
+            if (lead) {
                 // The dS image sent off above must have left shared memory before the update is
                 // released: its completion lets the state warps overwrite that image.
                 bulk_wait_read();
                 bulk_store(a.ddUT + tile * 16384, sddU, 16384);
                 bulk_commit();
+            }
+            __syncwarp();
+            {
                 {   // dS -= ddU^T W
                     const uint32_t idesc = make_idesc(128, 128, IDESC_A_NEG);
                     const uint64_t da0 = desc_kmajor(sddU), db0 = desc_kmajor(d + BS_WT);
                     for (int k = 0; k < 4; ++k)
-                        mma_ss(tS, desc_advance(da0, 32 * k), desc_advance(db0, 32 * k), idesc, 1);
+                        mma_ss(tS, desc_advance(da0, 32 * k), desc_advance(db0, 32 * k), idesc, 1, lead);
                 }
-                mma_commit(&bar_s_done);
-                mma_commit(&bar_empty[st]);
+                mma_commit(&bar_s_done, lead);
+                mma_commit(&bar_empty[st], lead);
             }
             __syncwarp();
             // the state-independent part of the next chunk's ddU^T, while the state warps convert dS
@@ -1300,7 +1311,7 @@ __device__ __forceinline__ void chain_bwd_role(const CUtensorMap& tmDO, const CU
             if (n + 1 < nchunks && chunk_len(n + 1) == CH) {
                 ok = mbar_wait(&bar_full[st ^ 1], ((n + 1) >> 1) & 1, a.status, ERR_CHAIN_TMA);
                 if (!ok) break;
-                if (lane == 0) issue_a1(sStage + (st ^ 1) * BSTAGE_BYTES);
+                issue_a1(sStage + (st ^ 1) * BSTAGE_BYTES);
                 __syncwarp();
                 a1_issued = true;
             }
@@ -1497,7 +1508,8 @@ __device__ __forceinline__ void chunk_bwd_role(const CUtensorMap& tmQ, const CUt
     __shared__ float sRed[2][CBW_WARPS];
 
     const int H = a.H;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
+    const bool lead = lane == 0;
     if (tid == 0) {
         for (uint64_t* b : {&bar_vec[0], &bar_vec[1], &bar_c, &bar_s, &bar_tok, &bar_v, &bar_mma[0], &bar_mma[1], &bar_mma[2], &bar_mma[3]}) mbar_init(b, 1);
         for (uint64_t* b : {&bar_zero, &bar_ea, &bar_ed, &bar_ef}) mbar_init(b, CBW_WARPS);
@@ -1762,74 +1774,74 @@ __device__ __forceinline__ void chunk_bwd_role(const CUtensorMap& tmQ, const CUt
             if (!mbar_wait(&bar_c, ph, a.status, ERR_TMA)) break;
             if (sInfo[ph][2] < CH && !mbar_wait(&bar_zero, ragged++ & 1, a.status, ERR_TMA)) break;
             tc_fence_after();
-            if (lane == 0) {   // phase A, first part
+            {   // phase A, first part
                 {   // dVb^T[v][j] = sum_i ddU^T[v][i] T[i][j]
                     const uint64_t da0 = desc_kmajor(sm + R_DDU), db0 = desc_mnmajor(sm + R_T, 0);
                     for (int k = 0; k < 4; ++k)
-                        mma_ss(cDVB, desc_advance(da0, 32 * k), desc_advance(db0, 2048 * k), make_idesc(128, 64, IDESC_B_MN), k > 0);
+                        mma_ss(cDVB, desc_advance(da0, 32 * k), desc_advance(db0, 2048 * k), make_idesc(128, 64, IDESC_B_MN), k > 0, lead);
                 }
                 {   // dP'[i][j] = sum_v dO[i][v] dU[j][v]                                      (M = 64)
                     const uint64_t db0 = desc_mnmajor(sm + R_DU, 0);
                     for (int k = 0; k < 8; ++k)
                         mma_ss(cDP, desc_advance(desc_kmajor(sm + R_DO + (k >> 2) * BOX), 32 * (k & 3)),
-                               desc_advance(db0, 2048 * k), make_idesc(64, 64, IDESC_B_MN), k > 0);
+                               desc_advance(db0, 2048 * k), make_idesc(64, 64, IDESC_B_MN), k > 0, lead);
                 }
-                mma_commit(&bar_mma[0]);
+                mma_commit(&bar_mma[0], lead);
             }
             __syncwarp();
             if (!mbar_wait(&bar_s, ph, a.status, ERR_TMA)) break;
             if (it > 0 && !mbar_wait(&bar_ef, ph ^ 1u, a.status, ERR_MMA1)) break;   // the previous dQ1 and dKtr have been read
             tc_fence_after();
-            if (lane == 0) {   // phase A, second part: only the later epilogues read it
+            {   // phase A, second part: only the later epilogues read it
                 const uint64_t das = desc_mnmajor(sm + R_S, 16384), dads = desc_mnmajor(sm + R_DS, 16384), dbu = desc_mnmajor(sm + R_DU, 0);
                 for (int k = 0; k < 8; ++k)   // dQ1^T[k][i] = sum_v S[v][k] dO[i][v]
                     mma_ss(cDQ1, desc_advance(das, 2048 * k), desc_advance(desc_kmajor(sm + R_DO + (k >> 2) * BOX), 32 * (k & 3)),
-                           make_idesc(128, 64, IDESC_A_MN), k > 0);
+                           make_idesc(128, 64, IDESC_A_MN), k > 0, lead);
                 for (int k = 0; k < 8; ++k)   // dKtr^T[k][j] = sum_v dS[v][k] dU[j][v]
                     mma_ss(cDKTR, desc_advance(dads, 2048 * k), desc_advance(dbu, 2048 * k),
-                           make_idesc(128, 64, IDESC_A_MN | IDESC_B_MN), k > 0);
+                           make_idesc(128, 64, IDESC_A_MN | IDESC_B_MN), k > 0, lead);
             }
             __syncwarp();
             if (!mbar_wait(&bar_tok, ph, a.status, ERR_TMA) || !mbar_wait(&bar_ea, ph, a.status, ERR_MMA1)) break;
             tc_fence_after();
-            if (lane == 0) {   // phase B
+            {   // phase B
                 const uint64_t dbv = desc_mnmajor(sm + R_DVB, 0);
                 {   // dA[a][b] = sum_v dVb[a][v] dU[b][v] (its negative, its strictly lower part)     (M = 64)
                     const uint64_t dbu = desc_mnmajor(sm + R_DU, 0);
                     for (int k = 0; k < 8; ++k)
                         mma_ss(cDA, desc_advance(dbv, 2048 * k), desc_advance(dbu, 2048 * k),
-                               make_idesc(64, 64, IDESC_A_MN | IDESC_B_MN), k > 0);
+                               make_idesc(64, 64, IDESC_A_MN | IDESC_B_MN), k > 0, lead);
                 }
-                mma_commit(&bar_mma[1]);
+                mma_commit(&bar_mma[1], lead);
                 {   // dKb^T[k][j] = -sum_v S[v][k] dVb[j][v]
                     const uint64_t das = desc_mnmajor(sm + R_S, 16384);
                     for (int k = 0; k < 8; ++k)
                         mma_ss(cDKB, desc_advance(das, 2048 * k), desc_advance(dbv, 2048 * k),
-                               make_idesc(128, 64, IDESC_A_MN | IDESC_B_MN | IDESC_A_NEG), k > 0);
+                               make_idesc(128, 64, IDESC_A_MN | IDESC_B_MN | IDESC_A_NEG), k > 0, lead);
                 }
                 {   // dq2^T[k][i] = sum_j Ktil[j][k] M1[i][j] ;  dktil^T[k][j] = sum_i Q[i][k] M1[i][j]
                     const uint64_t da0 = desc_mnmajor(sm + R_KT, BOX), da1 = desc_mnmajor(sm + R_Q, BOX);
                     const uint64_t dbk = desc_kmajor(sm + R_M1), dbm = desc_mnmajor(sm + R_M1, 0);
                     for (int k = 0; k < 4; ++k)
-                        mma_ss(cDQ2, desc_advance(da0, 2048 * k), desc_advance(dbk, 32 * k), make_idesc(128, 64, IDESC_A_MN), k > 0);
+                        mma_ss(cDQ2, desc_advance(da0, 2048 * k), desc_advance(dbk, 32 * k), make_idesc(128, 64, IDESC_A_MN), k > 0, lead);
                     for (int k = 0; k < 4; ++k)
                         mma_ss(cDKT, desc_advance(da1, 2048 * k), desc_advance(dbm, 2048 * k),
-                               make_idesc(128, 64, IDESC_A_MN | IDESC_B_MN), k > 0);
+                               make_idesc(128, 64, IDESC_A_MN | IDESC_B_MN), k > 0, lead);
                 }
-                mma_commit(&bar_mma[2]);
+                mma_commit(&bar_mma[2], lead);
             }
             __syncwarp();
             if (!mbar_wait(&bar_ed, ph, a.status, ERR_MMA2)) break;
             tc_fence_after();
-            if (lane == 0) {   // phase C: dktil^T += K^T M2 ; dkr^T[k][i] = sum_j Ktil[j][k] M2'[i][j]
+            {   // phase C: dktil^T += K^T M2 ; dkr^T[k][i] = sum_j Ktil[j][k] M2'[i][j]
                 const uint64_t da0 = desc_mnmajor(sm + R_K, BOX), da1 = desc_mnmajor(sm + R_KT, BOX);
                 const uint64_t dbm = desc_mnmajor(sm + R_M2, 0), dbk = desc_kmajor(sm + R_M2 + 8192);
                 for (int k = 0; k < 4; ++k)
                     mma_ss(cDKT, desc_advance(da0, 2048 * k), desc_advance(dbm, 2048 * k),
-                           make_idesc(128, 64, IDESC_A_MN | IDESC_B_MN), 1);
+                           make_idesc(128, 64, IDESC_A_MN | IDESC_B_MN), 1, lead);
                 for (int k = 0; k < 4; ++k)
-                    mma_ss(cDKR, desc_advance(da1, 2048 * k), desc_advance(dbk, 32 * k), make_idesc(128, 64, IDESC_A_MN), k > 0);
-                mma_commit(&bar_mma[3]);
+                    mma_ss(cDKR, desc_advance(da1, 2048 * k), desc_advance(dbk, 32 * k), make_idesc(128, 64, IDESC_A_MN), k > 0, lead);
+                mma_commit(&bar_mma[3], lead);
             }
             __syncwarp();
         }

@@ -255,33 +255,30 @@ __host__ __device__ constexpr uint32_t make_idesc(int M, int N, uint32_t flags =
            (static_cast<uint32_t>(M >> 4) << 24);
 }
 
-// D[tmem] (+)= A[smem] * B[smem]; issued by ONE thread.
+// D[tmem] (+)= A[smem] * B[smem].  The whole warp calls, in uniform control flow; the lane with `issue` set issues (one, the
+// same for a commit).  Descriptors then stay in uniform registers: formed in a branch that only one lane takes, every
+// instruction moved its operands over from the lane's registers and took about 100 cycles to issue, where the tensor core
+// needs 47 for N = 64.
 __device__ __forceinline__ void mma_ss(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                       uint32_t accumulate)
+                                       uint32_t accumulate, bool issue)
 {
     asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+        "{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 q, %5, 0;\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"((int)issue)
         : "memory");
 }
 
 // Makes `bar` complete once every MMA issued so far by this thread has finished.
-__device__ __forceinline__ void mma_commit(uint64_t* bar)
+__device__ __forceinline__ void mma_commit(uint64_t* bar, bool issue)
 {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
-                 ::"r"(smem_u32(bar)) : "memory");
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %1, 0;\n\t"
+                 "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}"
+                 ::"r"(smem_u32(bar)), "r"((int)issue) : "memory");
 }
 
-// A sequence of K steps of one product.  a_step / b_step: descriptor advance per K = 16 step in
-// bytes (32 for K-major, 2048 for MN-major).
-__device__ __forceinline__ void mma_ksteps(uint32_t d_tmem, uint64_t a_desc, uint32_t a_step, uint64_t b_desc,
-                                           uint32_t b_step, uint32_t idesc, int ksteps, bool accumulate_first)
-{
-    for (int s = 0; s < ksteps; ++s)
-        mma_ss(d_tmem, desc_advance(a_desc, a_step * s), desc_advance(b_desc, b_step * s), idesc,
-               (s > 0 || accumulate_first) ? 1u : 0u);
-}
+// The calling warp's index, known to be the same for all its lanes.
+__device__ __forceinline__ int warp_index() { return __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0); }
 
 // ---------------------------------------------------------------------------------------------
 // tensor memory <-> registers.  32x32b shape: thread t of the warp accesses lane (base + t),
