@@ -144,12 +144,12 @@ __device__ __forceinline__ void mma_tf32(float (&c)[4], const uint32_t (&a)[4], 
 
 // ---------------------------------------------------------------------------------------------
 // T = (I + A)^-1 for a 64 x 64 strictly lower triangular A, in place (fp32, shared memory, row
-// stride LCF), by 16 x 16 blocks: the four diagonal blocks by forward substitution with a column
-// per thread in registers, then block row by block row,
-//     T_bc = -T_bb sum_{m=c}^{b-1} A_bm T_mc            (c < b),
-// where row b of A is still untouched and the rows above already hold T.  The inner sums are
-// parked in the upper triangle (block (c, b)), so on return only entries with j <= i are meaningful.
-// Called by all threads of the CTA (at least 96); ends with a barrier.
+// stride LCF), by 16 x 16 blocks: warps 0 and 1 take a pair of diagonal blocks each, by forward substitution with a
+// column per thread in registers, and the block below it; then warps 0 to 3 the 32 x 32 block below those,
+//     T_21 = -T_22 (A_21 T_11).
+// The inner products are parked in the upper triangle, so on return only entries with j <= i are meaningful.
+// Called by all threads of the group (at least 128) behind a barrier; ends with a barrier.  Three barriers, where block row
+// by block row took eight; a chain of six block products instead of nine.
 // ---------------------------------------------------------------------------------------------
 constexpr int LCF = CH + 4;   // stride = 4 mod 32 words: conflict-free 16-byte row stores and A fragments
 
@@ -189,43 +189,56 @@ __device__ __forceinline__ void block16_store_ld(float* C, const float (&acc)[2]
 template <typename Sync> __device__ __forceinline__ void ut_inverse_64_inplace(float* sA, int tid, Sync sync)
 {
     const int warp = tid >> 5, lane = tid & 31;
-    {
-        float x[16];
-        const int b = (tid >> 4) & 3, col = tid & 15;
-        float* Ab = sA + (16 * b) * LCF + 16 * b;
-        if (tid < CH) {
+    if (warp < 2) {
+        {
+            float x[16];
+            float* Ab = sA + (16 * (tid >> 4)) * (LCF + 1);
+            const int col = tid & 15;
 #pragma unroll
-            for (int i = 0; i < 16; ++i) x[i] = i == col ? 1.f : 0.f;
+            for (int i = 0; i < 16; ++i) {
+                float sum = i == col ? 1.f : 0.f;
 #pragma unroll
-            for (int j = 0; j < 15; ++j) {
+                for (int j4 = 0; j4 < 16; j4 += 4)
+                    if (j4 < i) {
+                        const float4 r4 = *reinterpret_cast<const float4*>(Ab + i * LCF + j4);
+                        const float r[4] = {r4.x, r4.y, r4.z, r4.w};
 #pragma unroll
-                for (int i = j + 1; i < 16; ++i) x[i] = fmaf(-Ab[i * LCF + j], x[j], x[i]);
+                        for (int jj = 0; jj < 4; ++jj)
+                            if (j4 + jj < i) sum = fmaf(-r[jj], x[j4 + jj], sum);
+                    }
+                x[i] = sum;
             }
-        }
-        sync();   // every column has read the block before anyone overwrites it
-        if (tid < CH) {
+            __syncwarp();   // every column has read the block before anyone overwrites it
 #pragma unroll
             for (int i = 0; i < 16; ++i) Ab[i * LCF + col] = x[i];
+            __syncwarp();
         }
+        float* P = sA + 32 * warp * (LCF + 1);
+        float acc[2][4] = {}, acc2[2][4] = {};
+        block16_mma_ld<LCF>(acc, P + 16 * LCF, P, lane);
+        block16_store_ld<LCF>(P + 16, acc, 1.f, lane);
+        __syncwarp();
+        block16_mma_ld<LCF>(acc2, P + 16 * LCF + 16, P + 16, lane);
+        __syncwarp();
+        block16_store_ld<LCF>(P + 16 * LCF, acc2, -1.f, lane);
     }
     sync();
-    for (int b = 1; b < 4; ++b) {
-        // warp c < b: X = sum_m A_bm T_mc, parked in block (c, b); then T_bc = -T_bb X
-        float acc2[2][4] = {};
-        if (warp < b) {
-            const int c = warp;
-            float acc[2][4] = {};
-            for (int m = c; m < b; ++m)
-                block16_mma_ld<LCF>(acc, sA + (16 * b) * LCF + 16 * m, sA + (16 * m) * LCF + 16 * c, lane);
-            float* X = sA + (16 * c) * LCF + 16 * b;
-            block16_store_ld<LCF>(X, acc, 1.f, lane);
-            __syncwarp();
-            block16_mma_ld<LCF>(acc2, sA + (16 * b) * LCF + 16 * b, X, lane);
-        }
-        sync();   // row b of A has been read by every warp that needs it
-        if (warp < b) block16_store_ld<LCF>(sA + (16 * b) * LCF + 16 * warp, acc2, -1.f, lane);
-        sync();
+    const int r = 16 * ((warp >> 1) & 1), c = 16 * (warp & 1);   // this warp's block of the 32 x 32 one
+    float* X = sA + 32;                                          // rows 0 .. 31, columns 32 .. 63
+    if (warp < 4) {
+        float acc[2][4] = {};
+        block16_mma_ld<LCF>(acc, sA + (32 + r) * LCF + 16, sA + 16 * LCF + c, lane);   // T_11's upper block is zero
+        if (c == 0) block16_mma_ld<LCF>(acc, sA + (32 + r) * LCF, sA, lane);
+        block16_store_ld<LCF>(X + r * LCF + c, acc, 1.f, lane);
     }
+    sync();
+    if (warp < 4) {
+        float acc[2][4] = {};
+        block16_mma_ld<LCF>(acc, sA + (32 + r) * LCF + 32, X + c, lane);
+        if (r) block16_mma_ld<LCF>(acc, sA + (32 + r) * LCF + 48, X + 16 * LCF + c, lane);
+        block16_store_ld<LCF>(sA + (32 + r) * LCF + c, acc, -1.f, lane);
+    }
+    sync();
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -252,7 +265,8 @@ struct ClGroupShared {
     uint64_t bar_tma, bar_mma1, bar_mma2;
     int ticket;
     int pad;
-    float sG[CH], sBeta[CH];
+    float sG[CH];
+    alignas(16) float sGam[CH], sBeta[CH];
 };
 
 // One (chunk, head) tile by a group of CL_THREADS threads (local index `tid`) that synchronise on hardware
@@ -267,6 +281,7 @@ __device__ __forceinline__ void chunk_fwd_tile(const CUtensorMap& tmK, const CUt
     uint64_t& bar_mma1 = gs.bar_mma1;
     uint64_t& bar_mma2 = gs.bar_mma2;
     float* sG = gs.sG;
+    float* sGam = gs.sGam;
     float* sBeta = gs.sBeta;
     uint8_t* sKQ = sm;                 // per k-half h: [K rows 0-63 | Q rows 64-127], 16 KB each
     uint8_t* sKt = sKQ + 32768;        // per k-half: 8 KB
@@ -305,6 +320,8 @@ __device__ __forceinline__ void chunk_fwd_tile(const CUtensorMap& tmK, const CUt
         sb += __shfl_sync(0xffffffffu, sa, 31);
         sG[lane] = sa;
         sG[lane + 32] = sb;
+        sGam[lane] = __expf(sa);
+        sGam[lane + 32] = __expf(sb);
     }
     // The group's previous tile is published here, behind a barrier that is needed anyway: the barrier
     // orders every thread's stores before thread 0, whose fence (cumulative) then orders them before the flag.
@@ -343,7 +360,7 @@ __device__ __forceinline__ void chunk_fwd_tile(const CUtensorMap& tmK, const CUt
         const int hf = e >> 9, i = (e >> 3) & 63, ch = e & 7;
         const uint32_t off = sw128_chunk(i, ch);
         const uint4 w = *reinterpret_cast<const uint4*>(sKQ + hf * 16384 + BOX + off);
-        const float f = a.scale * __expf(sG[i]);
+        const float f = a.scale * sGam[i];
         const __nv_bfloat162* p2 = reinterpret_cast<const __nv_bfloat162*>(&w);
         uint32_t o[4];
 #pragma unroll
@@ -422,28 +439,35 @@ __device__ __forceinline__ void chunk_fwd_tile(const CUtensorMap& tmK, const CUt
     ut_inverse_64_inplace(sA, tid, sync);
 
     // ---- operand images: Tbg (shared), Tb and T (HBM) -----------------------------------------
-    for (int e = tid; e < CH * 8; e += CL_THREADS) {
-        const int i = e >> 3, ch = e & 7;
-        const float4 t0 = *reinterpret_cast<const float4*>(sA + i * LCF + ch * 8);
-        const float4 t1 = *reinterpret_cast<const float4*>(sA + i * LCF + ch * 8 + 4);
-        const float tv[8] = {t0.x, t0.y, t0.z, t0.w, t1.x, t1.y, t1.z, t1.w};
-        float t[8], tb8[8], tbg[8];
+    {
+        const int ch = tid & 7;   // the same eight columns in every round
+        float bj[8], gj[8];
 #pragma unroll
-        for (int x = 0; x < 8; ++x) {
-            const int j = ch * 8 + x;
-            t[x] = j <= i ? tv[x] : 0.f;   // above the diagonal the array holds scratch
-            tb8[x] = t[x] * sBeta[j];
-            tbg[x] = tb8[x] * __expf(sG[j]);
+        for (int x = 0; x < 8; x += 4) {
+            const float4 b4 = *reinterpret_cast<const float4*>(sBeta + ch * 8 + x), g4 = *reinterpret_cast<const float4*>(sGam + ch * 8 + x);
+            bj[x] = b4.x; bj[x + 1] = b4.y; bj[x + 2] = b4.z; bj[x + 3] = b4.w;
+            gj[x] = g4.x; gj[x + 1] = g4.y; gj[x + 2] = g4.z; gj[x + 3] = g4.w;
         }
-        const uint32_t off = sw128_chunk(i, ch);
-        *reinterpret_cast<uint4*>(sTb + off) = make_uint4(pack_bf16(tbg[0], tbg[1]), pack_bf16(tbg[2], tbg[3]),
-                                                         pack_bf16(tbg[4], tbg[5]), pack_bf16(tbg[6], tbg[7]));
-        *reinterpret_cast<uint4*>(a.Tb + tile * REC_BYTES + off) =
-            make_uint4(pack_bf16(tb8[0], tb8[1]), pack_bf16(tb8[2], tb8[3]), pack_bf16(tb8[4], tb8[5]),
-                       pack_bf16(tb8[6], tb8[7]));
-        if (a.save)
-            *reinterpret_cast<uint4*>(a.Tm + tile * 8192 + off) =
+#pragma unroll 1
+        for (int i = tid >> 3; i < CH; i += CL_THREADS / 8) {
+            const float4 t0 = *reinterpret_cast<const float4*>(sA + i * LCF + ch * 8);
+            const float4 t1 = *reinterpret_cast<const float4*>(sA + i * LCF + ch * 8 + 4);
+            float t[8] = {t0.x, t0.y, t0.z, t0.w, t1.x, t1.y, t1.z, t1.w};
+            const uint32_t off = sw128_chunk(i, ch);
+#pragma unroll
+            for (int x = 0; x < 8; ++x) t[x] = ch * 8 + x <= i ? t[x] : 0.f;   // above the diagonal the array holds scratch
+            if (a.save)
+                *reinterpret_cast<uint4*>(a.Tm + tile * 8192 + off) =
+                    make_uint4(pack_bf16(t[0], t[1]), pack_bf16(t[2], t[3]), pack_bf16(t[4], t[5]), pack_bf16(t[6], t[7]));
+#pragma unroll
+            for (int x = 0; x < 8; ++x) t[x] *= bj[x];
+            *reinterpret_cast<uint4*>(a.Tb + tile * REC_BYTES + off) =
                 make_uint4(pack_bf16(t[0], t[1]), pack_bf16(t[2], t[3]), pack_bf16(t[4], t[5]), pack_bf16(t[6], t[7]));
+#pragma unroll
+            for (int x = 0; x < 8; ++x) t[x] *= gj[x];
+            *reinterpret_cast<uint4*>(sTb + off) =
+                make_uint4(pack_bf16(t[0], t[1]), pack_bf16(t[2], t[3]), pack_bf16(t[4], t[5]), pack_bf16(t[6], t[7]));
+        }
     }
     fence_proxy_async();
     tc_fence_before();
@@ -1023,25 +1047,24 @@ __device__ __forceinline__ void chunk_fwd_workers(const CUtensorMap& tmK, const 
         fence_mbar_init();
     }
     gsync();
-    // The group's leader draws tickets one tile ahead, so the round trip of the atomic is hidden by the
-    // tile in progress.  A ticket that has been drawn is always worked off before the group stops.
-    auto draw = [&]() {
-        int t = -1;
-        if (*reinterpret_cast<volatile int*>(sc.tickets) < limit) {
-            t = atomicAdd(sc.tickets, 1);
-            if (t >= sc.ntickets) t = -1;
-        }
-        return t;
-    };
+    // Tickets are drawn one tile ahead by a thread that leads nothing else, and looked at only when the tile in
+    // progress is done: nobody waits for the atomic.  A ticket that has been drawn is always worked off before the group
+    // stops; it stops drawing when the tickets out, by its own last one and the groups at work, reach the limit.
+    constexpr int DRAWER = CL_THREADS - 32;
+    const int ahead = (int)gridDim.x * FWD_GROUPS;
     uint32_t ph = 0;
     int* publish = nullptr;   // flag of the tile the group finished last
-    int next = ltid == 0 ? draw() : -1;
+    int next = -1;
+    if (ltid == DRAWER && *reinterpret_cast<volatile int*>(sc.tickets) < limit) next = atomicAdd(sc.tickets, 1);
     while (true) {
-        if (ltid == 0) gs.ticket = next;
+        if (ltid == DRAWER) gs.ticket = next < sc.ntickets ? next : -1;
         gsync();
         const int t = gs.ticket;
         if (t < 0) break;
-        if (ltid == 0) next = draw();
+        if (ltid == DRAWER) {
+            next = -1;
+            if (t + ahead < limit || limit >= sc.ntickets) next = atomicAdd(sc.tickets, 1);
+        }
         int c, h;
         if (sc.order) {   // packed batch: position-major order from the sorted list, heads innermost
             const int j = t / cl.H;
