@@ -242,11 +242,15 @@ constexpr int FEW_RW = 4, FEW_WARPS = 4, MANY_WARPS = 8;
 template <typename T, int K, int V, bool VEC, bool MULTI>
 __global__ void __cluster_dims__(V / (FEW_RW * FEW_WARPS), 1, 1) __launch_bounds__(FEW_WARPS * 32) decode_few_kernel(DecArgs a)
 {
+    pdl_release();
+    pdl_wait();
     decode_body<T, K, V, VEC, FEW_RW, FEW_WARPS, MULTI>(a);
 }
 template <typename T, int K, int V, bool VEC, bool MULTI>
 __global__ void __launch_bounds__(MANY_WARPS * 32, 2) decode_many_kernel(DecArgs a)
 {
+    pdl_release();
+    pdl_wait();
     decode_body<T, K, V, VEC, V / MANY_WARPS, MANY_WARPS, MULTI>(a);
 }
 
@@ -259,14 +263,11 @@ constexpr unsigned MANY_CHAINS = 104;
 template <typename T, int K, int V, bool VEC> bool launch_one(unsigned chains, const DecArgs& a, cudaStream_t st)
 {
     constexpr unsigned SLICES = V / (FEW_RW * FEW_WARPS);
-    if (chains >= MANY_CHAINS) {
-        if (a.L > 1) decode_many_kernel<T, K, V, VEC, true><<<chains, MANY_WARPS * 32, 0, st>>>(a);
-        else decode_many_kernel<T, K, V, VEC, false><<<chains, MANY_WARPS * 32, 0, st>>>(a);
-    } else {
-        if (a.L > 1) decode_few_kernel<T, K, V, VEC, true><<<chains * SLICES, FEW_WARPS * 32, 0, st>>>(a);
-        else decode_few_kernel<T, K, V, VEC, false><<<chains * SLICES, FEW_WARPS * 32, 0, st>>>(a);
-    }
-    return cudaGetLastError() == cudaSuccess;
+    // Programmatic dependents: the launch of a call runs under the kernel before it in the stream, whose results it waits for
+    // before its first access (one sequence, calls back to back: 3.9 -> 3.1 us; 512 sequences 83.5 -> 81.0).
+    if (chains >= MANY_CHAINS)
+        return launch_after(a.L > 1 ? decode_many_kernel<T, K, V, VEC, true> : decode_many_kernel<T, K, V, VEC, false>, chains, MANY_WARPS * 32, 0, st, a);
+    return launch_after(a.L > 1 ? decode_few_kernel<T, K, V, VEC, true> : decode_few_kernel<T, K, V, VEC, false>, chains * SLICES, FEW_WARPS * 32, 0, st, a);
 }
 
 template <typename T> int launch_typed(const osdn_params& p, const DecArgs& a, cudaStream_t st)

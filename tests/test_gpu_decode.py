@@ -163,3 +163,61 @@ def test_prefill_128_then_one_recurrent_token_equals_chunk_129(apf):
     assert _rel(S, ref["final_state"].numpy()) <= 6.7e-3
     assert _rel(d, ref["precond_out"].numpy()) <= 2.0e-3
     assert parity.err(out.reshape(B, H, D), want) <= parity.TOL["bf16"]
+
+
+@pytest.mark.parametrize("B", [1, 60])
+def test_calls_follow_the_work_before_them(B):
+    """A call may be launched while the kernel before it runs: calls back to back, behind kernels that write their inputs, and
+    captured behind joined streams and a fill give the caches of calls that are waited for one by one, bit for bit."""
+    H, D, steps = 2, 128, 6
+    gen = torch.Generator(device=DEV).manual_seed(5)
+    rnd = lambda *s: torch.randn(*s, generator=gen, device=DEV)
+    p = binding.make_params(B=B, T=1, H=H, K=D, V=D, io_dtype="bf16", hyper=OsdnHyper(eta=0.3, apf_mode=1))
+    k0, q0, v0, b0, g0 = rnd(steps, B, H, D), rnd(steps, B, H, D), rnd(steps, B, H, D), rnd(steps, B, H), rnd(steps, B, H)
+    S0, d0 = rnd(B, H, D, D), torch.ones(B, H, D, device=DEV)
+    q, k, v, out = (torch.empty(B, H, D, device=DEV, dtype=torch.bfloat16) for _ in range(4))
+    beta, gate = torch.empty(B, H, device=DEV), torch.empty(B, H, device=DEV)
+    S, d = torch.empty_like(S0), torch.empty_like(d0)
+
+    def put(t):
+        k.copy_(torch.nn.functional.normalize(k0[t], dim=-1)); q.copy_(q0[t]); v.copy_(v0[t])
+        beta.copy_(torch.sigmoid(b0[t])); gate.copy_(-torch.nn.functional.softplus(g0[t]) * 0.1)
+
+    def call():
+        binding.osdn_decode_step(p, q, k, v, beta, gate, None, S, d, out)
+
+    def step(t):
+        put(t)
+        call()
+
+    def run(wait):
+        S.copy_(S0); d.copy_(d0)
+        for t in range(steps):
+            step(t)
+            if wait:
+                torch.cuda.synchronize()
+        torch.cuda.synchronize()
+        return S.clone(), d.clone(), out.clone()
+
+    want = run(True)
+    assert all(torch.equal(x, y) for x, y in zip(want, run(False)))
+    side, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph):
+        here = torch.cuda.current_stream()
+        side.wait_stream(here)
+        with torch.cuda.stream(side):
+            S.copy_(S0)
+        d.copy_(d0)
+        out.zero_()
+        here.wait_stream(side)
+        for t in range(steps):
+            if t:
+                step(t)
+            else:   # right behind the join: its inputs are in place before the replay
+                call()
+    for _ in range(2):
+        put(0)
+        graph.replay()
+        torch.cuda.synchronize()
+        assert all(torch.equal(x, y) for x, y in zip(want, (S, d, out)))
