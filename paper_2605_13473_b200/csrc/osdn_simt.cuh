@@ -148,6 +148,29 @@ __device__ __forceinline__ void load_gates(GateVecs& gv, const float* __restrict
     }
 }
 
+// 16 bytes on their way into shared memory, zeros where !in (nothing is read then); both addresses 16-byte aligned.
+__device__ __forceinline__ void copy16(float* dst, const float* src, bool in)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(umma::smem_u32(dst)), "l"(src), "r"(in ? 16 : 0) : "memory");
+}
+// Rows of N floats, contiguous in global memory, into rows of LD floats.
+template <int N, int LD, int NT> __device__ __forceinline__ void copy_rows(float* dst, const float* src, int rows)
+{
+#pragma unroll 4
+    for (int e = threadIdx.x; e < rows * N / 4; e += NT) copy16(dst + e / (N / 4) * LD + e % (N / 4) * 4, src + e * 4, true);
+}
+// An fp32 token tile like load_tile's, asynchronously.
+template <int D, int LD, int NT> __device__ __forceinline__ void copy_tile(float* dst, const float* src, int tok0, int len, int H, int h)
+{
+    const float* p = src + ((size_t)tok0 * H + h) * D;
+#pragma unroll 4
+    for (int e = threadIdx.x; e < CH * D / 4; e += NT) {
+        const int i = e / (D / 4), c = e % (D / 4) * 4;
+        copy16(dst + i * LD + c, p + (size_t)(i < len ? i : 0) * H * D + c, i < len);
+    }
+}
+__device__ __forceinline__ void copies_landed() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
 // Load a [64 x D] token tile into shared memory (rows beyond len are zero), 16 bytes at a time.
 template <typename T, int D, int NT>
 __device__ __forceinline__ void load_tile(float* dst, int ld, const T* __restrict__ src, int tok0, int len,
@@ -411,12 +434,13 @@ __global__ void __launch_bounds__(CL_NT, LocalFwd<T, K, V, CG>::MIN_CTAS) chunk_
     const int grp = threadIdx.x >> 8;
     const Lane l{(int)(threadIdx.x & 255) >> 4, (int)threadIdx.x & 15};
 
+    copy_tile<K, LD, CL_NT>(sKt, a.ktil, tok0, len, H, h);   // on their way while k and q are converted
+    if constexpr (CG) copy_tile<K, LD, CL_NT>(sG, a.gate, tok0, len, H, h);
     load_tile<T, K, CL_NT>(sK, LD, static_cast<const T*>(a.k), tok0, len, H, h);
-    load_tile<float, K, CL_NT>(sKt, LD, a.ktil, tok0, len, H, h);
     load_tile<T, K, CL_NT>(sQ, LD, static_cast<const T*>(a.q), tok0, len, H, h);
+    copies_landed();
     bool safe = true;
     if constexpr (CG) {
-        load_tile<float, K, CL_NT>(sG, LD, a.gate, tok0, len, H, h);
         if (threadIdx.x < CH) gv.beta[threadIdx.x] = threadIdx.x < len ? a.beta[(size_t)(tok0 + threadIdx.x) * H + h] : 0.f;
         __syncthreads();
         gate_prefix<K, LD>(sG, sL, tmp);
@@ -491,6 +515,14 @@ __global__ void __launch_bounds__(CL_NT, LocalFwd<T, K, V, CG>::MIN_CTAS) chunk_
             }
     }
     __syncthreads();
+    // v takes q's place while the first 64 threads substitute (read where it is, inside the product, it held the tile up for
+    // 20000 of 64000 cycles at K = V = 128)
+    if constexpr (V <= K) {
+        const Rows<T, V> v = rows_of<T, V>(a.v, tok0, len, H, h);
+        if (threadIdx.x >= 64)
+#pragma unroll 4
+            for (int e = threadIdx.x - 64; e < CH * V / 4; e += CL_NT - 64) st4(sQ + e / (V / 4) * LD + e % (V / 4) * 4, v(e / (V / 4), e % (V / 4) * 4));
+    }
     ut_inverse_64(sA, sT, tmp);
     if (a.Tm) {
         float* Tg = a.Tm + tile * CH * CH;
@@ -514,7 +546,10 @@ __global__ void __launch_bounds__(CL_NT, LocalFwd<T, K, V, CG>::MIN_CTAS) chunk_
         zero(acc);
         const Rows<T, V> v = rows_of<T, V>(a.v, tok0, len, H, h);
         tile_mm<false, false, TV>(acc, 0, jend, l, [&](int m, int j) { return ld4(sT + m * LC + j); },
-                                  [&](int j, int n) { return gv.beta[j] * v(j, n); });
+                                  [&](int j, int n) {
+                                    if constexpr (V <= K) return gv.beta[j] * ld4(sQ + j * LD + n);
+                                    else return gv.beta[j] * v(j, n);
+                                });
         float* Ug = a.U + tile * CH * V;
 #pragma unroll
         for (int i = 0; i < 4; ++i)
@@ -1011,6 +1046,11 @@ __global__ void __launch_bounds__(CL_NT) chunk_local_bwd_kernel(ChunkArgs a)
 
     bool safe = true;
     if constexpr (CG) safe = __syncthreads_and(threadIdx.x >= K || fabsf(Gg[(CH - 1) * K + (threadIdx.x & (K - 1))]) <= SAFE_RANGE);
+    // what is needed as it is comes asynchronously, under the gate factors
+    copy_rows<CH, LC, CL_NT>(sT, a.Tm + tile * CH * CH, CH);
+    copy_rows<V, LU, CL_NT>(sU, dUg, CH);
+    if constexpr (CG) copy_rows<K, LD, CL_NT>(sQ, a.Qg + tile * CH * K, CH);
+#pragma unroll 2
     for (int e = threadIdx.x; e < CH * K / 4; e += CL_NT) {
         const int i = e / (K / 4), n = e % (K / 4) * 4;
         const Rows<float, K> ktr = rows_of<float, K>(a.ktil, tok0, len, H, h);
@@ -1018,17 +1058,12 @@ __global__ void __launch_bounds__(CL_NT) chunk_local_bwd_kernel(ChunkArgs a)
         if constexpr (CG) {
             k = expG(i, n) * k;
             if (safe) kt = expmG(i, n) * kt;
-            st4(sQ + i * LD + n, ld4(a.Qg + tile * CH * K + e * 4));
         } else {
             st4(sQ + i * LD + n, qr(i, n));
         }
         st4(sK + i * LD + n, k);
         st4(sKt + i * LD + n, kt);
     }
-#pragma unroll 2
-    for (int e = threadIdx.x; e < CH * CH / 4; e += CL_NT) st4(sT + (e / 16) * LC + (e % 16) * 4, ld4(a.Tm + tile * CH * CH + e * 4));
-#pragma unroll 4
-    for (int e = threadIdx.x; e < CH * V / 4; e += CL_NT) st4(sU + e / (V / 4) * LU + e % (V / 4) * 4, ld4(dUg + e * 4));
     if constexpr (CG) {
         if (threadIdx.x < CH) gv.beta[threadIdx.x] = threadIdx.x < len ? a.beta[(size_t)(tok0 + threadIdx.x) * H + h] : 0.f;
     } else {
@@ -1037,10 +1072,11 @@ __global__ void __launch_bounds__(CL_NT) chunk_local_bwd_kernel(ChunkArgs a)
     {
         const int n = threadIdx.x % K, part = threadIdx.x / K;
         float s = 0.f;
-#pragma unroll 8
+#pragma unroll 16
         for (int v = part; v < V; v += PARTS) s = fmaf(Sg[v * K + n], dSg[v * K + n], s);
         sRed[part][n] = s;
     }
+    copies_landed();
     __syncthreads();
 
     // row sums <x_i, y_i> of a 4 x TN tile, written by one lane per row
