@@ -149,6 +149,7 @@ __global__ void __launch_bounds__(128) phase1_spec_kernel(P1Fwd a)
     const long tile = w >> 1;
     const int half = (int)(w & 1);
     pdl_release();
+    pdl_wait();
     clear_regions(a.clear);
     if (tile >= (long)a.NT * a.H) return;
     const int c = (int)(tile / a.H), h = (int)(tile % a.H);
@@ -1014,6 +1015,7 @@ __global__ void __launch_bounds__(FwdPipe<K, MANY>::THREADS, FwdPipe<K, MANY>::C
     const int lane = threadIdx.x & 31, warp = P::role(threadIdx.x >> 5);
     const int chain = blockIdx.x;
     const int s = chain / a.H, h = chain % a.H, H = a.H;
+    pdl_wait();
     // packed batch: T_dense is the packed token count; a malformed offset pair is clamped into it
     const int t0 = a.cu ? min(max(a.cu[s], 0), a.T_dense) : s * a.T_dense;
     const int len = a.cu ? min(max(a.cu[s + 1], t0), a.T_dense) - t0 : a.T_dense;
@@ -1616,8 +1618,7 @@ __global__ void __launch_bounds__(Pipe<K>::THREADS, 1) phase1_bwd_seq_kernel(P1B
     const int coord = warp * 32 + lane;   // core warps
     const size_t mine = ((size_t)s * H + h) * K + coord;
     if (threadIdx.x == 0) init_bars(sh.bars, RevShared<T, K, VEC>::QN, P::CORE);
-    pdl_release();
-    pdl_wait();
+    pdl_wait();   // no early release: the next call's parallel pass would crowd on the SMs that this one leaves idle (8 x 2048 tokens: + 5 us)
     clear_regions(a.clear);
     if (warp < P::CORE) sh.lam[coord] = a.dprecond_out ? a.dprecond_out[mine] : 0.f;
     uint32_t rounds = 0, uses = 0;
@@ -1656,8 +1657,7 @@ int fwd_launch(const P1Fwd& a, cudaStream_t st)
     const long warps = (long)a.NT * a.H * 2;
     const unsigned gspec = (unsigned)((warps + 3) / 4);
     stage_mark(st, "phase1_spec");
-    if (a.hy.apf_mode == 3) phase1_spec_kernel<TI, TO, K, true><<<gspec, 128, 0, st>>>(a);
-    else phase1_spec_kernel<TI, TO, K, false><<<gspec, 128, 0, st>>>(a);
+    if (!launch_after(a.hy.apf_mode == 3 ? phase1_spec_kernel<TI, TO, K, true> : phase1_spec_kernel<TI, TO, K, false>, gspec, 128, 0, st, a)) return -1;
     stage_mark(st, "phase1_seq");
     const unsigned chains = (unsigned)(a.S * a.H);
     const bool okl = p1_variant(a.hy.apf_mode == 3, chains, [&](auto vec, auto many) {
@@ -1758,8 +1758,7 @@ int phase1_update(const osdn_params& p, const Hyper& hy, const void* k, const fl
             constexpr size_t smem = sizeof(PipeShared<T, K, VEC, MANY>);
             const auto kernel = phase1_stream_kernel<T, T, K, VEC, MANY>;
             if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return false;
-            kernel<<<chains, FwdPipe<K, MANY>::THREADS, smem, st>>>(pa);
-            return true;
+            return launch_after(kernel, chains, FwdPipe<K, MANY>::THREADS, smem, st, pa);
         });
     };
     using K64 = std::integral_constant<int, 64>;

@@ -43,6 +43,7 @@ build_table_kernel(int S, int T_dense, const int* __restrict__ cu, int NTmax, Ta
     __shared__ int s_scan[TBL_THREADS];
     __shared__ int s_carry;
     const int tid = threadIdx.x;
+    pdl_wait();
     if (tid == 0) {
         s_carry = 0;
         if (status) *status = 0;
@@ -197,9 +198,7 @@ int launch_build_table(const osdn_params& p, const WsLayout& L, void* ws, cudaSt
     Table tab = carve_table(ws, L);
     if (L.dense_T) return 0;   // dense batch: the table is arithmetic, nothing to build
     stage_mark(st, "build_table");
-    build_table_kernel<<<1, TBL_THREADS, 0, st>>>(L.S, p.T, p.cu_seqlens, L.NTmax, tab,
-                                                  reinterpret_cast<int*>(static_cast<char*>(ws) + L.status));
-    return cudaGetLastError() == cudaSuccess ? 1 : -1;
+    return launch_after(build_table_kernel, 1, TBL_THREADS, 0, st, L.S, p.T, p.cu_seqlens, L.NTmax, tab, reinterpret_cast<int*>(static_cast<char*>(ws) + L.status)) ? 1 : -1;
 }
 
 int simt_forward(const osdn_params& p, const Hyper& hy, const WsLayout& L, void* ws, const Pointers& a,

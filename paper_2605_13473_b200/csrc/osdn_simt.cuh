@@ -413,6 +413,7 @@ template <typename T, int K, int V, bool CG> struct LocalFwd {
 template <typename T, int K, int V, bool CG>
 __global__ void __launch_bounds__(CL_NT, LocalFwd<T, K, V, CG>::MIN_CTAS) chunk_local_fwd_kernel(ChunkArgs a)
 {
+    pdl_wait();
     extern __shared__ __align__(16) float sm[];
     constexpr int LD = K + 4, TK = K / 16, TV = V / 16;
     float* sK = sm;                   // k; channel gate: gamma (.) k
@@ -576,6 +577,7 @@ template <typename T, int K, bool CG, int LD, int NT> __device__ __forceinline__
 template <typename T, int K, int V, bool CG>
 __global__ void __launch_bounds__(256) output_kernel(ChunkArgs a)
 {
+    pdl_wait();
     extern __shared__ __align__(16) float sm[];
     constexpr int TV = V / 16, LD = K + 4, NT = 256;
     float* sQ = sm;                  // [64][LD]
@@ -638,6 +640,7 @@ template <int K, int V> constexpr size_t pre_bwd_smem() { return sizeof(float) *
 template <typename T, int K, int V, bool CG>
 __global__ void __launch_bounds__(256) pre_bwd_kernel(ChunkArgs a)
 {
+    pdl_wait();
     extern __shared__ __align__(16) float sm[];
     constexpr int TV = V / 16, TK = K / 16, NT = 256;
     float* sP = sm;
@@ -792,6 +795,7 @@ template <int K> struct NarrowShared {
 template <int K, int V, bool BWD, bool CG>
 __global__ void __launch_bounds__(CNT) chain_narrow_kernel(ChainArgs a)
 {
+    pdl_wait();
     extern __shared__ __align__(16) float sm[];
     using Sh = NarrowShared<K>;
     constexpr int LD = Sh::LD, CW = Sh::CW, G = Sh::GROUPS, NI = CH / G, PER = VS * K / CNT;   // state values per thread
@@ -892,6 +896,7 @@ template <int K> struct WideShared {
 template <int K, int V, bool BWD, bool CG>
 __global__ void __launch_bounds__(K / 64 * 256) chain_wide_kernel(ChainArgs a)
 {
+    pdl_wait();
     extern __shared__ __align__(16) float sm[];
     using Sh = WideShared<K>;
     constexpr int LD = Sh::LD, LW = Sh::LW, G = Sh::G, NT = G * 256;
@@ -1007,6 +1012,7 @@ template <int K, int V> constexpr size_t local_bwd_smem() { return sizeof(float)
 template <typename T, int K, int V, bool CG>
 __global__ void __launch_bounds__(CL_NT) chunk_local_bwd_kernel(ChunkArgs a)
 {
+    pdl_wait();
     extern __shared__ __align__(16) float sm[];
     constexpr int LD = K + 4, LU = V + 4, TK = K / 16, TV = V / 16, PARTS = CL_NT / K;
     float* sK = sm;                 // as in the forward: channel gate gamma (.) k
@@ -1376,10 +1382,10 @@ template <int K, int V, bool BWD, bool CG> int launch_chain(const ChainArgs& ch,
     stage_mark(st, BWD ? "chain_bwd" : "chain_fwd");
     if (narrow * 10 <= wide * WIDE_STEP_TENTHS<K>) {
         if (!set_smem(chain_narrow_kernel<K, V, BWD, CG>, sizeof(NarrowShared<K>))) return -1;
-        chain_narrow_kernel<K, V, BWD, CG><<<dim3(chains, V / VS), CNT, sizeof(NarrowShared<K>), st>>>(ch);
+        if (!launch_after(chain_narrow_kernel<K, V, BWD, CG>, dim3(chains, V / VS), CNT, sizeof(NarrowShared<K>), st, ch)) return -1;
     } else {
         if (!set_smem(chain_wide_kernel<K, V, BWD, CG>, sizeof(WideShared<K>))) return -1;
-        chain_wide_kernel<K, V, BWD, CG><<<dim3(chains, V / WS), K / 64 * 256, sizeof(WideShared<K>), st>>>(ch);
+        if (!launch_after(chain_wide_kernel<K, V, BWD, CG>, dim3(chains, V / WS), K / 64 * 256, sizeof(WideShared<K>), st, ch)) return -1;
     }
     return 1;
 }
@@ -1405,7 +1411,7 @@ int chunk_forward(const osdn_params& p, const Hyper& hy, const WsLayout& L, void
     using LF = LocalFwd<T, K, V, CG>;
     if (!set_smem(chunk_local_fwd_kernel<T, K, V, CG>, LF::SMEM)) return -1;
     stage_mark(st, "chunk_local_fwd");
-    chunk_local_fwd_kernel<T, K, V, CG><<<tiles, CL_NT, LF::SMEM, st>>>(c);
+    if (!launch_after(chunk_local_fwd_kernel<T, K, V, CG>, tiles, CL_NT, LF::SMEM, st, c)) return -1;
     ChainArgs ch{};
     ch.H = p.H; ch.tab = c.tab; ch.X = c.W; ch.Y = c.Ktr; ch.D0 = c.U; ch.gC = c.gC; ch.gam = c.gam; ch.S0 = a.init_state;
     ch.D = const_cast<float*>(c.dU); ch.Sall = const_cast<float*>(c.Sn); ch.Sfin = a.final_state;
@@ -1413,7 +1419,7 @@ int chunk_forward(const osdn_params& p, const Hyper& hy, const WsLayout& L, void
     if (launch_chain<K, V, false, CG>(ch, L.S * p.H, st) < 0) return -1;
     if (!set_smem(output_kernel<T, K, V, CG>, output_smem<K, V>())) return -1;
     stage_mark(st, "chunk_output");
-    output_kernel<T, K, V, CG><<<tiles, 256, output_smem<K, V>(), st>>>(c);
+    if (!launch_after(output_kernel<T, K, V, CG>, tiles, 256, output_smem<K, V>(), st, c)) return -1;
     return cudaGetLastError() == cudaSuccess ? 3 : -1;
 }
 
@@ -1429,7 +1435,7 @@ int chunk_backward(const osdn_params& p, const Hyper& hy, const WsLayout& L, voi
     const dim3 tiles = tile_grid(L.NTmax, p.H);
     if (!set_smem(pre_bwd_kernel<T, K, V, CG>, pre_bwd_smem<K, V>())) return -1;
     stage_mark(st, "chunk_pre_bwd");
-    pre_bwd_kernel<T, K, V, CG><<<tiles, 256, pre_bwd_smem<K, V>(), st>>>(c);
+    if (!launch_after(pre_bwd_kernel<T, K, V, CG>, tiles, 256, pre_bwd_smem<K, V>(), st, c)) return -1;
     ChainArgs ch{};
     ch.H = p.H; ch.tab = c.tab; ch.X = c.Ktr; ch.Y = c.W; ch.D0 = c.ddU; ch.G0 = c.dSn; ch.gC = c.gC; ch.gam = c.gam; ch.S0 = a.dfinal_state;
     ch.D = c.ddU; ch.Sall = c.dSn; ch.Sfin = a.dinit_state;
@@ -1437,7 +1443,7 @@ int chunk_backward(const osdn_params& p, const Hyper& hy, const WsLayout& L, voi
     if (launch_chain<K, V, true, CG>(ch, L.S * p.H, st) < 0) return -1;
     if (!set_smem(chunk_local_bwd_kernel<T, K, V, CG>, local_bwd_smem<K, V>())) return -1;
     stage_mark(st, "chunk_local_bwd");
-    chunk_local_bwd_kernel<T, K, V, CG><<<tiles, CL_NT, local_bwd_smem<K, V>(), st>>>(c);
+    if (!launch_after(chunk_local_bwd_kernel<T, K, V, CG>, tiles, CL_NT, local_bwd_smem<K, V>(), st, c)) return -1;
     return cudaGetLastError() == cudaSuccess ? 3 : -1;
 }
 

@@ -196,6 +196,50 @@ def test_backward_tiles_at_their_edges(lens, kind):
         assert not torch.isnan(x.float()).any() and torch.equal(x, y)
 
 
+@pytest.mark.parametrize("io,K,cg,lens", [("bf16", 128, 0, [130, 130]), ("bf16", 128, 0, [70, 0, 200]), ("fp32", 64, 0, [130, 130]), ("fp32", 64, 1, [130])])
+def test_calls_follow_the_work_before_them(io, K, cg, lens):
+    """Every kernel of a call, the first one too, may be launched while the one before it in the stream runs.  Behind kernels
+    that write its inputs and its cotangents, and captured behind a fill: the results of calls that are waited for, bit for bit."""
+    hy = OsdnHyper(eta=0.003, apf_mode=2, channel_gate=cg)
+    inp = draw(f"follow_{io}_{cg}", 7950 + len(lens), lens, 2, K, K, io, dense_B=len(lens) if len(set(lens)) == 1 else 0, hyper=hy,
+               with_dout=True, with_log_ret=True, with_state_cotangents=True)
+    b = binding.DeviceBundle(inp, DEV, need_bwd=True)
+    names = [x for x in ("q", "k", "v", "beta", "gate", "log_ret", "dout") if getattr(b, x) is not None]
+    kept = {x: getattr(b, x).clone() for x in names}
+
+    def call():
+        for x in names:
+            getattr(b, x).copy_(kept[x])
+        b.fwd(save=True)
+        b.bwd(residuals_valid=True)
+
+    def spoil():
+        for x in names:
+            getattr(b, x).fill_(0.25)
+
+    results = []
+    for wait in (True, False):
+        spoil()
+        torch.cuda.synchronize()
+        call()
+        if wait:
+            torch.cuda.synchronize()
+        call()
+        torch.cuda.synchronize()
+        results.append([x.clone() for x in (b.out, b.final_state, b.precond_out, b.dq, b.dk, b.dv)])
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        b.dq.zero_()
+        call()
+    spoil()
+    graph.replay()
+    torch.cuda.synchronize()
+    assert b.device_status() == 0
+    results.append([b.out, b.final_state, b.precond_out, b.dq, b.dk, b.dv])
+    for other in results[1:]:
+        assert all(torch.equal(x, y) for x, y in zip(results[0], other))
+
+
 @pytest.mark.parametrize("B,H,L", [(49, 3, 8), (37, 4, 9), (191, 1, 1), (192, 1, 1), (50, 3, 17), (103, 1, 1), (104, 1, 1), (103, 1, 9), (52, 2, 9)])
 @pytest.mark.parametrize("io,K,V,apf", [("bf16", 128, 128, 1), ("fp32", 64, 128, 2), ("fp32", 128, 64, 3)])
 def test_decode_on_both_sides_of_its_dispatch(B, H, L, io, K, V, apf):
