@@ -120,11 +120,6 @@ __device__ __forceinline__ void zero_tail_rows(uint8_t* box, int len, int tid, i
         *reinterpret_cast<uint4*>(box + (len + e / 8) * 128 + (e % 8) * 16) = make_uint4(0, 0, 0, 0);
 }
 
-// ---------------------------------------------------------------------------------------------
-// fp32 scratch rows of the chunk-local backward: odd stride, one row per lane without bank conflicts
-// ---------------------------------------------------------------------------------------------
-constexpr int LC = CH + 1;
-
 // fp32 value as a TF32 operand (round to nearest)
 __device__ __forceinline__ uint32_t to_tf32(float x)
 {
