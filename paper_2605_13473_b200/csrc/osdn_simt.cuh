@@ -722,9 +722,8 @@ template <int K, int NT> __device__ __forceinline__ void fetch_group(Stage<K>& g
     }
     copies_group();
 }
-// One bulk copy per row by the first 128 threads.  Wide slices take this form: their step hides the issue, and the lookups of
-// the 16-byte copies would compete with its products (channel gate, 8 x 2048 tokens, 8 heads, reverse chain: 336 us
-// against 358).
+// One bulk copy per row by the first 128 threads.  Wide slices take this form: their step hides the issue (channel gate, 8 x 2048
+// tokens, 8 heads, reverse chain: 336 us against 358 with the copies above; forward chains equal).
 template <int K> __device__ __forceinline__ void fetch_stage(Stage<K>& g, const ChainArgs& a, size_t tile, uint64_t* bar)
 {
     if (threadIdx.x == 0) umma::mbar_expect_tx(bar, 2 * CH * K * 4);
@@ -1379,9 +1378,9 @@ template <typename F> bool set_smem(F* kernel, size_t bytes)
 
 // Narrow or wide slices: whichever walk is expected to end first.  What decides is how many waves of CTAs each cut makes; a
 // wave of wide slices (eight times the rows) takes as long as WIDE_STEP waves of narrow ones.  Measured, 512 tokens, forward
-// chain, microseconds for 1, 2, 3, 4, 5 waves of narrow slices against one of wide ones: K = 64 29, 48, 64 against 53;
-// K = 128 27, 46, 66, 86, 106 against 86.
-template <int K> constexpr int WIDE_STEP_TENTHS = K == 64 ? 25 : 35;
+// chain, microseconds for 1, 2, 3, 4, 5 waves of narrow slices against one of wide ones: K = 64 25 (18 with one CTA to an SM),
+// 45, 64, 82 against 53; K = 128 25, 43, 59, 78, 96 against 86 (channel gate, reverse chain 27, -, 64, 84, 104 against 88).
+template <int K> constexpr int WIDE_STEP_TENTHS = K == 64 ? 25 : 40;
 template <int K, int V, bool BWD, bool CG> int launch_chain(const ChainArgs& ch, int chains, cudaStream_t st)
 {
     const int SLOTS = num_sms() * (K == 64 ? 2 : 1);   // CTAs of either kind that fit an SM: by their shared memory

@@ -143,13 +143,23 @@ def test_chains_in_wide_slices(io, K):
 
 @pytest.mark.parametrize("io,cg,gates", [("fp32", 0, "softplus"), ("bf16", 0, "softplus"), ("fp32", 1, "softplus"), ("fp32", 1, "strong"), ("bf16", 1, "mixture")])
 def test_chains_in_wide_slices_of_128_rows(io, cg, gates):
-    """K = V = 128 in wide slices, two to a chain (from 28 chains on): scalar and channel gates, weak and strong."""
+    """K = V = 128 in wide slices, two to a chain (from 38 chains on): scalar and channel gates, weak and strong."""
     hy = OsdnHyper(eta=0.003, apf_mode=2, channel_gate=cg)
     inp = draw("wide128", 7250 + cg, [150] * 8, 5, 128, 128, io, dense_B=8, hyper=hy, gate_kind=gates, with_dout=True,
                with_log_ret=True, with_state=True, with_state_cotangents=True)
     got = run_inputs_bwd(inp, flags=binding.FLAG_FORCE_SIMT)
     ref = parity.oracle_all(inp, True, got["projection_masks"])
     parity.compare(got, ref, io, parity.FWD_KEYS + parity.BWD_KEYS, f"wide128_{io}_{cg}_{gates}")
+
+
+@pytest.mark.parametrize("B,L", [(37, 150), (38, 150), (37, 64), (9, 129)])
+@pytest.mark.parametrize("cg", [0, 1])
+def test_chains_on_both_sides_of_the_slice_rule(B, L, cg):
+    """K = V = 128: the most chains that narrow slices take (four waves), one more, one chunk only, one token past two chunks."""
+    hy = OsdnHyper(eta=0.003, apf_mode=2, channel_gate=cg)
+    inp = draw(f"slices_{B}_{L}", 7270 + B + cg, [L] * B, 1, 128, 128, "fp32", dense_B=B, hyper=hy, with_dout=True,
+               with_log_ret=True, with_state=True, with_state_cotangents=True)
+    _all_outputs(inp, f"slices_{B}_{L}_{cg}")
 
 
 def test_backward_twice_on_the_same_residuals():
