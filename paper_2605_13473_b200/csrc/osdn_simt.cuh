@@ -695,7 +695,7 @@ __global__ void __launch_bounds__(256) pre_bwd_kernel(ChunkArgs a)
 //   forward   X = W,   Y = Ktr, D0 = U,    G0 = 0,                  chunks ascending  (D = dU,  S = state)
 //   backward  X = Ktr, Y = W,   D0 = ddU0, G0 = scale dO^T Qg,      chunks descending (D = ddU, S = its cotangent)
 // and rows of S do not interact, so a chain is cut into slices of rows, one CTA each.  A tile's X and Y rows
-// arrive by bulk copies, one chunk ahead.
+// arrive by asynchronous copies, one chunk ahead.
 // ---------------------------------------------------------------------------------------
 struct ChainArgs {
     int H;
