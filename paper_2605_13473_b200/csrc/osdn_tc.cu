@@ -1507,6 +1507,11 @@ constexpr size_t CBW_SMEM = R_M1 + 8192 + 1024;
 //   e_a    images of M1 and dVb written                                                    epilogue -> issuer
 //   e_d    images of M2 written, dv staged, <dS, S> formed                                 epilogue -> issuer, producer
 //   e_f    everything of the tile is read; dq, dk staged, partial sums written             epilogue -> issuer, producer
+// and in a tile of fewer than 64 tokens
+//   zero   the rows beyond it are cleared                                                  epilogue -> issuer, epilogue
+//   rows   dq, dk, dv are staged                                                           epilogue -> epilogue
+// A wait that runs out ends its warp's loop and no other's: what a warp waits for between two tiles has to be an mbarrier,
+// whose wait is bounded. (A hardware barrier would wait for the warps that have left.)
 // A copy of the next tile is requested as soon as the space that it lands in is dead, the next tile's first products run
 // under this tile's last epilogue.
 // What bounds it: with three dependent phases (five when dL/dT was formed from dW K^T and ddU V^T and carried through
@@ -1518,7 +1523,7 @@ __device__ __forceinline__ void chunk_bwd_role(const CUtensorMap& tmQ, const CUt
                                                const CUtensorMap& tmDK, const CUtensorMap& tmDV, const TcChunkBwdArgs& a,
                                                uint8_t* sm, uint32_t tb, const TileQueue& tq)
 {
-    __shared__ uint64_t bar_vec[2], bar_c, bar_s, bar_tok, bar_v, bar_zero, bar_mma[4], bar_ea, bar_ed, bar_ef;
+    __shared__ uint64_t bar_vec[2], bar_c, bar_s, bar_tok, bar_v, bar_zero, bar_rows, bar_mma[4], bar_ea, bar_ed, bar_ef;
     __shared__ int sInfo[2][4];                            // tile (-1: no more), first token, length, head
     __shared__ unsigned sSkipW[2][2];
     __shared__ __align__(16) float sVec[2][4][CH];         // G_i, gamma_i = exp(G_i), rho_i = exp(G_C - G_i), beta_i
@@ -1530,7 +1535,7 @@ __device__ __forceinline__ void chunk_bwd_role(const CUtensorMap& tmQ, const CUt
     const bool lead = lane == 0;
     if (tid == 0) {
         for (uint64_t* b : {&bar_vec[0], &bar_vec[1], &bar_c, &bar_s, &bar_tok, &bar_v, &bar_mma[0], &bar_mma[1], &bar_mma[2], &bar_mma[3]}) mbar_init(b, 1);
-        for (uint64_t* b : {&bar_zero, &bar_ea, &bar_ed, &bar_ef}) mbar_init(b, CBW_WARPS);
+        for (uint64_t* b : {&bar_zero, &bar_rows, &bar_ea, &bar_ed, &bar_ef}) mbar_init(b, CBW_WARPS);
         fence_mbar_init();
     }
     tc_fence_before();
@@ -1890,9 +1895,9 @@ __device__ __forceinline__ void chunk_bwd_role(const CUtensorMap& tmQ, const CUt
                 for (const uint32_t reg : {R_DO, R_Q, R_K, R_KT, R_V})
                     for (int hf = 0; hf < 2; ++hf) zero_tail_rows(sm + reg + hf * BOX, len, tid, CBW_THREADS);
                 fence_proxy_async();
-                named_sync(1, CBW_THREADS);
+                __syncwarp();
                 if (lane == 0) mbar_arrive(&bar_zero);
-                ++ragged;
+                if (!mbar_wait(&bar_zero, ragged & 1, a.status, ERR_TMA)) break;
             }
             // ---- M1 = scale Gamma (.) lower(dP') and dVb^T as operands
             float gam[8], dvb[2][8];   // Gamma_ij = exp(G_i - G_j), j <= i (else 0); index 4 octet + 2 (row half) + column parity
@@ -2122,8 +2127,10 @@ __device__ __forceinline__ void chunk_bwd_role(const CUtensorMap& tmQ, const CUt
             }
             fence_proxy_async();
             tc_fence_before();
-            if (len < CH) {   // a ragged chunk leaves row by row
-                named_sync(1, CBW_THREADS);
+            if (len < CH) {   // a ragged chunk leaves row by row, once every warp has staged its part
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&bar_rows);
+                if (!mbar_wait(&bar_rows, ragged++ & 1, a.status, ERR_MMA2)) break;
                 for (int e = tid; e < len * 16; e += CBW_THREADS) {
                     const int j = e >> 4, ch = e & 15;
                     const size_t g = ((size_t)(tok0 + j) * H + h) * KD + ch * 8;

@@ -47,3 +47,24 @@ def test_malformed_cu_seqlens_is_reported_not_followed(cu):
     good.fwd()
     torch.cuda.synchronize()
     assert good.device_status() == 0
+
+
+@pytest.mark.parametrize("io,D", [("bf16", 128), ("fp32", 64)])
+@pytest.mark.parametrize("cu", [[0, 70, 60, 200], [5, 70, 130, 200], [0, 70, 130, 190]], ids=["decreasing", "first_not_zero", "last_not_T"])
+def test_malformed_cu_seqlens_through_the_backward(cu, io, D):
+    """The code is in the status word before the backward's first wait, and a long wait gives up for it: whatever each warp
+    decides, the kernels end, the code stays, and the next call is a good one."""
+    inp = draw("bad_cu_bwd", 33, [70, 60, 70], 2, D, D, io, hyper=OsdnHyper(eta=0.3, apf_mode=1), with_dout=True)
+    b = binding.DeviceBundle(inp, DEV)
+    b.cu.copy_(torch.tensor(cu, dtype=torch.int32))
+    for _ in range(2):
+        b.fwd(save=True)
+        b.bwd(residuals_valid=True)
+        torch.cuda.synchronize()
+        assert b.device_status() == 120
+    b.cu.copy_(inp.cu_seqlens)
+    b.fwd(save=True)
+    b.bwd(residuals_valid=True)
+    torch.cuda.synchronize()
+    assert b.device_status() == 0
+    assert all(bool(torch.isfinite(x.float()).all()) for x in (b.out, b.dq, b.dk, b.dv, b.dbeta, b.dgate))

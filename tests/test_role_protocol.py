@@ -1,0 +1,29 @@
+"""What the warp roles of the tensor-core kernels owe one another, read from the source: a missing wait or an unbounded one
+shows in no result, and a test that ran into it would hang the device."""
+import os
+import re
+
+import pytest
+
+import paper_2605_13473_b200
+
+CSRC = os.path.join(os.path.dirname(paper_2605_13473_b200.__file__), "csrc")
+
+
+def role(name):
+    """The body of a device function of the tensor-core file, without its comments."""
+    with open(os.path.join(CSRC, "osdn_tc.cu")) as f:
+        text = f.read()
+    body = re.search(r"\n__device__ __forceinline__ \w+ " + name + r"\(.*?\n\{\n(.*?)\n\}\n", text, re.S).group(1)
+    return re.sub(r"//[^\n]*", "", body)
+
+
+@pytest.mark.parametrize("name", ["chain_fwd_role", "chain_bwd_role", "chunk_bwd_role"])
+def test_roles_meet_at_bounded_waits_only(name):
+    """A warp whose wait runs out leaves its loop by itself.  Between the barrier that starts the roles and the one behind
+    them the others must not meet it at a hardware barrier, which has no limit."""
+    parts = re.split(r"__syncthreads(?:_\w+)?\(", role(name))
+    roles = max(parts, key=len)
+    assert roles.count("mbar_wait(") >= 5 and roles.count("break;") >= 5
+    assert not re.findall(r"named_sync\w*\(|\bbar\.|barrier\.", roles)
+    assert all("mbar_wait(" not in p for p in parts if p is not roles)
