@@ -2024,7 +2024,8 @@ __device__ __forceinline__ void chunk_bwd_role(const CUtensorMap& tmQ, const CUt
                 const float2 g0 = *reinterpret_cast<const float2*>(sGam + j0), g1 = *reinterpret_cast<const float2*>(sGam + j0 + 8);
                 gj[0] = g0.x; gj[1] = g0.y; gj[2] = g1.x; gj[3] = g1.y;
             }
-            if (!mbar_wait(&bar_mma[2], ph, a.status, ERR_MMA2)) break;
+            // (the products have waited for q, k and ktil, but only a wait of its own makes a copy visible to a thread)
+            if (!mbar_wait(&bar_tok, ph, a.status, ERR_TMA) || !mbar_wait(&bar_mma[2], ph, a.status, ERR_MMA2)) break;
             tc_fence_after();
 #pragma unroll
             for (int hf = 0; hf < 2; ++hf) {

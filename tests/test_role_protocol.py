@@ -27,3 +27,14 @@ def test_roles_meet_at_bounded_waits_only(name):
     assert roles.count("mbar_wait(") >= 5 and roles.count("break;") >= 5
     assert not re.findall(r"named_sync\w*\(|\bbar\.|barrier\.", roles)
     assert all("mbar_wait(" not in p for p in parts if p is not roles)
+
+
+def test_epilogue_waits_for_the_copies_that_it_reads():
+    """Chunk-local backward, full tiles: each operand that the epilogue warps read from shared memory has been waited for by
+    them on the barrier that its copy completes on."""
+    epilogue = role("chunk_bwd_role").split("const uint32_t offT", 1)[1]
+    epilogue = re.sub(r"\n {12}if \(len < CH\) \{.*?\n {12}\}", "", epilogue, flags=re.S)
+    for bar, regions in {"bar_tok": ("R_Q", "R_K", "R_KT"), "bar_v": ("R_V",), "bar_s": ("R_S", "R_DS")}.items():
+        for region in regions:
+            at = re.search(r"s0 \+ " + region + r" \+", epilogue).start()
+            assert "mbar_wait(&" + bar + "," in epilogue[:at], (region, bar)
