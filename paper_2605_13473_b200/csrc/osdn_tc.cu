@@ -257,7 +257,7 @@ constexpr size_t CL_SMEM = 32768 + CH * LCF * 4 + 1024;
 
 // Small per-group state of the chunk-local forward that lives in shared memory.
 struct ClGroupShared {
-    uint64_t bar_tma, bar_mma1, bar_mma2;
+    uint64_t bar_tma, bar_mma1, bar_mma2, bar_drain;
     int ticket;
     int pad;
     float sG[CH];
@@ -266,8 +266,9 @@ struct ClGroupShared {
 
 // One (chunk, head) tile by a group of CL_THREADS threads (local index `tid`) that synchronise on hardware
 // barrier `bar_id`; `sm`: CL_SMEM - 1024 bytes, 1024-byte aligned; `tb`: 128 tensor-memory columns;
-// `ph`: parity of the group's three barriers (they complete once per tile).
-__device__ __forceinline__ void chunk_fwd_tile(const CUtensorMap& tmK, const CUtensorMap& tmQ, const CUtensorMap& tmKt,
+// `ph`: parity of the group's three barriers (they complete once per tile).  False, for all threads alike, where a wait ran
+// out: the tile's copies and products have ended then, and the group takes no more (its barriers are out of step).
+__device__ __forceinline__ bool chunk_fwd_tile(const CUtensorMap& tmK, const CUtensorMap& tmQ, const CUtensorMap& tmKt,
                                                const TcChunkArgs& a, int c, int h, uint8_t* sm, ClGroupShared& gs,
                                                uint32_t tb, int tid, int bar_id, uint32_t ph, int* publish)
 {
@@ -286,7 +287,7 @@ __device__ __forceinline__ void chunk_fwd_tile(const CUtensorMap& tmK, const CUt
     uint8_t* sTb = sKQ + BOX;          // K-major [i][j]
     const int H = a.H;
     const int len = a.tab.chunk_len(c);
-    if (len == 0) return;
+    if (len == 0) return true;
     const int tok0 = a.tab.chunk_tok0(c);
     const size_t tile = (size_t)c * H + h;
     const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
@@ -500,7 +501,16 @@ __device__ __forceinline__ void chunk_fwd_tile(const CUtensorMap& tmK, const CUt
             }
     }
     tc_fence_before();
-    sync();
+    ok = named_sync_and(bar_id, CL_THREADS, ok);
+    if (!ok) {
+        mbar_drain(&bar_tma, ph);
+        if (warp == 0) {
+            mma_commit(&gs.bar_drain, lead);
+            mbar_drain(&gs.bar_drain, 0);
+        }
+        sync();
+    }
+    return ok;
 }
 
 // Stand-alone launch: one tile per CTA, four CTAs per SM.
@@ -518,6 +528,7 @@ tc_chunk_fwd_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
         mbar_init(&gs.bar_tma, 1);
         mbar_init(&gs.bar_mma1, 1);
         mbar_init(&gs.bar_mma2, 1);
+        mbar_init(&gs.bar_drain, 1);
         fence_mbar_init();
     }
     if ((tid >> 5) == 1) tmem_alloc(&tmem_base, 128);
@@ -598,7 +609,7 @@ __device__ __forceinline__ void chain_fwd_role(const CUtensorMap& tmV, const CUt
     uint8_t* sDU1 = sS + 32768;                 // dU^T, K-major [v][i]
     uint8_t* sDU2 = sDU1 + 16384;               // (rho dU)^T
     __shared__ uint64_t bar_full[2], bar_empty[2], bar_s_ready, bar_du_done, bar_du_ready, bar_s_done;
-    __shared__ uint64_t bar_o_done[2], bar_o_free[2];
+    __shared__ uint64_t bar_o_done[2], bar_o_free[2], bar_drain;
     __shared__ float sRho[2][CH], sGC[2];              // slot = chunk % 2
 
     const int H = a.H;
@@ -618,7 +629,7 @@ __device__ __forceinline__ void chain_fwd_role(const CUtensorMap& tmV, const CUt
     }
     uint64_t* const all_bars[] = {&bar_full[0], &bar_full[1], &bar_empty[0], &bar_empty[1], &bar_s_ready, &bar_du_done,
                                   &bar_du_ready, &bar_s_done, &bar_o_done[0], &bar_o_done[1], &bar_o_free[0],
-                                  &bar_o_free[1]};
+                                  &bar_o_free[1], &bar_drain};
     const int nchunks = c1 - c0;
     auto chunk_tok0 = [&](int n) { return seq_t0 + n * CH; };
     auto chunk_len = [&](int n) { return min(CH, seq_len - n * CH); };
@@ -636,6 +647,7 @@ __device__ __forceinline__ void chain_fwd_role(const CUtensorMap& tmV, const CUt
         mbar_init(&bar_o_done[1], 1);
         mbar_init(&bar_o_free[0], CFW_OUT_WARPS);
         mbar_init(&bar_o_free[1], CFW_OUT_WARPS);
+        mbar_init(&bar_drain, 1);
         fence_mbar_init();
     }
     tc_fence_before();
@@ -657,6 +669,7 @@ __device__ __forceinline__ void chain_fwd_role(const CUtensorMap& tmV, const CUt
         };
         float ga, gb;
         load_gates(0, ga, gb);
+        int asked = 0;   // chunks whose copies have been asked for
         for (int n = 0; n < nchunks && ok; ++n) {
             const int st = n & 1, gs = n & 1;
             const int tok0 = chunk_tok0(n);
@@ -695,7 +708,9 @@ __device__ __forceinline__ void chain_fwd_role(const CUtensorMap& tmV, const CUt
             if (lane == 0) mbar_arrive(&bar_full[st]);
             ga = ga_next;
             gb = gb_next;
+            asked = n + 1;
         }
+        for (int n = max(0, asked - 2); n < asked; ++n) mbar_drain(&bar_full[n & 1], (n >> 1) & 1);
     } else if (warp == CFW_MMA_WARP) {
         // ------------------------------------------------------------------ tensor-core issuer
         bool ok = true;
@@ -783,6 +798,8 @@ __device__ __forceinline__ void chain_fwd_role(const CUtensorMap& tmV, const CUt
                 ut_issued = true;
             }
         }
+        mma_commit(&bar_drain, lead);
+        mbar_drain(&bar_drain, 0);
         if (lane == 0) bulk_wait_all();
     } else if (warp >= CFW_OUT_WARP0) {
         // ------------------------------------------------------------------ output warps
@@ -953,6 +970,7 @@ __device__ __forceinline__ void chain_fwd_role(const CUtensorMap& tmV, const CUt
             __syncwarp();
             if (lane == 0) mbar_arrive(&bar_du_ready);
         }
+        tmem_st_wait();
         if (ok) ok = mbar_wait(&bar_s_done, (nchunks - 1) & 1, a.status, ERR_CHAIN_MMA2);
         tc_fence_after();
         if (ok && fin) {
@@ -1039,6 +1057,7 @@ __device__ __forceinline__ void chunk_fwd_workers(const CUtensorMap& tmK, const 
         mbar_init(&gs.bar_tma, 1);
         mbar_init(&gs.bar_mma1, 1);
         mbar_init(&gs.bar_mma2, 1);
+        mbar_init(&gs.bar_drain, 1);
         fence_mbar_init();
     }
     gsync();
@@ -1071,7 +1090,10 @@ __device__ __forceinline__ void chunk_fwd_workers(const CUtensorMap& tmK, const 
             h = chain - s * cl.H;
             c = s * sc.nchunks + n;
         }
-        chunk_fwd_tile(tmK, tmQ, tmKt, cl, c, h, sm + g * FWD_GROUP_SMEM, gs, tb + g * 128, ltid, 1 + g, ph, publish);
+        if (!chunk_fwd_tile(tmK, tmQ, tmKt, cl, c, h, sm + g * FWD_GROUP_SMEM, gs, tb + g * 128, ltid, 1 + g, ph, publish)) {
+            publish = nullptr;   // the chains that need the tile, and tickets drawn and not worked off, give up in their turn
+            break;
+        }
         publish = cl.ready + (size_t)c * cl.H + h;
         ph ^= 1;
     }
@@ -1087,6 +1109,7 @@ __device__ __forceinline__ void chunk_fwd_workers(const CUtensorMap& tmK, const 
         mbar_inval(&gs.bar_tma);
         mbar_inval(&gs.bar_mma1);
         mbar_inval(&gs.bar_mma2);
+        mbar_inval(&gs.bar_drain);
     }
     __syncthreads();
 }
@@ -1177,7 +1200,7 @@ __device__ __forceinline__ void chain_bwd_role(const CUtensorMap& tmDO, const CU
     uint8_t* sStage = sm;
     uint8_t* sdS = sm + 2 * BSTAGE_BYTES;       // dS as bf16, K-major, 2 k-halves x [128 x 128 B]
     uint8_t* sddU = sdS + 32768;                // ddU^T, K-major [v][i]
-    __shared__ uint64_t bar_full[2], bar_empty[2], bar_s_ready, bar_a_done, bar_a_ready, bar_s_done;
+    __shared__ uint64_t bar_full[2], bar_empty[2], bar_s_ready, bar_a_done, bar_a_ready, bar_s_done, bar_drain;
     __shared__ float sRho[2][CH], sGC[2];
 
     const int H = a.H;
@@ -1211,6 +1234,7 @@ __device__ __forceinline__ void chain_bwd_role(const CUtensorMap& tmDO, const CU
         mbar_init(&bar_a_done, 1);
         mbar_init(&bar_a_ready, CBK_EPI_WARPS);
         mbar_init(&bar_s_done, 1);
+        mbar_init(&bar_drain, 1);
         fence_mbar_init();
     }
     tc_fence_before();
@@ -1228,6 +1252,7 @@ __device__ __forceinline__ void chain_bwd_role(const CUtensorMap& tmDO, const CU
         };
         float ga, gb;
         load_gates(0, ga, gb);
+        int asked = 0;   // chunks whose copies have been asked for
         for (int n = 0; n < nchunks && ok; ++n) {
             const int st = n & 1;
             float ga_next = 0.f, gb_next = 0.f;
@@ -1259,7 +1284,9 @@ __device__ __forceinline__ void chain_bwd_role(const CUtensorMap& tmDO, const CU
             }
             ga = ga_next;
             gb = gb_next;
+            asked = n + 1;
         }
+        for (int n = max(0, asked - 2); n < asked; ++n) mbar_drain(&bar_full[n & 1], (n >> 1) & 1);
     } else if (warp == CBK_MMA_WARP) {
         // ------------------------------------------------------------------ tensor-core issuer
         bool ok = true;
@@ -1347,6 +1374,8 @@ __device__ __forceinline__ void chain_bwd_role(const CUtensorMap& tmDO, const CU
             }
             __syncwarp();
         }
+        mma_commit(&bar_drain, lead);
+        mbar_drain(&bar_drain, 0);
         if (lane == 0) {
             bulk_wait_all();
             if (ok) tq.push((int)chunk_tile(nchunks - 1), H, nchunks - published);
@@ -1460,6 +1489,7 @@ __device__ __forceinline__ void chain_bwd_role(const CUtensorMap& tmDO, const CU
     if (tid == 0) {   // the barrier words are initialised again for the CTA's next chain
         mbar_inval(&bar_full[0]); mbar_inval(&bar_full[1]); mbar_inval(&bar_empty[0]); mbar_inval(&bar_empty[1]);
         mbar_inval(&bar_s_ready); mbar_inval(&bar_a_done); mbar_inval(&bar_a_ready); mbar_inval(&bar_s_done);
+        mbar_inval(&bar_drain);
     }
     __syncthreads();
     tc_fence_after();
@@ -1523,7 +1553,7 @@ __device__ __forceinline__ void chunk_bwd_role(const CUtensorMap& tmQ, const CUt
                                                const CUtensorMap& tmDK, const CUtensorMap& tmDV, const TcChunkBwdArgs& a,
                                                uint8_t* sm, uint32_t tb, const TileQueue& tq)
 {
-    __shared__ uint64_t bar_vec[2], bar_c, bar_s, bar_tok, bar_v, bar_zero, bar_rows, bar_mma[4], bar_ea, bar_ed, bar_ef;
+    __shared__ uint64_t bar_vec[2], bar_c, bar_s, bar_tok, bar_v, bar_zero, bar_rows, bar_mma[4], bar_ea, bar_ed, bar_ef, bar_drain;
     __shared__ int sInfo[2][4];                            // tile (-1: no more), first token, length, head
     __shared__ unsigned sSkipW[2][2];
     __shared__ __align__(16) float sVec[2][4][CH];         // G_i, gamma_i = exp(G_i), rho_i = exp(G_C - G_i), beta_i
@@ -1534,7 +1564,7 @@ __device__ __forceinline__ void chunk_bwd_role(const CUtensorMap& tmQ, const CUt
     const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
     const bool lead = lane == 0;
     if (tid == 0) {
-        for (uint64_t* b : {&bar_vec[0], &bar_vec[1], &bar_c, &bar_s, &bar_tok, &bar_v, &bar_mma[0], &bar_mma[1], &bar_mma[2], &bar_mma[3]}) mbar_init(b, 1);
+        for (uint64_t* b : {&bar_vec[0], &bar_vec[1], &bar_c, &bar_s, &bar_tok, &bar_v, &bar_mma[0], &bar_mma[1], &bar_mma[2], &bar_mma[3], &bar_drain}) mbar_init(b, 1);
         for (uint64_t* b : {&bar_zero, &bar_rows, &bar_ea, &bar_ed, &bar_ef}) mbar_init(b, CBW_WARPS);
         fence_mbar_init();
     }
@@ -1586,17 +1616,22 @@ __device__ __forceinline__ void chunk_bwd_role(const CUtensorMap& tmQ, const CUt
             for (int hf = 0; hf < 2; ++hf) tma_store_2d(&m, x.h * KD + hf * 64, x.tok0, sm + region + hf * BOX);
         };
         auto load_t_ds = [&](const Tile& x) {
-            mbar_expect_tx(&bar_c, 8192 + 3 * 16384);
+            mbar_announce_tx(&bar_c, 8192);
             bulk_load(sm + R_T, a.Tm + (size_t)x.t * 8192, 8192, &bar_c);
-            mbar_expect_tx(&bar_s, 65536);
+            mbar_announce_tx(&bar_s, 32768);
             bulk_load(sm + R_DS, a.dSn + (size_t)x.t * 32768, 32768, &bar_s);
         };
         auto load_u_s = [&](const Tile& x) {
+            mbar_announce_tx(&bar_c, 32768);
+            mbar_expect_tx(&bar_s, 32768);
             bulk_load(sm + R_DDU, a.ddUT + (size_t)x.t * 16384, 16384, &bar_c);
             bulk_load(sm + R_DU, a.dUT + (size_t)x.t * 16384, 16384, &bar_c);
             bulk_load(sm + R_S, a.Sn + (size_t)x.t * 32768, 32768, &bar_s);
         };
-        auto load_do = [&](const Tile& x) { load_tok(tmDO, R_DO, x, &bar_c); };
+        auto load_do = [&](const Tile& x) {
+            mbar_expect_tx(&bar_c, 2 * BOX);
+            load_tok(tmDO, R_DO, x, &bar_c);
+        };
         auto load_kkq = [&](const Tile& x) {
             mbar_expect_tx(&bar_tok, 6 * BOX);
             load_tok(tmK, R_K, x, &bar_tok);
@@ -1695,6 +1730,9 @@ __device__ __forceinline__ void chunk_bwd_role(const CUtensorMap& tmQ, const CUt
                 }
         };
 
+        // copies asked for: those of the tiles before `newest`, and of this one T and dS (1), ddU, dU and S (2), dO (3),
+        // k, ktil and q (4), v (5)
+        int newest = -1, asked = 0;
         Tile cur{-1, 0, 0, 0};
         unsigned ticket = __shfl_sync(0xffffffffu, draw(), 0), after = draw();
         if (ticket < (unsigned)total) {
@@ -1711,6 +1749,8 @@ __device__ __forceinline__ void chunk_bwd_role(const CUtensorMap& tmQ, const CUt
                 load_v(cur);
             }
             __syncwarp();
+            newest = 0;
+            asked = 5;
             sc = fetch(cur);
         }
         publish(cur, sc, 0);
@@ -1741,6 +1781,10 @@ __device__ __forceinline__ void chunk_bwd_role(const CUtensorMap& tmQ, const CUt
                 if (known) load_t_ds(next);
             }
             __syncwarp();
+            if (known) {
+                newest = (int)it + 1;
+                asked = 1;
+            }
             if (!mbar_wait(&bar_mma[2], ph, a.status, ERR_MMA2)) break;
             if (lane == 0) {
                 if (known) load_u_s(next);   // S, dU and the dVb image (in the space of ddU) are dead
@@ -1750,6 +1794,7 @@ __device__ __forceinline__ void chunk_bwd_role(const CUtensorMap& tmQ, const CUt
                 }
             }
             __syncwarp();
+            if (known) asked = full ? 3 : 2;
             if (!mbar_wait(&bar_ef, ph, a.status, ERR_MMA2)) break;
             if (lane == 0) {
                 if (full) {
@@ -1763,6 +1808,7 @@ __device__ __forceinline__ void chunk_bwd_role(const CUtensorMap& tmQ, const CUt
                 }
             }
             __syncwarp();
+            if (known) asked = 4;
             finish_sums(cur, (int)ph);
             if (lane == 0 && full) bulk_wait_read();   // v lands where dq was staged, the next M2 images where dk was
             __syncwarp();
@@ -1780,11 +1826,26 @@ __device__ __forceinline__ void chunk_bwd_role(const CUtensorMap& tmQ, const CUt
                     load_v(next);
                 }
                 __syncwarp();
+                newest = (int)it + 1;
                 sc = fetch(next);
                 publish(next, sc, (int)(ph ^ 1u));
             }
             __syncwarp();
+            if (newest == (int)it + 1) asked = 5;
             cur = next;
+        }
+        // Whatever ended the loop, the copies asked for land before the memory is given up.  (A phase that was only announced
+        // in part gets its arrival here.)
+        if (newest >= 0) {
+            if (lane == 0) {
+                if (asked < 2) mbar_arrive(&bar_s);
+                if (asked < 3) mbar_arrive(&bar_c);
+            }
+            mbar_drain(&bar_c, newest & 1);
+            mbar_drain(&bar_s, newest & 1);
+            const int tok = asked < 4 ? newest - 1 : newest, vv = asked < 5 ? newest - 1 : newest;
+            if (tok >= 0) mbar_drain(&bar_tok, tok & 1);
+            if (vv >= 0) mbar_drain(&bar_v, vv & 1);
         }
         if (lane == 0) bulk_wait_all();
         __syncwarp();
@@ -1868,6 +1929,8 @@ __device__ __forceinline__ void chunk_bwd_role(const CUtensorMap& tmQ, const CUt
             }
             __syncwarp();
         }
+        mma_commit(&bar_drain, lead);
+        mbar_drain(&bar_drain, 0);
     } else {
         // ------------------------------------------------------------------ epilogue warps
         const int quad = warp & 3, colq = warp >> 2;      // lane quadrant (32 features or 16 rows), group of 16 columns

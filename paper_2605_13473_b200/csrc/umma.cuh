@@ -49,6 +49,12 @@ __device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes)
                  : "memory");
 }
 
+// The phase waits for these bytes too, without an arrival (which a later mbar_expect_tx or mbar_arrive makes).
+__device__ __forceinline__ void mbar_announce_tx(uint64_t* bar, uint32_t bytes)
+{
+    asm volatile("mbarrier.expect_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
+}
+
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar)
 {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
@@ -89,6 +95,10 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int* s
     }
     return __all_sync(0xffffffffu, done);
 }
+
+// The wait of a role that leaves for copies and products that are on their way: whatever the status word says (they land in
+// memory that is used again, or given back), and bounded all the same.
+__device__ __forceinline__ void mbar_drain(uint64_t* bar, uint32_t parity) { mbar_wait(bar, parity, nullptr, 0); }
 
 // ---------------------------------------------------------------------------------------------
 // proxies and fences
@@ -181,6 +191,16 @@ __device__ __forceinline__ void st_release_gpu(int* p, int v)
 __device__ __forceinline__ void named_sync(int id, int nthreads)
 {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
+}
+// ... that also ANDs a predicate over the participating threads.
+__device__ __forceinline__ bool named_sync_and(int id, int nthreads, bool pred)
+{
+    uint32_t out;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\tsetp.ne.b32 q, %3, 0;\n\t"
+        "barrier.cta.red.and.pred p, %1, %2, q;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(out) : "r"(id), "r"(nthreads), "r"((int)pred) : "memory");
+    return out != 0;
 }
 
 // One full warp allocates `ncols` (power of two >= 32) columns; the base address lands in *dst_smem.

@@ -38,3 +38,15 @@ def test_epilogue_waits_for_the_copies_that_it_reads():
         for region in regions:
             at = re.search(r"s0 \+ " + region + r" \+", epilogue).start()
             assert "mbar_wait(&" + bar + "," in epilogue[:at], (region, bar)
+
+
+@pytest.mark.parametrize("name", ["chunk_fwd_tile", "chain_fwd_role", "chain_bwd_role", "chunk_bwd_role"])
+def test_roles_leave_no_copy_or_product_behind(name):
+    """However a role ends, the copies that it has asked for have landed and its products are complete (both waits bounded, and
+    deaf to the status word) before the memory they work on is used again or given back."""
+    body = role(name)
+    targets = set(re.findall(r"(?:bulk_load|tma_load_2d|load_tok)\([^;]*&(?:gs\.)?(bar_\w+)", body))
+    assert targets
+    for bar in targets:
+        assert re.search(r"mbar_drain\(&" + bar + r"\b", body), bar
+    assert re.search(r"mma_commit\(&(gs\.)?bar_drain, lead\);\s*mbar_drain\(&(gs\.)?bar_drain, 0\);", body)
