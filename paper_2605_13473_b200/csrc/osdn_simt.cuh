@@ -944,8 +944,8 @@ __global__ void __launch_bounds__(K / 64 * 256) chain_wide_kernel(ChainArgs a)
             d0[x] = ld4(D0 + (size_t)(e / WS) * V + e % WS);
         }
         const bool ok = umma::mbar_wait(&s.full[j & 1], (j >> 1) & 1, a.status, CODE_SIMT_RING);
-        if (!__syncthreads_and(ok)) {   // give up, once the copy in flight has landed (or its wait runs out too)
-            if (j + 1 < w.n) umma::mbar_wait(&s.full[(j + 1) & 1], ((j + 1) >> 1) & 1, nullptr, 0);
+        if (!__syncthreads_and(ok)) {   // give up, once the copies in flight have landed
+            for (int x = j; x <= j + 1 && x < w.n; ++x) umma::mbar_drain(&s.full[x & 1], (x >> 1) & 1);
             break;
         }
         // S is complete and G0 has been read

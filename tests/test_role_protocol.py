@@ -10,11 +10,11 @@ import paper_2605_13473_b200
 CSRC = os.path.join(os.path.dirname(paper_2605_13473_b200.__file__), "csrc")
 
 
-def role(name):
-    """The body of a device function of the tensor-core file, without its comments."""
-    with open(os.path.join(CSRC, "osdn_tc.cu")) as f:
+def role(name, file="osdn_tc.cu"):
+    """The body of a function of a kernel file, without its comments."""
+    with open(os.path.join(CSRC, file)) as f:
         text = f.read()
-    body = re.search(r"\n__device__ __forceinline__ \w+ " + name + r"\(.*?\n\{\n(.*?)\n\}\n", text, re.S).group(1)
+    body = re.search(r"\n__(?:device__ __forceinline__|global__) [^\n]*\b" + name + r"\(.*?\n\{\n(.*?)\n\}\n", text, re.S).group(1)
     return re.sub(r"//[^\n]*", "", body)
 
 
@@ -50,3 +50,10 @@ def test_roles_leave_no_copy_or_product_behind(name):
     for bar in targets:
         assert re.search(r"mbar_drain\(&" + bar + r"\b", body), bar
     assert re.search(r"mma_commit\(&(gs\.)?bar_drain, lead\);\s*mbar_drain\(&(gs\.)?bar_drain, 0\);", body)
+
+
+def test_wide_chain_slices_leave_no_copy_behind():
+    """The two stage copies that may be on their way when a wide slice of a CUDA-core chain gives up: the one that was waited
+    for (a status code ends a wait early) and the one behind it."""
+    give_up = role("chain_wide_kernel", "osdn_simt.cuh").split("if (!__syncthreads_and(ok)) {", 1)[1].split("break;", 1)[0]
+    assert re.search(r"for \(int x = j; x <= j \+ 1 && x < w\.n; \+\+x\) umma::mbar_drain\(&s\.full\[x & 1\], \(x >> 1\) & 1\);", give_up)
