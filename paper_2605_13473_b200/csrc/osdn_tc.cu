@@ -1502,9 +1502,10 @@ __device__ __forceinline__ void chain_bwd_role(const CUtensorMap& tmDO, const CU
 //             (reads only what the chain kernels and the caller wrote: issued ahead)
 //   phase B : dA = -strictLower(dVb dU^T) ; dKb^T = -S^T dVb^T ; dq2^T = Ktil^T M1^T ; dktil^T = Q^T M1
 //             (M1 = scale Gamma (.) lower(dP'))
-//   phase C : dktil^T += K^T M2 ; dkr^T = Ktil^T M2'^T      (M2' = dA (.) Gamma, M2 = diag(beta) M2')
-//   final   : dq = scale gamma dQ1 + dq2 ; dv = beta dVb ; dktil += rho dKtr ; dk_read = beta (gamma dKb + dkr) ;
-//             dbeta = <dVb, v> + <gamma dKb + dkr, k> ; dgate from the products of the gradients with their inputs
+//             R0 = K Ktil^T                                   (issued ahead)
+//   phase C : dktil^T += K^T M2 ; dkr^T = Ktil^T M2^T       (M2 = diag(beta) (dA (.) Gamma))
+//   final   : dq = scale gamma dQ1 + dq2 ; dv = beta dVb ; dktil += rho dKtr ; dk_read = beta gamma dKb + dkr ;
+//             dbeta = <dVb, v> + <gamma dKb, k> + sum_j (dA Gamma R0)_ij ; dgate from the products of the gradients with their inputs
 // ---------------------------------------------------------------------------------------------
 struct TcChunkBwdArgs {
     int H, nseq;
@@ -1558,6 +1559,7 @@ __device__ __forceinline__ void chunk_bwd_role(const CUtensorMap& tmQ, const CUt
     __shared__ unsigned sSkipW[2][2];
     __shared__ __align__(16) float sVec[2][4][CH];         // G_i, gamma_i = exp(G_i), rho_i = exp(G_C - G_i), beta_i
     __shared__ float sSum[2][4][2][CH];                    // per quadrant of features: gate and beta terms of every token
+    __shared__ float sRow[2][4][CH];                       // per group of columns: the scores' share of a row's beta gradient
     __shared__ float sRed[2][CBW_WARPS];
 
     const int H = a.H;
@@ -1572,9 +1574,9 @@ __device__ __forceinline__ void chunk_bwd_role(const CUtensorMap& tmQ, const CUt
     __syncthreads();
     tc_fence_after();
 
-    // tensor memory columns (64 each); dkr takes the place of dA
+    // tensor memory columns (64 each); dA takes the place of dP', dkr that of R0
     const uint32_t cDP = tb, cDQ1 = tb + 64, cDKTR = tb + 128, cDVB = tb + 192;
-    const uint32_t cDA = tb + 256, cDKB = tb + 320, cDQ2 = tb + 384, cDKT = tb + 448, cDKR = cDA;
+    const uint32_t cR0 = tb + 256, cDKB = tb + 320, cDQ2 = tb + 384, cDKT = tb + 448, cDA = cDP, cDKR = cR0;
 
     if (warp == CBW_PROD_WARP) {
         // ------------------------------------------------------------------ producer
@@ -1709,7 +1711,8 @@ __device__ __forceinline__ void chunk_bwd_role(const CUtensorMap& tmQ, const CUt
             for (int u = 0; u < 2; ++u) {
                 const int j = lane + 32 * u;
                 s[u] = (sSum[buf][0][0][j] + sSum[buf][1][0][j]) + (sSum[buf][2][0][j] + sSum[buf][3][0][j]);
-                b[u] = (sSum[buf][0][1][j] + sSum[buf][1][1][j]) + (sSum[buf][2][1][j] + sSum[buf][3][1][j]);
+                b[u] = (sSum[buf][0][1][j] + sSum[buf][1][1][j]) + (sSum[buf][2][1][j] + sSum[buf][3][1][j]) +
+                       ((sRow[buf][0][j] + sRow[buf][1][j]) + (sRow[buf][2][j] + sRow[buf][3][j]));
             }
             float tot = lane < CBW_WARPS ? sRed[buf][lane] : 0.f;
 #pragma unroll
@@ -1886,7 +1889,12 @@ __device__ __forceinline__ void chunk_bwd_role(const CUtensorMap& tmQ, const CUt
                            make_idesc(128, 64, IDESC_A_MN | IDESC_B_MN), k > 0, lead);
             }
             __syncwarp();
-            if (!mbar_wait(&bar_tok, ph, a.status, ERR_TMA) || !mbar_wait(&bar_ea, ph, a.status, ERR_MMA1)) break;
+            if (!mbar_wait(&bar_tok, ph, a.status, ERR_TMA)) break;
+            for (int k = 0; k < 8; ++k)   // R0[i][j] = sum_c K[i][c] Ktil[j][c]                           (M = 64)
+                mma_ss(cR0, desc_advance(desc_kmajor(sm + R_K + (k >> 2) * BOX), 32 * (k & 3)),
+                       desc_advance(desc_kmajor(sm + R_KT + (k >> 2) * BOX), 32 * (k & 3)), make_idesc(64, 64), k > 0, lead);
+            __syncwarp();
+            if (!mbar_wait(&bar_ea, ph, a.status, ERR_MMA1)) break;
             tc_fence_after();
             {   // phase B
                 const uint64_t dbv = desc_mnmajor(sm + R_DVB, 0);
@@ -1917,9 +1925,9 @@ __device__ __forceinline__ void chunk_bwd_role(const CUtensorMap& tmQ, const CUt
             __syncwarp();
             if (!mbar_wait(&bar_ed, ph, a.status, ERR_MMA2)) break;
             tc_fence_after();
-            {   // phase C: dktil^T += K^T M2 ; dkr^T[k][i] = sum_j Ktil[j][k] M2'[i][j]
+            {   // phase C: dktil^T += K^T M2 ; dkr^T[k][i] = sum_j Ktil[j][k] M2[i][j]
                 const uint64_t da0 = desc_mnmajor(sm + R_K, BOX), da1 = desc_mnmajor(sm + R_KT, BOX);
-                const uint64_t dbm = desc_mnmajor(sm + R_M2, 0), dbk = desc_kmajor(sm + R_M2 + 8192);
+                const uint64_t dbm = desc_mnmajor(sm + R_M2, 0), dbk = desc_kmajor(sm + R_M2);
                 for (int k = 0; k < 4; ++k)
                     mma_ss(cDKT, desc_advance(da0, 2048 * k), desc_advance(dbm, 2048 * k),
                            make_idesc(128, 64, IDESC_A_MN | IDESC_B_MN), 1, lead);
@@ -2051,37 +2059,45 @@ __device__ __forceinline__ void chunk_bwd_role(const CUtensorMap& tmQ, const CUt
                 part = (lr >> 1) == (lane & 3) ? ((lr & 1) ? c[1] : c[0]) : 0.f;
             }
 
-            // ---- dA = -strictLower -> M2 = beta_i dA Gamma, M2' = dA Gamma
+            // ---- dA = -strictLower -> M2 = beta_i dA Gamma
+            float rw[2] = {};   // rows' sums of dA Gamma R0, from the accumulators (as <dkr, k>, through dkr's operand, they would be rounded to bf16)
             if (!mbar_wait(&bar_mma[1], ph, a.status, ERR_MMA2)) break;
             tc_fence_after();
             {
-                uint32_t r[8];
+                uint32_t r[8], r0[8];
                 tmem_ld_frag16(cDA + lane_addr + colq * 16, r);
+                tmem_ld_frag16(cR0 + lane_addr + colq * 16, r0);
                 const float bi[2] = {sBeta[i0], sBeta[i0 + 8]};
 #pragma unroll
                 for (int hf = 0; hf < 2; ++hf)
                     stmatrix_x4_trans(s0 + ST_DV + (offT ^ (32u * hf)), wv[hf][0], wv[hf][1], wv[hf][2], wv[hf][3]);
                 tmem_ld_wait();
-                uint32_t m[4], mp[4];
+                uint32_t m[4];
 #pragma unroll
                 for (int x = 0; x < 4; ++x) {   // x = 2 octet + row half
                     const int o = x >> 1, rh = x & 1;
                     float u[2];
 #pragma unroll
-                    for (int e = 0; e < 2; ++e)
+                    for (int e = 0; e < 2; ++e) {
                         u[e] = j0 + 8 * o + e < i0 + 8 * rh ? -__uint_as_float(r[2 * x + e]) * gam[2 * x + e] : 0.f;
-                    mp[x] = pack_bf16(u[0], u[1]);
+                        rw[rh] = fmaf(u[e], __uint_as_float(r0[2 * x + e]), rw[rh]);
+                    }
                     m[x] = pack_bf16(bi[rh] * u[0], bi[rh] * u[1]);
                 }
                 stmatrix_x4(s0 + R_M2 + offI, m[0], m[2], m[1], m[3]);
-                stmatrix_x4(s0 + R_M2 + 8192 + offI, mp[0], mp[2], mp[1], mp[3]);
             }
             fence_proxy_async();
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(&bar_ed);
 
-            // ---- while phase C runs: dq = scale gamma dQ1 + dq2, staged over v
+            // ---- while phase C runs: the row sums' four lanes together; dq = scale gamma dQ1 + dq2, staged over v
+            {
+                const bool up = lane & 1;
+                float y = (up ? rw[1] : rw[0]) + __shfl_xor_sync(0xffffffffu, up ? rw[0] : rw[1], 1);
+                y += __shfl_xor_sync(0xffffffffu, y, 2);
+                if (!(lane & 2)) sRow[ph][colq][i0 + (up ? 8 : 0)] = y;
+            }
             float gj[4];
             {
                 const float2 g0 = *reinterpret_cast<const float2*>(sGam + j0), g1 = *reinterpret_cast<const float2*>(sGam + j0 + 8);
@@ -2147,8 +2163,8 @@ __device__ __forceinline__ void chunk_bwd_role(const CUtensorMap& tmQ, const CUt
                             const float kv = e ? bf16_hi(kw) : bf16_lo(kw), ktv = e ? bf16_hi(tw) : bf16_lo(tw);
                             const float dktr = rj[j] * __uint_as_float(rt[x]);
                             dkt[x] = dktr + __uint_as_float(rd[x]);
-                            const float u = fmaf(gj[j], __uint_as_float(rb[x]), __uint_as_float(rk[x]));   // dk_read / beta
-                            dkr[x] = bj[j] * u;
+                            const float u = gj[j] * __uint_as_float(rb[x]);
+                            dkr[x] = fmaf(bj[j], u, __uint_as_float(rk[x]));
                             gv[j] += dkr[x] * kv - dkt[x] * ktv;
                             bv[j] = fmaf(u, kv, bv[j]);
                             rsum = fmaf(dktr, ktv, rsum);

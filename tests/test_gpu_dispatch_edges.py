@@ -268,3 +268,18 @@ def test_decode_on_both_sides_of_its_dispatch(B, H, L, io, K, V, apf):
     assert parity.err(S.cpu().numpy(), ref["final_state"]) <= 1e-4
     assert parity.err(d.cpu().numpy(), ref["precond_out"]) <= 1e-4
     assert parity.err(out.float().cpu().numpy(), ref["out"]) <= parity.TOL[io]
+
+
+def test_beta_gradient_takes_the_scores_in_fp32():
+    """One chunk whose operands are small integers, exact in bf16, and whose score gradients (up to eleven bits) are not: keys
+    one-hot and shared by two tokens each, beta 1/2, no gate, d = 1.  Sums of 128 integers are exact in fp32, so dbeta is."""
+    inp = draw("exact_beta", 7990, [64], 2, 128, 128, "bf16", dense_B=1, hyper=OsdnHyper(eta=0.0, apf_mode=0, scale=1.0), with_dout=True)
+    gen = torch.Generator().manual_seed(7991)
+    inp.q = inp.k = torch.nn.functional.one_hot(torch.arange(64) // 2, 128).float()[:, None].expand(64, 2, 128).contiguous()
+    inp.v, inp.dout = (torch.randint(-15, 16, (64, 2, 128), generator=gen).float() for _ in range(2))
+    inp.beta = torch.full((64, 2), 0.5)
+    inp.gate = torch.zeros(64, 2)
+    got = run_inputs_bwd(inp)
+    ref = oracle.bwd_inputs(inp)
+    assert float(np.abs(ref["dbeta"][1::2]).max()) > 256.0
+    assert parity.err(got["dbeta"], ref["dbeta"]) <= 1e-6
