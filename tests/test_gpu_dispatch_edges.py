@@ -206,48 +206,67 @@ def test_backward_tiles_at_their_edges(lens, kind):
         assert not torch.isnan(x.float()).any() and torch.equal(x, y)
 
 
-@pytest.mark.parametrize("io,K,cg,lens", [("bf16", 128, 0, [130, 130]), ("bf16", 128, 0, [70, 0, 200]), ("fp32", 64, 0, [130, 130]), ("fp32", 64, 1, [130])])
+def _follows(call, spoil, outputs):
+    """What `call` writes to `outputs` with its kernels held apart (the library's stage events stand between them), against one
+    call right behind `spoil`, which leaves other valid results everywhere, and one replayed from a graph behind it."""
+    spoil()
+    binding.stage_timing_enable(True)
+    call()
+    torch.cuda.synchronize()
+    binding.stage_timing_enable(False)
+    want = [x.clone() for x in outputs]
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        call()
+    for run in (call, graph.replay) * 2:
+        spoil()
+        torch.cuda.synchronize()
+        assert not any(torch.equal(x, y) for x, y in zip(want, outputs))
+        run()
+        torch.cuda.synchronize()
+        assert all(torch.equal(x, y) for x, y in zip(want, outputs))
+
+
+@pytest.mark.parametrize("io,K,cg,lens", [("bf16", 128, 0, [130, 130]), ("bf16", 128, 0, [70, 0, 200]), ("bf16", 128, 0, [70] * 60), ("fp32", 64, 0, [130, 130]),
+                                          ("fp32", 64, 0, [70, 0, 200]), ("fp32", 128, 0, [130] * 24), ("fp32", 64, 1, [130])])
 def test_calls_follow_the_work_before_them(io, K, cg, lens):
-    """Every kernel of a call, the first one too, may be launched while the one before it in the stream runs.  Behind kernels
-    that write its inputs and its cotangents, and captured behind a fill: the results of calls that are waited for, bit for bit."""
-    hy = OsdnHyper(eta=0.003, apf_mode=2, channel_gate=cg)
-    inp = draw(f"follow_{io}_{cg}", 7950 + len(lens), lens, 2, K, K, io, dense_B=len(lens) if len(set(lens)) == 1 else 0, hyper=hy,
-               with_dout=True, with_log_ret=True, with_state_cotangents=True)
-    b = binding.DeviceBundle(inp, DEV, need_bwd=True)
-    names = [x for x in ("q", "k", "v", "beta", "gate", "log_ret", "dout") if getattr(b, x) is not None]
+    """Every kernel of a call, the first one too, may be launched while the one before it in the stream runs.  Outputs and
+    workspace hold the results of other inputs when the call is enqueued, behind the kernels that write its own: a kernel that
+    does not wait for the one before it reads them."""
+    hy = OsdnHyper(eta=0.3, apf_mode=2, channel_gate=cg)
+    inp, other = (draw(f"follow_{io}_{cg}", 7950 + x + len(lens), lens, 2, K, K, io, dense_B=len(lens) if len(set(lens)) == 1 else 0, hyper=hy, key_kind="sparse",
+                       with_dout=True, with_log_ret=True, with_state=True, with_state_cotangents=True) for x in (0, 100))
+    b, o = binding.DeviceBundle(inp, DEV), binding.DeviceBundle(other, DEV)
+    names = ("q", "k", "v", "beta", "gate", "log_ret", "init_state", "precond_in", "dout", "dfinal_state", "dprecond_out")
     kept = {x: getattr(b, x).clone() for x in names}
 
-    def call():
+    def run(src):
         for x in names:
-            getattr(b, x).copy_(kept[x])
+            torch.mul(src[x], 1, out=getattr(b, x))
         b.fwd(save=True)
         b.bwd(residuals_valid=True)
 
-    def spoil():
-        for x in names:
-            getattr(b, x).fill_(0.25)
-
-    results = []
-    for wait in (True, False):
-        spoil()
-        torch.cuda.synchronize()
-        call()
-        if wait:
-            torch.cuda.synchronize()
-        call()
-        torch.cuda.synchronize()
-        results.append([x.clone() for x in (b.out, b.final_state, b.precond_out, b.dq, b.dk, b.dv)])
-    graph = torch.cuda.CUDAGraph()
-    with torch.cuda.graph(graph):
-        b.dq.zero_()
-        call()
-    spoil()
-    graph.replay()
-    torch.cuda.synchronize()
+    _follows(lambda: run(kept), lambda: run({x: getattr(o, x) for x in names}),
+             [b.out, b.final_state, b.precond_out, b.dq, b.dk, b.dv, b.dbeta, b.dgate, b.dlog_ret, b.dinit_state, b.dprecond_in])
     assert b.device_status() == 0
-    results.append([b.out, b.final_state, b.precond_out, b.dq, b.dk, b.dv])
-    for other in results[1:]:
-        assert all(torch.equal(x, y) for x, y in zip(results[0], other))
+
+
+@pytest.mark.parametrize("B", [2, 90])
+def test_standalone_update_follows_the_work_before_it(B):
+    """As above, the stand-alone update with its chains one and three to an SM."""
+    inp, other = (draw("follow_update", 7970 + x, [100] * B, 2, 128, 128, "bf16", dense_B=B, hyper=OsdnHyper(eta=0.3, apf_mode=2), key_kind="sparse",
+                       with_log_ret=True, with_state=True) for x in (0, 100))
+    b, o = (binding.DeviceBundle(x, DEV, need_bwd=False) for x in (inp, other))
+    kt, d = torch.empty_like(b.k), torch.empty_like(b.precond_in)
+    names = ("k", "beta", "log_ret", "precond_in")
+    kept = {x: getattr(b, x).clone() for x in names}
+
+    def run(src):
+        for x in names:
+            torch.mul(src[x], 1, out=getattr(b, x))
+        binding.osdn_precond_update(b.params, b.k, b.beta, b.log_ret, b.precond_in, kt, d)
+
+    _follows(lambda: run(kept), lambda: run({x: getattr(o, x) for x in names}), [kt, d])
 
 
 @pytest.mark.parametrize("B,H,L", [(49, 3, 8), (37, 4, 9), (191, 1, 1), (192, 1, 1), (50, 3, 17), (103, 1, 1), (104, 1, 1), (103, 1, 9), (52, 2, 9)])
