@@ -242,29 +242,29 @@ constexpr int FEW_RW = 4, FEW_WARPS = 4, MANY_WARPS = 8;
 template <typename T, int K, int V, bool VEC, bool MULTI>
 __global__ void __cluster_dims__(V / (FEW_RW * FEW_WARPS), 1, 1) __launch_bounds__(FEW_WARPS * 32) decode_few_kernel(DecArgs a)
 {
-    pdl_release();
     pdl_wait();
     decode_body<T, K, V, VEC, FEW_RW, FEW_WARPS, MULTI>(a);
 }
 template <typename T, int K, int V, bool VEC, bool MULTI>
 __global__ void __launch_bounds__(MANY_WARPS * 32, 2) decode_many_kernel(DecArgs a)
 {
-    pdl_release();
     pdl_wait();
     decode_body<T, K, V, VEC, V / MANY_WARPS, MANY_WARPS, MULTI>(a);
 }
 
 // From about two chains to three SMs on a CTA per chain is the faster one: it has no slices to wait for one another.  Measured
-// in a graph, K = V = 128, slices against a CTA per chain, us: one token 64 chains 2.96 / 3.40, 96 chains 3.35 / 3.42, 112
-// chains 3.92 / 3.68, 144 chains 5.09 / 3.92; 7 tokens 64 chains 7.6 / 9.3, 96 chains 9.6 / 9.4, 128 chains 13.4 / 9.5.  Slices
-// for every call against these rules: 4096 chains 106.5 -> 84.0 us (6.49 TB/s), 1110 chains x 7 tokens fp32 98 -> 52 us, 512
-// chains x 16 tokens 103 -> 52 us.
+// in a graph, K = V = 128, slices against a CTA per chain, us: one token 64 chains 2.65 / 3.02, 96 chains 3.02 / 3.10, 104
+// chains 3.12 / 3.12, 112 chains 3.29 / 3.18, 144 chains 4.62 / 3.40; 7 tokens 64 chains 7.1 / 8.9, 104 chains 9.0 / 9.0, 112
+// chains 12.5 / 9.0.  Slices for every call against these rules (plain launches): 4096 chains 106.5 -> 84.0 us, 1110 chains x 7
+// tokens fp32 98 -> 52 us, 512 chains x 16 tokens 103 -> 52 us.
 constexpr unsigned MANY_CHAINS = 104;
 template <typename T, int K, int V, bool VEC> bool launch_one(unsigned chains, const DecArgs& a, cudaStream_t st)
 {
     constexpr unsigned SLICES = V / (FEW_RW * FEW_WARPS);
     // Programmatic dependents: the launch of a call runs under the kernel before it in the stream, whose results it waits for
-    // before its first access (one sequence, calls back to back: 3.9 -> 3.1 us; 512 sequences 83.5 -> 81.0).
+    // before its first access (one sequence, 8 chains, in a graph 2.28 -> 1.98 us, back to back from the host 4.1 -> 3.1; 4096
+    // chains 83.9 -> 81.2 back to back).  No early release: the next call's CTAs would come in on the SMs that this one leaves
+    // idle, several to an SM (K = V = 128, 104 chains x 16 tokens 16.7 -> 26.3 us, 64 chains, K = V = 64, 9.7 -> 16.5).
     if (chains >= MANY_CHAINS)
         return launch_after(a.L > 1 ? decode_many_kernel<T, K, V, VEC, true> : decode_many_kernel<T, K, V, VEC, false>, chains, MANY_WARPS * 32, 0, st, a);
     return launch_after(a.L > 1 ? decode_few_kernel<T, K, V, VEC, true> : decode_few_kernel<T, K, V, VEC, false>, chains * SLICES, FEW_WARPS * 32, 0, st, a);

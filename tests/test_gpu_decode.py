@@ -221,3 +221,35 @@ def test_calls_follow_the_work_before_them(B):
         graph.replay()
         torch.cuda.synchronize()
         assert all(torch.equal(x, y) for x, y in zip(want, (S, d, out)))
+
+
+@pytest.mark.parametrize("D,B,L", [(64, 64, 16), (128, 104, 16), (128, 128, 7)])
+def test_calls_back_to_back_do_not_crowd(D, B, L):
+    """A call may come in while the one before it runs; it must not come in beside it, several blocks to an SM.  Calls right
+    behind one another take no longer than calls with a fill between them (they took up to 1.5 times as long)."""
+    gen = torch.Generator(device=DEV).manual_seed(6)
+    rnd = lambda *s: torch.randn(*s, generator=gen, device=DEV)
+    p = binding.make_params(B=B, T=L, H=1, K=D, V=D, io_dtype="bf16", hyper=OsdnHyper(eta=0.003, apf_mode=1))
+    q, k, v = (torch.nn.functional.normalize(rnd(B * L, 1, D), dim=-1).bfloat16() for _ in range(3))
+    beta, gate, S, d = torch.sigmoid(rnd(B * L, 1)), -torch.rand(B * L, 1, generator=gen, device=DEV), rnd(B, 1, D, D), torch.ones(B, 1, D, device=DEV)
+    out, other = torch.empty_like(v), torch.empty(1024, device=DEV)
+
+    def time(between):
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            for _ in range(50):
+                binding.osdn_decode_step(p, q, k, v, beta, gate, None, S, d, out)
+                if between:
+                    other.fill_(1.0)
+        ms = []
+        for _ in range(7):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            graph.replay()
+            b.record()
+            b.synchronize()
+            ms.append(a.elapsed_time(b))
+        return sorted(ms)[3]
+
+    binding.osdn_decode_step(p, q, k, v, beta, gate, None, S, d, out)
+    assert time(False) <= 1.05 * time(True)
