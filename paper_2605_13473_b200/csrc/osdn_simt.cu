@@ -8,7 +8,7 @@
 //   chain_fwd       dU = U - W S^T ; S <- gamma_C S + dU^T (rho Ktil)   (state recurrence)
 //   output          O = scale[(gamma Q) S^T + P dU]
 //   pre_bwd, chain_bwd  reverse state chain: ddU and dS (their parts that need no dS first)
-//   chunk_local_bwd all chunk-local gradients (through P, W, U, T, A and the gate prefix)
+//   chunk_local_bwd all chunk-local gradients (through P, the state's advance, the right side of the solve, A and the gate prefix)
 //
 // This file also builds the chunk table of packed batches.
 #include "osdn_simt.cuh"

@@ -713,7 +713,7 @@ template <int K> struct Stage {
 };
 // One group of 16-byte copies by all threads.  Narrow slices take this form: with one bulk copy per row, four warps issue 32
 // each, one after the other, in the middle of a step that is short (4 x 1000 tokens, 4 heads, K = V = 64: a chain 38.9 -> 28.8
-// us, forward and backward 193.7 -> 175.0).
+// us, forward and backward 196 -> 178).
 template <int K, int NT> __device__ __forceinline__ void fetch_group(Stage<K>& g, const ChainArgs& a, size_t tile, bool any)
 {
     if (any) {

@@ -6,7 +6,8 @@
 //   phase1_fwd (CUDA cores)      ktil = d (.) k in bf16, preconditioner at chunk starts
 //   tc_chunk_fwd  per (chunk, head), parallel:
 //        [K;Q] Ktil^T  -> A = strictLower(beta_i Gamma_ij <k_i,ktil_j>),  P' = scale * Lower(Gamma_ij <q_i,ktil_j>)
-//        T = (I + A)^-1 (fp32 forward substitution), Tb = T diag(beta), Tbg = T diag(beta gamma)
+//        T = (I + A)^-1 (blocks of 16 by fp32 substitution, the rest by TF32 block products), Tb = T diag(beta),
+//        Tbg = T diag(beta gamma)
 //        W^T = K^T Tbg^T                               (tensor memory: lane = feature, column = token)
 //   tc_chain_fwd  per chain, sequential over chunks, state S (V x K, fp32) resident in tensor memory:
 //        dU^T = V^T Tb^T - S W^T ;  O1^T = S Q^T
@@ -144,7 +145,9 @@ __device__ __forceinline__ void mma_tf32(float (&c)[4], const uint32_t (&a)[4], 
 //     T_21 = -T_22 (A_21 T_11).
 // The inner products are parked in the upper triangle, so on return only entries with j <= i are meaningful.
 // Called by all threads of the group (at least 128) behind a barrier; ends with a barrier.  Three barriers, where block row
-// by block row took eight; a chain of six block products instead of nine.
+// by block row took eight; a chain of four block products instead of six (that order with three barriers: 8 x 2048 tokens, 8
+// heads, forward 126.3 -> 130.1 us).  Another rounding, not a larger one: errors of the outputs against 64 bits, over those of
+// the other order, 1.0000 with gates and 0.9995 to 1.0005 without (24 seeds each).
 // ---------------------------------------------------------------------------------------------
 constexpr int LCF = CH + 4;   // stride = 4 mod 32 words: conflict-free 16-byte row stores and A fragments
 
@@ -1017,7 +1020,9 @@ tc_chain_fwd_kernel(const __grid_constant__ CUtensorMap tmV, const __grid_consta
 // turn into the state chains, whose loads wait for those flags; the other CTAs keep producing, and a CTA
 // whose chain is finished joins them again.  No worker ever waits, so the chains always make progress.
 // ---------------------------------------------------------------------------------------------
-constexpr float FWD_STEP_OVER_TILE_F = 0.65f;   // cost of a chain step in units of the time one SM needs for a tile
+// Cost of a chain step in units of the time one SM needs for a tile.  Forward, us, at 0.5 / 0.65 / 0.8: 8 x 2048 tokens, 8 heads
+// 130.1 / 126.3 / 132.3; 4 x 4096, 16 heads 232 / 214 / 221; 14 x 4096, 8 heads 378 / 367 / 387; up to 32 chains, and packed rows, alike.
+constexpr float FWD_STEP_OVER_TILE_F = 0.65f;
 struct FwdSched {
     int* tickets;     // zero at launch
     int ntickets;     // number of (chunk, head) tiles
@@ -1040,7 +1045,8 @@ __device__ __forceinline__ void fwd_sched_resolve(FwdSched& sc, const Table& tab
 }
 // Worker groups per CTA: four (1024 threads, 64 registers: the chain role loses about a tenth of its speed)
 // when the chunk-local tiles are the larger part of the work, three (768 threads, 80 registers) when the
-// longest chain is.
+// longest chain is.  Forward, us, with three / four: 2048 tokens, 8 heads, 1 sequence 93.6 / 102, 4 sequences 107 / 116,
+// 8 sequences 130 / 126; 4 x 4096, 16 heads 231 / 214; 131072 tokens in 8 packed sequences 1107 / 1235.
 constexpr uint32_t FWD_GROUP_SMEM = (uint32_t)CL_SMEM - 1024;
 static_assert(4 * FWD_GROUP_SMEM + 4 * sizeof(ClGroupShared) <= CF_SMEM - 1024, "worker groups fit");
 static_assert(3 * CL_THREADS >= CFW_THREADS, "the chain fits into the CTA");
@@ -1534,7 +1540,7 @@ constexpr size_t CBW_SMEM = R_M1 + 8192 + 1024;
 // completed once per tile (vec: one of the two):
 //   vec[2] per-token scalars and the tile's coordinates are in shared memory               producer -> all
 //   c, s, tok, v   copies: ddU T dO dU | S dS | q k ktil | v                               producer -> issuer, epilogue
-//   mma[0..3]      dVb, dP' | dA (and dQ1, dKtr) | dKb, dq2, first half of dktil | phase C  tensor core -> epilogue
+//   mma[0..3]      dVb, dP' | dA (and dQ1, dKtr, R0) | dKb, dq2, first half of dktil | phase C  tensor core -> epilogue
 //   e_a    images of M1 and dVb written                                                    epilogue -> issuer
 //   e_d    images of M2 written, dv staged, <dS, S> formed                                 epilogue -> issuer, producer
 //   e_f    everything of the tile is read; dq, dk staged, partial sums written             epilogue -> issuer, producer
@@ -1547,8 +1553,8 @@ constexpr size_t CBW_SMEM = R_M1 + 8192 + 1024;
 // under this tile's last epilogue.
 // What bounds it: with three dependent phases (five when dL/dT was formed from dW K^T and ddU V^T and carried through
 // T^T . T^T) the tile's copies, 184 KB in and 48 KB out.  Epilogues read the accumulators in the fragment layout of ldmatrix:
-// two packed instructions move what sixteen 2-byte accesses of a lane-per-feature layout did, and a token's sum over
-// the features is three shuffles.
+// two packed instructions move what sixteen 2-byte accesses of a lane-per-feature layout did, and eight sums of a token pair
+// over the warp's features take seven shuffles.
 __device__ __forceinline__ void chunk_bwd_role(const CUtensorMap& tmQ, const CUtensorMap& tmK, const CUtensorMap& tmKt,
                                                const CUtensorMap& tmV, const CUtensorMap& tmDO, const CUtensorMap& tmDQ,
                                                const CUtensorMap& tmDK, const CUtensorMap& tmDV, const TcChunkBwdArgs& a,
@@ -2280,8 +2286,7 @@ template <typename F> bool set_smem(F* kernel, size_t bytes)
 
 }  // namespace
 
-// Merged forward launch: SMs that must be left over to feed the chains, and the cost of one chain step in
-// units of the time one SM needs for a tile of the chunk-local pass (measured: 0.6 to 0.75 are equally good).
+// Merged forward launch: SMs that must be left over to feed the chains.
 constexpr int FWD_MIN_FEEDERS = 32;
 constexpr double FWD_STEP_OVER_TILE = FWD_STEP_OVER_TILE_F;
 
@@ -2339,8 +2344,8 @@ int tc_forward(const osdn_params& p, const Hyper& hy, const WsLayout& L, void* w
     ch.P = reinterpret_cast<uint8_t*>(w + t.P); ch.Sn = reinterpret_cast<uint8_t*>(w + t.Sn);
     ch.dUT = reinterpret_cast<uint8_t*>(w + t.dUT); ch.scale = hy.scale; ch.save = save ? 1 : 0;
     ch.status = status;
-    // One launch for both passes when the batch is dense (equal chunk counts give the tile order the
-    // chains want) and enough SMs are left over to feed the chains.
+    // One launch for both passes when enough SMs are left over to feed the chains.  The order of the tiles is arithmetic in
+    // a dense batch and comes from the chunk table in a packed one.
     const int grid = num_sms(), nchains = S * H;
     const int nchunks = p.nseq > 0 ? 0 : (p.T + CH - 1) / CH;
     if (nchains + FWD_MIN_FEEDERS <= grid) {
